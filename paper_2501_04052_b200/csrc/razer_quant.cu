@@ -1,10 +1,25 @@
-// razer_quant_act: online RaZeR quantization of bf16 activations (Sec. 4.2, Eq. 1-3, 6-7).
+// Quantizers: razer_quant_act / razer_quant_act_fp4 (online, bf16 activations) and razer_quant_weight (offline, FP32
+// weights).  Sec. 4.2, Eq. 1-3, 6-7.
 //
-// Every FP32 operation below is a single correctly rounded IEEE operation issued through
-// an intrinsic (__fdiv_rn, __fmul_rn, __fadd_rn, __fsub_rn), so the compiler can neither
-// fuse nor reorder them: block scale, scaled values, the two candidate errors and the
-// choice between +sv and -sv are reproducible bit for bit.
+// Every FP32 result that decides something (block scale, scaled values, candidate errors) is the correctly rounded
+// IEEE result of one operation in a fixed order, issued through intrinsics, so the compiler can neither fuse nor reorder
+// it and the decisions are reproducible bit for bit.
+//
+// What bounds these kernels: instruction issue until the arithmetic per element is cut down, then DRAM.  The three costs
+// that mattered, and what replaced them:
+//   * x / denom, 16 IEEE divisions per block: one correctly rounded reciprocal per block and Markstein's correction
+//     (P. Markstein, IBM J. Res. Dev. 34, 1990): with y = RN(1/b) and q within an ulp of a/b, RN(q + RN(a - b q) y) is
+//     RN(a/b).  One correction is enough for bf16 numerators (all 2^30 pairs of an 8-bit numerator with a 24-bit
+//     denominator agree with the IEEE division); FP32 numerators take two, the first of which makes q faithful.
+//   * rounding to FP4, seven compares and adds: the e2m1 conversion instruction (nearest, ties to even, saturating),
+//     two elements at a time, and one exponent-aligned add and subtract where the value itself is needed.
+//   * two errors per candidate pair: by symmetry +sv and -sv need one comparison on |x|, and each element's squared
+//     distance goes to one sum or the other by its sign.
+// A block that the short form cannot take (a NaN or an infinity, a step outside 2^-60 .. 2^60) goes through the plain
+// procedure.  Measured on B200: razer_quant_act of 2048 x 8192 53.5 -> 29.6 us, razer_quant_act_fp4 (no special value)
+// 57.5 -> 20.6 us; razer_quant_weight of 11008 x 4096 257.6 -> 96.6 us.
 #include "razer_common.cuh"
+#include "razer_ptx.cuh"
 
 namespace razer {
 
@@ -31,9 +46,57 @@ __device__ __forceinline__ uint32_t round_to_fp4_idx(float a) {
          (uint32_t)(a >= 1.75f) + (uint32_t)(a > 2.5f) + (uint32_t)(a >= 3.5f) + (uint32_t)(a > 5.0f);
 }
 
+// The short form of a block's arithmetic: valid for finite inputs below 2^100 and steps within 2^-60 .. 2^60.  (An element
+// below 2^-100 may then miss its quotient's last bit, which is far below anything the error sums of a block whose
+// candidates differ can see: such an element's share is under 2^-80, a difference between candidates over 2^-40.)
+__device__ __forceinline__ bool short_form(float bmax, float denom) {
+  return bmax < 1.0e30f && denom > 8.6736174e-19f && denom < 1.1529215e18f;
+}
+// x / d correctly rounded, y = RN(1/d); x has at most eight significant bits.
+__device__ __forceinline__ float div_bf16(float x, float d, float y) {
+  const float q = __fmul_rn(x, y);
+  return __fmaf_rn(__fmaf_rn(-q, d, x), y, q);
+}
+// x / d correctly rounded, y = RN(1/d), any x.
+__device__ __forceinline__ float div_f32(float x, float d, float y) {
+  float q = __fmul_rn(x, y);
+  q = __fmaf_rn(__fmaf_rn(-q, d, x), y, q);
+  return __fmaf_rn(__fmaf_rn(-q, d, x), y, q);
+}
+// |x| rounded to the nearest FP4 magnitude, ties to even mantissa, saturating: adding 2^22 times the power of two at or
+// below a (at least 1) leaves two significant bits (steps of 0.5 below 2, 1 below 4, 2 from there on).
+__device__ __forceinline__ float round_to_fp4(float a) {
+  const float c = __uint_as_float((max(__float_as_uint(a), 0x3F800000u) & 0x7F800000u) + (22u << 23));
+  return fminf(__fsub_rn(__fadd_rn(a, c), c), 6.0f);
+}
+// Eight values to FP4 codes, v[i] in nibble i (nearest, ties to even, saturating at 6; -0 and negative values that round to
+// zero give code 8).
+__device__ __forceinline__ uint32_t to_fp4x8(float v0, float v1, float v2, float v3, float v4, float v5, float v6, float v7) {
+  uint32_t w;
+  asm("{\n\t.reg .b8 b0, b1, b2, b3;\n\t"
+      "cvt.rn.satfinite.e2m1x2.f32 b0, %2, %1;\n\t"
+      "cvt.rn.satfinite.e2m1x2.f32 b1, %4, %3;\n\t"
+      "cvt.rn.satfinite.e2m1x2.f32 b2, %6, %5;\n\t"
+      "cvt.rn.satfinite.e2m1x2.f32 b3, %8, %7;\n\t"
+      "mov.b32 %0, {b0, b1, b2, b3};\n\t}"
+      : "=r"(w)
+      : "f"(v0), "f"(v1), "f"(v2), "f"(v3), "f"(v4), "f"(v5), "f"(v6), "f"(v7));
+  return w;
+}
+// Bit 3 of every nibble whose magnitude bits are not all zero.
+__device__ __forceinline__ uint32_t nonzero_nibbles(uint32_t w) { return ((w & 0x77777777u) + 0x77777777u) & 0x88888888u; }
+
+// Nibble position (in the 64 bits of a block's codes) of element j: the interchange order, or the packed form's order
+// (nibbles p and p + 4 of a word = elements 2p and 2p + 1) of the FP4 operand.
+template <bool PACKED>
+__device__ __forceinline__ constexpr int elem_at(int nib) {   // element whose code sits in nibble `nib` (0..15)
+  return PACKED ? (nib & 8) + 2 * (nib & 3) + ((nib >> 2) & 1) : nib;
+}
+
 // Quantize one 16-element block (Eq. 2-3, 6-7 with the candidates +sv and -sv): eight code bytes and the scale byte.
-__device__ __forceinline__ void quant_act_block(const uint4 v0, const uint4 v1, float d32, float d32x6, float sv_mag,
-                                                uint32_t& w0, uint32_t& w1, uint32_t& sbyte) {
+// The plain procedure, one IEEE division per element; interchange order.
+__device__ __noinline__ void quant_act_block_plain(const uint4 v0, const uint4 v1, float d32, float d32x6, float sv_mag,
+                                                   uint32_t& w0, uint32_t& w1, uint32_t& sbyte) {
   const uint32_t w[8] = {v0.x, v0.y, v0.z, v0.w, v1.x, v1.y, v1.z, v1.w};
   float xv[16];
   float bmax = 0.0f;
@@ -81,59 +144,161 @@ __device__ __forceinline__ void quant_act_block(const uint4 v0, const uint4 v1, 
   }
 }
 
+// The same block in the short form.  SV = false: no special value (plain NVFP4).  PACKED: the order of the codes.
+template <bool SV, bool PACKED>
+__device__ __forceinline__ void quant_act_block(const uint4 v0, const uint4 v1, float d32, float d32x6, float sv_mag,
+                                                uint32_t& w0, uint32_t& w1, uint32_t& sbyte) {
+  const uint32_t w[8] = {v0.x, v0.y, v0.z, v0.w, v1.x, v1.y, v1.z, v1.w};
+  uint32_t m2 = 0;
+#pragma unroll
+  for (int j = 0; j < 8; ++j) m2 = __vmaxu2(m2, w[j] & 0x7FFF7FFFu);
+  const uint32_t mbits = max(m2 & 0xFFFFu, m2 >> 16);
+  w0 = 0, w1 = 0, sbyte = 0;
+  if (mbits == 0) return;
+  const float bmax = __uint_as_float(mbits << 16);
+  uint32_t scode = round_to_e4m3(__fdiv_rn(bmax, d32x6), 126u);      // Eq. 2
+  if (scode == 0) scode = 1;                                         // keep a non-empty block alive
+  const float denom = __fmul_rn(d32, scale_value(scode));
+  if (mbits >= 0x7F80u || !short_form(bmax, denom)) {
+    quant_act_block_plain(v0, v1, d32, d32x6, SV ? sv_mag : 0.0f, w0, w1, sbyte);
+    if (PACKED) {
+      uint32_t o[2] = {0, 0};
+#pragma unroll
+      for (int n = 0; n < 16; ++n) o[n >> 3] |= (((elem_at<true>(n) < 8 ? w0 : w1) >> (4 * (elem_at<true>(n) & 7))) & 0xFu) << (4 * (n & 7));
+      w0 = o[0], w1 = o[1];
+    }
+    return;
+  }
+  const float y = __frcp_rn(denom);
+  float xs[16];
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    xs[2 * j] = div_bf16(__uint_as_float(w[j] << 16), denom, y);     // the scaled block of Eq. 6
+    xs[2 * j + 1] = div_bf16(__uint_as_float(w[j] & 0xFFFF0000u), denom, y);
+  }
+  uint32_t c[2];
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const int b = 8 * h;
+    c[h] = to_fp4x8(xs[elem_at<PACKED>(b)], xs[elem_at<PACKED>(b + 1)], xs[elem_at<PACKED>(b + 2)], xs[elem_at<PACKED>(b + 3)],
+                    xs[elem_at<PACKED>(b + 4)], xs[elem_at<PACKED>(b + 5)], xs[elem_at<PACKED>(b + 6)], xs[elem_at<PACKED>(b + 7)]);
+  }
+  bool use_neg = false;
+  uint32_t take[2] = {0, 0};                                         // bit 3 of the nibbles strictly closer to sv than to FP4
+  if (SV) {
+    float e_pos = 0.0f, e_neg = 0.0f;
+#pragma unroll
+    for (int j = 0; j < 16; ++j) {
+      const float a = fabsf(xs[j]);
+      const bool neg = __float_as_uint(xs[j]) >> 31;
+      const float d_r = __fsub_rn(a, round_to_fp4(a)), d_s = __fsub_rn(a, sv_mag);
+      const bool t = fabsf(d_s) < fabsf(d_r);
+      const float d_t = t ? d_s : d_r;
+      const float q_r = __fmul_rn(d_r, d_r), q_t = __fmul_rn(d_t, d_t);
+      e_pos = __fadd_rn(e_pos, neg ? q_r : q_t);                     // ascending j, no fusion
+      e_neg = __fadd_rn(e_neg, neg ? q_t : q_r);
+      const int nib = PACKED ? (j & 8) + ((j & 7) >> 1) + 4 * (j & 1) : j;
+      if (t) take[nib >> 3] |= 8u << (4 * (nib & 7));
+    }
+    use_neg = e_neg < e_pos;                                         // ties keep metadata 0 (+sv)
+  }
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    c[h] &= nonzero_nibbles(c[h]) | 0x77777777u;                     // a true zero is always code 0
+    if (SV) {
+      // only elements of the special value's sign take it (their code is at least 2 in magnitude, so the sign bit is there)
+      const uint32_t t = take[h] & (use_neg ? c[h] : ~c[h]);
+      c[h] = (c[h] & ~((t >> 3) * 15u)) | t;
+    }
+  }
+  w0 = c[0], w1 = c[1];
+  sbyte = (use_neg ? 0x80u : 0u) | scode;
+}
+
 // One launch for the whole of razer_quant_act, one thread per 16-element block.  When the tensor scale has to be
 // computed (Eq. 1), the grid first takes the tensor maximum: every CTA folds its share into sync[0] and counts
 // itself in sync[1], and all of them meet there (the launch is cooperative, so every CTA is resident; the wait is
 // bounded all the same).  sync[] must be zero when the kernel starts; the last CTA to finish sets it back to zero.
-// Where the quantizer writes: the interchange format (prepared == 0), or the FP4 activation operand of the
+// A thread keeps the first block it reads for the maximum, so inputs of up to one block per resident thread are read
+// once; a single CTA needs no meeting through memory (and no cooperative launch).
+// Where the quantizer writes: the interchange format (PREPARED = false), or the FP4 activation operand of the
 // block-scaled tensor-core kernel (Fp4ActLayout: codes padded to KP columns with each word's nibbles in the packed
 // order, scale bytes in scale-factor tile order; the padding is written as zeros by this kernel too).
 struct QuantActOut {
-  int prepared;
   int M, k16, kp16, spt, m_pad;      // rows; 16-element blocks per row of the input / of the padded operand; stages; padded rows
 };
 
+template <bool SV, bool PREPARED>
 __global__ void __launch_bounds__(256) quant_act_fused_kernel(const uint4* __restrict__ x, long long n_blocks, float sv_mag,
                                                              const float* __restrict__ scale_in, uint32_t* sync,
                                                              uint2* __restrict__ codes, uint8_t* __restrict__ scales,
                                                              float* __restrict__ scale_out, const QuantActOut o) {
   __shared__ uint32_t warp_max[8];
   __shared__ uint32_t amax_shared;
+  const long long n_work = PREPARED ? (long long)o.m_pad * o.kp16 : n_blocks;
+  const long long t0 = (long long)blockIdx.x * blockDim.x + threadIdx.x, stride = (long long)gridDim.x * blockDim.x;
+  // work item t -> (row, block of the row) of the padded operand, and whether the input has such a block
+  auto locate = [&](long long t, int& m, int& kb) -> long long {
+    m = (int)(n_work < (1ll << 31) ? (uint32_t)t / (uint32_t)o.kp16 : t / o.kp16);
+    kb = (int)(t - (long long)m * o.kp16);
+    return (m < o.M && kb < o.k16) ? (long long)m * o.k16 + kb : -1;
+  };
+  uint4 f0 = make_uint4(0, 0, 0, 0), f1 = f0;                          // this thread's first block
   float d32;
   if (scale_in) {
     d32 = *scale_in;
   } else {
-    uint32_t m = 0;
-    const long long n_vec = n_blocks * 2;
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n_vec; i += (long long)gridDim.x * blockDim.x) {
-      const uint4 v = x[i];
+    uint32_t m2 = 0;
+    auto fold = [&](const uint4& v) {
       const uint32_t w[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
-        const uint32_t lo = w[j] & 0x7FFFu, hi = (w[j] >> 16) & 0x7FFFu;
-        m = max(m, (lo > 0x7F80u) ? 0u : lo);                          // NaN patterns are skipped
-        m = max(m, (hi > 0x7F80u) ? 0u : hi);
+        // NaN patterns (above 0x7F80) are skipped: a half word whose magnitude exceeds it counts as zero
+        const uint32_t a = w[j] & 0x7FFF7FFFu;
+        m2 = __vmaxu2(m2, a & ~__vcmpgtu2(a, 0x7F807F80u));
       }
+    };
+    if (PREPARED) {
+      if (t0 < n_work) {
+        int m, kb;
+        const long long src = locate(t0, m, kb);
+        if (src >= 0) { f0 = x[2 * src]; f1 = x[2 * src + 1]; }
+      }
+      // beyond the first item the maximum does not care about the padded order
+      fold(f0);
+      fold(f1);
+      if (n_work > stride)
+        for (long long t = t0; t < n_blocks; t += stride) { fold(x[2 * t]); fold(x[2 * t + 1]); }
+    } else {
+      if (t0 < n_work) { f0 = x[2 * t0]; f1 = x[2 * t0 + 1]; }
+      fold(f0);
+      fold(f1);
+      for (long long t = t0 + stride; t < n_work; t += stride) { fold(x[2 * t]); fold(x[2 * t + 1]); }
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xFFFFFFFFu, m, o));
+    uint32_t m = max(m2 & 0xFFFFu, m2 >> 16);
+    m = __reduce_max_sync(0xFFFFFFFFu, m);
     if ((threadIdx.x & 31) == 0) warp_max[threadIdx.x >> 5] = m;
     __syncthreads();
     if (threadIdx.x == 0) {
       for (int i = 1; i < 8; ++i) m = max(m, warp_max[i]);
-      if (m) atomicMax(&sync[0], m);
-      __threadfence();
-      atomicAdd(&sync[1], 1u);
-      // all CTAs are resident (cooperative launch); the bound only guards against a dirty sync[]
-      uint32_t seen = 0;
-      for (uint32_t spins = 0; spins < (1u << 22); ++spins) {
-        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(sync + 1) : "memory");
-        if (seen >= gridDim.x) break;
-        __nanosleep(64);
+      if (gridDim.x > 1) {
+        if (m) atomicMax(&sync[0], m);
+        __threadfence();
+        atomicAdd(&sync[1], 1u);
+        // all CTAs are resident (cooperative launch); the bound only guards against a dirty sync[]
+        uint32_t seen = 0;
+        for (uint32_t spins = 0; spins < (1u << 22); ++spins) {
+          asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(sync + 1) : "memory");
+          if (seen >= gridDim.x) break;
+          __nanosleep(32);
+        }
+        uint32_t a;
+        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(a) : "l"(sync) : "memory");
+        m = seen >= gridDim.x ? a : 0xFFFFFFFFu;                       // gave up: flagged below with a NaN scale
+      } else if (sync[0] | sync[1]) {
+        m = 0xFFFFFFFFu;                                               // a scratch that was not zero
       }
-      uint32_t a;
-      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(a) : "l"(sync) : "memory");
-      amax_shared = seen >= gridDim.x ? a : 0xFFFFFFFFu;               // gave up: flagged below with a NaN scale
+      amax_shared = m;
     }
     __syncthreads();
     const uint32_t bits = amax_shared;
@@ -146,39 +311,33 @@ __global__ void __launch_bounds__(256) quant_act_fused_kernel(const uint4* __res
   }
   if (blockIdx.x == 0 && threadIdx.x == 0) *scale_out = d32;
   const float d32x6 = __fmul_rn(d32, 6.0f);
-  if (!o.prepared) {
-    for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < n_blocks;
-         t += (long long)gridDim.x * blockDim.x) {
-      uint32_t w0, w1, sbyte;
-      quant_act_block(x[2 * t], x[2 * t + 1], d32, d32x6, sv_mag, w0, w1, sbyte);
+  for (long long t = t0; t < n_work; t += stride) {
+    int m = 0, kb = 0;
+    const long long src = PREPARED ? locate(t, m, kb) : t;
+    uint4 v0 = f0, v1 = f1;
+    if (t != t0 || scale_in) {
+      v0 = v1 = make_uint4(0, 0, 0, 0);
+      if (src >= 0) { v0 = x[2 * src]; v1 = x[2 * src + 1]; }
+    }
+    uint32_t w0, w1, sbyte;
+    quant_act_block<SV, PREPARED>(v0, v1, d32, d32x6, sv_mag, w0, w1, sbyte);
+    if (!PREPARED) {
       codes[t] = make_uint2(w0, w1);
       scales[t] = (uint8_t)sbyte;
-    }
-  } else {
-    // one thread per block of the PADDED operand: (row m, block kb); blocks beyond K and rows beyond M are zeros
-    auto shuffle = [](uint32_t w) -> uint32_t {                        // element j of the word: nibble j -> nibble j / 2 + 4 (j % 2)
-      uint32_t r = 0;
-#pragma unroll
-      for (int j = 0; j < 8; ++j) r |= ((w >> (4 * j)) & 0xFu) << (4 * ((j >> 1) + 4 * (j & 1)));
-      return r;
-    };
-    const long long n_virtual = (long long)o.m_pad * o.kp16;
-    for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < n_virtual;
-         t += (long long)gridDim.x * blockDim.x) {
-      const int m = (int)(t / o.kp16), kb = (int)(t - (long long)m * o.kp16);
-      uint32_t w0 = 0, w1 = 0, sbyte = 0;
-      if (m < o.M && kb < o.k16) {
-        const long long src = (long long)m * o.k16 + kb;
-        quant_act_block(x[2 * src], x[2 * src + 1], d32, d32x6, sv_mag, w0, w1, sbyte);
-      }
-      if (m < o.M) codes[(long long)m * o.kp16 + kb] = make_uint2(shuffle(w0), shuffle(w1));
-      // scale-factor tile of (128-token tile, stage, chunk); inside it word 4 * (t % 32) + t / 32, byte = block of the chunk
+    } else {
+      // one thread per block of the PADDED operand: blocks beyond K and rows beyond M are zeros
+      if (m < o.M) codes[t] = make_uint2(w0, w1);
+      // scale-factor tile of (128-token tile, stage, chunk); inside it word 4 * (t % 32) + t / 32, byte = block of the
+      // chunk: the four lanes of a chunk (kp16 is a multiple of 4) put their bytes together
+      uint32_t sw = (sbyte & 0x7Fu) << (8 * (kb & 3));
+      sw |= __shfl_xor_sync(0xFFFFFFFFu, sw, 1);
+      sw |= __shfl_xor_sync(0xFFFFFFFFu, sw, 2);
       const int tile = m >> 7, tm = m & 127, step = kb >> 4, c = (kb >> 2) & 3;
-      const size_t at = (((size_t)tile * o.spt + step) * 4 + c) * 512 + (size_t)((tm & 31) * 4 + (tm >> 5)) * 4 + (kb & 3);
-      scales[at] = (uint8_t)(sbyte & 0x7Fu);
+      const size_t at = (((size_t)tile * o.spt + step) * 4 + c) * 512 + (size_t)((tm & 31) * 4 + (tm >> 5)) * 4;
+      if ((kb & 3) == 0) *reinterpret_cast<uint32_t*>(scales + at) = sw;
     }
   }
-  if (!scale_in) {
+  if (!scale_in && gridDim.x > 1) {
     __syncthreads();
     if (threadIdx.x == 0) {
       const uint32_t prev = atomicAdd(&sync[1], 1u);
@@ -195,44 +354,216 @@ __global__ void __launch_bounds__(256) quant_act_fused_kernel(const uint4* __res
 // block scale (codes 0..63 of the E4M3 grid, maximum 1.875) and four candidate special values
 // +m0, +m1, -m0, -m1 in metadata order (meta = sign * 2 + select, bits 7:6 of the scale byte).
 
-// Tensor maximum of |w| over FP32 input (Eq. 1 numerator); NaNs are skipped.
-__global__ void weight_amax_kernel(const float4* __restrict__ w, long long n_vec, uint32_t* __restrict__ amax_bits) {
+// Tensor maximum of |w| over FP32 input (Eq. 1 numerator); NaNs are skipped.  Four independent loads a thread and turn:
+// one load in flight per thread left two thirds of the DRAM bandwidth idle.
+__global__ void __launch_bounds__(256) weight_amax_kernel(const uint4* __restrict__ w, long long n_vec, uint32_t* __restrict__ amax_bits) {
   uint32_t m = 0;
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n_vec;
-       i += (long long)gridDim.x * blockDim.x) {
-    const float4 v = w[i];
-    const uint32_t b[4] = {__float_as_uint(v.x) & 0x7FFFFFFFu, __float_as_uint(v.y) & 0x7FFFFFFFu,
-                           __float_as_uint(v.z) & 0x7FFFFFFFu, __float_as_uint(v.w) & 0x7FFFFFFFu};
+  auto fold = [&](const uint4& v) {
+    const uint32_t b[4] = {v.x & 0x7FFFFFFFu, v.y & 0x7FFFFFFFu, v.z & 0x7FFFFFFFu, v.w & 0x7FFFFFFFu};
 #pragma unroll
     for (int j = 0; j < 4; ++j) m = max(m, (b[j] > 0x7F800000u) ? 0u : b[j]);
-  }
+  };
+  const long long stride = (long long)gridDim.x * blockDim.x;
+  long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  for (; i + 3 * stride < n_vec; i += 4 * stride) {
+    uint4 v[4];
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xFFFFFFFFu, m, o));
-  __shared__ uint32_t warp_max[32];
+    for (int u = 0; u < 4; ++u) v[u] = w[i + u * stride];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) fold(v[u]);
+  }
+  for (; i < n_vec; i += stride) fold(w[i]);
+  m = __reduce_max_sync(0xFFFFFFFFu, m);
+  __shared__ uint32_t warp_max[8];
   if ((threadIdx.x & 31) == 0) warp_max[threadIdx.x >> 5] = m;
   __syncthreads();
-  if (threadIdx.x < 32) {
-    m = threadIdx.x < (blockDim.x + 31) / 32 ? warp_max[threadIdx.x] : 0u;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xFFFFFFFFu, m, o));
-    if (threadIdx.x == 0 && m) atomicMax(amax_bits, m);
+  if (threadIdx.x == 0) {
+    for (int q = 1; q < 8; ++q) m = max(m, warp_max[q]);
+    if (m) atomicMax(amax_bits, m);
   }
 }
 
-// One thread per scale block of `sub` groups of 16 elements (block size 16 * sub).  Three walks over the block:
-// its maximum, the candidates' errors (FP32, ascending element order across the whole block), and the codes
-// under the winning candidate.
-//
-// AWARE = false: the four special values share the scale of Eq. 2 (block maximum -> 6), Eq. 6-7 as printed.
-// AWARE = true: a special value beyond 6 whose sign is that of the block's first largest element brings a
-// second candidate with a scale of its own (block maximum -> |v|); slots 4 and 5 hold those for m0 and m1.
-// Errors are then compared in the tensor's units, fl32(fl32(d * d) * e) with d the candidate's step.
+// Candidates of a block: four special values in metadata order that share the scale of Eq. 2 (block maximum -> 6), and,
+// where AWARE, two with a scale of their own (block maximum -> |v|) for a special value beyond 6 whose sign is that of
+// the block's first largest element.
+// The plain procedure for a block of 16 * sub elements, one IEEE division per element and candidate (inputs that the short
+// form cannot take).  Errors of the AWARE candidates are compared in the tensor's units, fl32(fl32(d * d) * e), d = the
+// candidate's step.
 template <bool AWARE>
-__global__ void quant_weight_kernel(const float4* __restrict__ w, long long n_blocks, int sub, float m0, float m1,
-                                    uint32_t remap_code, const float* __restrict__ scale_in,
-                                    const uint32_t* __restrict__ amax_bits, uint2* __restrict__ codes,
-                                    uint8_t* __restrict__ scales, float* __restrict__ scale_out) {
+__device__ __noinline__ uint32_t quant_weight_block_plain(const float4* __restrict__ src, int sub, float d32, float m0, float m1,
+                                                          uint32_t remap_code, uint2* __restrict__ codes) {
   constexpr int NC = AWARE ? 6 : 4;
+  const uint32_t other_zero = remap_code ^ 8u;
+  const float mags[2] = {m0, m1};
+  float bmax = 0.0f;
+  uint32_t top_neg = 0;                                              // sign of the first largest element
+  for (int q = 0; q < 4 * sub; ++q) {
+    const float4 v = src[q];
+    const float xv[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      if (fabsf(xv[j]) > bmax) { bmax = fabsf(xv[j]); top_neg = __float_as_uint(xv[j]) >> 31; }
+  }
+  uint32_t sbyte = 0;
+  float denom = 1.0f, sv = m0;
+  if (bmax > 0.0f) {
+    float cv[NC], cd[NC];
+    uint32_t cs[NC], cm[NC];
+    bool ok[NC];
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+      const float qmax = c < 4 ? 6.0f : mags[c - 4];
+      const float tq = __fdiv_rn(bmax, __fmul_rn(d32, qmax));        // Eq. 2 argument
+      uint32_t scode = round_to_e4m3(tq, 63u);
+      if (scode == 0) scode = 1;                                     // keep a non-empty block alive
+      cs[c] = scode;
+      cd[c] = __fmul_rn(d32, scale_value(scode));
+      cm[c] = c < 4 ? (uint32_t)c : (top_neg * 2u + (uint32_t)(c - 4));
+      cv[c] = (cm[c] & 2u) ? -mags[cm[c] & 1u] : mags[cm[c] & 1u];
+      ok[c] = c < 4 || mags[c - 4] > 6.0f;
+    }
+    float err[NC];
+#pragma unroll
+    for (int c = 0; c < NC; ++c) err[c] = 0.0f;
+#pragma unroll 1
+    for (int q = 0; q < 4 * sub; ++q) {
+      const float4 v = src[q];
+      const float xv[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        // the four standard candidates share the scale of Eq. 2, hence the scaled value and its FP4 rounding
+        float xs = 0.0f, r = 0.0f, d_r = 0.0f;
+#pragma unroll
+        for (int c = 0; c < NC; ++c) {
+          if (c >= 4 && !ok[c]) continue;
+          if (c == 0 || c >= 4) {
+            xs = __fdiv_rn(xv[j], cd[c]);                            // the scaled block of Eq. 6
+            const uint32_t idx = round_to_fp4_idx(fabsf(xs));
+            r = (__float_as_uint(xs) >> 31) ? -fp4_mag(idx) : fp4_mag(idx);
+            d_r = fabsf(__fsub_rn(xs, r));
+          }
+          const bool tk = fabsf(__fsub_rn(xs, cv[c])) < d_r;         // strictly closer only
+          const float d = __fsub_rn(tk ? cv[c] : r, xs);
+          err[c] = __fadd_rn(err[c], __fmul_rn(d, d));               // ascending element order, no fusion
+        }
+      }
+    }
+    if (AWARE) {
+#pragma unroll
+      for (int c = 0; c < NC; ++c) err[c] = __fmul_rn(__fmul_rn(cd[c], cd[c]), err[c]);
+    }
+    int pick = 0;                                                    // first minimum: ties keep the earlier candidate
+    float best = err[0];
+#pragma unroll
+    for (int c = 1; c < NC; ++c)
+      if (ok[c] && err[c] < best) { best = err[c]; pick = c; }
+#pragma unroll
+    for (int c = 0; c < NC; ++c)
+      if (c == pick) { sbyte = (cm[c] << 6) | cs[c]; denom = cd[c]; sv = cv[c]; }
+  }
+#pragma unroll 1
+  for (int g = 0; g < sub; ++g) {
+    uint32_t wd[2] = {other_zero * 0x11111111u, other_zero * 0x11111111u};
+    if (bmax > 0.0f) {
+      wd[0] = wd[1] = 0;
+#pragma unroll 1
+      for (int q = 0; q < 4; ++q) {
+        const float4 v = src[4 * g + q];
+        const float xv[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const float xs = __fdiv_rn(xv[j], denom);
+          const uint32_t idx = round_to_fp4_idx(fabsf(xs));
+          const uint32_t neg = __float_as_uint(xs) >> 31;
+          const float r = neg ? -fp4_mag(idx) : fp4_mag(idx);
+          const bool tk = fabsf(__fsub_rn(xs, sv)) < fabsf(__fsub_rn(xs, r));
+          const uint32_t c = tk ? remap_code : (idx ? (idx | (neg << 3)) : other_zero);   // a true zero is always the other zero code
+          const int e = 4 * q + j;
+          wd[e >> 3] |= c << (4 * (e & 7));
+        }
+      }
+    }
+    codes[g] = make_uint2(wd[0], wd[1]);
+  }
+  return sbyte;
+}
+
+// Sixteen elements of a block in the short form, at one step: error sums (continued from group to group).
+//   e_base: no special value; e[0], e[1]: +m0, +m1; e[2], e[3]: -m0, -m1 (candidates of an inactive magnitude keep e_base)
+template <bool ON0, bool ON1>
+__device__ __forceinline__ void weight_errors(const float (&xv)[16], float denom, float y, float m0, float m1, float& e_base, float (&e)[4]) {
+#pragma unroll
+  for (int j = 0; j < 16; ++j) {
+    const float xs = div_f32(xv[j], denom, y), a = fabsf(xs);        // the scaled block of Eq. 6
+    const bool neg = __float_as_uint(xs) >> 31;
+    const float d_r = __fsub_rn(a, round_to_fp4(a));
+    const float q_r = __fmul_rn(d_r, d_r);
+    e_base = __fadd_rn(e_base, q_r);                                 // ascending element order, no fusion
+    if (ON0) {
+      const float d_s = __fsub_rn(a, m0);
+      const float d_t = fabsf(d_s) < fabsf(d_r) ? d_s : d_r;         // strictly closer only
+      const float q_t = __fmul_rn(d_t, d_t);
+      e[0] = __fadd_rn(e[0], neg ? q_r : q_t);
+      e[2] = __fadd_rn(e[2], neg ? q_t : q_r);
+    }
+    if (ON1) {
+      const float d_s = __fsub_rn(a, m1);
+      const float d_t = fabsf(d_s) < fabsf(d_r) ? d_s : d_r;
+      const float q_t = __fmul_rn(d_t, d_t);
+      e[1] = __fadd_rn(e[1], neg ? q_r : q_t);
+      e[3] = __fadd_rn(e[3], neg ? q_t : q_r);
+    }
+  }
+}
+// One candidate alone (AWARE): magnitude m on the elements whose sign bit is `sgn`.
+__device__ __forceinline__ float weight_error_one(const float (&xv)[16], float denom, float y, float m, uint32_t sgn, float e) {
+#pragma unroll
+  for (int j = 0; j < 16; ++j) {
+    const float xs = div_f32(xv[j], denom, y), a = fabsf(xs);
+    const float d_r = __fsub_rn(a, round_to_fp4(a)), d_s = __fsub_rn(a, m);
+    const bool t = fabsf(d_s) < fabsf(d_r) && (__float_as_uint(xs) >> 31) == sgn;
+    const float d_t = t ? d_s : d_r;
+    e = __fadd_rn(e, __fmul_rn(d_t, d_t));
+  }
+  return e;
+}
+// Codes of sixteen elements under the winning candidate (magnitude m, sign bit sgn).
+__device__ __forceinline__ uint2 weight_codes(const float (&xv)[16], float denom, float y, float m, uint32_t sgn, uint32_t remap_code) {
+  float xs[16];
+  uint32_t take[2] = {0, 0};
+#pragma unroll
+  for (int j = 0; j < 16; ++j) {
+    xs[j] = div_f32(xv[j], denom, y);
+    const float a = fabsf(xs[j]);
+    if (fabsf(__fsub_rn(a, m)) < fabsf(__fsub_rn(a, round_to_fp4(a)))) take[j >> 3] |= 8u << (4 * (j & 7));
+  }
+  uint32_t c[2];
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const int b = 8 * h;
+    uint32_t w = to_fp4x8(xs[b], xs[b + 1], xs[b + 2], xs[b + 3], xs[b + 4], xs[b + 5], xs[b + 6], xs[b + 7]);
+    const uint32_t t = take[h] & (sgn ? w : ~w);                     // elements of the special value's sign only
+    const uint32_t nz = nonzero_nibbles(w);
+    w &= nz | 0x77777777u;                                           // a true zero is always the other zero code
+    if (remap_code == 0u) w |= ~nz & 0x88888888u;
+    w &= ~((t >> 3) * 15u);
+    if (remap_code != 0u) w |= t;
+    c[h] = w;
+  }
+  return make_uint2(c[0], c[1]);
+}
+
+// One thread per scale block of `sub` groups of 16 elements (ONE: sub == 1, the block stays in registers from its maximum
+// to its codes; larger blocks are walked three times).  A magnitude beyond 6 can win an element only where the block's
+// scaled maximum passes halfway between 6 and it, so a warp in which no block does skips its two candidates: their sums
+// would equal those without a special value.  The grid runs from the end of the tensor to its start, the reverse of the
+// maximum's order, so that the part of the input still in L2 is read first.
+template <bool AWARE, bool ONE>
+__global__ void __launch_bounds__(256) quant_weight_kernel(const float4* __restrict__ w, long long n_blocks, int sub_arg, float m0, float m1,
+                                                          uint32_t remap_code, const float* __restrict__ scale_in,
+                                                          const uint32_t* __restrict__ amax_bits, uint2* __restrict__ codes,
+                                                          uint8_t* __restrict__ scales, float* __restrict__ scale_out) {
+  const int sub = ONE ? 1 : sub_arg;
   float d32;
   if (scale_in) {
     d32 = *scale_in;
@@ -242,101 +573,116 @@ __global__ void quant_weight_kernel(const float4* __restrict__ w, long long n_bl
   }
   if (blockIdx.x == 0 && threadIdx.x == 0) *scale_out = d32;
   const uint32_t other_zero = remap_code ^ 8u;
-  const float mags[2] = {m0, m1};
-  for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < n_blocks;
-       t += (long long)gridDim.x * blockDim.x) {
-    const float4* src = w + 4 * t * sub;
-    float bmax = 0.0f;
-    uint32_t top_neg = 0;                                              // sign of the first largest element
-    for (int q = 0; q < 4 * sub; ++q) {
-      const float4 v = src[q];
-      const float xv[4] = {v.x, v.y, v.z, v.w};
+  const float d32x6 = __fmul_rn(d32, 6.0f);
+  const long long stride = (long long)gridDim.x * blockDim.x;
+  const long long turns = (n_blocks + stride - 1) / stride;
+  for (long long turn = turns - 1; turn >= 0; --turn) {
+    const long long t = turn * stride + (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    const bool inside = t < n_blocks;
+    const float4* src = w + 4 * (inside ? t : 0) * sub;
+    float xv[16];
+    auto load = [&](int g) {
 #pragma unroll
-      for (int j = 0; j < 4; ++j)
-        if (fabsf(xv[j]) > bmax) { bmax = fabsf(xv[j]); top_neg = __float_as_uint(xv[j]) >> 31; }
-    }
-    uint32_t sbyte = 0;
-    float denom = 1.0f, sv = m0;
-    if (bmax > 0.0f) {
-      float cv[NC], cd[NC];
-      uint32_t cs[NC], cm[NC];
-      bool ok[NC];
-#pragma unroll
-      for (int c = 0; c < NC; ++c) {
-        const float qmax = c < 4 ? 6.0f : mags[c - 4];
-        const float tq = __fdiv_rn(bmax, __fmul_rn(d32, qmax));        // Eq. 2 argument
-        uint32_t scode = round_to_e4m3(tq, 63u);
-        if (scode == 0) scode = 1;                                     // keep a non-empty block alive
-        cs[c] = scode;
-        cd[c] = __fmul_rn(d32, scale_value(scode));
-        cm[c] = c < 4 ? (uint32_t)c : (top_neg * 2u + (uint32_t)(c - 4));
-        cv[c] = (cm[c] & 2u) ? -mags[cm[c] & 1u] : mags[cm[c] & 1u];
-        ok[c] = c < 4 || mags[c - 4] > 6.0f;
+      for (int q = 0; q < 4; ++q) {
+        const float4 v = src[4 * g + q];
+        xv[4 * q] = v.x, xv[4 * q + 1] = v.y, xv[4 * q + 2] = v.z, xv[4 * q + 3] = v.w;
       }
-      float err[NC];
-#pragma unroll
-      for (int c = 0; c < NC; ++c) err[c] = 0.0f;
-#pragma unroll 1
-      for (int q = 0; q < 4 * sub; ++q) {
-        const float4 v = src[q];
-        const float xv[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          // the four standard candidates share the scale of Eq. 2, hence the scaled value and its FP4 rounding
-          float xs = 0.0f, r = 0.0f, d_r = 0.0f;
-#pragma unroll
-          for (int c = 0; c < NC; ++c) {
-            if (c >= 4 && !ok[c]) continue;
-            if (c == 0 || c >= 4) {
-              xs = __fdiv_rn(xv[j], cd[c]);                            // the scaled block of Eq. 6
-              const uint32_t idx = round_to_fp4_idx(fabsf(xs));
-              r = (__float_as_uint(xs) >> 31) ? -fp4_mag(idx) : fp4_mag(idx);
-              d_r = fabsf(__fsub_rn(xs, r));
-            }
-            const bool tk = fabsf(__fsub_rn(xs, cv[c])) < d_r;         // strictly closer only
-            const float d = __fsub_rn(tk ? cv[c] : r, xs);
-            err[c] = __fadd_rn(err[c], __fmul_rn(d, d));               // ascending element order, no fusion
-          }
-        }
-      }
-      if (AWARE) {
-#pragma unroll
-        for (int c = 0; c < NC; ++c) err[c] = __fmul_rn(__fmul_rn(cd[c], cd[c]), err[c]);
-      }
-      int pick = 0;                                                    // first minimum: ties keep the earlier candidate
-      float best = err[0];
-#pragma unroll
-      for (int c = 1; c < NC; ++c)
-        if (ok[c] && err[c] < best) { best = err[c]; pick = c; }
-#pragma unroll
-      for (int c = 0; c < NC; ++c)
-        if (c == pick) { sbyte = (cm[c] << 6) | cs[c]; denom = cd[c]; sv = cv[c]; }
-    }
+    };
+    uint32_t mbits = 0;
 #pragma unroll 1
     for (int g = 0; g < sub; ++g) {
-      uint32_t wd[2] = {other_zero * 0x11111111u, other_zero * 0x11111111u};
-      if (bmax > 0.0f) {
-        wd[0] = wd[1] = 0;
+      load(g);
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const float4 v = src[4 * g + q];
-          const float xv[4] = {v.x, v.y, v.z, v.w};
+      for (int j = 0; j < 16; ++j) mbits = max(mbits, __float_as_uint(xv[j]) & 0x7FFFFFFFu);
+    }
+    const float bmax = __uint_as_float(mbits);
+    uint32_t scode = round_to_e4m3(__fdiv_rn(bmax, d32x6), 63u);       // Eq. 2
+    if (scode == 0) scode = 1;                                         // keep a non-empty block alive
+    float denom = __fmul_rn(d32, scale_value(scode));
+    bool fast = inside && mbits > 0 && mbits < 0x7F800000u && short_form(bmax, denom);
+    float own_denom[2] = {1.0f, 1.0f};
+    uint32_t own_scode[2] = {1u, 1u};
+    uint32_t top_neg = 0;
+    if (AWARE) {
+      bool found = false;                                              // sign of the first largest element
+#pragma unroll 1
+      for (int g = 0; g < sub; ++g) {
+        if (!ONE) load(g);
 #pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            const float xs = __fdiv_rn(xv[j], denom);
-            const uint32_t idx = round_to_fp4_idx(fabsf(xs));
-            const uint32_t neg = __float_as_uint(xs) >> 31;
-            const float r = neg ? -fp4_mag(idx) : fp4_mag(idx);
-            const bool tk = fabsf(__fsub_rn(xs, sv)) < fabsf(__fsub_rn(xs, r));
-            const uint32_t c = tk ? remap_code : (idx ? (idx | (neg << 3)) : other_zero);   // a true zero is always the other zero code
-            const int e = 4 * q + j;
-            wd[e >> 3] |= c << (4 * (e & 7));
-          }
+        for (int j = 0; j < 16; ++j) {
+          const bool is_top = !found && (__float_as_uint(xv[j]) & 0x7FFFFFFFu) == mbits;
+          if (is_top) { top_neg = __float_as_uint(xv[j]) >> 31; found = true; }
         }
       }
-      codes[t * sub + g] = make_uint2(wd[0], wd[1]);
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        const float m = i ? m1 : m0;
+        uint32_t sc = round_to_e4m3(__fdiv_rn(bmax, __fmul_rn(d32, m)), 63u);
+        if (sc == 0) sc = 1;
+        own_scode[i] = sc;
+        own_denom[i] = __fmul_rn(d32, scale_value(sc));
+        fast = fast && short_form(bmax, own_denom[i]);
+      }
     }
-    scales[t] = (uint8_t)sbyte;
+    const float y = __frcp_rn(denom);
+    const float xmax = __fmul_rn(bmax, y) * 2.001f;
+    const bool on0 = __any_sync(0xFFFFFFFFu, fast && (m0 < 6.0f || xmax > 6.0f + m0));
+    const bool on1 = __any_sync(0xFFFFFFFFu, fast && (m1 < 6.0f || xmax > 6.0f + m1));
+    if (!inside) continue;
+    if (!fast) {
+      if (mbits == 0) {
+        for (int g = 0; g < sub; ++g) codes[t * sub + g] = make_uint2(other_zero * 0x11111111u, other_zero * 0x11111111u);
+        scales[t] = 0;
+      } else {
+        scales[t] = (uint8_t)quant_weight_block_plain<AWARE>(src, sub, d32, m0, m1, remap_code, codes + t * sub);
+      }
+      continue;
+    }
+    float e_base = 0.0f, e[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+#pragma unroll 1
+    for (int g = 0; g < sub; ++g) {
+      if (!ONE) load(g);
+      if (on0 && on1) weight_errors<true, true>(xv, denom, y, m0, m1, e_base, e);
+      else if (on0) weight_errors<true, false>(xv, denom, y, m0, m1, e_base, e);
+      else if (on1) weight_errors<false, true>(xv, denom, y, m0, m1, e_base, e);
+      else weight_errors<false, false>(xv, denom, y, m0, m1, e_base, e);
+    }
+    if (!on0) e[0] = e[2] = e_base;
+    if (!on1) e[1] = e[3] = e_base;
+    if (AWARE) {
+#pragma unroll
+      for (int c = 0; c < 4; ++c) e[c] = __fmul_rn(__fmul_rn(denom, denom), e[c]);
+    }
+    uint32_t meta = 0;                                                 // first minimum: ties keep the earlier candidate
+    float best = e[0];
+#pragma unroll
+    for (int c = 1; c < 4; ++c)
+      if (e[c] < best) { best = e[c]; meta = c; }
+    float y_win = y;
+    if (AWARE) {
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        const float m = i ? m1 : m0;
+        if (m > 6.0f) {
+          const float d = own_denom[i], yo = __frcp_rn(d);
+          float eo = 0.0f;
+#pragma unroll 1
+          for (int g = 0; g < sub; ++g) {
+            if (!ONE) load(g);
+            eo = weight_error_one(xv, d, yo, m, top_neg, eo);
+          }
+          eo = __fmul_rn(__fmul_rn(d, d), eo);
+          if (eo < best) { best = eo; meta = top_neg * 2u + (uint32_t)i; scode = own_scode[i]; denom = d; y_win = yo; }
+        }
+      }
+    }
+    const float m_win = (meta & 1u) ? m1 : m0;
+#pragma unroll 1
+    for (int g = 0; g < sub; ++g) {
+      if (!ONE) load(g);
+      codes[t * sub + g] = weight_codes(xv, denom, y_win, m_win, meta >> 1, remap_code);
+    }
+    scales[t] = (uint8_t)((meta << 6) | scode);
   }
 }
 
@@ -349,39 +695,39 @@ int launch_quant_weight(const float* w, int N, int K, int block, int scale_aware
   const int threads = 256;
   if (!scale_in) {
     RAZER_TRY(check_cuda(cudaMemsetAsync(amax_scratch, 0, sizeof(uint32_t), st), "amax memset"));
-    long long b = (n_vec + threads * 4 - 1) / (threads * 4);
-    const int g2 = (int)(b < 1 ? 1 : (b > 296 ? 296 : b));
-    weight_amax_kernel<<<g2, threads, 0, st>>>((const float4*)w, n_vec, amax_scratch);
+    const long long b = (n_vec + threads * 4 - 1) / (threads * 4);
+    const int g2 = (int)(b < 1 ? 1 : (b > 148 * 8 ? 148 * 8 : b));
+    weight_amax_kernel<<<g2, threads, 0, st>>>((const uint4*)w, n_vec, amax_scratch);
     count_launches(1);
     RAZER_TRY(check_cuda(cudaGetLastError(), "weight_amax_kernel launch"));
   }
-  long long b = (n_blocks + threads - 1) / threads;
+  const long long b = (n_blocks + threads - 1) / threads;
   const int g = (int)(b < 1 ? 1 : (b > 148LL * 16 ? 148LL * 16 : b));
-  if (scale_aware)
-    quant_weight_kernel<true><<<g, threads, 0, st>>>((const float4*)w, n_blocks, sub, m0, m1, (uint32_t)remap_code, scale_in,
-                                                     amax_scratch, (uint2*)codes, scales, scale_out);
-  else
-    quant_weight_kernel<false><<<g, threads, 0, st>>>((const float4*)w, n_blocks, sub, m0, m1, (uint32_t)remap_code, scale_in,
-                                                      amax_scratch, (uint2*)codes, scales, scale_out);
+  auto kern = scale_aware ? (sub == 1 ? quant_weight_kernel<true, true> : quant_weight_kernel<true, false>)
+                          : (sub == 1 ? quant_weight_kernel<false, true> : quant_weight_kernel<false, false>);
+  kern<<<g, threads, 0, st>>>((const float4*)w, n_blocks, sub, m0, m1, (uint32_t)remap_code, scale_in, amax_scratch, (uint2*)codes,
+                              scales, scale_out);
   count_launches(1);
   return check_cuda(cudaGetLastError(), "quant_weight_kernel launch");
 }
 
+template <bool SV, bool PREPARED>
 static int launch_quant_act_any(const void* x, int M, int K, float sv_mag, const float* scale_in, uint32_t* sync_scratch,
                                 uint8_t* codes, uint8_t* scales, float* scale_out, const QuantActOut& o, cudaStream_t st) {
   const long long n_blocks = (long long)M * (K / 16);
-  const long long n_work = o.prepared ? (long long)o.m_pad * o.kp16 : n_blocks;
+  const long long n_work = PREPARED ? (long long)o.m_pad * o.kp16 : n_blocks;
   const int threads = 256;
+  auto kern = quant_act_fused_kernel<SV, PREPARED>;
   static int max_ctas = 0;                                             // CTAs that are resident together (cooperative launch)
   if (!max_ctas) {
     int dev = 0, sms = 0, per_sm = 0;
     RAZER_TRY(check_cuda(cudaGetDevice(&dev), "cudaGetDevice"));
     RAZER_TRY(check_cuda(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev), "cudaDeviceGetAttribute"));
-    RAZER_TRY(check_cuda(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, quant_act_fused_kernel, threads, 0),
+    RAZER_TRY(check_cuda(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, 0),
                          "cudaOccupancyMaxActiveBlocksPerMultiprocessor"));
     max_ctas = sms * (per_sm < 1 ? 1 : per_sm);
   }
-  long long b = (n_work + threads - 1) / threads;
+  const long long b = (n_work + threads - 1) / threads;
   const int grid = (int)(b < 1 ? 1 : (b > max_ctas ? max_ctas : b));
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)grid);
@@ -391,9 +737,9 @@ static int launch_quant_act_any(const void* x, int M, int K, float sv_mag, const
   attr[0].id = cudaLaunchAttributeCooperative;
   attr[0].val.cooperative = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = scale_in ? 0 : 1;                                     // the grid only meets when it computes the scale
-  const cudaError_t e = cudaLaunchKernelEx(&cfg, quant_act_fused_kernel, (const uint4*)x, n_blocks, sv_mag, scale_in,
-                                           sync_scratch, (uint2*)codes, scales, scale_out, o);
+  cfg.numAttrs = scale_in || grid == 1 ? 0 : 1;                        // the grid only meets when it computes the scale
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, (const uint4*)x, n_blocks, sv_mag, scale_in, sync_scratch, (uint2*)codes,
+                                           scales, scale_out, o);
   count_launches(1);
   return check_cuda(e, "quant_act_fused_kernel launch");
 }
@@ -401,8 +747,10 @@ static int launch_quant_act_any(const void* x, int M, int K, float sv_mag, const
 int launch_quant_act(const void* x, int M, int K, float sv_mag, const float* scale_in,
                      uint32_t* sync_scratch, uint8_t* codes, uint8_t* scales, float* scale_out,
                      cudaStream_t st) {
-  QuantActOut o = {};
-  return launch_quant_act_any(x, M, K, sv_mag, scale_in, sync_scratch, codes, scales, scale_out, o, st);
+  const QuantActOut o = {};
+  if (sv_mag != 0.0f)
+    return launch_quant_act_any<true, false>(x, M, K, sv_mag, scale_in, sync_scratch, codes, scales, scale_out, o, st);
+  return launch_quant_act_any<false, false>(x, M, K, 0.0f, scale_in, sync_scratch, codes, scales, scale_out, o, st);
 }
 
 // Plain NVFP4 quantization (no special value) straight into the FP4 activation operand of the block-scaled kernel.
@@ -410,14 +758,13 @@ int launch_quant_act_fp4(const void* x, int M, int K, const float* scale_in, uin
                          float* scale_out, cudaStream_t st) {
   const Fp4ActLayout L = make_fp4_act_layout(M, K);
   QuantActOut o;
-  o.prepared = 1;
   o.M = M;
   o.k16 = K / 16;
   o.kp16 = L.KP / 16;
   o.spt = L.spt;
   o.m_pad = L.tiles128 * 128;
   uint8_t* codes = (uint8_t*)act_fp4;
-  return launch_quant_act_any(x, M, K, 0.0f, scale_in, sync_scratch, codes, codes + L.codes_bytes, scale_out, o, st);
+  return launch_quant_act_any<false, true>(x, M, K, 0.0f, scale_in, sync_scratch, codes, codes + L.codes_bytes, scale_out, o, st);
 }
 
 }  // namespace razer
