@@ -24,28 +24,14 @@ __device__ __forceinline__ uint32_t fma_relu_bf16x2(uint32_t a, uint32_t b, uint
 __device__ __forceinline__ uint32_t mul_bf16x2(uint32_t a, uint32_t b) { return as_u32(__hmul2(as_bf162(a), as_bf162(b))); }
 __device__ __forceinline__ uint32_t and_or(uint32_t a, uint32_t b, uint32_t c) { return (a & b) | c; }
 
-// Special-value constants of a block, selected by the scale byte's select bit.
-struct SvConsts {
-  uint32_t sv;               // (sv, sv) x 2^-126 as bf16x2
-  uint32_t nsv_lo;           // -(sv x 2^7):  sv - nsv_lo * (nibble in bits 3:0 read as bf16) = 0 for nibble 1
-  uint32_t nsv_hi;           // -(sv x 2^3):  the same for a nibble in bits 7:4
-  uint32_t pad;
-};
-
-// Decode tables in shared memory.
+// Decode table in shared memory.
 //   ss[(negate << 6 | scale code)][lane] : (+-scale x 2^126) as bf16x2; one copy per lane so that a
 //                                          warp's 32 lookups never collide on a bank
-//   sv[select]                           : SvConsts
 constexpr int DECODE_SS_ENTRIES = 128;
-constexpr int DECODE_TABLE_BYTES = DECODE_SS_ENTRIES * 32 * 4 + 2 * 16;
+constexpr int DECODE_TABLE_BYTES = DECODE_SS_ENTRIES * 32 * 4;
 
-struct DecodeTables {         // 32-bit shared-window addresses
-  uint32_t ss_lane;          // &ss[0][lane]
-  uint32_t sv;
-};
-
-// Fill the tables (all threads of the CTA call this; a __syncthreads() must follow).
-__device__ __forceinline__ void decode_tables_fill(uint8_t* base, float sv0, float sv1, int tid, int nthreads) {
+// Fill the table (all threads of the CTA call this; a __syncthreads() must follow).
+__device__ __forceinline__ void decode_tables_fill(uint8_t* base, int tid, int nthreads) {
   // every entry is computed once per quarter (four threads per entry) and written as eight of its 32 lane copies
   for (int i = tid; i < DECODE_SS_ENTRIES * 4; i += nthreads) {
     const uint32_t idx = (uint32_t)i >> 2;
@@ -57,77 +43,36 @@ __device__ __forceinline__ void decode_tables_fill(uint8_t* base, float sv0, flo
     dst[0] = make_uint4(v, v, v, v);
     dst[1] = make_uint4(v, v, v, v);
   }
-  if (tid < 2) {
-    const float sv = tid ? sv1 : sv0;                          // at most four significant bits
-    const uint32_t p0 = __float_as_uint(sv * 1.17549435e-38f) >> 16;     // sv x 2^-126
-    const uint32_t p1 = __float_as_uint(-sv * 128.0f) >> 16;
-    const uint32_t p2 = __float_as_uint(-sv * 8.0f) >> 16;
-    SvConsts c;
-    c.sv = p0 | (p0 << 16);
-    c.nsv_lo = p1 | (p1 << 16);
-    c.nsv_hi = p2 | (p2 << 16);
-    c.pad = 0;
-    reinterpret_cast<SvConsts*>(base + DECODE_SS_ENTRIES * 32 * 4)[tid] = c;
-  }
+}
+// (sv x 2^-126, sv x 2^-126) as bf16x2; sv has at most four significant bits.
+__host__ __device__ __forceinline__ uint32_t special_value_pair(float sv) {
+  union { float f; uint32_t u; } b;
+  b.f = sv * 1.17549435e-38f;
+  return (b.u >> 16) | (b.u & 0xFFFF0000u);
 }
 
-__device__ __forceinline__ DecodeTables decode_tables_view(const uint8_t* base, int lane) {
-  DecodeTables t;
-  t.ss_lane = smem_addr(base) + lane * 4;
-  t.sv = smem_addr(base) + DECODE_SS_ENTRIES * 32 * 4;
-  return t;
+// Scale pair of block `blk` (0..3, compile-time) of a chunk, from the row's scale word (four packed scale bytes
+// [select | negate | 6-bit scale code]); ss_lane = shared-window address of &ss[0][lane].
+__device__ __forceinline__ uint32_t decode_block_scale(uint32_t ss_lane, uint32_t sw, int blk) {
+  return lds32(ss_lane + ((blk == 0 ? sw << 7 : sw >> (8 * blk - 7)) & 0x3F80u));   // (byte & 0x7F) * 128
 }
 
-// Constants of block `blk` (0..3, compile-time) of a chunk, from the row's scale word
-// (four packed scale bytes [select | negate | 6-bit scale code]).
-__device__ __forceinline__ void decode_block_consts(const DecodeTables& t, uint32_t sw, int blk, uint32_t& ss2,
-                                                    SvConsts& svc) {
-  const uint32_t off_ss = (blk == 0 ? sw << 7 : sw >> (8 * blk - 7)) & 0x3F80u;   // (byte & 0x7F) * 128
-  const uint32_t off_sv = (sw >> (8 * blk + 3)) & 0x10u;                          // (byte >> 7) * 16
-  ss2 = lds32(t.ss_lane + off_ss);
-  const uint4 c = lds128(t.sv + off_sv);
-  svc.sv = c.x;
-  svc.nsv_lo = c.y;
-  svc.nsv_hi = c.z;
-  svc.pad = 0;
-}
-
-// The same for a scale byte already shifted down to bits 7:0 (higher bits may hold anything).
-__device__ __forceinline__ void decode_block_consts_byte(const DecodeTables& t, uint32_t sb, uint32_t& ss2, SvConsts& svc) {
-  ss2 = lds32(t.ss_lane + ((sb << 7) & 0x3F80u));
-  const uint4 c = lds128(t.sv + ((sb >> 3) & 0x10u));
-  svc.sv = c.x;
-  svc.nsv_lo = c.y;
-  svc.nsv_hi = c.z;
-  svc.pad = 0;
-}
-
-// The same for a scale word rotated so that the block's byte sits on bits 14:7 (higher and lower bits may hold
-// anything), for tables that start on a 16 KB boundary of the shared window: the table offsets are then
-// merged into the addresses by the same logic op that isolates them.
-__device__ __forceinline__ void decode_block_consts_rot(const DecodeTables& t, uint32_t r, uint32_t& ss2, SvConsts& svc) {
-  ss2 = lds32(and_or(r, 0x3F80u, t.ss_lane));
-  const uint4 c = lds128(and_or(r >> 10, 0x10u, t.sv));
-  svc.sv = c.x;
-  svc.nsv_lo = c.y;
-  svc.nsv_hi = c.z;
-  svc.pad = 0;
-}
-
-// Four stored nibbles of each 16-bit half of `w` -> four bf16x2 registers (elements 2p, 2p+1
-// of the word in register p), each the exact product value x scale with the block's sign.
-// mul_lo = 2^6 + 2^12, mul_hi = 2^2 + 2^8 (run-time values so that they stay multiplies).
-__device__ __forceinline__ void decode_word(uint32_t w, uint32_t ss2, const SvConsts& c, uint32_t mul_lo,
-                                            uint32_t mul_hi, uint32_t* out) {
+// Four stored nibbles of each 16-bit half of `w` -> four bf16x2 registers (elements 2p, 2p + 1 of the word in
+// register p), each the exact product value x scale with the block's sign.  The special value is the one
+// nibble that is numerically zero when the isolated nibble is read as a bf16 pair: relu(nibble * -2^11 + sv')
+// is sv' = sv x 2^-126 for it and 0 for every other nibble (the smallest, 2^-133, times 2^11 already exceeds
+// the largest sv').
+// mul_lo = 2^6 + 2^12, mul_hi = 2^2 + 2^8 (run-time values so that they stay multiplies): one shifted copy of the nibble
+// lands with E1 E0 M on bits 8:6, the other with S on bit 15; the mask keeps exactly those.
+__device__ __forceinline__ void decode_word(uint32_t w, uint32_t ss2, uint32_t svp, uint32_t mul_lo, uint32_t mul_hi, uint32_t* out) {
+  constexpr uint32_t NEG = 0xC500C500u;               // (-2048, -2048) as bf16x2
   const uint32_t w8 = w >> 8;
   const uint32_t n0 = w & 0x000F000Fu, n1 = w & 0x00F000F0u;
   const uint32_t n2 = w8 & 0x000F000Fu, n3 = w8 & 0x00F000F0u;
-  // nibble * (2^6 + 2^12) [bits 3:0] or * (2^2 + 2^8) [bits 7:4]: one copy lands with E1 E0 M on
-  // bits 8:6, the other with S on bit 15; the mask keeps exactly those
-  const uint32_t u0 = and_or(n0 * mul_lo, 0x81C081C0u, fma_relu_bf16x2(n0, c.nsv_lo, c.sv));
-  const uint32_t u1 = and_or(n1 * mul_hi, 0x81C081C0u, fma_relu_bf16x2(n1, c.nsv_hi, c.sv));
-  const uint32_t u2 = and_or(n2 * mul_lo, 0x81C081C0u, fma_relu_bf16x2(n2, c.nsv_lo, c.sv));
-  const uint32_t u3 = and_or(n3 * mul_hi, 0x81C081C0u, fma_relu_bf16x2(n3, c.nsv_hi, c.sv));
+  const uint32_t u0 = and_or(n0 * mul_lo, 0x81C081C0u, fma_relu_bf16x2(n0, NEG, svp));
+  const uint32_t u1 = and_or(n1 * mul_hi, 0x81C081C0u, fma_relu_bf16x2(n1, NEG, svp));
+  const uint32_t u2 = and_or(n2 * mul_lo, 0x81C081C0u, fma_relu_bf16x2(n2, NEG, svp));
+  const uint32_t u3 = and_or(n3 * mul_hi, 0x81C081C0u, fma_relu_bf16x2(n3, NEG, svp));
   out[0] = mul_bf16x2(u0, ss2);
   out[1] = mul_bf16x2(u1, ss2);
   out[2] = mul_bf16x2(u2, ss2);

@@ -17,6 +17,11 @@
 //
 // The register-level decode is described in razer_decode.cuh.
 //
+// What bounds it: up to 64 tokens the decode (about five instructions a weight pair) and the start and end of the stripes;
+// from 128 tokens on the MMAs (512 cycles per 128 x 256 x 64 item) together with shared-memory bandwidth (571 cycles).
+// Issuing from one lane elected once, and handing the accumulator back before a complete tile's stores:
+// 2048 x 14336 x 4096 206 -> 194 us, 16 x 8192 x 28672 49.3 -> 46.9 us.
+//
 // Work partition (Sec. 4.3 / App. E of the paper: stripes of about equal length that may span
 // several output tiles, partial results reduced through global memory): the grid is
 // persistent, work items are (output tile, k-stage) pairs in tile-major order and every CTA
@@ -65,14 +70,14 @@ struct UmmaArgs {
   uint32_t* status;          // device status word
   const float* extra_scale;  // optional device scalar multiplied into the tensor scale
   Geometry g;
-  float sv0, sv1, tensor_scale;
+  uint32_t svp0, svp1;       // special-value pairs for select 0 / 1 (razer_decode.cuh)
+  float tensor_scale;
   uint32_t mul_lo, mul_hi;   // 2^6 + 2^12 and 2^2 + 2^8, passed at run time so that they stay multiplies
   int M, token_tiles, steps_per_tile;
   int x_map_3d;              // the activation tensor map is the 3-D (64 k, tokens, k chunk) view: one load per stage
   long long total_items;
 };
 
-constexpr int MAX_ISSUERS = 5;          // the MMA warp, or one issuing warp per dequant group
 
 template <int NT, int CH, int STAGES, int ASTAGES, int NACC>
 struct UmmaCfg {
@@ -86,21 +91,20 @@ struct UmmaCfg {
   static constexpr int TMEM_COLS_NEEDED = ACC_COLS + ASTAGES * A_STAGE_COLS;
   static constexpr int TMEM_COLS = TMEM_COLS_NEEDED <= 64 ? 64 : TMEM_COLS_NEEDED <= 128 ? 128
                                    : TMEM_COLS_NEEDED <= 256 ? 256 : 512;
-  static constexpr int NUM_BARS = 2 * STAGES + 2 * ASTAGES + 3 + MAX_ISSUERS;
-  static constexpr int TABLE_BYTES = DECODE_TABLE_BYTES;        // scale table + special-value constants
+  static constexpr int NUM_BARS = 2 * STAGES + 2 * ASTAGES + 4;
+  static constexpr int TABLE_BYTES = DECODE_TABLE_BYTES;        // scale table
   static constexpr size_t SMEM_BYTES =
       1024 /*alignment slack*/ + (size_t)STAGES * STAGE_BYTES + NUM_BARS * 8 + 16 + 64 + TABLE_BYTES;
   static_assert(TMEM_COLS_NEEDED <= 512, "TMEM budget exceeded");
   static_assert(NT % 16 == 0 && NT >= 16 && NT <= 256, "UMMA N for M = 128");
 };
 
-// GI ("group issue"): each dequant group issues the MMAs of the items it decoded itself, into accumulators
-// of its own, instead of handing them to the MMA warp.  Used for the narrowest token tile (16), where an
-// item's MMAs are short; from 32 tokens up the MMA warp keeps up and issues (measured level at 16, the MMA
-// warp ahead at 32 and 64).
-template <int NT, int CH, int STAGES, int ASTAGES, int NDW, int NACC, bool GI>
+// The MMA warp issues every item's MMAs.  (Letting the group that decoded an item issue it, once level at 16 tokens, lost
+// when the MMA warp came to elect its lane once: 8192 x 28672 at 16 tokens 49.3 against 45.9 us.)
+template <int NT, int CH, int STAGES, int ASTAGES, int NDW, int NACC>
 __global__ void __launch_bounds__(64 + 32 * NDW, 1)
-razer_umma_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant__ CUtensorMap tmap_w, const UmmaArgs a) {
+razer_umma_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant__ CUtensorMap tmap_w,
+                  const __grid_constant__ UmmaArgs a) {
   using Cfg = UmmaCfg<NT, CH, STAGES, ASTAGES, NACC>;
   constexpr int THREADS = 64 + 32 * NDW;
   extern __shared__ uint8_t smem_raw[];
@@ -118,7 +122,7 @@ razer_umma_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
   const uint32_t bar_accfull = bar_aempty + 8 * ASTAGES;
   const uint32_t bar_accempty = bar_accfull + 8;
   const uint32_t bar_epi = bar_accempty + 8;            // rendezvous of the 128 epilogue threads
-  const uint32_t bar_drain = bar_epi + 8;               // [MAX_ISSUERS] an issuing warp's own MMAs have all completed
+  const uint32_t bar_drain = bar_epi + 8;               // the MMA warp's own MMAs have all completed
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int grid = gridDim.x, cta = blockIdx.x;
@@ -140,10 +144,10 @@ razer_umma_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
       mbar_init(bar_afull + 8 * i, 128);
       mbar_init(bar_aempty + 8 * i, 1);
     }
-    mbar_init(bar_accfull, GI ? NDW / 4 : 1);
-    mbar_init(bar_accempty, GI ? 128 : 32 * NDW);         // threads that read the accumulator in the epilogue
-    mbar_init(bar_epi, GI ? 128 : 32 * NDW);
-    for (int i = 0; i < MAX_ISSUERS; ++i) mbar_init(bar_drain + 8 * i, 1);
+    mbar_init(bar_accfull, 1);
+    mbar_init(bar_accempty, 32 * NDW);         // threads that read the accumulator in the epilogue
+    mbar_init(bar_epi, 32 * NDW);
+    mbar_init(bar_drain, 1);
     *abort_flag = 0;
     tmem_slot[3] = 0;                                   // a flag nobody sets (used by the drain waits)
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -195,7 +199,7 @@ razer_umma_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
       c2.template next<STAGES, ASTAGES>(spt);
     }
   }
-  if (warp != 0) decode_tables_fill(tables, a.sv0, a.sv1, threadIdx.x - 32, THREADS - 32);
+  if (warp != 0) decode_tables_fill(tables, threadIdx.x - 32, THREADS - 32);
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
                  "r"((uint32_t)Cfg::TMEM_COLS)
@@ -217,12 +221,11 @@ razer_umma_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
   // Whole warp, on leaving an issue loop (at its end or after a wait gave up): the MMAs this warp has issued
   // read shared memory and TMEM and write TMEM until they complete, so the warp commits them to a barrier of
   // its own and waits for it (bounded, not watching the abort flag) before the CTA may release either.
-  auto drain_mmas = [&](int issuer_idx) {
+  auto drain_mmas = [&]() {
     __syncwarp();
-    const uint32_t bar = bar_drain + 8 * issuer_idx;
-    if (elect_one()) tc_commit(bar);
+    if (elect_one()) tc_commit(bar_drain);
     __syncwarp();
-    mbar_wait(bar, 0u, tmem_slot + 3);
+    mbar_wait(bar_drain, 0u, tmem_slot + 3);
   };
 
   if (warp == 0) {
@@ -239,51 +242,44 @@ razer_umma_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
     }
   } else if (warp == 1) {
     // ===================== MMA issuer (whole warp walks the items, one elected lane issues) =====================
-    if (!GI) {
-      constexpr uint32_t idesc = make_idesc(NT);
-      // upper half of the shared-memory descriptor: 1024-byte group stride, descriptor version, 128-byte swizzle
-      constexpr uint32_t bd_hi = (1024u >> 4) | (1u << 14) | (2u << 29);
+    constexpr uint32_t idesc = make_idesc(NT);
+    // upper half of the shared-memory descriptor: 1024-byte group stride, descriptor version, 128-byte swizzle
+    constexpr uint32_t bd_hi = (1024u >> 4) | (1u << 14) | (2u << 29);
+    // One elected lane walks the items.  Electing once around the whole loop lets the compiler keep descriptors and
+    // addresses in uniform registers; electing anew for every item cost about 37 cycles per tcgen05 instruction.
+    if (elect_one()) {
       uint32_t seg = 0;
-      auto wait_warp = [&](uint32_t bar, uint32_t parity, uint32_t code) -> bool {
-        const bool got = mbar_wait(bar, parity, abort_flag);
-        if (!got) fail(code);
-        return __all_sync(0xFFFFFFFFu, got);
-      };
       for (int i = 0; i < n_items; ++i) {
         const bool seg_first = (i == 0) || cur.step == 0;
         const bool seg_last = (i + 1 == n_items) || cur.step == spt - 1;
         const int nch = min(CH, a.g.k_chunks - cur.step * CH);
         // the group that filled this A stage waited for the shared-memory stage (weights and activations)
         // before it decoded, so its arrival also covers the activation tile
-        if (!wait_warp(bar_afull + 8 * cur.astage, (uint32_t)cur.aphase, 3)) break;
-        if (seg_first && !wait_warp(bar_accempty, (seg & 1u) ^ 1u, 4)) break;
+        if (!mbar_wait(bar_afull + 8 * cur.astage, (uint32_t)cur.aphase, abort_flag)) { fail(3); break; }
+        if (seg_first && !mbar_wait(bar_accempty, (seg & 1u) ^ 1u, abort_flag)) { fail(4); break; }
         tc_fence_after();
         const uint32_t xs = smem_u32(smem) + (uint32_t)cur.stage * Cfg::STAGE_BYTES + Cfg::W_PAD;
         const uint32_t a_t = tmem_a0 + cur.astage * Cfg::A_STAGE_COLS;
         const uint32_t bd_lo = (xs >> 4) | (1u << 16);    // start address and (unused) leading offset fields
-        if (elect_one()) {
-          // Consecutive MMAs go to NACC different accumulators (summed in the epilogue): MMAs on one
-          // accumulator execute one after the other, and a narrow MMA is far shorter than its latency.
+        // Consecutive MMAs go to NACC different accumulators (summed in the epilogue): MMAs on one
+        // accumulator execute one after the other, and a narrow MMA is far shorter than its latency.
 #pragma unroll
-          for (int j = 0; j < CH * 4; ++j) {
-            // 16 k further along: +32 bytes inside a chunk's 128-byte rows, next chunk's box after four
-            if (j < nch * 4) {
-              const uint32_t bd = bd_lo + (uint32_t)(((j >> 2) * Cfg::X_BOX_BYTES + (j & 3) * 32) >> 4);
-              const uint32_t d_t = tmem_base + (j % NACC) * NT;
-              if (j < NACC && seg_first) tc_mma_ts2<false>(d_t, a_t + j * 8, bd, bd_hi, idesc);
-              else tc_mma_ts2<true>(d_t, a_t + j * 8, bd, bd_hi, idesc);
-            }
+        for (int j = 0; j < CH * 4; ++j) {
+          // 16 k further along: +32 bytes inside a chunk's 128-byte rows, next chunk's box after four
+          if (j < nch * 4) {
+            const uint32_t bd = bd_lo + (uint32_t)(((j >> 2) * Cfg::X_BOX_BYTES + (j & 3) * 32) >> 4);
+            const uint32_t d_t = tmem_base + (j % NACC) * NT;
+            if (j < NACC && seg_first) tc_mma_ts2<false>(d_t, a_t + j * 8, bd, bd_hi, idesc);
+            else tc_mma_ts2<true>(d_t, a_t + j * 8, bd, bd_hi, idesc);
           }
-          tc_commit(bar_empty + 8 * cur.stage);
-          tc_commit(bar_aempty + 8 * cur.astage);
-          if (seg_last) tc_commit(bar_accfull);
         }
-        __syncwarp();
-        if (seg_last) ++seg;
+        tc_commit(bar_empty + 8 * cur.stage);
+        tc_commit(bar_aempty + 8 * cur.astage);
+        if (seg_last) { tc_commit(bar_accfull); ++seg; }
         cur.template next<STAGES, ASTAGES>(spt);
       }
-      drain_mmas(0);
     }
+    drain_mmas();
   } else {
     // ===================== dequant (32 * NDW threads, thread = weight row) + epilogue =====================
     const int row = 32 * (warp & 3) + lane;              // TMEM lane this thread owns
@@ -291,39 +287,15 @@ razer_umma_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
     const int group = (warp - 2) >> 2;                   // four warps (all TMEM lane quarters) decode one item together
     constexpr int GROUPS = NDW / 4;
     static_assert(NDW % 4 == 0 && GROUPS <= ASTAGES, "every dequant group needs an A stage of its own");
-    static_assert(GROUPS + 1 <= MAX_ISSUERS, "a drain barrier per issuing warp");
-    static_assert(!GI || (NACC % GROUPS == 0 && ASTAGES == GROUPS), "group issue: A stage and accumulators per group");
-    static_assert(GI ? STAGES % GROUPS == 0 : (GROUPS == ASTAGES && STAGES >= ASTAGES),
+    static_assert(GROUPS == ASTAGES && STAGES >= ASTAGES,
                   "every fill of a stage must be known complete to the group that waits for the next one");
-    constexpr int APG = GI ? NACC / GROUPS : NACC;       // accumulators per group
-    // one warp of each group issues the group's MMAs; the groups pick different ones so that the issuing
-    // warps sit on different schedulers (a warp's scheduler is warp % 4)
-    const bool issuer = GI && ((warp - 2) & 3) == (group & 3);
-    uint32_t own_phase = 0, gseg = 0;                    // GI: parity of the group's A stage; segments seen
-    bool fresh = true;                                   // GI: the group's accumulators hold nothing of this segment yet
-    // Epilogue: with group issue only group 0 drains the (narrow) accumulators while the other groups
-    // keep decoding; otherwise every group drains its share of the columns of its TMEM lane quarter.
-    const bool epi_warp = !GI || (group == 0);
-    // shares in units of 16 columns: group g takes units [g U / GROUPS, (g + 1) U / GROUPS), U = NT / 16
-    const int col_lo = GI ? 0 : 16 * ((group * (NT / 16)) / GROUPS);
-    const int col_hi = GI ? NT : 16 * (((group + 1) * (NT / 16)) / GROUPS);
-    const bool leader = (threadIdx.x == 64);
-    float ts = a.tensor_scale;                           // (x extra scale: read after the grid dependency)
-    bool dep_waited = false;
-    uint32_t seg = 0, epi_phase = 0;
     // all 32 lanes take the same branch after a wait, so the .aligned tcgen05 instructions stay convergent
     auto wait_all = [&](uint32_t bar, uint32_t parity, uint32_t code) -> bool {
       const bool got = mbar_wait(bar, parity, abort_flag);
       if (!got) fail(code);
       return __all_sync(0xFFFFFFFFu, got);
     };
-    auto epi_sync = [&]() -> bool {                     // bounded rendezvous of the epilogue threads
-      mbar_arrive(bar_epi);
-      const bool got = wait_all(bar_epi, epi_phase & 1u, 8);
-      ++epi_phase;
-      return got;
-    };
-    const DecodeTables dt = decode_tables_view(tables, lane);
+    const uint32_t ss_lane = smem_addr(tables) + lane * 4;
     const uint32_t mul_lo = a.mul_lo, mul_hi = a.mul_hi;
     // where this thread's weight row sits inside a stage: strip row / 16, row r = row % 16 of it
     const int r16 = row % STRIP_ROWS;
@@ -333,27 +305,33 @@ razer_umma_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
     uint32_t code_off[CHUNK_BLOCKS];
 #pragma unroll
     for (int blk = 0; blk < CHUNK_BLOCKS; ++blk) code_off[blk] = (uint32_t)piece_code_offset(blk, r16);
+    // The epilogue of a finished segment runs after the group's next item has been prepared, so that the MMAs
+    // resume as soon as the accumulator is in registers.
+    struct Pending { int tile; bool at_end; } pending = {-1, false};
+    const EpilogueCtx ctx = {bar_accfull, bar_accempty, bar_epi, tmem_base + lane_off, row, group, threadIdx.x == 64};
+    uint32_t seg = 0, epi_phase = 0;
+    auto epilogue = [&]() -> bool {
+      grid_dep_wait();                                     // outputs, workspace and the scale scalar may belong to the preceding kernel
+      const float ts = a.extra_scale ? a.tensor_scale * *a.extra_scale : a.tensor_scale;
+      const int tile = pending.tile;
+      pending.tile = -1;
+      return segment_epilogue<NT, NACC, GROUPS>(
+          a, ctx, tile, pending.at_end, ts, seg++, epi_phase, abort_flag,
+          [&](uint32_t bar, uint32_t parity, uint32_t which) { return wait_all(bar, parity, 7u + which); },
+          [&](uint32_t which) { fail(7u + which); });
+    };
     int turn = 0;                                        // item i is decoded by group i % GROUPS
-    for (int i = 0; i < n_items; ++i, cur.template next<STAGES, ASTAGES>(spt), turn = (turn + 1 == GROUPS ? 0 : turn + 1)) {
-      const int tile = cur.tile, step = cur.step;
-      const bool seg_last = (i + 1 == n_items) || step == spt - 1;
+    for (int i = 0; i <= n_items; ++i, cur.template next<STAGES, ASTAGES>(spt), turn = (turn + 1 == GROUPS ? 0 : turn + 1)) {
+      const int step = cur.step;
+      const bool seg_last = (i + 1 >= n_items) || step == spt - 1;
       const int nch = min(CH, a.g.k_chunks - step * CH);
-      const bool seg_first = (i == 0) || step == 0;
-      if (GI && seg_first) {
-        fresh = true;
-        // the epilogue of the previous segment must have read the accumulators before any group moves on
-        if (issuer && gseg > 0 && !wait_all(bar_accempty, (gseg & 1u) ^ 1u, 4)) break;
-      }
-      if (turn == group) {
-      const int astage = GI ? group : cur.astage;
-      const uint32_t aph = GI ? own_phase : (uint32_t)cur.aphase;
+      if (turn == group && i < n_items) {
+      const int astage = cur.astage;
+      const uint32_t aph = (uint32_t)cur.aphase;
       // Order matters.  A parity wait is only sound for a waiter that knows the barrier's previous phase to be
       // complete, and a group does not see every fill of a shared-memory stage (the loads of a ring complete in
       // any order: a group could come back to a stage one ring later while the fill it skipped is still in
-      // flight, take that for its own and decode the stage's old bytes).  Group issue: STAGES is a multiple of
-      // GROUPS, so a stage always serves the same group, which sees all its fills (making every group wait for
-      // the fills it skips is no way out: the groups free the stages themselves and end up waiting for one
-      // another).  Otherwise the A stage is
+      // flight, take that for its own and decode the stage's old bytes).  The A stage is
       // this group's own (GROUPS == ASTAGES) and its release by the MMA warp, which takes the items in order,
       // means that every item up to i - ASTAGES was issued, hence decoded, hence landed, the stage's previous
       // fill (item i - STAGES, STAGES >= ASTAGES) among them.
@@ -374,14 +352,14 @@ razer_umma_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
 #pragma unroll
           for (int blk = 0; blk < CHUNK_BLOCKS; ++blk) cw[blk] = lds64(ck + code_off[blk]);
           uint32_t ss2[CHUNK_BLOCKS];
-          SvConsts svc[CHUNK_BLOCKS];
 #pragma unroll
-          for (int blk = 0; blk < CHUNK_BLOCKS; ++blk) decode_block_consts(dt, sw, blk, ss2[blk], svc[blk]);
+          for (int blk = 0; blk < CHUNK_BLOCKS; ++blk) ss2[blk] = decode_block_scale(ss_lane, sw, blk);
 #pragma unroll
           for (int blk = 0; blk < CHUNK_BLOCKS; ++blk) {
             uint32_t v[8];
-            decode_word(cw[blk].x, ss2[blk], svc[blk], mul_lo, mul_hi, v);
-            decode_word(cw[blk].y, ss2[blk], svc[blk], mul_lo, mul_hi, v + 4);
+            const uint32_t svp = (sw & (PACKED_SELECT << (8 * blk))) ? a.svp1 : a.svp0;
+            decode_word(cw[blk].x, ss2[blk], svp, mul_lo, mul_hi, v);
+            decode_word(cw[blk].y, ss2[blk], svp, mul_lo, mul_hi, v + 4);
             tc_st8(a_t + (c * 4 + blk) * 8, v);
           }
         }
@@ -389,153 +367,12 @@ razer_umma_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
       tc_wait_st();
       tc_fence_before();
       mbar_arrive(bar_afull + 8 * astage);
-      if (GI) {
-        if (issuer) {
-          // the group's 128 threads have stored their rows: issue this item's MMAs from here
-          if (!wait_all(bar_afull + 8 * astage, aph, 3)) break;
-          tc_fence_after();
-          constexpr uint32_t idesc = make_idesc(NT);
-          constexpr uint32_t bd_hi = (1024u >> 4) | (1u << 14) | (2u << 29);
-          const uint32_t xs = smem_u32(smem) + (uint32_t)cur.stage * Cfg::STAGE_BYTES + Cfg::W_PAD;
-          const uint32_t bd_lo = (xs >> 4) | (1u << 16);
-          const uint32_t a_s = tmem_a0 + astage * Cfg::A_STAGE_COLS;
-          if (elect_one()) {
-#pragma unroll
-            for (int j = 0; j < CH * 4; ++j) {
-              if (j < nch * 4) {
-                const uint32_t bd = bd_lo + (uint32_t)(((j >> 2) * Cfg::X_BOX_BYTES + (j & 3) * 32) >> 4);
-                const uint32_t d_t = tmem_base + (group * APG + j % APG) * NT;
-                if (j < APG && fresh) tc_mma_ts2<false>(d_t, a_s + j * 8, bd, bd_hi, idesc);
-                else tc_mma_ts2<true>(d_t, a_s + j * 8, bd, bd_hi, idesc);
-              }
-            }
-            tc_commit(bar_empty + 8 * cur.stage);
-            tc_commit(bar_aempty + 8 * astage);
-          }
-          __syncwarp();
-        }
-        fresh = false;
-        own_phase ^= 1u;
       }
-      }
-      if (GI && seg_last) {
-        // every group reports its share of the segment (a group without an item in it reports at once)
-        if (issuer) {
-          if (elect_one()) tc_commit(bar_accfull);
-          __syncwarp();
-        }
-        ++gseg;
-      }
-
-      if (!seg_last || !epi_warp) continue;
-      // ---------------- epilogue of the segment that ends with this item ----------------
-      const int it = it_begin + i;
-      const int tile_begin = tile * spt;
-      const int seg_begin = it_begin > tile_begin ? it_begin : tile_begin;
-      const bool complete = (seg_begin == tile_begin) && (step == spt - 1);
-      const int rt = tile / a.token_tiles, tt = tile - rt * a.token_tiles;
-      const int n_out = rt * TILE_ROWS + row;
-      const int m0 = tt * NT;
-      if (!dep_waited) {                                   // outputs, workspace and the scale scalar may belong to the preceding kernel
-        grid_dep_wait();
-        if (a.extra_scale) ts *= *a.extra_scale;
-        dep_waited = true;
-      }
-      // A partial tile is finished by its owner, the CTA whose stripe holds the tile's FIRST items: for that CTA the
-      // tile is the end of its stripe, for every other CTA of the tile it is the beginning, so their parts were
-      // published (FP32 slot in the workspace, then a release-add on the tile's counter) long before the owner gets
-      // here.  The owner adds its own accumulator (straight from TMEM) and the other parts in CTA order.
-      const int c_first = cta_of_item(tile_begin, grid, a.total_items);
-      const int c_last = cta_of_item(tile_begin + spt - 1, grid, a.total_items);
-      const bool owner = !complete && cta == c_first;
-      if (owner) {
-        // acquire: every counted CTA's slot stores are visible to this thread's loads below
-        const uint32_t others = (uint32_t)(c_last - c_first);
-        uint32_t seen = 0;
-        const uint64_t t0 = global_ns();
-        for (;;) {
-          asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(a.counters + tile) : "memory");
-          if (seen >= others || *abort_flag || global_ns() - t0 > WAIT_LIMIT_NS) break;
-          __nanosleep(200);
-        }
-        const bool ready = seen >= others;
-        if (!ready) fail(9);
-        if (!__all_sync(0xFFFFFFFFu, ready)) break;
-      }
-      if (!wait_all(bar_accfull, seg & 1u, 7)) break;
-      tc_fence_after();
-      float* my_slot = a.slots + (size_t)cta * 2 * (size_t)(NT * TILE_ROWS);   // a non-owner's part is its stripe's first segment
-      bool acc_valid[GROUPS];                                         // GI: which groups had an item in this segment
-      {
-        const int i0 = seg_begin - it_begin, len = i - i0 + 1;
-#pragma unroll
-        for (int q = 0; q < GROUPS; ++q) acc_valid[q] = (len >= GROUPS) || (((q - i0 % GROUPS + GROUPS) % GROUPS) < len);
-      }
-#pragma unroll 1
-      for (int c0 = col_lo; c0 < col_hi; c0 += 16) {
-        uint32_t v[16];
-        tc_ld16(tmem_base + lane_off + c0, v);
-        tc_wait_ld();
-        if (GI && !acc_valid[0]) {                                    // group 0 had no item in this segment
-#pragma unroll
-          for (int j = 0; j < 16; ++j) v[j] = 0;
-        }
-#pragma unroll
-        for (int q = 1; q < NACC; ++q) {
-          uint32_t w[16];
-          tc_ld16(tmem_base + lane_off + q * NT + c0, w);
-          tc_wait_ld();
-          if (!GI || acc_valid[q / APG]) {
-#pragma unroll
-            for (int j = 0; j < 16; ++j) v[j] = __float_as_uint(__uint_as_float(v[j]) + __uint_as_float(w[j]));
-          }
-        }
-        if (complete || owner) {
-          if (owner) {
-            const int m_valid = a.M - (m0 + c0);                       // tokens of this column group that exist
-            // ascending CTA order (a fixed summation order); the loads of two CTAs' slots are in flight together
-            for (int cb = c_first + 1; cb <= c_last; cb += 2) {
-              float part[2][16];
-#pragma unroll
-              for (int u = 0; u < 2; ++u) {
-                const int c = cb + u <= c_last ? cb + u : c_last;
-                const float* src = a.slots + (size_t)c * 2 * (size_t)(NT * TILE_ROWS);
-#pragma unroll
-                for (int j = 0; j < 16; ++j)
-                  part[u][j] = (cb + u <= c_last && j < m_valid) ? __ldcg(src + (c0 + j) * TILE_ROWS + row) : 0.0f;
-              }
-#pragma unroll
-              for (int u = 0; u < 2; ++u)
-#pragma unroll
-                for (int j = 0; j < 16; ++j) v[j] = __float_as_uint(__uint_as_float(v[j]) + part[u][j]);
-            }
-          }
-          if (n_out < a.g.N) {
-#pragma unroll
-            for (int j = 0; j < 16; ++j) {
-              const int m = m0 + c0 + j;
-              if (m < a.M) a.y[(size_t)m * a.g.N + n_out] = __float2bfloat16_rn(ts * __uint_as_float(v[j]));
-            }
-          }
-        } else {
-#pragma unroll
-          for (int j = 0; j < 16; ++j)
-            if (m0 + c0 + j < a.M) my_slot[(c0 + j) * TILE_ROWS + row] = __uint_as_float(v[j]);
-        }
-      }
-      tc_fence_before();
-      mbar_arrive(bar_accempty);
-      ++seg;
-      if (complete) continue;
-      if (!epi_sync()) break;                                         // every thread has read the counter / stored its part
-      if (leader) {
-        if (owner) a.counters[tile] = 0;                              // leave the counter ready for the next call
-        // release: the CTA's slot stores (ordered before this by the rendezvous) become visible with the count
-        else asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(a.counters + tile) : "memory");
-      }
-      (void)it;
+      // after the group's next item, or (a group without an item in a segment, the last segment) where there is none
+      if (pending.tile >= 0 && (turn == group || seg_last) && !epilogue()) break;
+      if (i == n_items) break;
+      if (seg_last) pending = {cur.tile, step == spt - 1};
     }
-    if (GI && issuer) drain_mmas(1 + group);
   }
 
   tc_fence_before();
@@ -592,10 +429,10 @@ size_t umma_workspace_zero_bytes(const razer_desc* d, int M) {
   return WS_STATUS_BYTES + make_plan(d, M).counters_bytes;
 }
 
-template <int NT, int CH, int STAGES, int ASTAGES, int NDW, int NACC, bool GI>
+template <int NT, int CH, int STAGES, int ASTAGES, int NDW, int NACC>
 static int launch_cfg(const CUtensorMap& tmap, const CUtensorMap& tmap_w, const UmmaArgs& args, int grid, cudaStream_t st) {
   using Cfg = UmmaCfg<NT, CH, STAGES, ASTAGES, NACC>;
-  auto kern = razer_umma_kernel<NT, CH, STAGES, ASTAGES, NDW, NACC, GI>;
+  auto kern = razer_umma_kernel<NT, CH, STAGES, ASTAGES, NDW, NACC>;
   static bool attr_set = false;
   if (!attr_set) {
     RAZER_TRY(check_cuda(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::SMEM_BYTES),
@@ -672,8 +509,8 @@ int launch_gemm_umma(const razer_desc* d, const void* packed, const void* x, int
   a.slots = (float*)((char*)ws + WS_STATUS_BYTES + p.counters_bytes);
   a.extra_scale = extra_scale_dev;
   a.g = g;
-  a.sv0 = d->sv_mag[0];
-  a.sv1 = d->sv_mag[1];
+  a.svp0 = special_value_pair(d->sv_mag[0]);
+  a.svp1 = special_value_pair(d->sv_mag[1]);
   a.mul_lo = (1u << 6) + (1u << 12);
   a.mul_hi = (1u << 2) + (1u << 8);
   a.tensor_scale = d->tensor_scale * extra_scale;
@@ -683,12 +520,11 @@ int launch_gemm_umma(const razer_desc* d, const void* packed, const void* x, int
   a.total_items = p.total_items;
   a.x_map_3d = map_3d;
   switch (p.NT) {
-    case 16:
-      return launch_cfg<16, 4, 6, 3, 12, 6, true>(tmap, tmap_w, a, p.grid, st);
-    case 32: return launch_cfg<32, 4, 6, 3, 12, 2, false>(tmap, tmap_w, a, p.grid, st);
-    case 64: return launch_cfg<64, 4, 4, 3, 12, 2, false>(tmap, tmap_w, a, p.grid, st);
-    case 128: return launch_cfg<128, 2, 4, 4, 16, 1, false>(tmap, tmap_w, a, p.grid, st);
-    default: return launch_cfg<256, 1, 5, 4, 16, 1, false>(tmap, tmap_w, a, p.grid, st);
+    case 16: return launch_cfg<16, 4, 6, 3, 12, 2>(tmap, tmap_w, a, p.grid, st);
+    case 32: return launch_cfg<32, 4, 6, 3, 12, 2>(tmap, tmap_w, a, p.grid, st);
+    case 64: return launch_cfg<64, 4, 4, 3, 12, 2>(tmap, tmap_w, a, p.grid, st);
+    case 128: return launch_cfg<128, 2, 4, 4, 16, 1>(tmap, tmap_w, a, p.grid, st);
+    default: return launch_cfg<256, 1, 5, 4, 16, 1>(tmap, tmap_w, a, p.grid, st);
   }
 }
 

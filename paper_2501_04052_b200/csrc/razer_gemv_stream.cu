@@ -49,10 +49,10 @@ __device__ __forceinline__ void strip_step(float (&acc)[4], uint32_t piece, cons
   const uint2 t0 = lds64(__byte_perm(sb, v.tbl, 0x7604) >> TABLE_SHIFT);
   const uint2 t1 = lds64(__byte_perm(sb, v.tbl, 0x7614) >> TABLE_SHIFT);
   uint32_t e0[8], e1[8];
-  decode_word2(c0.x, t0.x, t0.y, mul_lo, mul_hi, e0);
-  decode_word2(c0.y, t0.x, t0.y, mul_lo, mul_hi, e0 + 4);
-  decode_word2(c1.x, t1.x, t1.y, mul_lo, mul_hi, e1);
-  decode_word2(c1.y, t1.x, t1.y, mul_lo, mul_hi, e1 + 4);
+  decode_word(c0.x, t0.x, t0.y, mul_lo, mul_hi, e0);
+  decode_word(c0.y, t0.x, t0.y, mul_lo, mul_hi, e0 + 4);
+  decode_word(c1.x, t1.x, t1.y, mul_lo, mul_hi, e1);
+  decode_word(c1.y, t1.x, t1.y, mul_lo, mul_hi, e1 + 4);
 #pragma unroll
   for (int q = 0; q < 4; ++q) mma_16816(acc, e0[2 * q], e1[2 * q], e0[2 * q + 1], e1[2 * q + 1], xq[q][0], xq[q][1]);
 }

@@ -162,27 +162,6 @@ __device__ __forceinline__ Work make_work(const Args& a, int b) {
   return w;
 }
 
-// Four stored nibbles of each 16-bit half of `w` -> four bf16x2 registers (elements 2p, 2p + 1 of the word in
-// register p), each the exact product value x scale with the block's sign.  The special value is the one
-// nibble that is numerically zero when the isolated nibble is read as a bf16 pair: relu(nibble * -2^11 + sv')
-// is sv' = sv x 2^-126 for it and 0 for every other nibble (the smallest, 2^-133, times 2^11 already exceeds
-// the largest sv').
-__device__ __forceinline__ void decode_word2(uint32_t w, uint32_t ss2, uint32_t svp, uint32_t mul_lo, uint32_t mul_hi,
-                                             uint32_t* out) {
-  constexpr uint32_t NEG = 0xC500C500u;               // (-2048, -2048) as bf16x2
-  const uint32_t w8 = w >> 8;
-  const uint32_t n0 = w & 0x000F000Fu, n1 = w & 0x00F000F0u;
-  const uint32_t n2 = w8 & 0x000F000Fu, n3 = w8 & 0x00F000F0u;
-  const uint32_t u0 = and_or(n0 * mul_lo, 0x81C081C0u, fma_relu_bf16x2(n0, NEG, svp));
-  const uint32_t u1 = and_or(n1 * mul_hi, 0x81C081C0u, fma_relu_bf16x2(n1, NEG, svp));
-  const uint32_t u2 = and_or(n2 * mul_lo, 0x81C081C0u, fma_relu_bf16x2(n2, NEG, svp));
-  const uint32_t u3 = and_or(n3 * mul_hi, 0x81C081C0u, fma_relu_bf16x2(n3, NEG, svp));
-  out[0] = mul_bf16x2(u0, ss2);
-  out[1] = mul_bf16x2(u1, ss2);
-  out[2] = mul_bf16x2(u2, ss2);
-  out[3] = mul_bf16x2(u3, ss2);
-}
-
 // Wait for a barrier phase.  One cheap poll first; the slow path looks at the clock and the abort flag only once
 // per 32 polls and, for the service warps (SLEEP_NS > 0), sleeps between polls, so that a waiting warp costs the
 // decoding warps few issue slots.

@@ -4,7 +4,10 @@
 
 #include <cuda.h>
 #include <cuda_runtime.h>
+#include <cuda_bf16.h>
 #include <stdint.h>
+
+#include "razer_ptx.cuh"
 
 namespace razer {
 
@@ -72,6 +75,146 @@ struct ItemCursor {
     if (++astage == ASTAGES) { astage = 0; aphase ^= 1; }
   }
 };
+
+// ------------------------------------------------------------------ end of a CTA's part of an output tile
+// What both tcgen05 kernels do with the accumulator of a segment (the items of one output tile inside a CTA's stripe): a
+// tile the CTA covers completely is scaled, rounded and stored; of a partial tile every CTA but the first publishes its
+// part (FP32 slot in the workspace, then a release-add on the tile's counter), and the CTA that holds the tile's FIRST
+// items (for it the tile is the end of its stripe, for the others the beginning, so their parts were published long
+// before) adds the parts in CTA order, a fixed summation order, and stores.
+// A complete tile's accumulator goes into registers whole (rounded, two columns to a register) and is handed back to the
+// MMAs before the stores.  Nothing here may spill: with all of the SM's memory configured as shared memory a spilled
+// register is an L2 round trip (64 FP32 registers a thread, a few of them spilled, instead of 32 packed ones: 157
+// against 118 us at 2048 x 8192 x 8192 on the FP4 kernel; 124 us with the stores before the hand-back).
+struct EpilogueCtx {
+  uint32_t bar_accfull, bar_accempty, bar_epi;   // barriers (shared-window addresses)
+  uint32_t tmem;             // accumulator, with the warp's lane quarter
+  int row, group;            // the thread's weight row inside the tile; which share of the columns
+  bool leader;
+};
+
+// a: kernel arguments (y, slots, counters, g, M, token_tiles, steps_per_tile, total_items).  at_end: the segment reaches the
+// end of its tile.  GROUPS sets of four warps share the columns in units of 16.  wait(barrier, parity, which) is a bounded
+// wait of the whole warp, fail(which) records one that gave up: which = 0 accumulator, 1 rendezvous, 2 other CTAs.
+template <int NT, int NACC, int GROUPS, class KernelArgs, class Wait, class Fail>
+__device__ __forceinline__ bool segment_epilogue(const KernelArgs& a, const EpilogueCtx& x, int tile, bool at_end, float ts, uint32_t seg,
+                                                 uint32_t& epi_phase, volatile uint32_t* abort_flag, Wait wait, Fail fail) {
+  constexpr int UNITS = NT / 16, MAXC = 16 * ((UNITS + GROUPS - 1) / GROUPS);
+  constexpr size_t SLOT = (size_t)2 * NT * 128;
+  const int grid = gridDim.x, cta = blockIdx.x, spt = a.steps_per_tile;
+  const int col_lo = 16 * ((x.group * UNITS) / GROUPS), n_cols = 16 * (((x.group + 1) * UNITS) / GROUPS) - col_lo;
+  const int tile_begin = tile * spt;
+  const bool complete = (int)((a.total_items * cta) / grid) <= tile_begin && at_end;
+  const int rt = tile / a.token_tiles, m0 = (tile - rt * a.token_tiles) * NT + col_lo;
+  const int valid = min(n_cols, a.M - m0);                   // columns that are tokens
+  const int n_out = rt * 128 + x.row;
+  __nv_bfloat16* dst = a.y + (size_t)m0 * a.g.N + n_out;
+  // sixteen columns of the accumulator, summed over the NACC accumulators used in turn
+  auto load16 = [&](int c, float (&v)[16]) {
+    uint32_t w[16];
+    tc_ld16(x.tmem + col_lo + c, w);
+    tc_wait_ld();
+#pragma unroll
+    for (int j = 0; j < 16; ++j) v[j] = __uint_as_float(w[j]);
+#pragma unroll
+    for (int q = 1; q < NACC; ++q) {
+      tc_ld16(x.tmem + q * NT + col_lo + c, w);
+      tc_wait_ld();
+#pragma unroll
+      for (int j = 0; j < 16; ++j) v[j] += __uint_as_float(w[j]);
+    }
+  };
+  if (complete) {
+    if (!wait(x.bar_accfull, seg & 1u, 0)) return false;
+    tc_fence_after();
+    uint32_t packed[MAXC / 2];
+#pragma unroll
+    for (int c = 0; c < MAXC; c += 16) {
+      if (c < n_cols) {
+        float v[16];
+        load16(c, v);
+#pragma unroll
+        for (int j = 0; j < 16; j += 2) {
+          const __nv_bfloat162 p = __floats2bfloat162_rn(ts * v[j], ts * v[j + 1]);
+          packed[(c + j) / 2] = *reinterpret_cast<const uint32_t*>(&p);
+        }
+      }
+    }
+    tc_fence_before();
+    mbar_arrive(x.bar_accempty);
+    if (n_out < a.g.N) {
+#pragma unroll
+      for (int j = 0; j < MAXC; ++j) {
+        if (j < valid) *dst = __ushort_as_bfloat16((unsigned short)(packed[j / 2] >> (16 * (j & 1))));
+        dst += a.g.N;
+        asm volatile("" : "+l"(dst));                        // one running pointer, not MAXC addresses held ready
+      }
+    }
+    return true;
+  }
+  const int c_first = cta_of_item(tile_begin, grid, a.total_items);
+  const bool owner = cta == c_first;
+  int c_last = c_first;
+  if (owner) {
+    // acquire: every counted CTA's slot stores are visible to this thread's loads below
+    c_last = cta_of_item(tile_begin + spt - 1, grid, a.total_items);
+    const uint32_t others = (uint32_t)(c_last - c_first);
+    uint32_t seen = 0;
+    const uint64_t t0 = global_ns();
+    for (;;) {
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(a.counters + tile) : "memory");
+      if (seen >= others || *abort_flag || global_ns() - t0 > WAIT_LIMIT_NS) break;
+      __nanosleep(100);
+    }
+    const bool ready = seen >= others;
+    if (!ready) fail(2);
+    if (!__all_sync(0xFFFFFFFFu, ready)) return false;
+  }
+  if (!wait(x.bar_accfull, seg & 1u, 0)) return false;
+  tc_fence_after();
+  float* mine = a.slots + (size_t)cta * SLOT + col_lo * 128 + x.row;
+#pragma unroll 1
+  for (int c = 0; c < n_cols; c += 16) {
+    float v[16];
+    load16(c, v);
+    if (owner) {
+      // ascending CTA order; the loads of two CTAs' slots are in flight together
+      for (int cb = c_first + 1; cb <= c_last; cb += 2) {
+        float part[2][16];
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+          const float* src = a.slots + (size_t)min(cb + u, c_last) * SLOT + (col_lo + c) * 128 + x.row;
+#pragma unroll
+          for (int j = 0; j < 16; ++j) part[u][j] = (cb + u <= c_last && c + j < valid) ? __ldcg(src + j * 128) : 0.0f;
+        }
+#pragma unroll
+        for (int u = 0; u < 2; ++u)
+#pragma unroll
+          for (int j = 0; j < 16; ++j) v[j] += part[u][j];
+      }
+#pragma unroll
+      for (int j = 0; j < 16; ++j) {
+        if (c + j < valid && n_out < a.g.N) *dst = __float2bfloat16_rn(ts * v[j]);
+        dst += a.g.N;
+      }
+    } else {
+#pragma unroll
+      for (int j = 0; j < 16; ++j)
+        if (c + j < valid) mine[(c + j) * 128] = v[j];
+    }
+  }
+  tc_fence_before();
+  mbar_arrive(x.bar_accempty);
+  mbar_arrive(x.bar_epi);                                    // every thread has read the counter / stored its part
+  if (!wait(x.bar_epi, epi_phase & 1u, 1)) return false;
+  ++epi_phase;
+  if (x.leader) {
+    if (owner) a.counters[tile] = 0;                         // leave the counter ready for the next call
+    // release: the CTA's slot stores (ordered before this by the rendezvous) become visible with the count
+    else asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(a.counters + tile) : "memory");
+  }
+  return true;
+}
 
 // ------------------------------------------------------------------ host side
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
