@@ -9,18 +9,24 @@
 // is the hardware's UE4M3 scale factor as it stands.  The two passes are two MMAs per 64-column chunk into
 // the same TMEM accumulator; neither matrix exists in global memory.
 //
-// Mapping: the weight tile is the MMA's A operand (128 rows), the token tile its B operand (128 tokens, or 256
-// when there are more than 128), both K-major FP4 in shared memory with the 128-byte swizzle (one row = 256
-// codes = one stage of four chunks).  Warp 0 = weight producer (TMA box of packed bytes into a ring of its own,
-// released by the remap warps as soon as they have read it), warp 1 = TMEM owner and MMA issuer, warps 2..17 =
+// Mapping: the weight tile is the MMA's A operand in TMEM (128 rows = 128 lanes, 8 columns per pass and chunk), the token
+// tile its B operand (128 tokens, or 256 when there are more than 128), K-major FP4 in shared memory with the 128-byte
+// swizzle (one row = 256 codes = one stage of four chunks).  Warp 0 = weight producer (TMA box of packed bytes into a ring
+// of its own, released by the remap warps as soon as they have read it), warp 1 = TMEM owner and MMA issuer, warps 2..17 =
 // remap (thread = weight row and one of a stage's four chunks; all sixteen warps take every stage, alternating
 // between two operand slots so that one stage is remapped while the previous one is multiplied)
 // and epilogue, warp 18 = activation producer (codes by TMA, scale-factor tiles by bulk copy, into a ring
 // released by the MMAs' completion).  A remap thread reads its row's packed blocks, finds the special-value
 // nibbles (the only nibbles that are 0x0 in the packed form), builds the two code words with two integer
-// multiply-adds, applies the block's stored-negated flag to the sign bits, and writes both rows plus the row's
-// four scale bytes (scale-factor layout: 32 x 16-byte rows, row r % 32, word r / 32).  The MMA warp copies
-// the scale factors of both operands to TMEM (tcgen05.cp) and issues main and comp MMAs.
+// multiply-adds, applies the block's stored-negated flag to the sign bits, and stores both passes of its row to TMEM plus the
+// row's four scale bytes to shared memory (scale-factor layout: 32 x 16-byte rows, row r % 32, word r / 32).  The MMA warp
+// copies the scale factors of both operands to TMEM (tcgen05.cp) and issues main and comp MMAs.
+//
+// What bounds it: a stage at 256 tokens is 1028 cycles of MMA (128.5 each, measured) against 138 KB of shared-memory
+// traffic (1080 cycles at 128 B/clk) and about 1400 cycles until its remap has gone through (measured with the MMAs left
+// out).  With both passes of A written to and read from shared memory the traffic was 202 KB, and an issuing lane elected
+// anew for every stage took about 37 cycles per tcgen05 instruction: 2048 x 8192 x 8192 137 -> 118 us for A in TMEM, one
+// election and the accumulator handed back before the stores; 256 x 8192 x 8192 28.1 -> 25.6 us.
 //
 // The activation operand is prepared by a small kernel before the matmul: codes padded to whole stages with
 // the nibbles of every 32-bit word in the packed form's order (the contraction does not care about the order
@@ -47,28 +53,29 @@ constexpr int THREADS = 64 + 32 * NRW + 32;           // + W producer, MMA warp,
 constexpr int W_BYTES = CH * CHUNK_BYTES;             // 18432 packed weight bytes of a stage
 constexpr int SF_TILE_BYTES = 512;                    // scale factors of 128 rows x one chunk
 constexpr int SF_BYTES = CH * SF_TILE_BYTES;          // ... x one stage
-constexpr int A_TILE_BYTES = TILE_ROWS * 128;         // 128 rows x 256 codes
-constexpr int ASTAGE_BYTES = 2 * A_TILE_BYTES + SF_BYTES;
+constexpr int A_PASS_COLS = CH * 8;                   // TMEM columns of 128 rows x 256 codes (one pass of a stage)
+constexpr int A_COLS = 2 * A_PASS_COLS;               // main, then comp
 
 // NT = tokens per tile (the MMA's N): 128, or 256 when there are more than 128 tokens (half the weight traffic
 // and remap work per flop).
 template <int NT>
 struct Cfg {
-  static constexpr int XSTAGES = NT == 128 ? 3 : 2;               // activation ring (released by the MMAs' completion)
+  static constexpr int XSTAGES = NT == 128 ? 6 : 4;               // activation ring (released by the MMAs' completion)
   static constexpr int X_CODE_BYTES = NT * 128;
   static constexpr int X_BYTES = X_CODE_BYTES + (NT / 128) * SF_BYTES;   // codes + scale-factor tiles
   static constexpr int NACC = NT == 128 ? 2 : 1;                  // accumulators (main / comp passes apart when they fit)
   static constexpr int ACC_COLS = NACC * NT;
   static constexpr int SFB_COLS = CH * 4 * (NT / 128);
   static constexpr int SF_COLS = CH * 4 + SFB_COLS;               // per operand ring slot: A and B scale factors of a stage
+  static constexpr int SLOT_COLS = A_COLS + SF_COLS;               // operand ring slot in TMEM: A codes, scale factors
   static constexpr int TMEM_COLS = 512;
   static constexpr int NUM_BARS = 2 * WSTAGES + 2 * XSTAGES + 2 * ASTAGES + 4;
   static constexpr size_t SMEM_BYTES =
-      1024 + (size_t)WSTAGES * W_BYTES + (size_t)XSTAGES * X_BYTES + (size_t)ASTAGES * ASTAGE_BYTES + NUM_BARS * 8 + 64;
+      1024 + (size_t)WSTAGES * W_BYTES + (size_t)XSTAGES * X_BYTES + (size_t)ASTAGES * SF_BYTES + NUM_BARS * 8 + 64;
   // E2M1 x E2M1 -> FP32, UE4M3 scale factors, both operands K-major, M = 128, N = NT
   static constexpr uint32_t IDESC = (1u << 7) | (1u << 10) | ((uint32_t)(NT >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
-  static_assert(W_BYTES % 1024 == 0 && X_BYTES % 1024 == 0 && ASTAGE_BYTES % 1024 == 0, "swizzled tiles sit on 1024 bytes");
-  static_assert(ACC_COLS + ASTAGES * SF_COLS <= TMEM_COLS, "TMEM budget");
+  static_assert(W_BYTES % 1024 == 0 && X_BYTES % 1024 == 0, "swizzled tiles sit on 1024 bytes");
+  static_assert(ACC_COLS + ASTAGES * SLOT_COLS <= TMEM_COLS, "TMEM budget");
   static_assert(SMEM_BYTES <= 232448, "shared memory budget");
 };
 
@@ -86,16 +93,15 @@ struct Args {
   long long total_items;
 };
 
-// D[tmem] (+)= A[smem] * B[smem], FP4 operands with one UE4M3 scale factor per 16 elements read from TMEM.
-__device__ __forceinline__ void mma_fp4(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t desc_hi, uint32_t idesc,
+// D[tmem] (+)= A[tmem] * B[smem], FP4 operands with one UE4M3 scale factor per 16 elements read from TMEM.
+__device__ __forceinline__ void mma_fp4(uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo, uint32_t desc_hi, uint32_t idesc,
                                         uint32_t sfa_tmem, uint32_t sfb_tmem, uint32_t accumulate) {
   asm volatile(
-      "{\n\t.reg .pred p;\n\t.reg .b64 ad, bd;\n\t"
+      "{\n\t.reg .pred p;\n\t.reg .b64 bd;\n\t"
       "setp.ne.b32 p, %7, 0;\n\t"
-      "mov.b64 ad, {%1, %3};\n\t"
       "mov.b64 bd, {%2, %3};\n\t"
-      "tcgen05.mma.cta_group::1.kind::mxf4nvf4.block_scale.block16 [%0], ad, bd, %4, [%5], [%6], p;\n\t}" ::"r"(d_tmem),
-      "r"(a_lo), "r"(b_lo), "r"(desc_hi), "r"(idesc), "r"(sfa_tmem), "r"(sfb_tmem), "r"(accumulate)
+      "tcgen05.mma.cta_group::1.kind::mxf4nvf4.block_scale.block16 [%0], [%1], bd, %4, [%5], [%6], p;\n\t}" ::"r"(d_tmem),
+      "r"(a_tmem), "r"(b_lo), "r"(desc_hi), "r"(idesc), "r"(sfa_tmem), "r"(sfb_tmem), "r"(accumulate)
       : "memory");
 }
 // 32 rows x 16 bytes of shared memory -> 4 TMEM columns, the same in all four 32-lane quarters.
@@ -109,9 +115,6 @@ __device__ __forceinline__ void copy_sf_to_tmem(uint32_t tmem, uint32_t saddr) {
       "tcgen05.cp.cta_group::1.32x128b.warpx4 [%0], sd;\n\t}" ::"r"(tmem),
       "r"(lo), "r"(hi)
       : "memory");
-}
-__device__ __forceinline__ void sts128(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
-  asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
 }
 __device__ __forceinline__ void sts32(uint32_t addr, uint32_t v) {
   asm volatile("st.shared.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
@@ -137,7 +140,8 @@ struct Cursor {
 
 template <int NT>
 __global__ void __launch_bounds__(THREADS, 1)
-razer_fp4_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant__ CUtensorMap tmap_w, const Args a) {
+razer_fp4_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant__ CUtensorMap tmap_w,
+                 const __grid_constant__ Args a) {
   using C = Cfg<NT>;
   constexpr int XSTAGES = C::XSTAGES;
   constexpr int X_WARP = 2 + NRW;                       // the activation producer
@@ -145,7 +149,7 @@ razer_fp4_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_consta
   uint8_t* smem_w = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   uint8_t* smem_x = smem_w + (size_t)WSTAGES * W_BYTES;
   uint8_t* smem_a = smem_x + (size_t)XSTAGES * C::X_BYTES;
-  uint64_t* bars = reinterpret_cast<uint64_t*>(smem_a + (size_t)ASTAGES * ASTAGE_BYTES);
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem_a + (size_t)ASTAGES * SF_BYTES);
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + C::NUM_BARS);
   volatile uint32_t* abort_flag = tmem_slot + 1;
 
@@ -219,7 +223,7 @@ razer_fp4_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_consta
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
-  const uint32_t tmem_sf0 = tmem_base + C::ACC_COLS;
+  const uint32_t tmem_slot0 = tmem_base + C::ACC_COLS;
 
   auto fail = [&](uint32_t code) {
     *abort_flag = 1;
@@ -265,27 +269,22 @@ razer_fp4_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_consta
     }
   } else if (warp == 1) {
     // ===================== MMA issuer (whole warp walks the items, one elected lane issues) =====================
-    uint32_t seg = 0;
-    auto wait_warp = [&](uint32_t bar, uint32_t parity, uint32_t code) -> bool {
-      const bool got = mbar_wait(bar, parity, abort_flag);
-      if (!got) fail(code);
-      return __all_sync(0xFFFFFFFFu, got);
-    };
-    for (int i = 0; i < n_items; ++i) {
-      const bool seg_first = (i == 0) || cur.step == 0;
-      const bool seg_last = (i + 1 == n_items) || cur.step == spt - 1;
-      const int nch = min(CH, a.g.k_chunks - cur.step * CH);
-      if (!wait_warp(bar_afull + 8 * cur.as, (uint32_t)cur.aph, 23)) break;
-      if (!wait_warp(bar_xfull + 8 * cur.xs, (uint32_t)cur.xph, 30)) break;
-      if (seg_first && !wait_warp(bar_accempty, (seg & 1u) ^ 1u, 24)) break;
-      tc_fence_after();
-      const uint32_t xs = smem_u32(smem_x) + (uint32_t)cur.xs * C::X_BYTES;
-      const uint32_t sfb_s = xs + C::X_CODE_BYTES;
-      const uint32_t am = smem_u32(smem_a) + (uint32_t)cur.as * ASTAGE_BYTES;
-      const uint32_t ac = am + A_TILE_BYTES;
-      const uint32_t sfa_s = am + 2 * A_TILE_BYTES;
-      const uint32_t sf_t = tmem_sf0 + cur.as * C::SF_COLS;
-      if (elect_one()) {
+    // elected once for the whole loop: descriptors and addresses stay in uniform registers
+    if (elect_one()) {
+      uint32_t seg = 0;
+      for (int i = 0; i < n_items; ++i) {
+        const bool seg_first = (i == 0) || cur.step == 0;
+        const bool seg_last = (i + 1 == n_items) || cur.step == spt - 1;
+        const int nch = min(CH, a.g.k_chunks - cur.step * CH);
+        if (!mbar_wait(bar_afull + 8 * cur.as, (uint32_t)cur.aph, abort_flag)) { fail(23); break; }
+        if (!mbar_wait(bar_xfull + 8 * cur.xs, (uint32_t)cur.xph, abort_flag)) { fail(30); break; }
+        if (seg_first && !mbar_wait(bar_accempty, (seg & 1u) ^ 1u, abort_flag)) { fail(24); break; }
+        tc_fence_after();
+        const uint32_t xs = smem_u32(smem_x) + (uint32_t)cur.xs * C::X_BYTES;
+        const uint32_t sfb_s = xs + C::X_CODE_BYTES;
+        const uint32_t sfa_s = smem_u32(smem_a) + (uint32_t)cur.as * SF_BYTES;
+        const uint32_t am_t = tmem_slot0 + cur.as * C::SLOT_COLS, ac_t = am_t + A_PASS_COLS;
+        const uint32_t sf_t = am_t + A_COLS;
         // the stage's scale factors first, then its MMAs back to back
 #pragma unroll
         for (int c = 0; c < CH; ++c) {
@@ -302,21 +301,18 @@ razer_fp4_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_consta
         for (int c = 0; c < CH; ++c) {
           if (c < nch) {
             const uint32_t sfa_t = sf_t + c * 4, sfb_t = sf_t + CH * 4 + c * 4 * (NT / 128);
-            // 64 codes further along k: +32 bytes inside the 128-byte rows
+            // 64 codes further along k: +32 bytes inside the 128-byte rows, +8 TMEM columns
             const uint32_t b_lo = ((xs + c * 32) >> 4) | (1u << 16);
             const uint32_t first = (seg_first && c == 0) ? 0u : 1u;
-            mma_fp4(tmem_base, ((am + c * 32) >> 4) | (1u << 16), b_lo, DESC_HI, C::IDESC, sfa_t, sfb_t, first);
-            mma_fp4(tmem_base + (C::NACC - 1) * NT, ((ac + c * 32) >> 4) | (1u << 16), b_lo, DESC_HI, C::IDESC, sfa_t, sfb_t,
-                    C::NACC == 2 ? first : 1u);
+            mma_fp4(tmem_base, am_t + c * 8, b_lo, DESC_HI, C::IDESC, sfa_t, sfb_t, first);
+            mma_fp4(tmem_base + (C::NACC - 1) * NT, ac_t + c * 8, b_lo, DESC_HI, C::IDESC, sfa_t, sfb_t, C::NACC == 2 ? first : 1u);
           }
         }
         tc_commit(bar_xempty + 8 * cur.xs);
         tc_commit(bar_aempty + 8 * cur.as);
-        if (seg_last) tc_commit(bar_accfull);
+        if (seg_last) { tc_commit(bar_accfull); ++seg; }
+        cur.next(spt);
       }
-      __syncwarp();
-      if (seg_last) ++seg;
-      cur.next(spt);
     }
     // the MMAs issued so far read shared memory and TMEM until they complete: wait for them (bounded, not
     // watching the abort flag) before the CTA may release either
@@ -333,23 +329,10 @@ razer_fp4_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_consta
     // The item after it goes into the other operand slot, so its remap runs while this item's MMAs execute.
     const int chunk = (warp - 2) >> 2;
     static_assert(NRW == 4 * CH, "one set of four warps per chunk");
-    constexpr int EPI_SETS = NRW / 4;                     // sets of four warps (all lane quarters) share the columns
-    const int col_lo = 16 * ((((warp - 2) >> 2) * (NT / 16)) / EPI_SETS);
-    const int col_hi = 16 * (((((warp - 2) >> 2) + 1) * (NT / 16)) / EPI_SETS);
-    const bool leader = (threadIdx.x == 64);
-    float ts = a.tensor_scale;
-    bool dep_waited = false;
-    uint32_t seg = 0, epi_phase = 0;
     auto wait_all = [&](uint32_t bar, uint32_t parity, uint32_t code) -> bool {
       const bool got = mbar_wait(bar, parity, abort_flag);
       if (!got) fail(code);
       return __all_sync(0xFFFFFFFFu, got);
-    };
-    auto epi_sync = [&]() -> bool {
-      mbar_arrive(bar_epi);
-      const bool got = wait_all(bar_epi, epi_phase & 1u, 28);
-      ++epi_phase;
-      return got;
     };
     const int r16 = row % STRIP_ROWS;
     const uint32_t strip_off = (uint32_t)(row / STRIP_ROWS) * (CH * PIECE_BYTES);
@@ -358,21 +341,34 @@ razer_fp4_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_consta
     uint32_t code_off[CHUNK_BLOCKS];
 #pragma unroll
     for (int blk = 0; blk < CHUNK_BLOCKS; ++blk) code_off[blk] = (uint32_t)piece_code_offset(blk, r16);
-    const uint32_t row_off = (uint32_t)row * 128;        // this row inside an operand tile
-    const uint32_t sw7 = (uint32_t)row & 7u;              // 128-byte swizzle: 16-byte unit u of row r sits at u ^ (r % 8)
     const uint32_t sf_word = (uint32_t)((row & 31) * 4 + (row >> 5)) * 4;
-    for (int i = 0; i < n_items; ++i, cur.next(spt)) {
-      const int tile = cur.tile, step = cur.step;
+    // The epilogue of a finished segment runs after the next item has been prepared, so that the MMAs
+    // resume as soon as the accumulator is in registers.
+    struct Pending { int tile; bool at_end; } pending = {-1, false};
+    const EpilogueCtx ctx = {bar_accfull, bar_accempty, bar_epi, tmem_base + lane_off, row, chunk, threadIdx.x == 64};
+    uint32_t seg = 0, epi_phase = 0;
+    auto epilogue = [&]() -> bool {
+      grid_dep_wait();                                     // outputs, workspace and the scale scalar may belong to the preceding kernel
+      const float ts = a.extra_scale ? a.tensor_scale * *a.extra_scale : a.tensor_scale;
+      const int tile = pending.tile;
+      pending.tile = -1;
+      return segment_epilogue<NT, C::NACC, NRW / 4>(
+          a, ctx, tile, pending.at_end, ts, seg++, epi_phase, abort_flag,
+          [&](uint32_t bar, uint32_t parity, uint32_t which) { return wait_all(bar, parity, 27u + which); },
+          [&](uint32_t which) { fail(27u + which); });
+    };
+    for (int i = 0; i <= n_items; ++i, cur.next(spt)) {
+      const int step = cur.step;
       const bool seg_last = (i + 1 == n_items) || step == spt - 1;
       const int nch = min(CH, a.g.k_chunks - step * CH);
-      {
+      if (i < n_items) {
         // every remap thread sees every phase of the barriers it waits on, so the parity waits are sound
         if (!wait_all(bar_aempty + 8 * cur.as, (uint32_t)cur.aph ^ 1u, 26)) break;
         if (!wait_all(bar_wfull + 8 * cur.ws, (uint32_t)cur.wph, 25)) break;
         const uint32_t st = smem_addr(smem_w) + (uint32_t)cur.ws * W_BYTES + strip_off;
-        const uint32_t am = smem_addr(smem_a) + (uint32_t)cur.as * ASTAGE_BYTES + row_off;
-        const uint32_t ac = am + A_TILE_BYTES;
-        const uint32_t sfa = smem_addr(smem_a) + (uint32_t)cur.as * ASTAGE_BYTES + 2 * A_TILE_BYTES + sf_word;
+        tc_fence_after();
+        const uint32_t am_t = tmem_slot0 + cur.as * C::SLOT_COLS + lane_off;
+        const uint32_t sfa = smem_addr(smem_a) + (uint32_t)cur.as * SF_BYTES + sf_word;
         {
           const int c = chunk;
           if (c < nch) {
@@ -398,112 +394,21 @@ razer_fp4_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_consta
                 pw[2 * blk + h] = (z * rem) ^ neg8;
               }
             }
-            const uint32_t u0 = ((uint32_t)(2 * c) ^ sw7) << 4, u1 = ((uint32_t)(2 * c + 1) ^ sw7) << 4;
-            sts128(am + u0, mw[0], mw[1], mw[2], mw[3]);
-            sts128(am + u1, mw[4], mw[5], mw[6], mw[7]);
-            sts128(ac + u0, pw[0], pw[1], pw[2], pw[3]);
-            sts128(ac + u1, pw[4], pw[5], pw[6], pw[7]);
+            tc_st8(am_t + c * 8, mw);
+            tc_st8(am_t + A_PASS_COLS + c * 8, pw);
             sts32(sfa + c * SF_TILE_BYTES, sw & 0x3F3F3F3Fu);
           }
         }
         mbar_arrive(bar_wempty + 8 * cur.ws);               // the packed bytes are in registers or written out
         fence_async_smem();
+        tc_wait_st();
+        tc_fence_before();
         mbar_arrive(bar_afull + 8 * cur.as);
       }
 
-      if (!seg_last) continue;
-      // ---------------- epilogue of the segment that ends with this item ----------------
-      const int tile_begin = tile * spt;
-      const int seg_begin = it_begin > tile_begin ? it_begin : tile_begin;
-      const bool complete = (seg_begin == tile_begin) && (step == spt - 1);
-      const int rt = tile / a.token_tiles, tt = tile - rt * a.token_tiles;
-      const int n_out = rt * TILE_ROWS + row;
-      const int m0 = tt * NT;
-      if (!dep_waited) {
-        grid_dep_wait();
-        if (a.extra_scale) ts *= *a.extra_scale;
-        dep_waited = true;
-      }
-      // A partial tile is finished by its owner, the CTA whose stripe holds the tile's FIRST items: for that CTA the
-      // tile is the end of its stripe, for every other CTA of the tile it is the beginning, so their parts were
-      // published (FP32 slot in the workspace, then a release-add on the tile's counter) long before the owner gets
-      // here.  The owner adds its own accumulator (straight from TMEM) and the other parts in CTA order.
-      const int c_first = cta_of_item(tile_begin, grid, a.total_items);
-      const int c_last = cta_of_item(tile_begin + spt - 1, grid, a.total_items);
-      const bool owner = !complete && cta == c_first;
-      if (owner) {
-        // acquire: every counted CTA's slot stores are visible to this thread's loads below
-        const uint32_t others = (uint32_t)(c_last - c_first);
-        uint32_t seen = 0;
-        const uint64_t t0 = global_ns();
-        for (;;) {
-          asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(a.counters + tile) : "memory");
-          if (seen >= others || *abort_flag || global_ns() - t0 > WAIT_LIMIT_NS) break;
-          __nanosleep(200);
-        }
-        const bool ready = seen >= others;
-        if (!ready) fail(29);
-        if (!__all_sync(0xFFFFFFFFu, ready)) break;
-      }
-      if (!wait_all(bar_accfull, seg & 1u, 27)) break;
-      tc_fence_after();
-      float* my_slot = a.slots + (size_t)cta * 2 * (size_t)(NT * TILE_ROWS);   // a non-owner's part is its stripe's first segment
-#pragma unroll 1
-      for (int c0 = col_lo; c0 < col_hi; c0 += 16) {
-        uint32_t v[16];
-        tc_ld16(tmem_base + lane_off + c0, v);
-        if (C::NACC == 2) {
-          uint32_t v1[16];
-          tc_ld16(tmem_base + lane_off + NT + c0, v1);
-          tc_wait_ld();
-#pragma unroll
-          for (int j = 0; j < 16; ++j) v[j] = __float_as_uint(__uint_as_float(v[j]) + __uint_as_float(v1[j]));
-        } else {
-          tc_wait_ld();
-        }
-        if (complete || owner) {
-          if (owner) {
-            const int m_valid = a.M - (m0 + c0);                       // tokens of this column group that exist
-            // ascending CTA order (a fixed summation order); the loads of two CTAs' slots are in flight together
-            for (int cb = c_first + 1; cb <= c_last; cb += 2) {
-              float part[2][16];
-#pragma unroll
-              for (int u = 0; u < 2; ++u) {
-                const int c = cb + u <= c_last ? cb + u : c_last;
-                const float* src = a.slots + (size_t)c * 2 * (size_t)(NT * TILE_ROWS);
-#pragma unroll
-                for (int j = 0; j < 16; ++j)
-                  part[u][j] = (cb + u <= c_last && j < m_valid) ? __ldcg(src + (c0 + j) * TILE_ROWS + row) : 0.0f;
-              }
-#pragma unroll
-              for (int u = 0; u < 2; ++u)
-#pragma unroll
-                for (int j = 0; j < 16; ++j) v[j] = __float_as_uint(__uint_as_float(v[j]) + part[u][j]);
-            }
-          }
-          if (n_out < a.g.N) {
-#pragma unroll
-            for (int j = 0; j < 16; ++j) {
-              const int m = m0 + c0 + j;
-              if (m < a.M) a.y[(size_t)m * a.g.N + n_out] = __float2bfloat16_rn(ts * __uint_as_float(v[j]));
-            }
-          }
-        } else {
-#pragma unroll
-          for (int j = 0; j < 16; ++j)
-            if (m0 + c0 + j < a.M) my_slot[(c0 + j) * TILE_ROWS + row] = __uint_as_float(v[j]);
-        }
-      }
-      tc_fence_before();
-      mbar_arrive(bar_accempty);
-      ++seg;
-      if (complete) continue;
-      if (!epi_sync()) break;                                         // every thread has read the counter / stored its part
-      if (leader) {
-        if (owner) a.counters[tile] = 0;                              // leave the counter ready for the next call
-        // release: the CTA's slot stores (ordered before this by the rendezvous) become visible with the count
-        else asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(a.counters + tile) : "memory");
-      }
+      if (pending.tile >= 0 && !epilogue()) break;
+      if (i == n_items) break;
+      if (seg_last) pending = {cur.tile, step == spt - 1};
     }
   }
 
