@@ -73,8 +73,12 @@ __host__ __device__ inline Geometry make_geometry(int N, int K) {
   return g;
 }
 
-// Every matmul workspace starts with the device status word (0 = ok), on a block of its own.
+// Every matmul workspace starts with the device status word (0 = ok), on a block of its own, and the arrival counters of
+// the partial tiles, zero between calls.  The counters' place and size do not depend on the shape: what one shape keeps
+// behind them (FP32 parts) must never lie where another one has its counters.
 constexpr size_t WS_STATUS_BYTES = 256;
+constexpr size_t WS_COUNTER_BYTES = 8192;
+constexpr size_t WS_ZERO_BYTES = WS_STATUS_BYTES + WS_COUNTER_BYTES;
 
 // Layout of the FP4 activation operand as the block-scaled tensor-core kernel reads it (written by the activation
 // re-layout kernel or directly by the quantizer): codes [M][KP / 2] bytes (KP = K rounded up to whole 256-column

@@ -83,7 +83,7 @@ struct Args {
   __nv_bfloat16* y;
   const uint8_t* sfb;        // activation scale factors: [128-token tile][stage][chunk] tiles of 512 bytes
   float* slots;              // [grid][2][NT][128] FP32 partial tiles
-  uint32_t* counters;        // one per output tile, zero between calls
+  uint32_t* counters;        // one per CTA: that of the partial tile it finishes; zero between calls
   uint32_t* status;          // device status word
   const float* extra_scale;  // device scalar multiplied into the tensor scale (the activations' tensor scale)
   Geometry g;
@@ -481,7 +481,7 @@ struct Plan {
   Fp4ActLayout act;
   int grid;
   long long tiles, total_items;
-  size_t counters_bytes, slots_bytes;
+  size_t slots_bytes;
 };
 
 static Plan make_plan(const razer_desc* d, int M) {
@@ -492,7 +492,6 @@ static Plan make_plan(const razer_desc* d, int M) {
   p.total_items = p.tiles * p.act.spt;
   const int sms = sm_count();
   p.grid = (int)(p.total_items < sms ? p.total_items : sms);
-  p.counters_bytes = align256((size_t)p.tiles * sizeof(uint32_t));
   p.slots_bytes = (size_t)(p.grid > 148 ? p.grid : 148) * 2 * p.act.NT * TILE_ROWS * sizeof(float);
   return p;
 }
@@ -555,13 +554,13 @@ Fp4ActLayout make_fp4_act_layout(int M, int K) {
 // workspace of the matmul proper: status word, tile counters, partial-tile slots
 size_t gemm_fp4_core_workspace_bytes(const razer_desc* d, int M) {
   const fp4_path::Plan p = fp4_path::make_plan(d, M);
-  return WS_STATUS_BYTES + p.counters_bytes + p.slots_bytes;
+  return WS_ZERO_BYTES + p.slots_bytes;
 }
 
 // ... plus the re-laid-out activation operand when the caller brings the interchange format
 size_t gemm_fp4_workspace_bytes(const razer_desc* d, int M) {
   const fp4_path::Plan p = fp4_path::make_plan(d, M);
-  return WS_STATUS_BYTES + p.counters_bytes + p.slots_bytes + p.act.codes_bytes + p.act.sfb_bytes;
+  return WS_ZERO_BYTES + p.slots_bytes + p.act.codes_bytes + p.act.sfb_bytes;
 }
 
 // The matmul on a prepared activation operand (act_fp4: codes, then scale-factor tiles).
@@ -570,7 +569,7 @@ int launch_gemm_fp4_prepared(const razer_desc* d, const void* packed, const void
   using namespace fp4_path;
   const Geometry g = make_geometry(d->N, d->K);
   const Plan p = make_plan(d, M);
-  const size_t need = WS_STATUS_BYTES + p.counters_bytes + p.slots_bytes;
+  const size_t need = WS_ZERO_BYTES + p.slots_bytes;
   if (!ws || ws_bytes < need)
     return set_error(RAZER_ERR_WORKSPACE, "workspace of %zu bytes needed, %zu given", need, ws_bytes);
   Args a;
@@ -589,7 +588,7 @@ int launch_gemm_fp4_prepared(const razer_desc* d, const void* packed, const void
   char* base_ws = (char*)ws;
   a.status = (uint32_t*)base_ws;
   a.counters = (uint32_t*)(base_ws + WS_STATUS_BYTES);
-  a.slots = (float*)(base_ws + WS_STATUS_BYTES + p.counters_bytes);
+  a.slots = (float*)(base_ws + WS_ZERO_BYTES);
   uint8_t* codes_pad = (uint8_t*)const_cast<void*>(act_fp4);
   a.sfb = codes_pad + p.act.codes_bytes;
   a.y = (__nv_bfloat16*)y;
@@ -661,7 +660,7 @@ int launch_gemm_fp4(const razer_desc* d, const void* packed, const uint8_t* act_
                     const float* act_tensor_scale_dev, int M, void* y, void* ws, size_t ws_bytes, cudaStream_t st) {
   using namespace fp4_path;
   const Plan p = make_plan(d, M);
-  const size_t core = WS_STATUS_BYTES + p.counters_bytes + p.slots_bytes;
+  const size_t core = WS_ZERO_BYTES + p.slots_bytes;
   const size_t need = core + p.act.codes_bytes + p.act.sfb_bytes;
   if (!ws || ws_bytes < need)
     return set_error(RAZER_ERR_WORKSPACE, "workspace of %zu bytes needed, %zu given", need, ws_bytes);

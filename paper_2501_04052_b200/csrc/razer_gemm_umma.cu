@@ -66,7 +66,7 @@ struct UmmaArgs {
   const uint8_t* packed;
   __nv_bfloat16* y;
   float* slots;              // [grid][2][NT][128] FP32 partial tiles
-  uint32_t* counters;        // one per output tile, zero between calls
+  uint32_t* counters;        // one per CTA: that of the partial tile it finishes; zero between calls
   uint32_t* status;          // device status word
   const float* extra_scale;  // optional device scalar multiplied into the tensor scale
   Geometry g;
@@ -390,7 +390,7 @@ struct UmmaPlan {
   int NT, CH;
   int token_tiles, steps_per_tile, grid;
   long long tiles, total_items;
-  size_t counters_bytes, slots_bytes;
+  size_t slots_bytes;
 };
 
 static UmmaPlan make_plan(const razer_desc* d, int M) {
@@ -404,7 +404,6 @@ static UmmaPlan make_plan(const razer_desc* d, int M) {
   p.total_items = p.tiles * p.steps_per_tile;
   const int sms = sm_count();
   p.grid = (int)(p.total_items < sms ? p.total_items : sms);
-  p.counters_bytes = align256((size_t)p.tiles * sizeof(uint32_t));
   p.slots_bytes = (size_t)p.grid * 2 * p.NT * TILE_ROWS * sizeof(float);
   return p;
 }
@@ -421,12 +420,7 @@ size_t umma_workspace_bytes(const razer_desc* d, int M) {
   // sized for the largest grid (all SMs); the status word comes first
   UmmaPlan p = make_plan(d, M);
   const size_t slots = (size_t)(p.grid > 148 ? p.grid : 148) * 2 * p.NT * TILE_ROWS * sizeof(float);
-  return WS_STATUS_BYTES + p.counters_bytes + slots;
-}
-
-// Leading part of the workspace that has to be zero before a launch (status word + counters).
-size_t umma_workspace_zero_bytes(const razer_desc* d, int M) {
-  return WS_STATUS_BYTES + make_plan(d, M).counters_bytes;
+  return WS_ZERO_BYTES + slots;
 }
 
 template <int NT, int CH, int STAGES, int ASTAGES, int NDW, int NACC>
@@ -461,7 +455,7 @@ int launch_gemm_umma(const razer_desc* d, const void* packed, const void* x, int
                      const float* extra_scale_dev, void* y, void* ws, size_t ws_bytes, cudaStream_t st) {
   const Geometry g = make_geometry(d->N, d->K);
   const UmmaPlan p = make_plan(d, M);
-  const size_t need = WS_STATUS_BYTES + p.counters_bytes + p.slots_bytes;
+  const size_t need = WS_ZERO_BYTES + p.slots_bytes;
   if (!ws || ws_bytes < need)
     return set_error(RAZER_ERR_WORKSPACE, "workspace of %zu bytes needed, %zu given", need, ws_bytes);
   EncodeTiledFn enc = encode_fn();
@@ -506,7 +500,7 @@ int launch_gemm_umma(const razer_desc* d, const void* packed, const void* x, int
   a.y = (__nv_bfloat16*)y;
   a.status = (uint32_t*)ws;
   a.counters = (uint32_t*)((char*)ws + WS_STATUS_BYTES);
-  a.slots = (float*)((char*)ws + WS_STATUS_BYTES + p.counters_bytes);
+  a.slots = (float*)((char*)ws + WS_ZERO_BYTES);
   a.extra_scale = extra_scale_dev;
   a.g = g;
   a.svp0 = special_value_pair(d->sv_mag[0]);

@@ -105,8 +105,7 @@ size_t simt_workspace_bytes(const razer_desc* d, int M) {
   const Geometry g = make_geometry(d->N, d->K);
   const int MT = M >= 8 ? 8 : (M >= 4 ? 4 : (M >= 2 ? 2 : 1));
   const int s = simt_splits(g, M, MT);
-  // the first 256 bytes of every workspace hold the device status word
-  return 256 + (s > 1 ? (size_t)s * M * d->N * sizeof(float) : 0);
+  return WS_ZERO_BYTES + (s > 1 ? (size_t)s * M * d->N * sizeof(float) : 0);
 }
 
 int launch_gemv_simt(const razer_desc* d, const void* packed, const void* x, int M,
@@ -118,8 +117,8 @@ int launch_gemv_simt(const razer_desc* d, const void* packed, const void* x, int
   int cps = (g.k_chunks + splits - 1) / splits;
   cps = (cps + SIMT_GROUP_CHUNKS - 1) / SIMT_GROUP_CHUNKS * SIMT_GROUP_CHUNKS;
   const int n_splits = (g.k_chunks + cps - 1) / cps;
-  const size_t need = n_splits > 1 ? 256 + (size_t)n_splits * M * d->N * sizeof(float) : 0;
-  float* partial = ws ? reinterpret_cast<float*>(static_cast<char*>(ws) + 256) : nullptr;
+  const size_t need = n_splits > 1 ? WS_ZERO_BYTES + (size_t)n_splits * M * d->N * sizeof(float) : 0;
+  float* partial = ws ? reinterpret_cast<float*>(static_cast<char*>(ws) + WS_ZERO_BYTES) : nullptr;
   if (need > ws_bytes || (need && !ws))
     return set_error(RAZER_ERR_WORKSPACE, "workspace of %zu bytes needed, %zu given", need, ws_bytes);
   dim3 grid(g.row_tiles, n_splits, (M + MT - 1) / MT);

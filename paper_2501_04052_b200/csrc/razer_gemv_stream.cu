@@ -311,7 +311,7 @@ bool gemv_stream_supported(const razer_desc* d, int M) {
 
 size_t gemv_stream_workspace_bytes(const razer_desc* d, int M) {
   const StreamPlan p = stream_plan(d, M);
-  return WS_STATUS_BYTES + p.counters_bytes + p.slots_bytes;
+  return WS_ZERO_BYTES + p.slots_bytes;
 }
 
 template <int TM, int SPW>
@@ -342,7 +342,7 @@ static int launch_stream_cfg(const stream_path::Args& a, int grid, cudaStream_t 
 int launch_gemv_stream(const razer_desc* d, const void* packed, const void* x, int M, float extra_scale,
                        const float* extra_scale_dev, void* y, void* ws, size_t ws_bytes, cudaStream_t st) {
   const StreamPlan p = stream_plan(d, M);
-  const size_t need = WS_STATUS_BYTES + p.counters_bytes + p.slots_bytes;
+  const size_t need = WS_ZERO_BYTES + p.slots_bytes;
   if (!ws || ws_bytes < need)
     return set_error(RAZER_ERR_WORKSPACE, "workspace of %zu bytes needed, %zu given", need, ws_bytes);
   stream_path::Args a;
@@ -351,7 +351,7 @@ int launch_gemv_stream(const razer_desc* d, const void* packed, const void* x, i
   a.y = (__nv_bfloat16*)y;
   a.status = (uint32_t*)ws;
   a.counters = (uint32_t*)((char*)ws + WS_STATUS_BYTES);
-  a.slots = (float*)((char*)ws + WS_STATUS_BYTES + p.counters_bytes);
+  a.slots = (float*)((char*)ws + WS_ZERO_BYTES);
   a.extra_scale = extra_scale_dev;
   a.N = d->N;
   a.K = d->K;

@@ -15,7 +15,6 @@ namespace razer {
 int launch_gemm_umma(const razer_desc*, const void* packed, const void* x, int M, int ldx_K, float extra_scale,
                      const float* extra_scale_dev, void* y, void* ws, size_t ws_bytes, cudaStream_t);
 size_t umma_workspace_bytes(const razer_desc*, int M);
-size_t umma_workspace_zero_bytes(const razer_desc*, int M);
 
 // Every GPU that loads the library holds this array until the process exits.
 constexpr size_t STATIC_SCRATCH_BYTES = 4u << 20;
@@ -56,9 +55,9 @@ extern "C" int razer_gemv_static(const razer_desc* d, const void* packed_dev, co
   if (reinterpret_cast<uintptr_t>(packed_dev) % 16 || reinterpret_cast<uintptr_t>(x_dev) % 16 ||
       reinterpret_cast<uintptr_t>(y_dev) % 2)
     return set_error(RAZER_ERR_INVALID_ARG, "packed_dev and x_dev must be 16-byte aligned, y_dev 2-byte aligned");
-  const size_t need = umma_workspace_bytes(d, M);
-  const size_t zeroed = umma_workspace_zero_bytes(d, M);   // status word + arrival counters
-  if (need > STATIC_SCRATCH_BYTES || zeroed > need)
+  // one word per 128-row tile is counted in: the documented limit on the number of rows
+  const size_t need = umma_workspace_bytes(d, M) + (size_t)make_geometry(d->N, d->K).row_tiles * sizeof(uint32_t);
+  if (need > STATIC_SCRATCH_BYTES)
     return set_error(RAZER_ERR_UNSUPPORTED,
                      "this shape needs %zu bytes of scratch; the built-in array holds %zu (use razer_gemv with a "
                      "caller-owned workspace)", need, (size_t)STATIC_SCRATCH_BYTES);
@@ -66,6 +65,6 @@ extern "C" int razer_gemv_static(const razer_desc* d, const void* packed_dev, co
   RAZER_TRY(static_scratch(&scratch));
   cudaStream_t st = (cudaStream_t)stream;
   // The array keeps whatever the previous call left: the status word and the counters must start at zero.
-  RAZER_TRY(check_cuda(cudaMemsetAsync(scratch, 0, zeroed, st), "static scratch clear"));
+  RAZER_TRY(check_cuda(cudaMemsetAsync(scratch, 0, WS_ZERO_BYTES, st), "static scratch clear"));
   return launch_gemm_umma(d, packed_dev, x_dev, M, d->K, 1.0f, nullptr, y_dev, scratch, STATIC_SCRATCH_BYTES, st);
 }

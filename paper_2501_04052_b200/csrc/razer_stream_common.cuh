@@ -298,10 +298,8 @@ struct StreamPlan {
   int TM, SPW, grid, units, kc;
   int whole_base, whole_per_cta, rem_ctas, pieces_per_unit;
   double cost;
-  size_t counters_bytes, slots_bytes;
+  size_t slots_bytes;
 };
-
-static inline size_t align256s(size_t v) { return (v + 255) / 256 * 256; }
 
 // One candidate: units of TM strips; every CTA takes whole units only (split == false), or q whole units after a
 // piece of one of the remaining units, each of which is cut along K into equal pieces (processed first, combined
@@ -352,7 +350,6 @@ static inline StreamPlan stream_candidate(const razer_desc* d, int M, int G, int
     p.grid = (p.units + qa - 1) / qa;
     p.cost = (double)qa * p.kc * per_slice;
   }
-  p.counters_bytes = align256s((size_t)G * sizeof(uint32_t));           // at most G - 1 split units
   p.slots_bytes = (size_t)G * 2 * SLOT_FLOATS * sizeof(float);
   return p;
 }

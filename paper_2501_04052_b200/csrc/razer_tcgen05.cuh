@@ -79,7 +79,7 @@ struct ItemCursor {
 // ------------------------------------------------------------------ end of a CTA's part of an output tile
 // What both tcgen05 kernels do with the accumulator of a segment (the items of one output tile inside a CTA's stripe): a
 // tile the CTA covers completely is scaled, rounded and stored; of a partial tile every CTA but the first publishes its
-// part (FP32 slot in the workspace, then a release-add on the tile's counter), and the CTA that holds the tile's FIRST
+// part (FP32 slot in the workspace, then a release-add on the tile's counter, which is its first CTA's), and the CTA that holds the tile's FIRST
 // items (for it the tile is the end of its stripe, for the others the beginning, so their parts were published long
 // before) adds the parts in CTA order, a fixed summation order, and stores.
 // A complete tile's accumulator goes into registers whole (rounded, two columns to a register) and is handed back to the
@@ -162,7 +162,7 @@ __device__ __forceinline__ bool segment_epilogue(const KernelArgs& a, const Epil
     uint32_t seen = 0;
     const uint64_t t0 = global_ns();
     for (;;) {
-      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(a.counters + tile) : "memory");
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(a.counters + c_first) : "memory");
       if (seen >= others || *abort_flag || global_ns() - t0 > WAIT_LIMIT_NS) break;
       __nanosleep(100);
     }
@@ -209,9 +209,9 @@ __device__ __forceinline__ bool segment_epilogue(const KernelArgs& a, const Epil
   if (!wait(x.bar_epi, epi_phase & 1u, 1)) return false;
   ++epi_phase;
   if (x.leader) {
-    if (owner) a.counters[tile] = 0;                         // leave the counter ready for the next call
+    if (owner) a.counters[cta] = 0;                          // leave the counter ready for the next call
     // release: the CTA's slot stores (ordered before this by the rendezvous) become visible with the count
-    else asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(a.counters + tile) : "memory");
+    else asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(a.counters + c_first) : "memory");
   }
   return true;
 }

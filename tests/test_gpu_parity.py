@@ -565,6 +565,27 @@ def test_workspace_too_small_is_an_error(b):
         assert e.value.code == b.ERR_WORKSPACE
 
 
+def test_one_workspace_serves_all_shapes_and_token_counts_in_turn(b):
+    """A workspace prepared once serves any calls one after another: what the partial sums of one shape or kernel leave
+    behind must not be where another one has its arrival counters.  (66000 rows: more row tiles than the counters of the
+    small-batch kernel once took, so that its partial sums lay on the counters of the larger token counts.)"""
+    cases, sizes = [], []
+    for i, (N, K) in enumerate([(1024, 4096), (66000, 512), (2000, 8192)]):
+        codes, scales = inputs.random_codes(N, K, seed=180 + i)
+        desc, packed = _pack(b, codes.numpy(), scales.numpy(), 0.002)
+        for M in (2, 16, 7, 64):
+            x = inputs.activations(M, K, 190 + i).cuda()
+            cases.append((desc, packed, x, b.razer_gemv(desc, packed, x)))    # a workspace of its own
+            sizes.append(b.razer_workspace_bytes(desc, M, b.OP_GEMV))
+    ws = torch.empty(max(sizes), dtype=torch.uint8, device="cuda")
+    b.razer_workspace_init(ws)
+    for step in (1, 5, 7):                                                    # three orders of the twelve calls
+        for i in range(len(cases)):
+            desc, packed, x, want = cases[(i * step) % len(cases)]
+            assert torch.equal(b.razer_gemv(desc, packed, x, workspace=ws), want)
+    b.razer_workspace_status(ws)
+
+
 def test_weights_written_just_ahead_of_the_matmul_are_seen(b):
     """Stream-ordering contract of the header: the matmul kernels start reading the packed weights before the kernel
     directly ahead of them is known to have finished (programmatic dependent launch).  What is guaranteed: weights
