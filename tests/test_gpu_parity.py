@@ -224,6 +224,58 @@ def test_quant_act_given_scale_and_zero_input(b):
     assert ts.item() == 1.0 and not codes.any() and not scales.any()
 
 
+@pytest.mark.parametrize("log2_scale", [None, -80, 0, 80])
+@pytest.mark.parametrize("sv_mag", [5.0, 8.0, None])
+def test_quant_act_extreme_magnitudes(b, log2_scale, sv_mag):
+    """Rows from bf16 subnormals to 2^100, zero blocks among them, against the oracle: the blocks that the kernel's short form
+    cannot take go through the plain procedure, with the same decisions."""
+    M, K = 60, 272
+    x = inputs.activations(M, K, 84).float() * torch.pow(2.0, torch.linspace(-132, 100, M))[:, None]
+    x[5, 32:64] = 0.0
+    x = x.to(torch.bfloat16)
+    ts = None if log2_scale is None else torch.tensor([2.0 ** log2_scale])
+    codes, scales, out = b.razer_quant_act(x.cuda(), sv_mag=sv_mag or 0.0, tensor_scale=None if ts is None else ts.cuda())
+    with np.errstate(all="ignore"):
+        want_c, want_s, want_d, dbg = ro.quantize_act(inputs.bf16_to_bits(x), sv_mag=sv_mag and (sv_mag,), return_debug=True,
+                                                      tensor_scale=None if ts is None else np.float32(ts.item()))
+    assert np.float32(out.item()) == want_d
+    blk_ok = (scales.cpu().numpy() == want_s) & np.all((codes.cpu().numpy() == want_c).reshape(M, K // 16, 8), axis=2)
+    assert np.all(blk_ok | dbg["near_tie"])
+
+
+@pytest.mark.parametrize("block,aware", [(16, False), (16, True), (64, False), (128, True)])
+def test_quant_weight_extreme_magnitudes(b, block, aware):
+    """The same for the weight quantizer, at a given tensor scale that puts some rows' steps outside the short form."""
+    N, K = 70, 384
+    w = inputs.student_t_weights(N, K, 8, outlier_frac=0.01) * torch.pow(2.0, torch.linspace(-140, 100, N))[:, None]
+    w[3, 128:256] = 0.0
+    for log2_scale in (-70, -4, 70):
+        ts = torch.tensor([2.0 ** log2_scale])
+        codes, scales, _ = b.razer_quant_weight(w.cuda(), tensor_scale=ts.cuda(), block=block, scale_aware=aware)
+        with np.errstate(all="ignore"):
+            quantize = ro.quantize_scale_aware if aware else ro.quantize_weight
+            want_c, want_s, _, dbg = quantize(w.numpy(), tensor_scale=np.float32(ts.item()), block=block, return_debug=True)
+        blk_ok = (scales.cpu().numpy() == want_s) & np.all((codes.cpu().numpy() == want_c).reshape(N, K // block, block // 2), axis=2)
+        assert np.all(blk_ok | dbg["near_tie"])
+
+
+@pytest.mark.parametrize("N,K", [(16, 1024), (17, 1040), (31, 2032), (1, 2064)])
+def test_dequant_spans_and_unaligned_output(b, N, K):
+    """Widths at and around the sixteen chunks that a CTA lays out or decodes at a time, and outputs that are not 16-byte aligned."""
+    codes, scales = inputs.random_codes(N, K, seed=12, scale_lo=0, scale_hi=64, zero_block_frac=0.05)
+    desc, packed = _pack(b, codes.numpy(), scales.numpy(), 0.0123)
+    want1 = ro.f64_to_bf16_bits(ro.dequant_d1(codes.numpy(), scales.numpy()).astype(np.float64))
+    want2 = ro.dequant_d2(codes.numpy(), scales.numpy(), np.float32(0.0123))
+    for off in (0, 1):
+        o1 = torch.empty(N * K + 1, dtype=torch.bfloat16, device="cuda")[off:off + N * K]
+        o2 = torch.empty(N * K + 1, dtype=torch.float32, device="cuda")[off:off + N * K]
+        for out, fp32 in ((o1, 0), (o2, 1)):
+            b._check(b.lib().razer_dequant(desc, packed.data_ptr(), out.data_ptr(), fp32, None))
+        torch.cuda.synchronize()
+        assert np.array_equal(inputs.bf16_to_bits(o1.cpu()).reshape(N, K), want1)
+        assert np.array_equal(o2.cpu().numpy().view(np.uint32).reshape(N, K), want2.view(np.uint32))
+
+
 @pytest.mark.parametrize("N,K,seed,sv_mag,remap_code", [(1024, 1024, 0, (5.0, 8.0), 0x8), (200, 80, 3, (5.0, 8.0), 0x8),
                                                          (129, 4160, 5, (5.0, 9.0), 0x0), (300, 528, 6, (2.5, 12.0), 0x8)])
 def test_quant_weight_bit_exact(b, N, K, seed, sv_mag, remap_code):
