@@ -82,7 +82,7 @@ struct Cfg {
 struct Args {
   __nv_bfloat16* y;
   const uint8_t* sfb;        // activation scale factors: [128-token tile][stage][chunk] tiles of 512 bytes
-  float* slots;              // [grid][2][NT][128] FP32 partial tiles
+  float* slots;              // [grid] FP32 partial tiles of NT x 128
   uint32_t* counters;        // one per CTA: that of the partial tile it finishes; zero between calls
   uint32_t* status;          // device status word
   const float* extra_scale;  // device scalar multiplied into the tensor scale (the activations' tensor scale)
@@ -90,6 +90,7 @@ struct Args {
   float tensor_scale;
   uint32_t base0, rem0, base1, rem1;   // FP4 codes of the base value and the remainder for select 0 / 1
   int M, token_tiles, steps_per_tile;
+  int split;                 // > 1: every tile is cut evenly among this many CTAs (grid = tiles x split)
   long long total_items;
 };
 
@@ -492,7 +493,7 @@ static Plan make_plan(const razer_desc* d, int M) {
   p.total_items = p.tiles * p.act.spt;
   const int sms = sm_count();
   p.grid = (int)(p.total_items < sms ? p.total_items : sms);
-  p.slots_bytes = (size_t)(p.grid > 148 ? p.grid : 148) * 2 * p.act.NT * TILE_ROWS * sizeof(float);
+  p.slots_bytes = (size_t)(p.grid > 148 ? p.grid : 148) * p.act.NT * TILE_ROWS * sizeof(float);
   return p;
 }
 
@@ -598,6 +599,7 @@ int launch_gemm_fp4_prepared(const razer_desc* d, const void* packed, const void
   a.M = M;
   a.token_tiles = p.act.token_tiles;
   a.steps_per_tile = p.act.spt;
+  a.split = p.grid % p.tiles == 0 ? (int)(p.grid / p.tiles) : 0;
   a.total_items = p.total_items;
 
   const cuuint32_t estr[3] = {1, 1, 1};

@@ -191,6 +191,20 @@ def test_gemm_config4_full_size_every_output(b):
     _check_matmul(b, b.razer_gemm, desc, packed, codes, scales, 0.002, x)
 
 
+@pytest.mark.parametrize("M,N,K", [(9, 108, 1344), (9, 137, 64), (17, 672, 3264), (150, 132, 64), (33, 1049, 1904), (33, 3914, 80),
+                                   (65, 666, 1920), (65, 2299, 80), (100, 4750, 3376), (100, 5457, 80), (300, 2323, 3456),
+                                   (333, 3093, 4704), (150, 4968, 80), (200, 3116, 3392), (512, 3178, 4480), (400, 5620, 80),
+                                   (2048, 19000, 80)])
+def test_gemm_token_tiles_and_partitions(b, M, N, K):
+    """Every token tile of the tcgen05 kernel (16, 32, 64, 96, 128, 192, 256) with tiles that stay on one CTA, tiles cut evenly
+    among several CTAs, and stripes, as the host picks them for these sizes; ragged in every dimension."""
+    codes, scales = inputs.random_codes(N, K, seed=74)
+    codes, scales = codes.numpy(), scales.numpy()
+    desc, packed = _pack(b, codes, scales, 0.002)
+    x = inputs.activations(M, K, 75, outlier_channel_frac=0.01)
+    _check_matmul(b, b.razer_gemm, desc, packed, codes, scales, 0.002, x, rows=rows_with_edge_tiles(N, 96, 76))
+
+
 # ------------------------------------------------------------------ activation quantization / W4A4
 
 @pytest.mark.parametrize("M,K,seed", [(256, 8192, 80), (7, 48, 81), (33, 1040, 82)])
