@@ -91,8 +91,15 @@ def _check(rc: int) -> None:
         raise RazerError(rc, last_error())
 
 
-def _stream() -> int:
-    return torch.cuda.current_stream().cuda_stream
+# The current device's current stream as a raw pointer: building a torch.cuda.Stream object for it takes 3.3 us of an 8.3 us
+# call, this 0.1 us.
+_raw_stream, _device = getattr(torch._C, "_cuda_getCurrentRawStream", None), getattr(torch._C, "_cuda_getDevice", None)
+if _raw_stream is not None and _device is not None:
+    def _stream() -> int:
+        return _raw_stream(_device())
+else:
+    def _stream() -> int:
+        return torch.cuda.current_stream().cuda_stream
 
 
 def _ptr(t) -> int:
