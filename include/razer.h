@@ -142,7 +142,9 @@ int razer_gemm(const razer_desc* d, const void* packed_dev, const void* x_dev, i
  * x_host / y_host should be pinned for the copies to be asynchronous.  When y_host is
  * pinned memory that the device can address (what cudaHostAlloc / cudaHostRegister give
  * under unified addressing), the kernel stores y straight into it and y_stage_dev is not
- * touched; otherwise y goes through y_stage_dev and one more copy. */
+ * touched; otherwise y goes through y_stage_dev and one more copy.  Pinned x_host of up to 256 KB on a
+ * 16-byte boundary is fetched by a kernel instead of a copy.  Each calling thread keeps 64 bytes of pinned host memory
+ * (the workspace's status is shown there) until it ends. */
 int razer_gemv_host(const razer_desc* d, const void* packed_dev, const void* x_host, int M,
                     void* y_host, void* x_stage_dev, void* y_stage_dev, void* workspace_dev,
                     size_t workspace_bytes, void* stream);

@@ -65,6 +65,7 @@ static int check_ptr(const void* p, size_t align, const char* name) {
 // kernels' host launchers (defined next to the kernels)
 int launch_pack(const razer_desc*, const uint8_t*, const uint8_t*, void*, cudaStream_t);
 int launch_dequant(const razer_desc*, const void*, void*, int, cudaStream_t);
+int launch_copy_from_host(const void*, void*, size_t, cudaStream_t);
 int launch_decode_act(const uint8_t*, const uint8_t*, int, int, float, void*, cudaStream_t);
 int launch_quant_weight(const float*, int, int, int, int, float, float, int, const float*, uint32_t*, uint8_t*,
                         uint8_t*, float*, cudaStream_t);
@@ -79,11 +80,11 @@ size_t gemm_fp4_workspace_bytes(const razer_desc*, int M);
 int launch_gemm_fp4_prepared(const razer_desc*, const void*, const void*, const float*, int, void*, void*, size_t, cudaStream_t);
 int launch_quant_act_fp4(const void*, int, int, const float*, uint32_t*, void*, float*, cudaStream_t);
 int launch_gemm_umma(const razer_desc*, const void* packed, const void* x, int M, int ldx_K, float extra_scale,
-                     const float* extra_scale_dev, void* y, void* ws, size_t ws_bytes, cudaStream_t);
+                     const float* extra_scale_dev, void* y, void* ws, size_t ws_bytes, cudaStream_t, uint32_t* status_host);
 size_t umma_workspace_bytes(const razer_desc*, int M);
 bool umma_supported(const razer_desc*, int M);
 int launch_gemv_stream(const razer_desc*, const void* packed, const void* x, int M, float extra_scale,
-                       const float* extra_scale_dev, void* y, void* ws, size_t ws_bytes, cudaStream_t);
+                       const float* extra_scale_dev, void* y, void* ws, size_t ws_bytes, cudaStream_t, uint32_t* status_host);
 size_t gemv_stream_workspace_bytes(const razer_desc*, int M);
 bool gemv_stream_supported(const razer_desc*, int M);
 
@@ -197,16 +198,16 @@ int razer_workspace_status(const void* workspace_dev, void* stream) {
 
 static int matmul_common(const razer_desc* d, const void* packed_dev, const void* x_dev, int M, void* y_dev,
                          void* ws, size_t ws_bytes, float extra_scale, const float* extra_scale_dev,
-                         cudaStream_t st) {
+                         cudaStream_t st, uint32_t* status_host = nullptr) {
   RAZER_TRY(check_ptr(packed_dev, 16, "packed_dev"));
   RAZER_TRY(check_ptr(x_dev, 16, "x_dev"));
   RAZER_TRY(check_ptr(y_dev, 2, "y_dev"));
   if (ws && reinterpret_cast<uintptr_t>(ws) % 256)
     return set_error(RAZER_ERR_INVALID_ARG, "workspace is not 256-byte aligned");
   if (use_stream(d, M))
-    return launch_gemv_stream(d, packed_dev, x_dev, M, extra_scale, extra_scale_dev, y_dev, ws, ws_bytes, st);
+    return launch_gemv_stream(d, packed_dev, x_dev, M, extra_scale, extra_scale_dev, y_dev, ws, ws_bytes, st, status_host);
   if (umma_supported(d, M))
-    return launch_gemm_umma(d, packed_dev, x_dev, M, d->K, extra_scale, extra_scale_dev, y_dev, ws, ws_bytes, st);
+    return launch_gemm_umma(d, packed_dev, x_dev, M, d->K, extra_scale, extra_scale_dev, y_dev, ws, ws_bytes, st, status_host);
   razer_desc dd = *d;
   dd.tensor_scale = d->tensor_scale * extra_scale;
   return launch_gemv_simt(&dd, packed_dev, x_dev, M, extra_scale_dev, y_dev, ws, ws_bytes, st);
@@ -228,6 +229,52 @@ int razer_gemm(const razer_desc* d, const void* packed_dev, const void* x_dev, i
                        (cudaStream_t)stream);
 }
 
+}  // extern "C"
+
+namespace razer {
+// Device address of pinned host memory, or NULL.
+static void* device_view(const void* host) {
+  cudaPointerAttributes at;
+  if (cudaPointerGetAttributes(&at, host) != cudaSuccess) {
+    cudaGetLastError();                                      // not a CUDA-known pointer
+    return nullptr;
+  }
+  return at.type == cudaMemoryTypeHost ? at.devicePointer : nullptr;
+}
+
+// A pinned word of the calling thread in which a kernel shows that a wait gave up; given back when the thread ends.
+struct HostStatus {
+  volatile uint32_t* word = nullptr;
+  uint32_t* device_word = nullptr;
+  bool tried = false;
+  bool ready() {
+    if (!tried) {
+      tried = true;
+      void *h = nullptr, *v = nullptr;
+      if (cudaHostAlloc(&h, 64, cudaHostAllocPortable | cudaHostAllocMapped) == cudaSuccess) {
+        if (cudaHostGetDevicePointer(&v, h, 0) == cudaSuccess) {
+          word = (volatile uint32_t*)h;
+          device_word = (uint32_t*)v;
+        } else {
+          cudaFreeHost(h);
+        }
+      }
+      if (!word) cudaGetLastError();                         // the copy serves instead
+    }
+    return word != nullptr;
+  }
+  ~HostStatus() {
+    if (word) cudaFreeHost((void*)word);
+  }
+};
+
+// Up to here a kernel fetches x over the bus; beyond, the copy engine.
+constexpr size_t HOST_X_KERNEL_BYTES = 256 * 1024;
+static bool use_simt(const razer_desc* d, int M) { return !use_stream(d, M) && !umma_supported(d, M); }
+}  // namespace razer
+
+extern "C" {
+
 int razer_gemv_host(const razer_desc* d, const void* packed_dev, const void* x_host, int M, void* y_host,
                     void* x_stage_dev, void* y_stage_dev, void* workspace_dev, size_t workspace_bytes,
                     void* stream) {
@@ -237,25 +284,32 @@ int razer_gemv_host(const razer_desc* d, const void* packed_dev, const void* x_h
   RAZER_TRY(check_ptr(x_stage_dev, 16, "x_stage_dev"));
   RAZER_TRY(check_ptr(y_stage_dev, 2, "y_stage_dev"));
   cudaStream_t st = (cudaStream_t)stream;
-  // pinned host memory that the device can address takes the kernel's stores directly (no copy back)
-  void* y_target = y_stage_dev;
-  {
-    cudaPointerAttributes at;
-    if (cudaPointerGetAttributes(&at, y_host) == cudaSuccess) {
-      if (at.type == cudaMemoryTypeHost && at.devicePointer) y_target = at.devicePointer;
-    } else {
-      cudaGetLastError();                                    // not a CUDA-known pointer: use the staging buffer
-    }
+  // Pinned host memory that the device can address takes the kernel's stores directly (no copy back), and gives x to a small
+  // kernel that the matmul can follow as a dependent launch: a copy of a few KB by the copy engine costs about 6 us of this call.
+  void* y_mapped = device_view(y_host);
+  void* x_mapped = device_view(x_host);
+  void* y_target = y_mapped ? y_mapped : y_stage_dev;
+  const size_t x_bytes = (size_t)M * d->K * 2;
+  if (x_mapped && reinterpret_cast<uintptr_t>(x_mapped) % 16 == 0 && x_bytes <= HOST_X_KERNEL_BYTES)
+    RAZER_TRY(launch_copy_from_host(x_mapped, x_stage_dev, x_bytes, st));
+  else
+    RAZER_TRY(check_cuda(cudaMemcpyAsync(x_stage_dev, x_host, x_bytes, cudaMemcpyHostToDevice, st), "copy of x to the device"));
+  static thread_local HostStatus status;
+  if (!workspace_dev || use_simt(d, M) || !status.ready()) {               // no status word, or no way to see it but a copy
+    RAZER_TRY(matmul_common(d, packed_dev, x_stage_dev, M, y_target, workspace_dev, workspace_bytes, 1.0f, nullptr, st));
+    if (!y_mapped)
+      RAZER_TRY(check_cuda(cudaMemcpyAsync(y_host, y_stage_dev, (size_t)M * d->N * 2, cudaMemcpyDeviceToHost, st), "copy of y to the host"));
+    if (workspace_dev) return razer_workspace_status(workspace_dev, stream);   // synchronizes
+    return check_cuda(cudaStreamSynchronize(st), "stream synchronize");
   }
-  RAZER_TRY(check_cuda(cudaMemcpyAsync(x_stage_dev, x_host, (size_t)M * d->K * 2, cudaMemcpyHostToDevice, st),
-                       "copy of x to the device"));
-  RAZER_TRY(matmul_common(d, packed_dev, x_stage_dev, M, y_target, workspace_dev, workspace_bytes, 1.0f,
-                          nullptr, st));
-  if (y_target == y_stage_dev)
-    RAZER_TRY(check_cuda(cudaMemcpyAsync(y_host, y_stage_dev, (size_t)M * d->N * 2, cudaMemcpyDeviceToHost, st),
-                         "copy of y to the host"));
-  if (workspace_dev) return razer_workspace_status(workspace_dev, stream);   // synchronizes
-  return check_cuda(cudaStreamSynchronize(st), "stream synchronize");
+  // The kernel shows a status other than 0 in a host word too, so that the common case needs no copy of it (11 us).
+  *status.word = 0;
+  RAZER_TRY(matmul_common(d, packed_dev, x_stage_dev, M, y_target, workspace_dev, workspace_bytes, 1.0f, nullptr, st, status.device_word));
+  if (!y_mapped)
+    RAZER_TRY(check_cuda(cudaMemcpyAsync(y_host, y_stage_dev, (size_t)M * d->N * 2, cudaMemcpyDeviceToHost, st), "copy of y to the host"));
+  RAZER_TRY(check_cuda(cudaStreamSynchronize(st), "stream synchronize"));
+  const uint32_t code = *status.word;
+  return code == 0 ? RAZER_OK : set_error(RAZER_ERR_DEVICE_TIMEOUT, "a device-side wait gave up (wait id %u)", code);
 }
 
 int razer_quant_act(const void* x_dev, int M, int K, float sv_mag, const float* tensor_scale_in_dev,

@@ -64,6 +64,7 @@ struct UmmaArgs {
   float* slots;              // [grid] FP32 partial tiles of NT x 128
   uint32_t* counters;        // one per CTA: that of the partial tile it finishes; zero between calls
   uint32_t* status;          // device status word
+  uint32_t* status_host;     // the same for a host that waits for this call (pinned memory), or NULL
   const float* extra_scale;  // optional device scalar multiplied into the tensor scale
   Geometry g;
   uint32_t svp0, svp1;       // special-value pairs for select 0 / 1 (razer_decode.cuh)
@@ -214,6 +215,7 @@ razer_umma_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
     *abort_flag = 1;
     grid_dep_wait();                                      // the status word lives in the (possibly shared) workspace
     atomicCAS(a.status, 0u, code);
+    show_status(a.status_host, code);
   };
 
   if (warp == 0) {
@@ -233,6 +235,7 @@ razer_umma_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
     if (lane == 0) {
       asm volatile("prefetch.tensormap [%0];" ::"l"(&tmap_x) : "memory");
       grid_dep_wait();                                    // activations may belong to the preceding kernel
+      if (cta == 0 && a.status_host) show_status(a.status_host, *(volatile uint32_t*)a.status);   // what an earlier call left
       Ring<XST> xr;
       int done = 0;                                       // stages
       bool alive = true;
@@ -542,7 +545,7 @@ static int launch_cfg(const CUtensorMap& tmap, const CUtensorMap& tmap_w, const 
 }
 
 int launch_gemm_umma(const razer_desc* d, const void* packed, const void* x, int M, int ldx_K, float extra_scale,
-                     const float* extra_scale_dev, void* y, void* ws, size_t ws_bytes, cudaStream_t st) {
+                     const float* extra_scale_dev, void* y, void* ws, size_t ws_bytes, cudaStream_t st, uint32_t* status_host) {
   const Geometry g = make_geometry(d->N, d->K);
   const UmmaPlan p = make_plan(d, M);
   const size_t need = WS_ZERO_BYTES + p.slots_bytes;
@@ -591,6 +594,7 @@ int launch_gemm_umma(const razer_desc* d, const void* packed, const void* x, int
   a.status = (uint32_t*)ws;
   a.counters = (uint32_t*)((char*)ws + WS_STATUS_BYTES);
   a.slots = (float*)((char*)ws + WS_ZERO_BYTES);
+  a.status_host = status_host;
   a.extra_scale = extra_scale_dev;
   a.g = g;
   a.svp0 = special_value_pair(d->sv_mag[0]);

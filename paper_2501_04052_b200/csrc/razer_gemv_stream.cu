@@ -175,7 +175,7 @@ __global__ void __launch_bounds__(THREADS, OCC) razer_stream_kernel(const Args a
   grid_dep_launch();                                          // the next launch of the stream may become resident
   __syncthreads();
   if (stages < 2) {                                           // cannot happen with the sizes the host admits
-    if (threadIdx.x == 0) { grid_dep_wait(); atomicCAS(a.status, 0u, 20u); }
+    if (threadIdx.x == 0) { grid_dep_wait(); atomicCAS(a.status, 0u, 20u); show_status(a.status_host, 20u); }
     return;
   }
 
@@ -183,6 +183,7 @@ __global__ void __launch_bounds__(THREADS, OCC) razer_stream_kernel(const Args a
     *abort_flag = 1;
     grid_dep_wait();                                          // the status word lives in the (possibly shared) workspace
     atomicCAS(a.status, 0u, code);
+    show_status(a.status_host, code);
   };
 
   if (warp == 0) {
@@ -213,6 +214,7 @@ __global__ void __launch_bounds__(THREADS, OCC) razer_stream_kernel(const Args a
   } else if (warp == 1) {
     // ===================== epilogue: add the consumer warps' partial sums, write y, combine split units =====================
     grid_dep_wait();                                          // y, workspace and the scale scalar may belong to the preceding kernel
+    if (b == 0 && lane == 0 && a.status_host) show_status(a.status_host, *(volatile uint32_t*)a.status);   // what an earlier call left
     float ts = a.tensor_scale;
     if (a.extra_scale) ts *= *a.extra_scale;
     epilogue_loop<C::ROWS>(a, work, b, lane, red, bar_red_full, bar_red_free, abort_flag, ts, fail);
@@ -340,7 +342,7 @@ static int launch_stream_cfg(const stream_path::Args& a, int grid, cudaStream_t 
 }
 
 int launch_gemv_stream(const razer_desc* d, const void* packed, const void* x, int M, float extra_scale,
-                       const float* extra_scale_dev, void* y, void* ws, size_t ws_bytes, cudaStream_t st) {
+                       const float* extra_scale_dev, void* y, void* ws, size_t ws_bytes, cudaStream_t st, uint32_t* status_host) {
   const StreamPlan p = stream_plan(d, M);
   const size_t need = WS_ZERO_BYTES + p.slots_bytes;
   if (!ws || ws_bytes < need)
@@ -352,6 +354,7 @@ int launch_gemv_stream(const razer_desc* d, const void* packed, const void* x, i
   a.status = (uint32_t*)ws;
   a.counters = (uint32_t*)((char*)ws + WS_STATUS_BYTES);
   a.slots = (float*)((char*)ws + WS_ZERO_BYTES);
+  a.status_host = status_host;
   a.extra_scale = extra_scale_dev;
   a.N = d->N;
   a.K = d->K;

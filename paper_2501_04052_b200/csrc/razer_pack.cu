@@ -215,6 +215,36 @@ int launch_dequant(const razer_desc* d, const void* packed, void* out, int fp32,
   return check_cuda(cudaGetLastError(), "dequant_kernel launch");
 }
 
+// Up to a few hundred KB from pinned host memory, read over the bus, one 16-byte load a thread.  Bound by the bus's round trip;
+// it replaces a copy by the copy engine, whose start and hand-over to the next kernel cost more than the transfer.
+__global__ void __launch_bounds__(128) copy_from_host_kernel(const uint4* __restrict__ src, uint4* __restrict__ dst, int n) {
+  const int i = (int)(blockIdx.x * blockDim.x + threadIdx.x);
+  grid_dep_wait();                                        // source and destination may belong to the preceding kernel
+  grid_dep_launch();                                      // only now: the matmul behind reads packed weights at once
+  if (i < n) {
+    uint4 v;                                              // volatile: the host may have changed it since an earlier call
+    asm volatile("ld.volatile.global.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(src + i));
+    dst[i] = v;
+  }
+}
+
+int launch_copy_from_host(const void* src, void* dst, size_t bytes, cudaStream_t st) {
+  static const bool pdl = [] { const char* e = getenv("RAZER_PDL"); return !(e && e[0] == '0'); }();
+  const int n = (int)(bytes / 16);                                     // K is a multiple of 16 elements
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)((n + 127) / 128));
+  cfg.blockDim = dim3(128);
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = pdl ? 1 : 0;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, copy_from_host_kernel, (const uint4*)src, (uint4*)dst, n);
+  count_launches(1);
+  return check_cuda(e, "copy_from_host_kernel launch");
+}
+
 int launch_decode_act(const uint8_t* codes, const uint8_t* scales, int M, int K, float sv_mag,
                       void* out, cudaStream_t st) {
   const long long nb = (long long)M * (K / 16);

@@ -89,4 +89,9 @@ __device__ __forceinline__ bool elect_one() {
 __device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
+// A status other than 0 for a host that waits on the call (`host`: pinned memory, or NULL).
+__device__ __forceinline__ void show_status(uint32_t* host, uint32_t code) {
+  if (host && code) *(volatile uint32_t*)host = code;
+}
+
 }  // namespace razer

@@ -13,7 +13,7 @@
 namespace razer {
 
 int launch_gemm_umma(const razer_desc*, const void* packed, const void* x, int M, int ldx_K, float extra_scale,
-                     const float* extra_scale_dev, void* y, void* ws, size_t ws_bytes, cudaStream_t);
+                     const float* extra_scale_dev, void* y, void* ws, size_t ws_bytes, cudaStream_t, uint32_t* status_host);
 size_t umma_workspace_bytes(const razer_desc*, int M);
 
 // Every GPU that loads the library holds this array until the process exits.
@@ -66,5 +66,5 @@ extern "C" int razer_gemv_static(const razer_desc* d, const void* packed_dev, co
   cudaStream_t st = (cudaStream_t)stream;
   // The array keeps whatever the previous call left: the status word and the counters must start at zero.
   RAZER_TRY(check_cuda(cudaMemsetAsync(scratch, 0, WS_ZERO_BYTES, st), "static scratch clear"));
-  return launch_gemm_umma(d, packed_dev, x_dev, M, d->K, 1.0f, nullptr, y_dev, scratch, STATIC_SCRATCH_BYTES, st);
+  return launch_gemm_umma(d, packed_dev, x_dev, M, d->K, 1.0f, nullptr, y_dev, scratch, STATIC_SCRATCH_BYTES, st, nullptr);
 }

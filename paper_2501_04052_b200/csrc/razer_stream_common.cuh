@@ -54,6 +54,7 @@ struct Args {
   float* slots;              // [grid][2][SLOT_FLOATS]
   uint32_t* counters;        // one per split unit, zero between calls
   uint32_t* status;          // device status word
+  uint32_t* status_host;     // the same for a host that waits for this call (pinned memory), or NULL
   const float* extra_scale;  // optional device scalar multiplied into the tensor scale
   int N, K, kc, M;
   int units;                 // units of TM strips that hold rows < N

@@ -618,6 +618,27 @@ def test_gemv_host_entry_point(b, pinned, M, N, K):
         y.fill_(float("nan"))
 
 
+@pytest.mark.parametrize("M,N,K,offset", [(1, 300, 528, 0), (2, 300, 528, 4), (64, 256, 2048, 0), (64, 256, 2064, 0)])
+def test_gemv_host_routes_of_x(b, M, N, K, offset):
+    """x fetched by a kernel, or copied because it is not on a 16-byte boundary or larger than 256 KB; new values in the same host
+    buffer on the second call; a status that an earlier call left in the workspace is reported."""
+    codes, scales = inputs.random_codes(N, K, seed=99)
+    desc, packed = _pack(b, codes.numpy(), scales.numpy(), 0.01)
+    buf = torch.empty(M * K + offset, dtype=torch.bfloat16).pin_memory()
+    x = buf[offset:].view(M, K)
+    y = torch.empty((M, N), dtype=torch.bfloat16).pin_memory()
+    xs, ys = torch.empty((M, K), dtype=torch.bfloat16, device="cuda"), torch.empty((M, N), dtype=torch.bfloat16, device="cuda")
+    ws = b.alloc_workspace(desc, M, b.OP_GEMV, "cuda")
+    for seed in (99, 100):
+        x.copy_(inputs.activations(M, K, seed))
+        b.razer_gemv_host(desc, packed, x, y, xs, ys, ws)
+        assert torch.equal(y, b.razer_gemv(desc, packed, x.cuda()).cpu())
+    ws[:4] = torch.tensor([7, 0, 0, 0], dtype=torch.uint8)
+    with pytest.raises(b.RazerError) as e:
+        b.razer_gemv_host(desc, packed, x, y, xs, ys, ws)
+    assert e.value.code == b.ERR_DEVICE_TIMEOUT and "7" in str(e.value)
+
+
 def test_workspace_too_small_is_an_error(b):
     N, K = 512, 4096
     codes, scales = inputs.random_codes(N, K, seed=98)
