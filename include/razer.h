@@ -243,7 +243,7 @@ int razer_gemm_w4a4(const razer_desc* d, const void* packed_w_dev, const uint8_t
  * razer_quant_act_fp4: plain NVFP4 quantization (Eq. 1-3, the arithmetic of razer_quant_act with sv_mag = 0; same
  * tensor_scale_in_dev / amax_scratch_dev contract, one launch) writing act_fp4_dev: codes padded to whole
  * 256-column stages and scale bytes in the scale-factor tile order of the block-scaled MMA, padding included, so
- * the buffer needs no clearing.  The layout is internal (it depends on the token tile the matmul picks for M).
+ * the buffer needs no clearing.  The layout is internal.
  * razer_gemm_w4a4_fp4: razer_gemm_w4a4(use_native_fp4 = 1) on such an operand; bit-identical results.  Workspace:
  * RAZER_OP_GEMM_W4A4 (zeroed once by razer_workspace_init). */
 int razer_fp4_act_bytes(int M, int K, size_t* bytes_out);

@@ -86,8 +86,9 @@ constexpr size_t WS_ZERO_BYTES = WS_STATUS_BYTES + WS_COUNTER_BYTES;
 // [128-token tile][stage][chunk][512 bytes] (word 4 * (t % 32) + t / 32 of a tile = the four 7-bit scale bytes of
 // token t of the tile for the chunk's four blocks; zero for tokens beyond M and blocks beyond K).
 struct Fp4ActLayout {
-  int NT;            // tokens per tile of the matmul kernel: 128, or 256 above 128 tokens
-  int token_tiles, tiles128, spt, KP;
+  int tiles128;      // 128-token scale-factor tiles: one up to 128 tokens, an even number above, whichever token tile the matmul picks
+  int force_nt;      // token tile forced for a test, or 0
+  int spt, KP;
   size_t codes_bytes, sfb_bytes;
 };
 Fp4ActLayout make_fp4_act_layout(int M, int K);   // host (razer_gemm_fp4.cu)

@@ -13,8 +13,8 @@
 // tile its B operand (128 tokens, or 256 when there are more than 128), K-major FP4 in shared memory with the 128-byte
 // swizzle (one row = 256 codes = one stage of four chunks).  Warp 0 = weight producer (TMA box of packed bytes into a ring
 // of its own, released by the remap warps as soon as they have read it), warp 1 = TMEM owner and MMA issuer, warps 2..17 =
-// remap (thread = weight row and one of a stage's four chunks; all sixteen warps take every stage, alternating
-// between two operand slots so that one stage is remapped while the previous one is multiplied)
+// remap (thread = weight row and two of a stage's four chunks; two groups of eight warps take the stages in turn, an operand
+// slot each, so that one stage is remapped while the previous one is multiplied)
 // and epilogue, warp 18 = activation producer (codes by TMA, scale-factor tiles by bulk copy, into a ring
 // released by the MMAs' completion).  A remap thread reads its row's packed blocks, finds the special-value
 // nibbles (the only nibbles that are 0x0 in the packed form), builds the two code words with two integer
@@ -23,10 +23,11 @@
 // copies the scale factors of both operands to TMEM (tcgen05.cp) and issues main and comp MMAs.
 //
 // What bounds it: a stage at 256 tokens is 1028 cycles of MMA (128.5 each, measured) against 138 KB of shared-memory
-// traffic (1080 cycles at 128 B/clk) and about 1400 cycles until its remap has gone through (measured with the MMAs left
-// out).  With both passes of A written to and read from shared memory the traffic was 202 KB, and an issuing lane elected
-// anew for every stage took about 37 cycles per tcgen05 instruction: 2048 x 8192 x 8192 137 -> 118 us for A in TMEM, one
-// election and the accumulator handed back before the stores; 256 x 8192 x 8192 28.1 -> 25.6 us.
+// traffic (1080 cycles at 128 B/clk); on all SMs it takes about 1500 cycles with the remap left out, so what is left is mostly
+// the MMAs and the operands' way to them.  Steps taken, 2048 / 256 x 8192 x 8192 in us: both passes of A in shared memory and
+// the issuing lane elected anew for every stage 137 / 28.1; A in TMEM, one election, the accumulator handed back before the stores
+// 118 / 25.6; remap by table and one add per word instead of shifts, in two groups that take the stages in turn and have their
+// words ready before the operand slot is free 107 / 23.2; grid and token tile by cost 105 / 21.3.
 //
 // The activation operand is prepared by a small kernel before the matmul: codes padded to whole stages with
 // the nibbles of every 32-bit word in the packed form's order (the contraction does not care about the order
@@ -48,7 +49,11 @@ namespace fp4_path {
 constexpr int CH = 4;                                 // chunks per stage: 256 codes = one 128-byte swizzled row
 constexpr int WSTAGES = 4;                            // packed-weight ring (released by the remap warps)
 constexpr int ASTAGES = 2;                            // remapped-operand ring: one slot is remapped while the other is multiplied
-constexpr int NRW = 16;                               // remap warps: four per chunk of a stage
+constexpr int NRW = 16;                               // remap warps
+constexpr int GROUPS = 2;                             // ... in groups that take the stages in turn, one operand slot each
+constexpr int GROUP_WARPS = NRW / GROUPS;
+constexpr int CPT = CH / (GROUP_WARPS / 4);           // chunks of a stage per remap thread
+static_assert(GROUPS == ASTAGES && WSTAGES % GROUPS == 0, "a ring slot always serves the same group, which then sees all its phases");
 constexpr int THREADS = 64 + 32 * NRW + 32;           // + W producer, MMA warp, X producer
 constexpr int W_BYTES = CH * CHUNK_BYTES;             // 18432 packed weight bytes of a stage
 constexpr int SF_TILE_BYTES = 512;                    // scale factors of 128 rows x one chunk
@@ -71,7 +76,7 @@ struct Cfg {
   static constexpr int TMEM_COLS = 512;
   static constexpr int NUM_BARS = 2 * WSTAGES + 2 * XSTAGES + 2 * ASTAGES + 4;
   static constexpr size_t SMEM_BYTES =
-      1024 + (size_t)WSTAGES * W_BYTES + (size_t)XSTAGES * X_BYTES + (size_t)ASTAGES * SF_BYTES + NUM_BARS * 8 + 64;
+      1024 + (size_t)WSTAGES * W_BYTES + (size_t)XSTAGES * X_BYTES + (size_t)ASTAGES * SF_BYTES + NUM_BARS * 8 + 16 + 64 + 64;
   // E2M1 x E2M1 -> FP32, UE4M3 scale factors, both operands K-major, M = 128, N = NT
   static constexpr uint32_t IDESC = (1u << 7) | (1u << 10) | ((uint32_t)(NT >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
   static_assert(W_BYTES % 1024 == 0 && X_BYTES % 1024 == 0, "swizzled tiles sit on 1024 bytes");
@@ -150,7 +155,8 @@ razer_fp4_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_consta
   uint8_t* smem_w = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   uint8_t* smem_x = smem_w + (size_t)WSTAGES * W_BYTES;
   uint8_t* smem_a = smem_x + (size_t)XSTAGES * C::X_BYTES;
-  uint64_t* bars = reinterpret_cast<uint64_t*>(smem_a + (size_t)ASTAGES * SF_BYTES);
+  uint4* remap_table = reinterpret_cast<uint4*>(smem_a + (size_t)ASTAGES * SF_BYTES);   // [select * 2 + negate]: sign flips, base, signed remainder
+  uint64_t* bars = reinterpret_cast<uint64_t*>(remap_table + 4);
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + C::NUM_BARS);
   volatile uint32_t* abort_flag = tmem_slot + 1;
 
@@ -179,14 +185,14 @@ razer_fp4_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_consta
   if (threadIdx.x == 0) {
     for (int i = 0; i < WSTAGES; ++i) {
       mbar_init(bar_wfull + 8 * i, 1);
-      mbar_init(bar_wempty + 8 * i, 32 * NRW);
+      mbar_init(bar_wempty + 8 * i, GROUP_WARPS);
     }
     for (int i = 0; i < XSTAGES; ++i) {
       mbar_init(bar_xfull + 8 * i, 1);
       mbar_init(bar_xempty + 8 * i, 1);
     }
     for (int i = 0; i < ASTAGES; ++i) {
-      mbar_init(bar_afull + 8 * i, 32 * NRW);
+      mbar_init(bar_afull + 8 * i, 32 * GROUP_WARPS);
       mbar_init(bar_aempty + 8 * i, 1);
     }
     mbar_init(bar_accfull, 1);
@@ -219,6 +225,10 @@ razer_fp4_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_consta
                  "r"((uint32_t)C::TMEM_COLS)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  if (threadIdx.x >= 64 && threadIdx.x < 68) {
+    const uint32_t i = threadIdx.x - 64, neg = i & 1u;
+    remap_table[i] = make_uint4(neg * 0x88888888u, (i & 2u) ? a.base1 : a.base0, ((i & 2u) ? a.rem1 : a.rem0) | neg * 8u, 0u);
   }
   tc_fence_before();
   __syncthreads();
@@ -325,11 +335,12 @@ razer_fp4_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_consta
     // ===================== remap (thread = weight row) + epilogue =====================
     const int row = 32 * (warp & 3) + lane;              // weight row of the tile = TMEM lane of its outputs
     const uint32_t lane_off = (uint32_t)(32 * (warp & 3)) << 16;
-    // All sixteen warps remap every item: warps w, w + 4, w + 8, w + 12 own the same 32 rows (a warp reaches only the
-    // TMEM lanes 32 * (warp % 4) .. + 31, which the epilogue needs) and take one of the stage's four chunks each.
-    // The item after it goes into the other operand slot, so its remap runs while this item's MMAs execute.
-    const int chunk = (warp - 2) >> 2;
-    static_assert(NRW == 4 * CH, "one set of four warps per chunk");
+    // Group i % 2 remaps item i into its own operand slot, so that one item is remapped while the other group's is multiplied.
+    // Warps w and w + 4 of a group own the same 32 rows (a warp reaches only the TMEM lanes 32 * (warp % 4) .. + 31) and take
+    // two of a stage's four chunks each.  (All sixteen warps on every stage, a chunk each, paid the waits and the bookkeeping
+    // of an item twice as often.)
+    const int set = (warp - 2) >> 2, group = (warp - 2) / GROUP_WARPS;
+    const int chunk0 = (set % (GROUP_WARPS / 4)) * CPT;
     auto wait_all = [&](uint32_t bar, uint32_t parity, uint32_t code) -> bool {
       const bool got = mbar_wait(bar, parity, abort_flag);
       if (!got) fail(code);
@@ -339,77 +350,95 @@ razer_fp4_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_consta
     const uint32_t strip_off = (uint32_t)(row / STRIP_ROWS) * (CH * PIECE_BYTES);
     const uint32_t scale_off = (uint32_t)PIECE_CODE_BYTES + (uint32_t)(r16 & 7) * 8;
     const uint32_t scale_sel = (r16 >> 3) ? 0x7531u : 0x6420u;
-    uint32_t code_off[CHUNK_BLOCKS];
-#pragma unroll
-    for (int blk = 0; blk < CHUNK_BLOCKS; ++blk) code_off[blk] = (uint32_t)piece_code_offset(blk, r16);
+    const uint32_t code_off = (uint32_t)r16 * 8;         // ^ 32 blk: row r of block blk sits in slot r ^ (4 blk)
+    const uint32_t table = smem_addr(remap_table);       // on a 64-byte boundary
     const uint32_t sf_word = (uint32_t)((row & 31) * 4 + (row >> 5)) * 4;
     // The epilogue of a finished segment runs after the next item has been prepared, so that the MMAs
     // resume as soon as the accumulator is in registers.
     struct Pending { int tile; bool at_end; } pending = {-1, false};
-    const EpilogueCtx ctx = {bar_accfull, bar_accempty, bar_epi, tmem_base + lane_off, row, chunk, threadIdx.x == 64};
+    const EpilogueCtx ctx = {bar_accfull, bar_accempty, bar_epi, tmem_base + lane_off, row, set, threadIdx.x == 64};
     uint32_t seg = 0, epi_phase = 0;
     auto epilogue = [&]() -> bool {
       grid_dep_wait();                                     // outputs, workspace and the scale scalar may belong to the preceding kernel
       const float ts = a.extra_scale ? a.tensor_scale * *a.extra_scale : a.tensor_scale;
-      const int tile = pending.tile;
+      const int done_tile = pending.tile;
       pending.tile = -1;
       return segment_epilogue<NT, C::NACC, NRW / 4>(
-          a, ctx, tile, pending.at_end, ts, seg++, epi_phase, abort_flag,
+          a, ctx, done_tile, pending.at_end, ts, seg++, epi_phase, abort_flag,
           [&](uint32_t bar, uint32_t parity, uint32_t which) { return wait_all(bar, parity, 27u + which); },
           [&](uint32_t which) { fail(27u + which); });
     };
-    for (int i = 0; i <= n_items; ++i, cur.next(spt)) {
-      const int step = cur.step;
-      const bool seg_last = (i + 1 == n_items) || step == spt - 1;
+    const int last_tile = (it_end - 1) / spt;            // tile of the CTA's last item
+    int tile = cur.tile, step = cur.step + group;        // the group's item at hand: it walks its own only
+    bool ahead = false, all_closed = n_items == 0;
+    for (int i = group;;) {
+      const bool crossed = step >= spt && tile < last_tile;   // a segment ends before the group's next item
+      if (pending.tile >= 0 && (crossed || i >= n_items || ahead)) {
+        if (!epilogue()) break;
+        continue;
+      }
+      if (crossed) {
+        pending = {tile, true};
+        ahead = false;
+        step -= spt;
+        ++tile;
+        continue;
+      }
+      if (i >= n_items) {
+        if (all_closed) break;
+        all_closed = true;
+        pending = {tile, it_end == (last_tile + 1) * spt};
+        continue;
+      }
       const int nch = min(CH, a.g.k_chunks - step * CH);
-      if (i < n_items) {
-        // every remap thread sees every phase of the barriers it waits on, so the parity waits are sound
-        if (!wait_all(bar_aempty + 8 * cur.as, (uint32_t)cur.aph ^ 1u, 26)) break;
-        if (!wait_all(bar_wfull + 8 * cur.ws, (uint32_t)cur.wph, 25)) break;
-        const uint32_t st = smem_addr(smem_w) + (uint32_t)cur.ws * W_BYTES + strip_off;
-        tc_fence_after();
-        const uint32_t am_t = tmem_slot0 + cur.as * C::SLOT_COLS + lane_off;
-        const uint32_t sfa = smem_addr(smem_a) + (uint32_t)cur.as * SF_BYTES + sf_word;
-        {
-          const int c = chunk;
-          if (c < nch) {
-            const uint32_t ck = st + c * PIECE_BYTES;
-            const uint2 sq = lds64(ck + scale_off);
-            const uint32_t sw = __byte_perm(sq.x, sq.y, scale_sel);   // this row's four scale bytes, in block order
-            uint2 cw[CHUNK_BLOCKS];
+      const uint32_t ws = (uint32_t)i % WSTAGES, wph = ((uint32_t)i / WSTAGES) & 1u, as = (uint32_t)i % ASTAGES, aph = ((uint32_t)i / ASTAGES) & 1u;
+      const uint32_t st = smem_addr(smem_w) + ws * W_BYTES + strip_off;
+      const uint32_t am_t = tmem_slot0 + as * C::SLOT_COLS + lane_off;
+      const uint32_t sfa = smem_addr(smem_a) + as * SF_BYTES + sf_word;
+      if (!wait_all(bar_wfull + 8 * ws, wph, 25)) break;
+      // everything up to the stores is done before the operand slot is free
+      uint32_t mw[CPT][8], pw[CPT][8], sw[CPT];
 #pragma unroll
-            for (int blk = 0; blk < CHUNK_BLOCKS; ++blk) cw[blk] = lds64(ck + code_off[blk]);
-            uint32_t mw[8], pw[8];
+      for (int cc = 0; cc < CPT; ++cc) {                 // chunks past the end of K arrive as zeros
+        const uint32_t ck = st + (chunk0 + cc) * PIECE_BYTES;
+        const uint2 sq = lds64(ck + scale_off);
+        uint2 cw[CHUNK_BLOCKS];
 #pragma unroll
-            for (int blk = 0; blk < CHUNK_BLOCKS; ++blk) {
-              const uint32_t sb = (sw >> (8 * blk)) & 0xFFu;
-              const uint32_t neg8 = (sb & PACKED_NEGATE) ? 0x88888888u : 0u;   // stored negated: flip every sign bit
-              const uint32_t base = (sb & PACKED_SELECT) ? a.base1 : a.base0;
-              const uint32_t rem = (sb & PACKED_SELECT) ? a.rem1 : a.rem0;
+        for (int blk = 0; blk < CHUNK_BLOCKS; ++blk) cw[blk] = lds64(ck + blk * (STRIP_ROWS * 8) + (code_off ^ (32u * blk)));
+        sw[cc] = __byte_perm(sq.x, sq.y, scale_sel);     // this row's four scale bytes, in block order
 #pragma unroll
-              for (int h = 0; h < 2; ++h) {
-                const uint32_t w = h ? cw[blk].y : cw[blk].x;
-                const uint32_t any = w | (w >> 1) | (w >> 2) | (w >> 3);
-                const uint32_t z = ~any & 0x11111111u;                         // 1 in every nibble that is 0x0
-                mw[2 * blk + h] = (w + z * base) ^ neg8;
-                pw[2 * blk + h] = (z * rem) ^ neg8;
-              }
-            }
-            tc_st8(am_t + c * 8, mw);
-            tc_st8(am_t + A_PASS_COLS + c * 8, pw);
-            sts32(sfa + c * SF_TILE_BYTES, sw & 0x3F3F3F3Fu);
+        for (int blk = 0; blk < CHUNK_BLOCKS; ++blk) {
+          const uint4 k = lds128(((blk == 0 ? sw[cc] >> 2 : sw[cc] >> (8 * blk + 2)) & 0x30u) | table);
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            const uint32_t w = h ? cw[blk].y : cw[blk].x;
+            const uint32_t t = (w & 0x77777777u) + 0x77777777u;            // bit 3: magnitude not zero
+            const uint32_t z = (~(t | w) & 0x88888888u) >> 3;              // 1 in every nibble that is 0x0
+            mw[cc][2 * blk + h] = (w ^ k.x) + z * k.y;
+            pw[cc][2 * blk + h] = z * k.z;
           }
         }
-        mbar_arrive(bar_wempty + 8 * cur.ws);               // the packed bytes are in registers or written out
-        fence_async_smem();
-        tc_wait_st();
-        tc_fence_before();
-        mbar_arrive(bar_afull + 8 * cur.as);
       }
-
-      if (pending.tile >= 0 && !epilogue()) break;
-      if (i == n_items) break;
-      if (seg_last) pending = {cur.tile, step == spt - 1};
+      __syncwarp();                                      // every lane has read the stage
+      if (lane == 0) mbar_arrive(bar_wempty + 8 * ws);
+      if (!wait_all(bar_aempty + 8 * as, aph ^ 1u, 26)) break;
+      tc_fence_after();
+#pragma unroll
+      for (int cc = 0; cc < CPT; ++cc) {
+        const int c = chunk0 + cc;
+        if (c < nch) {
+          tc_st8(am_t + c * 8, mw[cc]);
+          tc_st8(am_t + A_PASS_COLS + c * 8, pw[cc]);
+          sts32(sfa + c * SF_TILE_BYTES, sw[cc] & 0x3F3F3F3Fu);
+        }
+      }
+      fence_async_smem();
+      tc_wait_st();
+      tc_fence_before();
+      mbar_arrive(bar_afull + 8 * as);
+      ahead = true;
+      i += GROUPS;
+      step += GROUPS;
     }
   }
 
@@ -480,21 +509,35 @@ __global__ void fp4_act_prep_kernel(const uint32_t* __restrict__ codes, const ui
 
 struct Plan {
   Fp4ActLayout act;
-  int grid;
+  int NT, token_tiles, grid;
   long long tiles, total_items;
   size_t slots_bytes;
 };
 
+// Fitted to a sweep of 16 shapes (M 16 .. 2048, K and N 300 .. 14336, both widths, all grids).  With 256 tokens wherever there are
+// more than 128, and stripes on all SMs, 512 x 4096 x 4096 took 18.0 us (14.0 by this choice), 300 x 390 x 2320 10.6 (7.9),
+// 2048 x 1024 x 1024 13.0 (6.4), 1000 x 300 x 8192 27.5 (12.2), 128 x 14336 x 4096 16.4 (13.8).
+static const TileCost tile_costs[] = {{128, CH, CH, 0.139f, 0.08f, 0.6f, 2.9f, 0.30f, 4.6f, 0.50f},
+                                      {256, CH, CH, 0.177f, 0.18f, 1.3f, 3.1f, 0.30f, 6.5f, 1.30f}};
+
 static Plan make_plan(const razer_desc* d, int M) {
-  Plan p;
+  Plan best;
+  float best_cost = 0.0f;
   const Geometry g = make_geometry(d->N, d->K);
-  p.act = make_fp4_act_layout(M, d->K);
-  p.tiles = (long long)g.row_tiles * p.act.token_tiles;
-  p.total_items = p.tiles * p.act.spt;
-  const int sms = sm_count();
-  p.grid = (int)(p.total_items < sms ? p.total_items : sms);
-  p.slots_bytes = (size_t)(p.grid > 148 ? p.grid : 148) * p.act.NT * TILE_ROWS * sizeof(float);
-  return p;
+  const Fp4ActLayout act = make_fp4_act_layout(M, d->K);
+  for (const TileCost& t : tile_costs) {
+    if (act.force_nt ? t.NT != act.force_nt : t.NT > act.tiles128 * 128) continue;
+    Plan p;
+    p.act = act;
+    p.NT = t.NT;
+    p.token_tiles = (M + p.NT - 1) / p.NT;
+    p.tiles = (long long)g.row_tiles * p.token_tiles;
+    p.total_items = p.tiles * act.spt;
+    const float cost = best_grid(t, p.tiles, act.spt, sm_count(), p.grid);
+    if (best_cost == 0.0f || cost < best_cost) { best_cost = cost; best = p; }
+  }
+  best.slots_bytes = (size_t)best.grid * best.NT * TILE_ROWS * sizeof(float);
+  return best;
 }
 
 // FP4 magnitude code (0 .5 1 1.5 2 3 4 6 -> 0..7) of v, or -1.
@@ -537,13 +580,13 @@ static bool split_special_values(const float sv[2], uint32_t base[2], uint32_t r
 
 Fp4ActLayout make_fp4_act_layout(int M, int K) {
   Fp4ActLayout L;
-  L.NT = M > 128 ? 256 : 128;
+  L.force_nt = 0;
   if (const char* e = getenv("RAZER_FP4_NT")) {                        // tuning and test aid: force the token tile
     const int v = atoi(e);
-    if (v == 128 || v == 256) L.NT = v;
+    if (v == 128 || v == 256) L.force_nt = v;
   }
-  L.token_tiles = (M + L.NT - 1) / L.NT;
-  L.tiles128 = L.token_tiles * (L.NT / 128);
+  L.tiles128 = (M + 127) / 128;
+  if (L.tiles128 > 1 || L.force_nt == 256) L.tiles128 = (L.tiles128 + 1) / 2 * 2;   // either token tile reads whole ones
   const int k_chunks = (K + CHUNK_K - 1) / CHUNK_K;
   L.spt = (k_chunks + fp4_path::CH - 1) / fp4_path::CH;
   L.KP = L.spt * fp4_path::CH * CHUNK_K;
@@ -597,7 +640,7 @@ int launch_gemm_fp4_prepared(const razer_desc* d, const void* packed, const void
   a.g = g;
   a.tensor_scale = d->tensor_scale;
   a.M = M;
-  a.token_tiles = p.act.token_tiles;
+  a.token_tiles = p.token_tiles;
   a.steps_per_tile = p.act.spt;
   a.split = p.grid % p.tiles == 0 ? (int)(p.grid / p.tiles) : 0;
   a.total_items = p.total_items;
@@ -608,7 +651,7 @@ int launch_gemm_fp4_prepared(const razer_desc* d, const void* packed, const void
     // padded activation codes as bytes: [M][KP / 2]; box = 128 bytes (one stage of k) x NT tokens
     const cuuint64_t dims[2] = {(cuuint64_t)(p.act.KP / 2), (cuuint64_t)M};
     const cuuint64_t strides[1] = {(cuuint64_t)(p.act.KP / 2)};
-    const cuuint32_t box[2] = {128, (cuuint32_t)p.act.NT};
+    const cuuint32_t box[2] = {128, (cuuint32_t)p.NT};
     const CUresult r = enc(&tmap_x, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, codes_pad, dims, strides, box, estr,
                            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
@@ -634,7 +677,7 @@ int launch_gemm_fp4_prepared(const razer_desc* d, const void* packed, const void
   cfg.attrs = attr;
   cfg.numAttrs = pdl ? 1 : 0;
   cudaError_t e;
-  if (p.act.NT == 128) {
+  if (p.NT == 128) {
     static bool attr_set = false;
     if (!attr_set) {
       RAZER_TRY(check_cuda(cudaFuncSetAttribute(razer_fp4_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize,

@@ -448,26 +448,20 @@ struct UmmaPlan {
   size_t slots_bytes;
 };
 
-// Token tile and grid.  Every token-tile width is weighed with every grid that keeps a tile on one CTA, cuts every tile evenly
-// among 2 .. 16 CTAs, or gives all SMs equal stripes, by a model in microseconds fitted to a sweep of 18 shapes (M 16 .. 2048, K and N
-// 300 .. 28672, all widths, all grids): a start (1.6, and 1.8 more with a CTA on every SM), the chunks of the busiest CTA, and the
-// end of a tile.  `chunk`: one 64-column chunk of a 128-row tile; it grows by `load` with all SMs at work.  `whole`: storing a
-// tile; `cut`, `part`: combining one cut among several CTAs, and each CTA of it; `stripe`: the two partial tiles of a stripe.
-// On the swept shapes the choice is within 11 % of the best of the sweep (16 x 28672 x 1024 aside), where the fixed rule before
-// it (the narrowest tile that holds M, all SMs) was up to 4 times slower: 300 x 390 x 2320 36.2 -> 8.1 us, 256 x 1024 x 1024 20.8 ->
-// 4.8, 1000 x 300 x 8192 33.1 -> 14.5, 333 x 4096 x 11008 38.8 -> 32.4.
-struct TileCost { int NT, CH, CHX; float chunk, load, whole, cut, part, stripe; };
+// Token tile and grid: the cheapest pair by the cost model (razer_tcgen05.cuh), fitted to a sweep of 18 shapes (M 16 .. 2048, K and N
+// 300 .. 28672, all widths, all grids).  On these the choice is within 11 % of the best of the sweep (16 x 28672 x 1024
+// aside), where the fixed rule before it (the narrowest tile that holds M, all SMs) was up to 4 times slower: 300 x 390 x 2320
+// 36.2 -> 8.1 us, 256 x 1024 x 1024 20.8 -> 4.8, 1000 x 300 x 8192 33.1 -> 14.5, 333 x 4096 x 11008 38.8 -> 32.4.
 static const TileCost tile_costs[] = {
-    {16, 4, 4, 0.168f, 0.20f, 0.0f, 2.0f, 0.20f, 4.0f},  {32, 4, 4, 0.170f, 0.20f, 0.1f, 2.6f, 0.20f, 4.0f},
-    {64, 4, 4, 0.178f, 0.15f, 0.4f, 2.3f, 0.35f, 4.5f},  {96, 4, 2, 0.186f, 0.15f, 0.5f, 2.4f, 0.37f, 5.0f},
-    {128, 4, 1, 0.228f, 0.15f, 0.7f, 2.9f, 0.75f, 6.0f}, {192, 2, 1, 0.268f, 0.20f, 1.2f, 3.7f, 0.60f, 6.3f},
-    {256, 2, 1, 0.315f, 0.25f, 1.6f, 4.0f, 0.55f, 7.0f}};
+    {16, 4, 4, 0.168f, 0.20f, 0.0f, 2.0f, 0.20f, 4.0f, 0.06f},  {32, 4, 4, 0.170f, 0.20f, 0.1f, 2.6f, 0.20f, 4.0f, 0.11f},
+    {64, 4, 4, 0.178f, 0.15f, 0.4f, 2.3f, 0.35f, 4.5f, 0.22f},  {96, 4, 2, 0.186f, 0.15f, 0.5f, 2.4f, 0.37f, 5.0f, 0.34f},
+    {128, 4, 1, 0.228f, 0.15f, 0.7f, 2.9f, 0.75f, 6.0f, 0.45f}, {192, 2, 1, 0.268f, 0.20f, 1.2f, 3.7f, 0.60f, 6.3f, 0.67f},
+    {256, 2, 1, 0.315f, 0.25f, 1.6f, 4.0f, 0.55f, 7.0f, 0.90f}};
 
 static UmmaPlan make_plan(const razer_desc* d, int M) {
   UmmaPlan best;
   float best_cost = 0.0f;
   const Geometry g = make_geometry(d->N, d->K);
-  const int sms = sm_count();
   for (const TileCost& t : tile_costs) {
     if (t.NT > 16 && t.NT >= 2 * M) continue;              // half of the tile or more would be padding
     UmmaPlan p;
@@ -478,29 +472,8 @@ static UmmaPlan make_plan(const razer_desc* d, int M) {
     p.steps_per_tile = (g.k_chunks + p.CH - 1) / p.CH;
     p.tiles = (long long)g.row_tiles * p.token_tiles;
     p.total_items = p.tiles * p.steps_per_tile;
-    auto consider = [&](long long grid, int tiles_per_cta, int cut) {   // whole tiles per CTA, or CTAs per tile, or stripes (0, 0)
-      p.grid = (int)grid;
-      const float busy = (float)grid / sms;
-      const long long items = (p.total_items + grid - 1) / grid;
-      float c = 1.6f + 1.8f * busy + (float)(items * p.CH) * t.chunk * (1.0f + t.load * busy);
-      if (tiles_per_cta > 0) {
-        c += t.whole * (0.6f + 0.4f * tiles_per_cta);
-      } else if (cut > 0) {
-        c += t.cut + t.part * cut;
-      } else {
-        const float tiles = (float)p.total_items / grid / p.steps_per_tile, parts = 1.0f / tiles + 1.0f;
-        c += t.stripe + 0.4f * t.whole * tiles + (parts > 3.0f ? (parts - 3.0f) * 0.0035f * p.NT : 0.0f);
-      }
-      if (best_cost == 0.0f || c < best_cost) { best_cost = c; best = p; }
-    };
-    if (p.tiles <= sms) {
-      consider(p.tiles, 1, 0);
-      for (int cut = 2; cut <= 16 && p.tiles * cut <= sms && cut <= p.steps_per_tile; ++cut) consider(p.tiles * cut, 0, cut);
-    } else {
-      for (int q = (int)((p.tiles + sms - 1) / sms), n = 0; n < 2 && q <= 8; ++q, ++n)
-        if (p.tiles % q == 0) consider(p.tiles / q, q, 0);
-    }
-    consider(p.total_items < sms ? p.total_items : sms, 0, 0);
+    const float cost = best_grid(t, p.tiles, p.steps_per_tile, sm_count(), p.grid);
+    if (best_cost == 0.0f || cost < best_cost) { best_cost = cost; best = p; }
   }
   best.slots_bytes = (size_t)best.grid * best.NT * TILE_ROWS * sizeof(float);
   return best;

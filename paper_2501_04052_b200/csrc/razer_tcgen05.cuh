@@ -305,6 +305,41 @@ static inline EncodeTiledFn encode_fn() {
   return fn;
 }
 
+// What a token-tile width costs, in microseconds, fitted to sweeps over sizes, widths and grids (razer_gemm_umma.cu,
+// razer_gemm_fp4.cu).  `chunk`: one 64-column chunk of a 128-row tile; it grows by `load` with a CTA on every SM.  `whole`: storing
+// a tile; `cut`, `part`: combining one cut evenly among several CTAs, and each CTA of it; `stripe`: the two partial tiles of a
+// stripe, `extra`: each CTA beyond three that shares one.
+struct TileCost { int NT, CH, CHX; float chunk, load, whole, cut, part, stripe, extra; };
+
+// The cheapest grid for `tiles` output tiles of `steps` items: every tile on one CTA, every tile cut evenly among 2 .. 16 CTAs, or
+// equal stripes on all SMs.  Returns the modelled time.
+static inline float best_grid(const TileCost& t, long long tiles, int steps, int sms, int& grid) {
+  float best = 0.0f;
+  const long long total = tiles * steps;
+  auto consider = [&](long long g, int tiles_per_cta, int cut) {            // whole tiles per CTA, or CTAs per tile, or stripes (0, 0)
+    const float busy = (float)g / sms;
+    float c = 1.6f + 1.8f * busy + (float)((total + g - 1) / g * t.CH) * t.chunk * (1.0f + t.load * busy);
+    if (tiles_per_cta > 0) {
+      c += t.whole * (0.6f + 0.4f * tiles_per_cta);
+    } else if (cut > 0) {
+      c += t.cut + t.part * cut;
+    } else {
+      const float per_cta = (float)total / g / steps, parts = 1.0f / per_cta + 1.0f;
+      c += t.stripe + 0.4f * t.whole * per_cta + (parts > 3.0f ? (parts - 3.0f) * t.extra : 0.0f);
+    }
+    if (best == 0.0f || c < best) { best = c; grid = (int)g; }
+  };
+  if (tiles <= sms) {
+    consider(tiles, 1, 0);
+    for (int cut = 2; cut <= 16 && tiles * cut <= sms && cut <= steps; ++cut) consider(tiles * cut, 0, cut);
+  } else {
+    for (int q = (int)((tiles + sms - 1) / sms), n = 0; n < 2 && q <= 8; ++q, ++n)
+      if (tiles % q == 0) consider(tiles / q, q, 0);
+  }
+  consider(total < sms ? total : sms, 0, 0);
+  return best;
+}
+
 static inline int sm_count() {
   static int n = 0;
   if (!n) {

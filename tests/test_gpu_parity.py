@@ -461,6 +461,19 @@ def test_w4a4_native_fp4_forced_token_tile(b, monkeypatch, nt, M):
     _w4a4_native_check(b, desc, packed, wc, ws, wd, ac, as_, ats)
 
 
+@pytest.mark.parametrize("M,N,K", [(16, 1000, 1024), (64, 300, 4112), (100, 19000, 336), (2000, 1100, 528), (250, 600, 8208),
+                                   (333, 4090, 5520), (140, 260, 80), (2, 16, 16)])
+def test_w4a4_native_fp4_token_tiles_and_partitions(b, M, N, K):
+    """Both token tiles of the FP4 kernel with tiles that stay on one CTA, tiles cut evenly among several, and stripes, as the host
+    picks them for these sizes."""
+    wc, ws = inputs.random_codes(N, K, seed=99)
+    wc, ws = wc.numpy(), ws.numpy()
+    desc, packed = _pack(b, wc, ws, 0.002)
+    x = inputs.activations(M, K, 99, outlier_channel_frac=0.01)
+    ac, as_, ats = b.razer_quant_act(x.cuda(), sv_mag=0.0)
+    _w4a4_native_check(b, desc, packed, wc, ws, 0.002, ac, as_, ats, rows=rows_with_edge_tiles(N, 64, 98))
+
+
 @pytest.mark.parametrize("M,N,K", [(256, 512, 8192), (17, 200, 464), (300, 260, 1040), (130, 390, 2320)])
 def test_w4a4_fp4_prepared_operand_matches_the_interchange_route(b, M, N, K):
     """razer_quant_act_fp4 + razer_gemm_w4a4_fp4 (the quantizer writes the tensor core's operand layout itself)
