@@ -15,36 +15,31 @@ namespace razer {
 
 namespace stream_path {
 
-#ifndef STREAM_CW
-#define STREAM_CW 8
-#endif
-constexpr int CW = STREAM_CW;                       // consumer warps; a stage holds CW * SPW slices, SPW per warp
-constexpr int THREADS = 32 * (CW + 2);              // + producer warp + epilogue warp
+constexpr int CW = 16;                              // consumer warps
+constexpr int EW = 2;                               // epilogue warps, each with its half of a unit's outputs
+constexpr int THREADS = 32 * (CW + EW + 2);         // + a producer warp each for weights and activations
 constexpr int MAX_STAGES = 8;
 constexpr int MAX_M = 8;
-#ifndef STREAM_OCC
-#define STREAM_OCC 2
-#endif
-#ifndef STREAM_TABLE_SHIFT
-#define STREAM_TABLE_SHIFT 2
-#endif
-constexpr int OCC = STREAM_OCC;                     // CTAs per SM the kernel is built for
-constexpr int TABLE_SHIFT = STREAM_TABLE_SHIFT;     // 1: 16 copies of each entry, 2: 8 copies, 3: 4 copies
-constexpr int TABLE_COPIES = 32 >> TABLE_SHIFT;
-constexpr int TABLE_BYTES = 256 * TABLE_COPIES * 8; // 256 scale bytes x copies x {scale, special value}
-constexpr int RED_STRIDE = 36;                      // floats per (warp, token) in the partial-sum buffers
-constexpr int SLOT_FLOATS = 32 * MAX_M;             // one CTA's partial result of a unit
-constexpr int SMEM_BYTES = (OCC == 2 ? 112 : 74) * 1024;   // OCC CTAs per SM (each also holds 1 KB of system shared memory)
-constexpr int BAR_BYTES = (2 * MAX_STAGES + 4) * 8 + 32;
+constexpr int LUT_BYTES = 65536;                    // [weight byte][special value][lane]: two elements as bf16x2
+constexpr int SCALES_BYTES = 128 * 32 * 4;                  // [scale byte without the select bit][lane]: +-scale as bf16x2
+constexpr int MAX_ROWS = 64;
+constexpr int SLOT_FLOATS = MAX_ROWS * MAX_M;       // one CTA's partial result of a unit
+constexpr int SMEM_BYTES = 226 * 1024;              // one CTA per SM
+constexpr int BAR_BYTES = (2 * MAX_STAGES + 4) * 8;
 
-template <int TM, int SPW>
+// SW x KW = CW consumer warps: SW side by side over the unit's strips (TM strips each), KW over its chunks; a warp takes
+// SPW chunks of a stage.
+template <int SW_, int TM_, int SPW_>
 struct Cfg {
-  static constexpr int ROWS = 16 * TM;
-  static constexpr int CPS = CW * SPW;                     // chunks (slices) per stage
+  static constexpr int SW = SW_, TM = TM_, SPW = SPW_, KW = CW / SW_;
+  static constexpr int STRIPS = SW * TM, ROWS = 16 * STRIPS;
+  static constexpr int CPS = KW * SPW;                     // chunks per stage
   static constexpr int STRIP_BYTES = CPS * PIECE_BYTES;    // one strip's pieces of a stage
-  static constexpr int W_BYTES = TM * STRIP_BYTES;         // weights of a stage
+  static constexpr int W_BYTES = STRIPS * STRIP_BYTES;     // weights of a stage
   static constexpr int XS = CPS * 128 + 16;                // bytes between tokens in a stage (16 mod 128: no bank conflicts)
+  static constexpr int RED_STRIDE = ROWS + 4;              // floats per (warp, token) in the partial-sum buffers
   static_assert(XS % 16 == 0, "bulk copies land on 16-byte boundaries");
+  static_assert(ROWS <= MAX_ROWS, "a unit's partial result fits its slot");
 };
 
 struct Args {
@@ -52,18 +47,18 @@ struct Args {
   const __nv_bfloat16* x;    // [M][K]
   __nv_bfloat16* y;          // [M][N]
   float* slots;              // [grid][2][SLOT_FLOATS]
-  uint32_t* counters;        // one per split unit, zero between calls
+  uint32_t* counters;        // [split unit][epilogue warp], zero between calls
   uint32_t* status;          // device status word
   uint32_t* status_host;     // the same for a host that waits for this call (pinned memory), or NULL
   const float* extra_scale;  // optional device scalar multiplied into the tensor scale
   int N, K, kc, M;
-  int units;                 // units of TM strips that hold rows < N
+  int red_bufs;              // partial-sum buffers: 1 or 2
+  int units;                 // units (Cfg::STRIPS strips) that hold rows < N
   int whole_base, whole_per_cta;   // CTA b owns the whole units whole_base + b * whole_per_cta .. (clipped to units)
   int rem_ctas;              // CTAs that share the split units [0, whole_base); 0 = nothing is split
   int pieces_per_unit;       // a split unit is cut along K into this many equal pieces; the pieces of all split units,
                              // in unit order, are dealt out to the rem_ctas CTAs in equal contiguous ranges
   float sv0, sv1, tensor_scale;
-  uint32_t mul_lo, mul_hi;   // 2^6 + 2^12 and 2^2 + 2^8 (razer_decode.cuh)
 };
 
 // D (+)= A(16 x 16, row) * B(16 x 8, col), bf16 inputs, FP32 accumulation.
@@ -164,52 +159,54 @@ __device__ __forceinline__ Work make_work(const Args& a, int b) {
 }
 
 // Wait for a barrier phase.  One cheap poll first; the slow path looks at the clock and the abort flag only once
-// per 32 polls and, for the service warps (SLEEP_NS > 0), sleeps between polls, so that a waiting warp costs the
+// per 32 polls and, for the service warps (sleep_ns > 0), sleeps between polls, so that a waiting warp costs the
 // decoding warps few issue slots.
-template <int SLEEP_NS>
-__device__ __noinline__ bool wait_phase_slow(uint32_t bar, uint32_t parity, volatile uint32_t* abort_flag) {
+static __device__ __noinline__ bool wait_phase_slow(uint32_t bar, uint32_t parity, volatile uint32_t* abort_flag, uint32_t sleep_ns) {
   const uint64_t t0 = global_ns();
   for (uint32_t i = 0; i < (WAIT_LIMIT >> 5); ++i) {
 #pragma unroll 1
     for (int j = 0; j < 32; ++j) {
       if (mbar_try_wait(bar, parity)) return true;
-      if (SLEEP_NS > 0) __nanosleep(SLEEP_NS);
+      if (sleep_ns > 0) __nanosleep(sleep_ns);
     }
     if (*abort_flag) return false;
     if (global_ns() - t0 > WAIT_LIMIT_NS) return false;
   }
   return false;
 }
-template <int SLEEP_NS = 0>
-__device__ __forceinline__ bool wait_phase(uint32_t bar, uint32_t parity, volatile uint32_t* abort_flag) {
+__device__ __forceinline__ bool wait_phase(uint32_t bar, uint32_t parity, volatile uint32_t* abort_flag, uint32_t sleep_ns = 0) {
   if (mbar_try_wait(bar, parity)) return true;
-  return wait_phase_slow<SLEEP_NS>(bar, parity, abort_flag);
+  return wait_phase_slow(bar, parity, abort_flag, sleep_ns);
 }
 
-// The epilogue warp's loop over the CTA's segments: add the consumer warps' partial sums of a segment in warp order,
-// then either write y (whole unit) or publish the piece, count, and let the last arrival add the pieces in CTA order.
-// `ts` multiplies every output.  `fail(code)` records a wait that gave up.
-template <int ROWS, class Fail>
-__device__ __forceinline__ void epilogue_loop(const Args& a, const Work& work, int b, int lane, uint32_t red,
+// An epilogue warp's loop over the CTA's segments: add the consumer warps' partial sums of its outputs of a segment in
+// warp order, then either write y (whole unit) or publish the piece, count, and let the last arrival add the pieces in CTA
+// order (the warps of a CTA count apart).  `ts` multiplies every output.  `fail(code)` records a wait that gave up.
+template <class C, class Fail>
+__device__ __forceinline__ void epilogue_loop(const Args& a, const Work& work, int b, int ew, int lane, uint32_t red,
                                               uint32_t bar_red_full, uint32_t bar_red_free, volatile uint32_t* abort_flag,
                                               float ts, Fail fail) {
+  constexpr int ROWS = C::ROWS, KW = C::KW, RED_STRIDE = C::RED_STRIDE;
+  constexpr int STEP = 32 * EW, PER_LANE = ROWS * MAX_M / STEP;
   const int outputs = ROWS * a.M;                           // output o = token (o / ROWS), row (o % ROWS)
+  const int first = lane + 32 * ew;                         // this lane's outputs: first, first + STEP, ..
   for (int i = 0; i < work.n_seg; ++i) {
     const Seg s = work.seg(i);
-    const int buf = i & 1;
-    const bool got = wait_phase<32>(bar_red_full + 8 * buf, (uint32_t)(i >> 1) & 1u, abort_flag);
+    const uint32_t sleep_ns = min(256, 32 * ((s.c1 - s.c0) / C::CPS + 1));   // a stage takes the consumers several hundred ns
+    const int buf = a.red_bufs == 2 ? i & 1 : 0;
+    const bool got = wait_phase(bar_red_full + 8 * buf, (uint32_t)(a.red_bufs == 2 ? i >> 1 : i) & 1u, abort_flag, sleep_ns);
     if (!got) fail(10);
     if (!__all_sync(0xFFFFFFFFu, got)) break;
-    float v[MAX_M];
+    float v[PER_LANE];
 #pragma unroll
-    for (int j = 0; j < MAX_M; ++j) {
-      const int o = lane + 32 * j;
+    for (int j = 0; j < PER_LANE; ++j) {
+      const int o = first + STEP * j;
       float sum = 0.0f;
       if (o < outputs) {
         const int m = o / ROWS, row = o % ROWS;
-        const uint32_t src = red + (uint32_t)(((buf * CW) * a.M + m) * RED_STRIDE + row) * 4u;
+        const uint32_t src = red + (uint32_t)((buf * KW * a.M + m) * RED_STRIDE + row) * 4u;
 #pragma unroll
-        for (int w = 0; w < CW; ++w) sum += __uint_as_float(lds32(src + (uint32_t)(w * a.M * RED_STRIDE) * 4u));   // warp order
+        for (int w = 0; w < KW; ++w) sum += __uint_as_float(lds32(src + (uint32_t)(w * a.M * RED_STRIDE) * 4u));   // warp order
       }
       v[j] = sum;
     }
@@ -219,8 +216,8 @@ __device__ __forceinline__ void epilogue_loop(const Args& a, const Work& work, i
     const bool whole = s.c0 == 0 && s.c1 == a.kc;
     if (whole) {
 #pragma unroll
-      for (int j = 0; j < MAX_M; ++j) {
-        const int o = lane + 32 * j;
+      for (int j = 0; j < PER_LANE; ++j) {
+        const int o = first + STEP * j;
         if (o < outputs) {
           const int m = o / ROWS, n = n0 + o % ROWS;
           if (n < a.N) a.y[(size_t)m * a.N + n] = __float2bfloat16_rn(ts * v[j]);
@@ -231,25 +228,26 @@ __device__ __forceinline__ void epilogue_loop(const Args& a, const Work& work, i
     // ---- a piece of a split unit: publish, count, the last arrival adds the pieces in CTA order ----
     float* mine = a.slots + ((size_t)b * 2 + i) * SLOT_FLOATS;          // split segments come first: i is 0 or 1
 #pragma unroll
-    for (int j = 0; j < MAX_M; ++j)
-      if (lane + 32 * j < outputs) mine[lane + 32 * j] = v[j];
+    for (int j = 0; j < PER_LANE; ++j)
+      if (first + STEP * j < outputs) mine[first + STEP * j] = v[j];
     __syncwarp();
     const int c_first = cta_of_piece(a, s.unit * a.pieces_per_unit);
     const int c_last = cta_of_piece(a, (s.unit + 1) * a.pieces_per_unit - 1);
+    uint32_t* count = a.counters + EW * s.unit + ew;
     uint32_t last = 0;
     if (lane == 0) {
       uint32_t prev;
       // release: this warp's slot stores (ordered before by the warp barrier) become visible with the count;
       // acquire: the last arrival sees every earlier arrival's slot stores
-      asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(prev) : "l"(a.counters + s.unit) : "memory");
+      asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(prev) : "l"(count) : "memory");
       last = (prev + 1 == (uint32_t)(c_last - c_first + 1)) ? 1u : 0u;
-      if (last) a.counters[s.unit] = 0;                     // leave the counter ready for the next call
+      if (last) *count = 0;                     // leave the counter ready for the next call
     }
     last = __shfl_sync(0xFFFFFFFFu, last, 0);
     if (!last) continue;
-    float acc[MAX_M];
+    float acc[PER_LANE];
 #pragma unroll
-    for (int j = 0; j < MAX_M; ++j) acc[j] = 0.0f;
+    for (int j = 0; j < PER_LANE; ++j) acc[j] = 0.0f;
     // CTA order (a fixed summation order); the loads of four CTAs' slots are in flight together
     for (int cb = c_first; cb <= c_last; cb += 4) {
       const float* src[4];
@@ -260,11 +258,11 @@ __device__ __forceinline__ void epilogue_loop(const Args& a, const Work& work, i
         src[u] = a.slots + ((size_t)c * 2 + sl) * SLOT_FLOATS;
       }
 #pragma unroll
-      for (int j = 0; j < MAX_M; ++j) {
-        if (lane + 32 * j < outputs) {
+      for (int j = 0; j < PER_LANE; ++j) {
+        if (first + STEP * j < outputs) {
           float part[4];
 #pragma unroll
-          for (int u = 0; u < 4; ++u) part[u] = __ldcg(src[u] + lane + 32 * j);
+          for (int u = 0; u < 4; ++u) part[u] = __ldcg(src[u] + first + STEP * j);
 #pragma unroll
           for (int u = 0; u < 4; ++u)
             if (cb + u <= c_last) acc[j] += part[u];
@@ -272,8 +270,8 @@ __device__ __forceinline__ void epilogue_loop(const Args& a, const Work& work, i
       }
     }
 #pragma unroll
-    for (int j = 0; j < MAX_M; ++j) {
-      const int o = lane + 32 * j;
+    for (int j = 0; j < PER_LANE; ++j) {
+      const int o = first + STEP * j;
       if (o < outputs) {
         const int m = o / ROWS, n = n0 + o % ROWS;
         if (n < a.N) a.y[(size_t)m * a.N + n] = __float2bfloat16_rn(ts * acc[j]);
@@ -295,45 +293,55 @@ static inline int stream_sm_count() {
   return n;
 }
 
+static inline int force_spw() {   // tuning aid
+  static const int v = [] { const char* e = getenv("RAZER_STREAM_SPW"); return e ? atoi(e) : 0; }();
+  return v;
+}
+
 struct StreamPlan {
-  int TM, SPW, grid, units, kc;
+  int SW, TM, SPW, grid, units, kc, red_bufs;
   int whole_base, whole_per_cta, rem_ctas, pieces_per_unit;
   double cost;
   size_t slots_bytes;
 };
 
-// One candidate: units of TM strips; every CTA takes whole units only (split == false), or q whole units after a
+// One candidate: units of SW * TM strips; every CTA takes whole units only (split == false), or q whole units after a
 // piece of one of the remaining units, each of which is cut along K into equal pieces (processed first, combined
-// through the workspace).  The cost is the busiest CTA's work in strip-slices: a slice of TM strips costs TM plus
-// what is per slice (activation fragment, loop), and a split whose combination nothing follows (q == 0) pays
-// for it at the end of the launch.
-static inline StreamPlan stream_candidate(const razer_desc* d, int M, int G, int TM, bool split) {
+// through the workspace).  The cost is the busiest CTA's time in SM cycles.  A round (each consumer warp takes TM strips of one
+// chunk) costs the shared-memory wavefronts of its loads, 23 per strip and 8 per chunk and warp, which is what the decode is
+// bound by; a stage about 200 more, and 14 per token for the activations' copies; a segment 260 (partial sums); a split whose
+// combination nothing follows (q == 0) another 1700 at the end of the launch.  (Measured in place with the SM's clock: 870 to
+// 910 a round at TM = 2, 240 to 300 between the rounds of two stages.)
+static inline StreamPlan stream_candidate(const razer_desc* d, int M, int G, int SW, int TM, bool split) {
   using namespace stream_path;
   StreamPlan p;
   const Geometry g = make_geometry(d->N, d->K);
-  const int strips = (d->N + STRIP_ROWS - 1) / STRIP_ROWS;
+  const int strips = (d->N + STRIP_ROWS - 1) / STRIP_ROWS, KW = CW / SW;
+  p.SW = SW;
   p.TM = TM;
-  p.units = (strips + TM - 1) / TM;
+  p.units = (strips + SW * TM - 1) / (SW * TM);
   p.kc = g.k_chunks;
-  // slices per warp and stage: as many as leave three stages in what a CTA has for its ring
-  p.SPW = 1;
-  const int ring_bytes = SMEM_BYTES - TABLE_BYTES - 2 * CW * M * RED_STRIDE * 4 - 2048;
-  for (int spw = (TM == 1 ? 4 : 2); spw >= 1; spw >>= 1) {
-    const int stage = TM * CW * spw * PIECE_BYTES + M * (CW * spw * 128 + 16);
-    if (3 * stage <= ring_bytes) { p.SPW = spw; break; }
-  }
-  const double per_slice = TM + 0.12 + 0.04 * M;
+  // two chunks per warp and stage where that leaves three stages in what a CTA has for its ring, and two partial-sum
+  // buffers where that leaves as many
+  const int red1 = KW * M * (16 * SW * TM + 4) * 4;
+  const int ring = SMEM_BYTES - LUT_BYTES - SCALES_BYTES - BAR_BYTES - red1 - 128;
+  const int stage1 = SW * TM * KW * PIECE_BYTES + M * (KW * 128 + 16);
+  p.SPW = TM <= 2 && 6 * stage1 <= ring ? 2 : 1;
+  if (force_spw() == 1 || (force_spw() == 2 && TM <= 2 && 4 * stage1 <= ring)) p.SPW = force_spw();
+  const int stages = ring / (p.SPW * stage1);
+  p.red_bufs = (ring - red1) / (p.SPW * stage1) >= std::min(stages, 3) ? 2 : 1;
+  const double round = 16.0 * (23 * TM + 8) * (stages < 3 ? 1.12 : 1.0) + (200.0 + 14 * M) / p.SPW;
+  auto cycles = [&](int chunks) { return ((chunks + KW - 1) / KW) * round + 260; };
   const int q = p.units / G, rem = p.units - q * G;
   if (split && rem > 0) {
-    // pieces per unit: the count that leaves the busiest CTA the least to do; every further segment of a CTA costs a
-    // little (partial sums, combination), so ties go to fewer pieces
+    // pieces per unit: the count that leaves the busiest CTA the least to do
     int best_p = 1;
     double best_cost = 0;
-    const int max_p = std::max(1, std::min(8, p.kc / CW));              // a piece is at least one slice per warp
+    const int max_p = std::max(1, std::min(8, p.kc / KW));              // a piece is at least one chunk per warp
     for (int pc = 1; pc <= max_p; ++pc) {
       const int ctas = std::min(G, rem * pc);
       const int most = (rem * pc + ctas - 1) / ctas;                    // pieces of the busiest CTA
-      const double c = most * ((p.kc + pc - 1) / pc) * per_slice + (most > 1 ? 4.0 : 0.0) + 0.5 * pc;
+      const double c = cycles(most * ((p.kc + pc - 1) / pc)) + (most > 1 ? 260 : 0) + 50 * pc;
       if (pc == 1 || c < best_cost) { best_cost = c; best_p = pc; }
     }
     p.whole_base = rem;
@@ -341,7 +349,7 @@ static inline StreamPlan stream_candidate(const razer_desc* d, int M, int G, int
     p.pieces_per_unit = best_p;
     p.rem_ctas = std::min(G, rem * best_p);
     p.grid = q > 0 ? G : p.rem_ctas;
-    p.cost = (double)q * p.kc * per_slice + best_cost + (q == 0 && best_p > 1 ? 40.0 : 0.0);
+    p.cost = q * cycles(p.kc) + best_cost + (q == 0 && best_p > 1 ? 1700 : 0);
   } else {
     const int qa = (p.units + G - 1) / G;
     p.whole_base = 0;
@@ -349,31 +357,34 @@ static inline StreamPlan stream_candidate(const razer_desc* d, int M, int G, int
     p.pieces_per_unit = 1;
     p.rem_ctas = 0;
     p.grid = (p.units + qa - 1) / qa;
-    p.cost = (double)qa * p.kc * per_slice;
+    p.cost = qa * cycles(p.kc);
   }
   p.slots_bytes = (size_t)G * 2 * SLOT_FLOATS * sizeof(float);
   return p;
 }
 
-// The cheapest of the four candidates (one or two strips per unit, with or without a split).
+// The cheapest candidate (one, two or four strips per unit, with or without a split).
 static inline StreamPlan stream_plan(const razer_desc* d, int M) {
   using namespace stream_path;
-  static const int per_sm = [] { const char* e = getenv("RAZER_STREAM_CTAS"); const int v = e ? atoi(e) : 0; return v >= 1 && v <= OCC ? v : OCC; }();   // tuning aids
-  static const char force_split = [] { const char* e = getenv("RAZER_STREAM_SPLIT"); return e ? e[0] : '\0'; }();
+  static const char force_split = [] { const char* e = getenv("RAZER_STREAM_SPLIT"); return e ? e[0] : '\0'; }();   // tuning aids
   static const char force_tm = [] { const char* e = getenv("RAZER_STREAM_TM"); return e ? e[0] : '\0'; }();
-  const int G = per_sm * stream_sm_count();
+  static const char force_sw = [] { const char* e = getenv("RAZER_STREAM_SW"); return e ? e[0] : '\0'; }();
+  const int G = stream_sm_count();
   StreamPlan best;
   bool have = false;
-  for (int TM = 1; TM <= 2; ++TM) {
-    if ((force_tm == '1' && TM != 1) || (force_tm == '2' && TM != 2)) continue;
-    for (int split = 0; split <= 1; ++split) {
-      if (force_split == '0' && split) continue;
-      const StreamPlan c = stream_candidate(d, M, G, TM, split != 0);
-      if (force_split == '1' && !split && c.units % G != 0) continue;
-      if (!have || c.cost < best.cost) { best = c; have = true; }
+  for (int SW = 1; SW <= 2; ++SW) {
+    if (force_sw && force_sw != '0' + SW) continue;
+    for (int TM = 1; TM * SW <= 4; TM *= 2) {
+      if (force_tm && force_tm != '0' + TM) continue;
+      for (int split = 0; split <= 1; ++split) {
+        if (force_split == '0' && split) continue;
+        const StreamPlan c = stream_candidate(d, M, G, SW, TM, split != 0);
+        if (force_split == '1' && !split && c.units % G != 0) continue;
+        if (!have || c.cost < best.cost) { best = c; have = true; }
+      }
     }
   }
-  if (!have) best = stream_candidate(d, M, G, 1, false);
+  if (!have) best = stream_candidate(d, M, G, 1, 1, false);
   return best;
 }
 

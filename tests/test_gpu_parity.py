@@ -764,6 +764,21 @@ def test_alternative_kernels_match_the_oracle(kernel, extra_env):
     assert r.returncode == 0 and "ok" in r.stdout, r.stdout + r.stderr
 
 
+@pytest.mark.parametrize("sw,tm,spw,split", [(1, 1, 1, 1), (1, 1, 2, 0), (1, 2, 1, 1), (1, 2, 2, 1), (1, 4, 1, 0), (1, 4, 1, 1),
+                                             (2, 1, 1, 0), (2, 1, 2, 1), (2, 2, 1, 1), (2, 2, 2, 0)])
+def test_decode_kernel_unit_shapes(sw, tm, spw, split):
+    """Every unit shape of the decode kernel (warps along the rows, strips per warp, chunks per warp and stage), each forced on
+    shapes that fill no unit, end inside a chunk, and leave stages and pieces ragged."""
+    import os
+    import subprocess
+    import sys
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    env = dict(os.environ, RAZER_KERNEL="stream", RAZER_STREAM_SW=str(sw), RAZER_STREAM_TM=str(tm), RAZER_STREAM_SPW=str(spw),
+               RAZER_STREAM_SPLIT=str(split))
+    r = subprocess.run([sys.executable, "-c", _ALT_KERNEL_CHECK, root], env=env, capture_output=True, text=True, timeout=600)
+    assert r.returncode == 0 and "ok" in r.stdout, r.stdout + r.stderr
+
+
 def test_back_to_back_dependent_launches(b):
     """The matmul kernels start their weight stream while the preceding kernel of the stream still runs
     (programmatic dependent launch) and must read activations, workspace and outputs only after it has
