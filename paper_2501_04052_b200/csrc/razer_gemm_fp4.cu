@@ -203,7 +203,7 @@ razer_fp4_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_consta
     tmem_slot[3] = 0;                                   // a flag nobody sets (used by the drain waits)
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  // Weight producer state (thread 0 only).  The first ring of weight loads goes out before the rest of the
+  // Weight producer state (one elected thread of warp 0).  The first ring of weight loads goes out before the rest of the
   // prologue: the packed weights depend on nothing that precedes this kernel in the stream.
   int issued = 0;
   int p_rt = cur.tile / a.token_tiles, p_tt = cur.tile - p_rt * a.token_tiles;
@@ -215,7 +215,8 @@ razer_fp4_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_consta
     if (cur.step == spt - 1 && ++p_tt == a.token_tiles) { p_tt = 0; ++p_rt; }
     cur.next(spt);
   };
-  if (threadIdx.x == 0) {
+  __syncwarp();
+  if (warp == 0 && elect_one()) {
     asm volatile("prefetch.tensormap [%0];" ::"l"(&tmap_w) : "memory");
     grid_dep_launch();
     for (; issued < n_items && issued < WSTAGES; ++issued) produce_w();
@@ -244,7 +245,7 @@ razer_fp4_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_consta
 
   if (warp == 0) {
     // ===================== weight producer =====================
-    if (lane == 0) {
+    if (elect_one()) {
       for (; issued < n_items; ++issued) {
         if (!mbar_wait(bar_wempty + 8 * cur.ws, (uint32_t)cur.wph ^ 1u, abort_flag)) { fail(21); break; }
         produce_w();
@@ -256,7 +257,7 @@ razer_fp4_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_consta
     }
   } else if (warp == X_WARP) {
     // ===================== activation producer (codes and scale factors written by the preparation kernel) =====================
-    if (lane == 0) {
+    if (elect_one()) {
       asm volatile("prefetch.tensormap [%0];" ::"l"(&tmap_x) : "memory");
       grid_dep_wait();
       int tt = cur.tile % a.token_tiles;

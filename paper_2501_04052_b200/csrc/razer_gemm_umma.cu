@@ -19,7 +19,10 @@
 // 64) together with shared-memory bandwidth (571 cycles), and the combination of cut tiles.  Device times on B200, first for one
 // ring of weights and activations and items of one chunk at 256 tokens, then for rings apart, two-chunk items and groups that
 // walk only their own items: 2048 x 14336 x 4096 204 -> 171 us (149 with the decode left out), 256 x 8192 x 8192 38.4 -> 32.7,
-// 64 x 8192 x 28672 50.1 -> 46.7, 16 x 8192 x 28672 45.7 -> 42.2.
+// 64 x 8192 x 28672 50.1 -> 45.0, 16 x 8192 x 28672 45.7 -> 40.8.  At 16 tokens the decode takes 2500 cycles of the 4070 that a
+// group spends on an item; most of the rest it waits for its operand stage, 700 cycles from its last store to the MMAs'
+// completion.  Half-item operand stages, two to a group, came to 45.7 us (the MMA warp's waits double), all groups on one item with
+// two stages to 44.3, without the MMAs the launch takes 40.4.
 //
 // Work partition (Sec. 4.3 / App. E of the paper: stripes of about equal length that may span
 // several output tiles, partial results reduced through global memory): the grid is
@@ -179,7 +182,7 @@ razer_umma_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
     tmem_slot[3] = 0;                                   // a flag nobody sets (used by the drain waits)
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  // Weight producer state (thread 0 only).  The first ring of weight loads goes out before the rest of the prologue
+  // Weight producer state (one elected thread of warp 0).  The first ring of weight loads goes out before the rest of the prologue
   // (table, TMEM allocation): the packed weights depend on nothing, and the first HBM round trip then overlaps it.
   int issued = 0;
   int p_rt = tile / a.token_tiles, p_tt = tile - p_rt * a.token_tiles;
@@ -193,7 +196,8 @@ razer_umma_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
     next_item();
     wr.next();
   };
-  if (threadIdx.x == 0) {
+  __syncwarp();
+  if (warp == 0 && elect_one()) {
     asm volatile("prefetch.tensormap [%0];" ::"l"(&tmap_w) : "memory");
     grid_dep_launch();                                    // the next kernel may start its own prologue
     for (; issued < n_items && issued < WST; ++issued) produce_w();
@@ -220,7 +224,7 @@ razer_umma_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
 
   if (warp == 0) {
     // ===================== weight producer =====================
-    if (lane == 0) {
+    if (elect_one()) {                                    // as for the MMAs; 128 x 14336 x 4096 20.0 -> 18.7 us with both producers elected
       for (; issued < n_items; ++issued) {
         if (!mbar_wait(bar_wempty + 8 * wr.slot, wr.phase ^ 1u, abort_flag)) { fail(1); break; }
         produce_w();
@@ -232,7 +236,7 @@ razer_umma_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
     }
   } else if (warp == X_WARP) {
     // ===================== activation producer =====================
-    if (lane == 0) {
+    if (elect_one()) {
       asm volatile("prefetch.tensormap [%0];" ::"l"(&tmap_x) : "memory");
       grid_dep_wait();                                    // activations may belong to the preceding kernel
       if (cta == 0 && a.status_host) show_status(a.status_host, *(volatile uint32_t*)a.status);   // what an earlier call left
@@ -403,14 +407,16 @@ razer_umma_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
             uint32_t sw_next = 0;
             uint2 cw_next[CHUNK_BLOCKS];
             if (c + 1 < CH) load(c + 1, sw_next, cw_next);
+            // (One store for the chunk lets the four blocks' decodes mix: 16 x 8192 x 28672 42.0 -> 40.9 us.  A lookup table instead,
+            // as in the decode kernel, came out level: its loads cost what its fewer instructions save.)
+            uint32_t v[8 * CHUNK_BLOCKS];
 #pragma unroll
             for (int blk = 0; blk < CHUNK_BLOCKS; ++blk) {
               const uint32_t svp = (sw & (PACKED_SELECT << (8 * blk))) ? a.svp1 : a.svp0;
-              uint32_t v[8];
-              decode_word(cw[blk].x, ss2[blk], svp, mul_lo, mul_hi, v);
-              decode_word(cw[blk].y, ss2[blk], svp, mul_lo, mul_hi, v + 4);
-              tc_st8(a_t + (c * 4 + blk) * 8, v);
+              decode_word(cw[blk].x, ss2[blk], svp, mul_lo, mul_hi, v + 8 * blk);
+              decode_word(cw[blk].y, ss2[blk], svp, mul_lo, mul_hi, v + 8 * blk + 4);
             }
+            tc_st32(a_t + c * 32, v);
             if (c + 1 < CH) {
               sw = sw_next;
 #pragma unroll
