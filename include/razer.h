@@ -179,8 +179,9 @@ int razer_gemv_static(const razer_desc* d, const void* packed_dev, const void* x
  * aligned) that are ZERO before the first call; every call leaves them zero again, so one
  * scratch serves any number of calls one after another (calls that may overlap on the GPU
  * need a scratch each; after a call that was interrupted mid-kernel clear it again).  The
- * whole call is one kernel launch; with a computed scale its CTAs meet once (cooperative
- * launch), and a scale of NaN in tensor_scale_out_dev reports a scratch that was not zero.
+ * call is one kernel launch, whose CTAs meet once when the scale is computed (cooperative
+ * launch), or from 2^20 elements on with a computed scale two (maximum, then the rest); a scale
+ * of NaN in tensor_scale_out_dev reports a scratch that was not zero.
  * Writes act_codes_dev [M][K/2], act_scales_dev [M][K/16] in the interchange format
  * (remapped code 0x8) and the scale used to tensor_scale_out_dev. */
 int razer_quant_act(const void* x_dev, int M, int K, float sv_mag,
@@ -241,7 +242,7 @@ int razer_gemm_w4a4(const razer_desc* d, const void* packed_w_dev, const uint8_t
  * re-layout kernel between quantizer and matmul.
  * razer_fp4_act_bytes: size of that operand for M x K activations (256-byte aligned buffer, caller-owned).
  * razer_quant_act_fp4: plain NVFP4 quantization (Eq. 1-3, the arithmetic of razer_quant_act with sv_mag = 0; same
- * tensor_scale_in_dev / amax_scratch_dev contract, one launch) writing act_fp4_dev: codes padded to whole
+ * tensor_scale_in_dev / amax_scratch_dev contract, the same launches) writing act_fp4_dev: codes padded to whole
  * 256-column stages and scale bytes in the scale-factor tile order of the block-scaled MMA, padding included, so
  * the buffer needs no clearing.  The layout is internal.
  * razer_gemm_w4a4_fp4: razer_gemm_w4a4(use_native_fp4 = 1) on such an operand; bit-identical results.  Workspace:

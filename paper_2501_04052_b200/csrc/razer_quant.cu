@@ -221,6 +221,10 @@ __device__ __forceinline__ void quant_act_block(const uint4 v0, const uint4 v1, 
 // bounded all the same).  sync[] must be zero when the kernel starts; the last CTA to finish sets it back to zero.
 // A thread keeps the first block it reads for the maximum, so inputs of up to one block per resident thread are read
 // once; a single CTA needs no meeting through memory (and no cooperative launch).
+// Inputs of TWO_LAUNCH_BLOCKS and more take two launches instead: act_amax_kernel leaves the maximum in sync[0] and its CTA count in
+// the lower half of sync[1], and this kernel (amax_ctas > 0), resident early as a dependent launch and with its first block
+// in registers, reads them when that one has completed.  Its CTAs count in the upper half; the last one clears sync[].  A lower
+// half that is not the first kernel's CTA count gives away a scratch that was not zero.
 // Where the quantizer writes: the interchange format (PREPARED = false), or the FP4 activation operand of the
 // block-scaled tensor-core kernel (Fp4ActLayout: codes padded to KP columns with each word's nibbles in the packed
 // order, scale bytes in scale-factor tile order; the padding is written as zeros by this kernel too).
@@ -228,11 +232,48 @@ struct QuantActOut {
   int M, k16, kp16, spt, m_pad;      // rows; 16-element blocks per row of the input / of the padded operand; stages; padded rows
 };
 
+// Maximum magnitude of a bf16 tensor, as its bit pattern, folded into sync[0]; NaNs are skipped (patterns above 0x7F80 count as
+// zero).  Four independent loads a thread and turn.
+__device__ __forceinline__ void fold_bf16_max(uint32_t& m2, const uint4& v) {
+  const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const uint32_t a = w[j] & 0x7FFF7FFFu;
+    m2 = __vmaxu2(m2, a & ~__vcmpgtu2(a, 0x7F807F80u));
+  }
+}
+__global__ void __launch_bounds__(256) act_amax_kernel(const uint4* __restrict__ x, long long n_vec, uint32_t* __restrict__ sync) {
+  __shared__ uint32_t warp_max[8];
+  grid_dep_wait();                                        // x and sync[] may belong to the preceding kernel
+  grid_dep_launch();
+  uint32_t m2 = 0;
+  const long long stride = (long long)gridDim.x * 256;
+  long long i = (long long)blockIdx.x * 256 + threadIdx.x;
+  for (; i + 3 * stride < n_vec; i += 4 * stride) {
+    const uint4 v0 = x[i], v1 = x[i + stride], v2 = x[i + 2 * stride], v3 = x[i + 3 * stride];
+    fold_bf16_max(m2, v0);
+    fold_bf16_max(m2, v1);
+    fold_bf16_max(m2, v2);
+    fold_bf16_max(m2, v3);
+  }
+  for (; i < n_vec; i += stride) fold_bf16_max(m2, x[i]);
+  const uint32_t m = __reduce_max_sync(0xFFFFFFFFu, max(m2 & 0xFFFFu, m2 >> 16));
+  if ((threadIdx.x & 31) == 0) warp_max[threadIdx.x >> 5] = m;
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    const uint32_t all = __reduce_max_sync(0xFFFFFFFFu, warp_max[threadIdx.x & 7]);
+    if (threadIdx.x == 0) {
+      if (all) atomicMax(&sync[0], all);
+      atomicAdd(&sync[1], 1u);
+    }
+  }
+}
+
 template <bool SV, bool PREPARED>
 __global__ void __launch_bounds__(256) quant_act_fused_kernel(const uint4* __restrict__ x, long long n_blocks, float sv_mag,
                                                              const float* __restrict__ scale_in, uint32_t* sync,
                                                              uint2* __restrict__ codes, uint8_t* __restrict__ scales,
-                                                             float* __restrict__ scale_out, const QuantActOut o) {
+                                                             float* __restrict__ scale_out, const QuantActOut o, uint32_t amax_ctas) {
   __shared__ uint32_t warp_max[8];
   __shared__ uint32_t amax_shared;
   const long long n_work = PREPARED ? (long long)o.m_pad * o.kp16 : n_blocks;
@@ -249,15 +290,7 @@ __global__ void __launch_bounds__(256) quant_act_fused_kernel(const uint4* __res
     d32 = *scale_in;
   } else {
     uint32_t m2 = 0;
-    auto fold = [&](const uint4& v) {
-      const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        // NaN patterns (above 0x7F80) are skipped: a half word whose magnitude exceeds it counts as zero
-        const uint32_t a = w[j] & 0x7FFF7FFFu;
-        m2 = __vmaxu2(m2, a & ~__vcmpgtu2(a, 0x7F807F80u));
-      }
-    };
+    auto fold = [&](const uint4& v) { if (amax_ctas == 0) fold_bf16_max(m2, v); };
     if (PREPARED) {
       if (t0 < n_work) {
         int m, kb;
@@ -267,40 +300,55 @@ __global__ void __launch_bounds__(256) quant_act_fused_kernel(const uint4* __res
       // beyond the first item the maximum does not care about the padded order
       fold(f0);
       fold(f1);
-      if (n_work > stride)
+      if (amax_ctas == 0 && n_work > stride)
         for (long long t = t0; t < n_blocks; t += stride) { fold(x[2 * t]); fold(x[2 * t + 1]); }
     } else {
       if (t0 < n_work) { f0 = x[2 * t0]; f1 = x[2 * t0 + 1]; }
       fold(f0);
       fold(f1);
-      for (long long t = t0 + stride; t < n_work; t += stride) { fold(x[2 * t]); fold(x[2 * t + 1]); }
+      if (amax_ctas == 0)
+        for (long long t = t0 + stride; t < n_work; t += stride) { fold(x[2 * t]); fold(x[2 * t + 1]); }
     }
-    uint32_t m = max(m2 & 0xFFFFu, m2 >> 16);
-    m = __reduce_max_sync(0xFFFFFFFFu, m);
-    if ((threadIdx.x & 31) == 0) warp_max[threadIdx.x >> 5] = m;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      for (int i = 1; i < 8; ++i) m = max(m, warp_max[i]);
-      if (gridDim.x > 1) {
-        if (m) atomicMax(&sync[0], m);
+    if (amax_ctas > 0) {
+      grid_dep_wait();
+      grid_dep_launch();                                               // only now: a matmul behind reads packed weights at once
+      if (threadIdx.x == 0) {
+        const uint32_t a = *(volatile uint32_t*)&sync[0];
         __threadfence();
-        atomicAdd(&sync[1], 1u);
-        // all CTAs are resident (cooperative launch); the bound only guards against a dirty sync[]
-        uint32_t seen = 0;
-        for (uint32_t spins = 0; spins < (1u << 22); ++spins) {
-          asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(sync + 1) : "memory");
-          if (seen >= gridDim.x) break;
-          __nanosleep(32);
-        }
-        uint32_t a;
-        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(a) : "l"(sync) : "memory");
-        m = seen >= gridDim.x ? a : 0xFFFFFFFFu;                       // gave up: flagged below with a NaN scale
-      } else if (sync[0] | sync[1]) {
-        m = 0xFFFFFFFFu;                                               // a scratch that was not zero
+        const uint32_t prev = atomicAdd(&sync[1], 0x10000u);
+        const bool clean = (prev & 0xFFFFu) == amax_ctas;
+        if (clean && (prev >> 16) == gridDim.x - 1) sync[0] = sync[1] = 0;   // everyone has read the maximum
+        amax_shared = clean ? a : 0xFFFFFFFFu;
       }
-      amax_shared = m;
+      __syncthreads();
+    } else {
+      uint32_t m = max(m2 & 0xFFFFu, m2 >> 16);
+      m = __reduce_max_sync(0xFFFFFFFFu, m);
+      if ((threadIdx.x & 31) == 0) warp_max[threadIdx.x >> 5] = m;
+      __syncthreads();
+      if (threadIdx.x == 0) {
+        for (int i = 1; i < 8; ++i) m = max(m, warp_max[i]);
+        if (gridDim.x > 1) {
+          if (m) atomicMax(&sync[0], m);
+          __threadfence();
+          atomicAdd(&sync[1], 1u);
+          // all CTAs are resident (cooperative launch); the bound only guards against a dirty sync[]
+          uint32_t seen = 0;
+          for (uint32_t spins = 0; spins < (1u << 22); ++spins) {
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(sync + 1) : "memory");
+            if (seen >= gridDim.x) break;
+            __nanosleep(32);
+          }
+          uint32_t a;
+          asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(a) : "l"(sync) : "memory");
+          m = seen >= gridDim.x ? a : 0xFFFFFFFFu;                       // gave up: flagged below with a NaN scale
+        } else if (sync[0] | sync[1]) {
+          m = 0xFFFFFFFFu;                                               // a scratch that was not zero
+        }
+        amax_shared = m;
+      }
+      __syncthreads();
     }
-    __syncthreads();
     const uint32_t bits = amax_shared;
     if (bits == 0xFFFFFFFFu) {
       if (blockIdx.x == 0 && threadIdx.x == 0) *scale_out = __uint_as_float(0x7FC00000u);
@@ -337,7 +385,7 @@ __global__ void __launch_bounds__(256) quant_act_fused_kernel(const uint4* __res
       if ((kb & 3) == 0) *reinterpret_cast<uint32_t*>(scales + at) = sw;
     }
   }
-  if (!scale_in && gridDim.x > 1) {
+  if (!scale_in && amax_ctas == 0 && gridDim.x > 1) {
     __syncthreads();
     if (threadIdx.x == 0) {
       const uint32_t prev = atomicAdd(&sync[1], 1u);
@@ -711,6 +759,12 @@ int launch_quant_weight(const float* w, int N, int K, int block, int scale_aware
   return check_cuda(cudaGetLastError(), "quant_weight_kernel launch");
 }
 
+// One cooperative launch or two dependent ones: a meeting of the whole grid costs more on the GPU (us, replayed: 256 x 8192 8.5 against
+// 6.3 for the FP4 operand, 9.9 against 7.1 with a special value; 1000 x 4096 10.1 against 8.6; 64 x 8192 5.4 against 4.2), the second
+// launch 1 us on the host.  Level for a caller that launches from the host at 128 x 8192 (7.8 against 8.0, and 256 x 8192 10.3
+// against 7.8), where the line is drawn.
+constexpr long long TWO_LAUNCH_BLOCKS = 65536;
+
 template <bool SV, bool PREPARED>
 static int launch_quant_act_any(const void* x, int M, int K, float sv_mag, const float* scale_in, uint32_t* sync_scratch,
                                 uint8_t* codes, uint8_t* scales, float* scale_out, const QuantActOut& o, cudaStream_t st) {
@@ -718,7 +772,7 @@ static int launch_quant_act_any(const void* x, int M, int K, float sv_mag, const
   const long long n_work = PREPARED ? (long long)o.m_pad * o.kp16 : n_blocks;
   const int threads = 256;
   auto kern = quant_act_fused_kernel<SV, PREPARED>;
-  static int max_ctas = 0;                                             // CTAs that are resident together (cooperative launch)
+  static int max_ctas = 0;                                             // CTAs that are resident together
   if (!max_ctas) {
     int dev = 0, sms = 0, per_sm = 0;
     RAZER_TRY(check_cuda(cudaGetDevice(&dev), "cudaGetDevice"));
@@ -729,17 +783,30 @@ static int launch_quant_act_any(const void* x, int M, int K, float sv_mag, const
   }
   const long long b = (n_work + threads - 1) / threads;
   const int grid = (int)(b < 1 ? 1 : (b > max_ctas ? max_ctas : b));
+  const bool two = !scale_in && grid > 1 && n_blocks >= TWO_LAUNCH_BLOCKS;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)grid);
   cfg.blockDim = dim3(threads);
   cfg.stream = st;
   cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeCooperative;
-  attr[0].val.cooperative = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = scale_in || grid == 1 ? 0 : 1;                        // the grid only meets when it computes the scale
+  uint32_t amax_ctas = 0;
+  if (two) {
+    const long long n_vec = 2 * n_blocks, a = (n_vec + 4 * threads - 1) / (4 * threads);
+    amax_ctas = (uint32_t)(a > 8 * 148 ? 8 * 148 : a);
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.gridDim = dim3(amax_ctas);
+    cfg.numAttrs = 1;
+    RAZER_TRY(check_cuda(cudaLaunchKernelEx(&cfg, act_amax_kernel, (const uint4*)x, n_vec, sync_scratch), "act_amax_kernel launch"));
+    count_launches(1);
+  } else {
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
+    cfg.numAttrs = scale_in || grid == 1 ? 0 : 1;                      // the grid only meets when it computes the scale
+  }
+  cfg.gridDim = dim3((unsigned)grid);
   const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, (const uint4*)x, n_blocks, sv_mag, scale_in, sync_scratch, (uint2*)codes,
-                                           scales, scale_out, o);
+                                           scales, scale_out, o, amax_ctas);
   count_launches(1);
   return check_cuda(e, "quant_act_fused_kernel launch");
 }

@@ -238,6 +238,31 @@ def test_quant_act_given_scale_and_zero_input(b):
     assert ts.item() == 1.0 and not codes.any() and not scales.any()
 
 
+@pytest.mark.parametrize("M,K", [(64, 16368), (64, 16384), (129, 8208), (1100, 4096)])
+def test_quant_act_computed_scale_large(b, M, K):
+    """Below, at and above the size from which the tensor maximum has a launch of its own: the scale is that of Eq. 1, everything
+    else is what the same scale gives when it is handed in, and the scratch is zero again; one that was not is reported."""
+    x = inputs.activations(M, K, 85).cuda()
+    x[M - 1, K - 1] = -37.5 * x.abs().max().float()       # the maximum is the last element
+    want = torch.tensor([float(np.float32(x.abs().max().float().item()) / np.float32(448.0 * 6.0))], dtype=torch.float32).cuda()
+    for sv in (5.0, 0.0):
+        scratch = torch.zeros(2, dtype=torch.int32, device="cuda")
+        for _ in range(3):                                # back to back on one scratch
+            codes, scales, ts = b.razer_quant_act(x, sv_mag=sv, scratch=scratch)
+        assert torch.equal(ts.reshape(-1), want) and not scratch.any()
+        for got, given in zip((codes, scales), b.razer_quant_act(x, sv_mag=sv, tensor_scale=want)):
+            assert torch.equal(got, given)
+    # zeroed buffers: the alignment gap between codes and scale factors belongs to neither
+    act, act_given = torch.zeros((2, b.razer_fp4_act_bytes(M, K)), dtype=torch.uint8, device="cuda")
+    _, ts = b.razer_quant_act_fp4(x, act_fp4=act, scratch=scratch)
+    b.razer_quant_act_fp4(x, tensor_scale=want, act_fp4=act_given)
+    assert torch.equal(act, act_given) and torch.equal(ts.reshape(-1), want) and not scratch.any()
+    if M * K >= 1 << 20:
+        for dirty in (1, 7):
+            scratch = torch.tensor([0, dirty], dtype=torch.int32, device="cuda")
+            assert torch.isnan(b.razer_quant_act(x, scratch=scratch)[2]).all()
+
+
 @pytest.mark.parametrize("log2_scale", [None, -80, 0, 80])
 @pytest.mark.parametrize("sv_mag", [5.0, 8.0, None])
 def test_quant_act_extreme_magnitudes(b, log2_scale, sv_mag):
