@@ -52,22 +52,58 @@ __device__ __forceinline__ uint32_t round_to_fp4_idx(float a) {
 __device__ __forceinline__ bool short_form(float bmax, float denom) {
   return bmax < 1.0e30f && denom > 8.6736174e-19f && denom < 1.1529215e18f;
 }
-// x / d correctly rounded, y = RN(1/d); x has at most eight significant bits.
-__device__ __forceinline__ float div_bf16(float x, float d, float y) {
-  const float q = __fmul_rn(x, y);
-  return __fmaf_rn(__fmaf_rn(-q, d, x), y, q);
+// Two FP32 values in one 64-bit register: the packed instructions round each half like their scalar forms and take one issue
+// slot for both, which is what the quantizers are bound by.
+struct F2 { uint64_t v; };
+__device__ __forceinline__ F2 f2(float a, float b) { F2 r; asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(a), "f"(b)); return r; }
+__device__ __forceinline__ void split(F2 x, float& a, float& b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(x.v)); }
+__device__ __forceinline__ F2 add2(F2 a, F2 b) { F2 r; asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v)); return r; }
+__device__ __forceinline__ F2 mul2(F2 a, F2 b) { F2 r; asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v)); return r; }
+__device__ __forceinline__ F2 fma2(F2 a, F2 b, F2 c) { F2 r; asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v)); return r; }
+__device__ __forceinline__ F2 sub2(F2 a, F2 b) { return fma2(b, f2(-1.0f, -1.0f), a); }   // one rounding, of a - b
+__device__ __forceinline__ F2 abs2(F2 x) { float a, b; split(x, a, b); return f2(fabsf(a), fabsf(b)); }
+
+// x / d correctly rounded, nd = -d, y = RN(1/d); x has at most eight significant bits.
+__device__ __forceinline__ F2 div_bf16(F2 x, F2 nd, F2 y) {
+  const F2 q = mul2(x, y);
+  return fma2(fma2(q, nd, x), y, q);
 }
-// x / d correctly rounded, y = RN(1/d), any x.
-__device__ __forceinline__ float div_f32(float x, float d, float y) {
-  float q = __fmul_rn(x, y);
-  q = __fmaf_rn(__fmaf_rn(-q, d, x), y, q);
-  return __fmaf_rn(__fmaf_rn(-q, d, x), y, q);
+// x / d correctly rounded, nd = -d, y = RN(1/d), any x.
+__device__ __forceinline__ F2 div_f32(F2 x, F2 nd, F2 y) {
+  F2 q = mul2(x, y);
+  q = fma2(fma2(q, nd, x), y, q);
+  return fma2(fma2(q, nd, x), y, q);
 }
 // |x| rounded to the nearest FP4 magnitude, ties to even mantissa, saturating: adding 2^22 times the power of two at or
 // below a (at least 1) leaves two significant bits (steps of 0.5 below 2, 1 below 4, 2 from there on).
-__device__ __forceinline__ float round_to_fp4(float a) {
-  const float c = __uint_as_float((max(__float_as_uint(a), 0x3F800000u) & 0x7F800000u) + (22u << 23));
-  return fminf(__fsub_rn(__fadd_rn(a, c), c), 6.0f);
+__device__ __forceinline__ F2 round_to_fp4(F2 a) {
+  float a0, a1;
+  split(a, a0, a1);
+  const F2 c = f2(__uint_as_float((max(__float_as_uint(a0), 0x3F800000u) & 0x7F800000u) + (22u << 23)),
+                  __uint_as_float((max(__float_as_uint(a1), 0x3F800000u) & 0x7F800000u) + (22u << 23)));
+  float r0, r1;
+  split(sub2(add2(a, c), c), r0, r1);
+  return f2(fminf(r0, 6.0f), fminf(r1, 6.0f));
+}
+// Error of two scaled magnitudes under special value m (`d_r`: their distances to FP4): squares of the smaller distance, and
+// which elements are strictly closer to m.
+__device__ __forceinline__ F2 special_error(F2 a, F2 d_r, F2 minus_m, bool& t0, bool& t1) {
+  float r0, r1, s0, s1;
+  split(d_r, r0, r1);
+  split(add2(a, minus_m), s0, s1);
+  t0 = fabsf(s0) < fabsf(r0);
+  t1 = fabsf(s1) < fabsf(r1);
+  const F2 d = f2(t0 ? s0 : r0, t1 ? s1 : r1);
+  return mul2(d, d);
+}
+// Error sums of a positive and a negative special value, both continued by two elements (in order): an element's error is q_t under
+// the special value of its own sign and q_r under the other.
+__device__ __forceinline__ void add_errors(F2& e, F2 q_r, F2 q_t, bool neg0, bool neg1) {
+  float r0, r1, t0, t1;
+  split(q_r, r0, r1);
+  split(q_t, t0, t1);
+  e = add2(e, neg0 ? f2(r0, t0) : f2(t0, r0));
+  e = add2(e, neg1 ? f2(r1, t1) : f2(t1, r1));
 }
 // Eight values to FP4 codes, v[i] in nibble i (nearest, ties to even, saturating at 6; -0 and negative values that round to
 // zero give code 8).
@@ -170,12 +206,11 @@ __device__ __forceinline__ void quant_act_block(const uint4 v0, const uint4 v1, 
     return;
   }
   const float y = __frcp_rn(denom);
+  const F2 y2 = f2(y, y), nd2 = f2(-denom, -denom);
   float xs[16];
 #pragma unroll
-  for (int j = 0; j < 8; ++j) {
-    xs[2 * j] = div_bf16(__uint_as_float(w[j] << 16), denom, y);     // the scaled block of Eq. 6
-    xs[2 * j + 1] = div_bf16(__uint_as_float(w[j] & 0xFFFF0000u), denom, y);
-  }
+  for (int j = 0; j < 8; ++j)                                        // the scaled block of Eq. 6
+    split(div_bf16(f2(__uint_as_float(w[j] << 16), __uint_as_float(w[j] & 0xFFFF0000u)), nd2, y2), xs[2 * j], xs[2 * j + 1]);
   uint32_t c[2];
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
@@ -186,20 +221,20 @@ __device__ __forceinline__ void quant_act_block(const uint4 v0, const uint4 v1, 
   bool use_neg = false;
   uint32_t take[2] = {0, 0};                                         // bit 3 of the nibbles strictly closer to sv than to FP4
   if (SV) {
-    float e_pos = 0.0f, e_neg = 0.0f;
+    F2 e = f2(0.0f, 0.0f);
+    const F2 minus_sv = f2(-sv_mag, -sv_mag);
 #pragma unroll
-    for (int j = 0; j < 16; ++j) {
-      const float a = fabsf(xs[j]);
-      const bool neg = __float_as_uint(xs[j]) >> 31;
-      const float d_r = __fsub_rn(a, round_to_fp4(a)), d_s = __fsub_rn(a, sv_mag);
-      const bool t = fabsf(d_s) < fabsf(d_r);
-      const float d_t = t ? d_s : d_r;
-      const float q_r = __fmul_rn(d_r, d_r), q_t = __fmul_rn(d_t, d_t);
-      e_pos = __fadd_rn(e_pos, neg ? q_r : q_t);                     // ascending j, no fusion
-      e_neg = __fadd_rn(e_neg, neg ? q_t : q_r);
-      const int nib = PACKED ? (j & 8) + ((j & 7) >> 1) + 4 * (j & 1) : j;
-      if (t) take[nib >> 3] |= 8u << (4 * (nib & 7));
+    for (int j = 0; j < 16; j += 2) {
+      const F2 a = f2(fabsf(xs[j]), fabsf(xs[j + 1])), d_r = sub2(a, round_to_fp4(a));
+      bool t0, t1;
+      const F2 q_t = special_error(a, d_r, minus_sv, t0, t1);
+      add_errors(e, mul2(d_r, d_r), q_t, __float_as_uint(xs[j]) >> 31, __float_as_uint(xs[j + 1]) >> 31);   // ascending j, no fusion
+      const int n0 = PACKED ? (j & 8) + ((j & 7) >> 1) : j, n1 = PACKED ? n0 + 4 : j + 1;
+      if (t0) take[n0 >> 3] |= 8u << (4 * (n0 & 7));
+      if (t1) take[n1 >> 3] |= 8u << (4 * (n1 & 7));
     }
+    float e_pos, e_neg;
+    split(e, e_pos, e_neg);
     use_neg = e_neg < e_pos;                                         // ties keep metadata 0 (+sv)
   }
 #pragma unroll
@@ -537,54 +572,54 @@ __device__ __noinline__ uint32_t quant_weight_block_plain(const float4* __restri
 }
 
 // Sixteen elements of a block in the short form, at one step: error sums (continued from group to group).
-//   e_base: no special value; e[0], e[1]: +m0, +m1; e[2], e[3]: -m0, -m1 (candidates of an inactive magnitude keep e_base)
-template <bool ON0, bool ON1>
-__device__ __forceinline__ void weight_errors(const float (&xv)[16], float denom, float y, float m0, float m1, float& e_base, float (&e)[4]) {
+//   e_base: no special value; e[0], e[1]: +-m0, +-m1 (candidates of an inactive magnitude keep e_base)
+// KEEP: the scaled elements replace xv, and take[i] receives bit 3 of the nibbles strictly closer to magnitude i than to FP4.
+template <bool ON0, bool ON1, bool KEEP>
+__device__ __forceinline__ void weight_errors(float (&xv)[16], float denom, float y, float m0, float m1, float& e_base, F2 (&e)[2],
+                                              uint32_t (&take)[2][2]) {
+  const F2 nd2 = f2(-denom, -denom), y2 = f2(y, y), minus_m0 = f2(-m0, -m0), minus_m1 = f2(-m1, -m1);
 #pragma unroll
-  for (int j = 0; j < 16; ++j) {
-    const float xs = div_f32(xv[j], denom, y), a = fabsf(xs);        // the scaled block of Eq. 6
-    const bool neg = __float_as_uint(xs) >> 31;
-    const float d_r = __fsub_rn(a, round_to_fp4(a));
-    const float q_r = __fmul_rn(d_r, d_r);
-    e_base = __fadd_rn(e_base, q_r);                                 // ascending element order, no fusion
+  for (int j = 0; j < 16; j += 2) {
+    const F2 xs = div_f32(f2(xv[j], xv[j + 1]), nd2, y2);            // the scaled block of Eq. 6
+    float x0, x1, q0, q1;
+    split(xs, x0, x1);
+    const bool neg0 = __float_as_uint(x0) >> 31, neg1 = __float_as_uint(x1) >> 31;
+    const F2 a = abs2(xs), d_r = sub2(a, round_to_fp4(a)), q_r = mul2(d_r, d_r);
+    split(q_r, q0, q1);
+    if (!(ON0 && ON1)) e_base = __fadd_rn(__fadd_rn(e_base, q0), q1);   // ascending element order, no fusion
+    bool t0, t1;
     if (ON0) {
-      const float d_s = __fsub_rn(a, m0);
-      const float d_t = fabsf(d_s) < fabsf(d_r) ? d_s : d_r;         // strictly closer only
-      const float q_t = __fmul_rn(d_t, d_t);
-      e[0] = __fadd_rn(e[0], neg ? q_r : q_t);
-      e[2] = __fadd_rn(e[2], neg ? q_t : q_r);
+      add_errors(e[0], q_r, special_error(a, d_r, minus_m0, t0, t1), neg0, neg1);
+      if (KEEP && t0) take[0][j >> 3] |= 8u << (4 * (j & 7));
+      if (KEEP && t1) take[0][j >> 3] |= 8u << (4 * ((j + 1) & 7));
     }
     if (ON1) {
-      const float d_s = __fsub_rn(a, m1);
-      const float d_t = fabsf(d_s) < fabsf(d_r) ? d_s : d_r;
-      const float q_t = __fmul_rn(d_t, d_t);
-      e[1] = __fadd_rn(e[1], neg ? q_r : q_t);
-      e[3] = __fadd_rn(e[3], neg ? q_t : q_r);
+      add_errors(e[1], q_r, special_error(a, d_r, minus_m1, t0, t1), neg0, neg1);
+      if (KEEP && t0) take[1][j >> 3] |= 8u << (4 * (j & 7));
+      if (KEEP && t1) take[1][j >> 3] |= 8u << (4 * ((j + 1) & 7));
     }
+    if (KEEP) xv[j] = x0, xv[j + 1] = x1;
   }
 }
 // One candidate alone (AWARE): magnitude m on the elements whose sign bit is `sgn`.
 __device__ __forceinline__ float weight_error_one(const float (&xv)[16], float denom, float y, float m, uint32_t sgn, float e) {
+  const F2 nd2 = f2(-denom, -denom), y2 = f2(y, y), minus_m = f2(-m, -m);
 #pragma unroll
-  for (int j = 0; j < 16; ++j) {
-    const float xs = div_f32(xv[j], denom, y), a = fabsf(xs);
-    const float d_r = __fsub_rn(a, round_to_fp4(a)), d_s = __fsub_rn(a, m);
-    const bool t = fabsf(d_s) < fabsf(d_r) && (__float_as_uint(xs) >> 31) == sgn;
-    const float d_t = t ? d_s : d_r;
-    e = __fadd_rn(e, __fmul_rn(d_t, d_t));
+  for (int j = 0; j < 16; j += 2) {
+    const F2 xs = div_f32(f2(xv[j], xv[j + 1]), nd2, y2), a = abs2(xs), d_r = sub2(a, round_to_fp4(a));
+    float x0, x1, r0, r1, s0, s1;
+    split(xs, x0, x1);
+    split(d_r, r0, r1);
+    split(add2(a, minus_m), s0, s1);
+    const bool t0 = fabsf(s0) < fabsf(r0) && (__float_as_uint(x0) >> 31) == sgn, t1 = fabsf(s1) < fabsf(r1) && (__float_as_uint(x1) >> 31) == sgn;
+    const F2 d = f2(t0 ? s0 : r0, t1 ? s1 : r1);
+    split(mul2(d, d), r0, r1);
+    e = __fadd_rn(__fadd_rn(e, r0), r1);
   }
   return e;
 }
-// Codes of sixteen elements under the winning candidate (magnitude m, sign bit sgn).
-__device__ __forceinline__ uint2 weight_codes(const float (&xv)[16], float denom, float y, float m, uint32_t sgn, uint32_t remap_code) {
-  float xs[16];
-  uint32_t take[2] = {0, 0};
-#pragma unroll
-  for (int j = 0; j < 16; ++j) {
-    xs[j] = div_f32(xv[j], denom, y);
-    const float a = fabsf(xs[j]);
-    if (fabsf(__fsub_rn(a, m)) < fabsf(__fsub_rn(a, round_to_fp4(a)))) take[j >> 3] |= 8u << (4 * (j & 7));
-  }
+// Codes of sixteen scaled elements, those in `take` (bit 3 of their nibbles) that have sign bit `sgn` to the special value.
+__device__ __forceinline__ uint2 codes_of_scaled(const float (&xs)[16], const uint32_t (&take)[2], uint32_t sgn, uint32_t remap_code) {
   uint32_t c[2];
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
@@ -600,6 +635,38 @@ __device__ __forceinline__ uint2 weight_codes(const float (&xv)[16], float denom
   }
   return make_uint2(c[0], c[1]);
 }
+// Codes of sixteen elements under the winning candidate (magnitude m, sign bit sgn).
+__device__ __forceinline__ uint2 weight_codes(const float (&xv)[16], float denom, float y, float m, uint32_t sgn, uint32_t remap_code) {
+  const F2 nd2 = f2(-denom, -denom), y2 = f2(y, y), minus_m = f2(-m, -m);
+  float xs[16];
+  uint32_t take[2] = {0, 0};
+#pragma unroll
+  for (int j = 0; j < 16; j += 2) {
+    const F2 q = div_f32(f2(xv[j], xv[j + 1]), nd2, y2), a = abs2(q);
+    split(q, xs[j], xs[j + 1]);
+    float r0, r1, s0, s1;
+    split(sub2(a, round_to_fp4(a)), r0, r1);
+    split(add2(a, minus_m), s0, s1);
+    if (fabsf(s0) < fabsf(r0)) take[j >> 3] |= 8u << (4 * (j & 7));
+    if (fabsf(s1) < fabsf(r1)) take[j >> 3] |= 8u << (4 * ((j + 1) & 7));
+  }
+  return codes_of_scaled(xs, take, sgn, remap_code);
+}
+
+// Eight floats from a 16-byte aligned address, in one 32-byte load where the tensor is aligned to that (`wide`, uniform): a block
+// of its own per thread makes every load of a warp touch 32 separate sectors, and halves fetched apart cost twice the requests
+// (blocks of 32 to 128 elements: 140 us for 11008 x 4096, now 88; blocks of 16: 67, now 62).
+__device__ __forceinline__ void load8(const float4* p, float* v, bool wide) {
+  if (wide) {
+    asm volatile("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7])
+                 : "l"(p));
+  } else {
+    const float4 a = p[0], b = p[1];
+    v[0] = a.x, v[1] = a.y, v[2] = a.z, v[3] = a.w, v[4] = b.x, v[5] = b.y, v[6] = b.z, v[7] = b.w;
+  }
+}
+__device__ __forceinline__ bool aligned32(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 31) == 0; }
 
 // One thread per scale block of `sub` groups of 16 elements (ONE: sub == 1, the block stays in registers from its maximum
 // to its codes; larger blocks are walked three times).  A magnitude beyond 6 can win an element only where the block's
@@ -607,11 +674,12 @@ __device__ __forceinline__ uint2 weight_codes(const float (&xv)[16], float denom
 // would equal those without a special value.  The grid runs from the end of the tensor to its start, the reverse of the
 // maximum's order, so that the part of the input still in L2 is read first.
 template <bool AWARE, bool ONE>
-__global__ void __launch_bounds__(256) quant_weight_kernel(const float4* __restrict__ w, long long n_blocks, int sub_arg, float m0, float m1,
+__global__ void __launch_bounds__(256, 4) quant_weight_kernel(const float4* __restrict__ w, long long n_blocks, int sub_arg, float m0, float m1,
                                                           uint32_t remap_code, const float* __restrict__ scale_in,
                                                           const uint32_t* __restrict__ amax_bits, uint2* __restrict__ codes,
                                                           uint8_t* __restrict__ scales, float* __restrict__ scale_out) {
   const int sub = ONE ? 1 : sub_arg;
+  const bool wide = aligned32(w);
   float d32;
   if (scale_in) {
     d32 = *scale_in;
@@ -631,10 +699,7 @@ __global__ void __launch_bounds__(256) quant_weight_kernel(const float4* __restr
     float xv[16];
     auto load = [&](int g) {
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const float4 v = src[4 * g + q];
-        xv[4 * q] = v.x, xv[4 * q + 1] = v.y, xv[4 * q + 2] = v.z, xv[4 * q + 3] = v.w;
-      }
+      for (int q = 0; q < 2; ++q) load8(src + 4 * g + 2 * q, xv + 8 * q, wide);
     };
     uint32_t mbits = 0;
 #pragma unroll 1
@@ -686,15 +751,21 @@ __global__ void __launch_bounds__(256) quant_weight_kernel(const float4* __restr
       }
       continue;
     }
-    float e_base = 0.0f, e[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+    float e_base = 0.0f;
+    F2 e2[2] = {f2(0.0f, 0.0f), f2(0.0f, 0.0f)};
+    uint32_t take[2][2] = {{0, 0}, {0, 0}};
+    constexpr bool KEEP = ONE && !AWARE;
 #pragma unroll 1
     for (int g = 0; g < sub; ++g) {
       if (!ONE) load(g);
-      if (on0 && on1) weight_errors<true, true>(xv, denom, y, m0, m1, e_base, e);
-      else if (on0) weight_errors<true, false>(xv, denom, y, m0, m1, e_base, e);
-      else if (on1) weight_errors<false, true>(xv, denom, y, m0, m1, e_base, e);
-      else weight_errors<false, false>(xv, denom, y, m0, m1, e_base, e);
+      if (on0 && on1) weight_errors<true, true, KEEP>(xv, denom, y, m0, m1, e_base, e2, take);
+      else if (on0) weight_errors<true, false, KEEP>(xv, denom, y, m0, m1, e_base, e2, take);
+      else if (on1) weight_errors<false, true, KEEP>(xv, denom, y, m0, m1, e_base, e2, take);
+      else weight_errors<false, false, KEEP>(xv, denom, y, m0, m1, e_base, e2, take);
     }
+    float e[4];                                                        // metadata order: +m0, +m1, -m0, -m1
+    split(e2[0], e[0], e[2]);
+    split(e2[1], e[1], e[3]);
     if (!on0) e[0] = e[2] = e_base;
     if (!on1) e[1] = e[3] = e_base;
     if (AWARE) {
@@ -728,7 +799,12 @@ __global__ void __launch_bounds__(256) quant_weight_kernel(const float4* __restr
 #pragma unroll 1
     for (int g = 0; g < sub; ++g) {
       if (!ONE) load(g);
-      codes[t * sub + g] = weight_codes(xv, denom, y_win, m_win, meta >> 1, remap_code);
+      if (KEEP) {
+        const uint32_t won[2] = {(meta & 1u) ? take[1][0] : take[0][0], (meta & 1u) ? take[1][1] : take[0][1]};
+        codes[t] = codes_of_scaled(xv, won, meta >> 1, remap_code);
+      } else {
+        codes[t * sub + g] = weight_codes(xv, denom, y_win, m_win, meta >> 1, remap_code);
+      }
     }
     scales[t] = (uint8_t)((meta << 6) | scode);
   }

@@ -282,6 +282,18 @@ def test_quant_act_extreme_magnitudes(b, log2_scale, sv_mag):
     assert np.all(blk_ok | dbg["near_tie"])
 
 
+@pytest.mark.parametrize("block,aware", [(16, False), (16, True), (32, False), (128, True)])
+def test_quant_weight_any_alignment(b, block, aware):
+    """A weight tensor on a 16-byte boundary that is not a 32-byte one gives what the same tensor gives on a 256-byte boundary."""
+    N, K = 131, 384
+    w = inputs.student_t_weights(N, K, 9, outlier_frac=0.01).cuda()
+    buf = torch.empty(N * K + 4, device="cuda")
+    off = buf[4:].view(N, K).copy_(w)
+    assert off.data_ptr() % 32 == 16 and w.data_ptr() % 32 == 0
+    for got, want in zip(b.razer_quant_weight(off, block=block, scale_aware=aware), b.razer_quant_weight(w, block=block, scale_aware=aware)):
+        assert torch.equal(got, want)
+
+
 @pytest.mark.parametrize("block,aware", [(16, False), (16, True), (64, False), (128, True)])
 def test_quant_weight_extreme_magnitudes(b, block, aware):
     """The same for the weight quantizer, at a given tensor scale that puts some rows' steps outside the short form."""
