@@ -15,7 +15,7 @@
 // (razer_decode.cuh) costs five and a quarter, two of them on the half-rate FMA pipe: 61 instructions per 16 weights came down to
 // 47, and what binds is now the shared-memory pipe (14 wavefronts per warp and 16 weights a lane, 94 % of it busy while a launch
 // streams).  Decoding an eighth to a half of the words in registers instead, to even the two out, measured 1 to 13 % slower;
-// 20 or 24 consumer warps 6 to 10 %; reading the next slice ahead of the current one's decode 15 %.
+// 20 or 24 consumer warps 6 to 10 %.
 // Unit: SW * TM strips; a warp that takes more strips of a chunk (TM) reads its activation fragment less often.
 // Each producer issues from one lane elected once: with the issue of both in one lane chosen by its index, a copy cost 200 to 300
 // cycles of that warp, and at 8 tokens (10 copies a stage) the launch waited for the issue: 8 x 28672 x 8192 60.4 us, now 33.9.
@@ -27,8 +27,8 @@
 // Work: a unit is SW * TM strips of 16 weight rows over the whole of K; a slice is one unit x one 64-column chunk.
 // A stage of the ring holds KW * SPW consecutive slices of one unit and the matching activation columns.  A CTA has an SM to
 // itself (the tables are large); the CTAs of the next launch in the stream start as those of this one exit (programmatic
-// dependent launch), fill their tables and rings and wait.  Two CTAs of half the ring per SM, so that the next launch is resident
-// earlier, measured 1.4 to 2 times slower.
+// dependent launch), fill their tables and rings and wait.  Two CTAs per SM, so that the next launch is resident
+// earlier, would leave each a ring of 36 KB beside its tables.
 // Partition (host, stream_plan): either every CTA takes whole units only, or every CTA takes q whole units
 // and the remaining units are cut along K into equal slice ranges, one range per CTA, processed FIRST: a
 // unit shared by several CTAs is combined through FP32 slots in the workspace by the last CTA to arrive (one
