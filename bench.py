@@ -34,8 +34,8 @@ DECODE_SHAPES = [(4096, 4096), (11008, 4096), (4096, 11008)]
 SKINNY_SHAPES = [(8192, 8192), (28672, 8192), (8192, 28672)]
 PREFILL_SHAPES = [(14336, 4096), (4096, 14336)]
 # DRAM bytes of one step (its three launches) read from the ncu capture of the kernel as committed:
-# 9,506,304 + 25,430,272 + 25,445,120 read, 0 written.  Set to None whenever the kernel changes until re-captured.
-NCU_DRAM_BYTES_PER_STEP = 60381696
+# 9,492,992 + 25,426,688 + 25,432,320 read, 0 written.  Set to None whenever the kernel changes until re-captured.
+NCU_DRAM_BYTES_PER_STEP = 60352000
 METRIC = "razer_gemv_effective_hbm_bandwidth"
 
 
