@@ -1,4 +1,4 @@
-// Register-level decode of packed RaZeR blocks to bf16 pairs, shared by the matmul kernels.
+// Register-level decode of packed RaZeR blocks to bf16 pairs: the tcgen05 matmul kernel, and what the others share of it.
 //
 // Per pair of elements, with no comparison and no conversion instruction: the stored nibble
 // is isolated in both 16-bit halves of the word, one integer multiply-add drops two shifted
