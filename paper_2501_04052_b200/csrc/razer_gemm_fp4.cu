@@ -364,8 +364,8 @@ razer_fp4_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_consta
       const float ts = a.extra_scale ? a.tensor_scale * *a.extra_scale : a.tensor_scale;
       const int done_tile = pending.tile;
       pending.tile = -1;
-      return segment_epilogue<NT, C::NACC, NRW / 4>(
-          a, ctx, done_tile, pending.at_end, ts, seg++, epi_phase, abort_flag,
+      return segment_epilogue<NT, C::NACC, 1, NRW / 4>(
+          a, ctx, done_tile, pending.at_end, 1u, ts, seg++, epi_phase, abort_flag,
           [&](uint32_t bar, uint32_t parity, uint32_t which) { return wait_all(bar, parity, 27u + which); },
           [&](uint32_t which) { fail(27u + which); });
     };

@@ -94,6 +94,11 @@ struct UmmaCfg {
   static constexpr int X_BOX_BYTES = NT * 128;                 // NT tokens x 64 k x 2 B
   static constexpr int X_BYTES = CHX * X_BOX_BYTES;
   static constexpr int ACC_COLS = NACC * NT < 32 ? 32 : NACC * NT;   // NACC accumulators, used round robin
+  // More than two accumulators: a set for each operand slot, so that an item's products meet only those of every AST-th item.  The
+  // tensor core's FP32 additions truncate, and their error grows with the length of a chain: with six accumulators instead of
+  // two, which 16 tokens leave TMEM for, it is a third (16 x 8192 x 28672: 3.7e-9 of |x||w| instead of 1.24e-8, outputs off the
+  // correctly rounded value 5 in 10^4 instead of 15), at 42.3 instead of 41.8 us a pass.
+  static constexpr int SETS = NACC > 2 ? AST : 1, PER_SET = NACC / SETS;
   static constexpr int A_STAGE_COLS = CH * 32;                 // 4 blocks x 8 columns per chunk
   static constexpr int TMEM_COLS_NEEDED = ACC_COLS + AST * A_STAGE_COLS;
   static constexpr int TMEM_COLS = TMEM_COLS_NEEDED <= 64 ? 64 : TMEM_COLS_NEEDED <= 128 ? 128
@@ -105,6 +110,7 @@ struct UmmaCfg {
   static_assert(TMEM_COLS_NEEDED <= 512, "TMEM budget exceeded");
   static_assert(SMEM_BYTES <= 232448, "shared memory budget exceeded");
   static_assert(CH % CHX == 0, "an item is whole activation stages");
+  static_assert(NACC % SETS == 0 && PER_SET <= 4, "a set is within an item's first chunk, which every item has");
   static_assert(NT % 16 == 0 && NT >= 16 && NT <= 256, "UMMA N for M = 128");
   // A parity wait is only sound for a waiter that knows the barrier's previous phase to be complete.  The groups take the
   // items in turn, so a stage has to come round to the same group every time: then that group has seen all its phases.
@@ -274,6 +280,7 @@ razer_umma_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
     // addresses in uniform registers; electing anew for every item cost about 37 cycles per tcgen05 instruction.
     if (elect_one()) {
       uint32_t seg = 0;
+      int seg_items = 0;                                  // of the segment, issued
       bool alive = true;
       Ring<XST> xr;
       Ring<AST> ar;
@@ -285,7 +292,10 @@ razer_umma_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
         if (seg_first && !mbar_wait(bar_accempty, (seg & 1u) ^ 1u, abort_flag)) { fail(4); break; }
         tc_fence_after();
         const uint32_t a_t = tmem_a0 + ar.slot * Cfg::A_STAGE_COLS;
-        // Consecutive MMAs go to NACC different accumulators (summed in the epilogue): MMAs on one
+        if (seg_first) seg_items = 0;
+        const bool fresh = seg_items++ < Cfg::SETS;       // the item's set of accumulators holds nothing of this segment yet
+        const uint32_t d_0 = tmem_base + (Cfg::SETS > 1 ? ar.slot * (Cfg::PER_SET * NT) : 0);
+        // Consecutive MMAs go to different accumulators (summed in the epilogue): MMAs on one
         // accumulator execute one after the other, and a narrow MMA is far shorter than its latency.
 #pragma unroll
         for (int h = 0; h < CH / CHX; ++h) {
@@ -299,8 +309,8 @@ razer_umma_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
               // 16 k further along: +32 bytes inside a chunk's 128-byte rows, next chunk's box after four
               if (j < nch * 4) {
                 const uint32_t bd = bd_lo + (uint32_t)(((k >> 2) * Cfg::X_BOX_BYTES + (k & 3) * 32) >> 4);
-                const uint32_t d_t = tmem_base + (j % NACC) * NT;
-                if (j < NACC && seg_first) tc_mma_ts2<false>(d_t, a_t + j * 8, bd, bd_hi, idesc);
+                const uint32_t d_t = d_0 + (j % Cfg::PER_SET) * NT;
+                if (j < Cfg::PER_SET && fresh) tc_mma_ts2<false>(d_t, a_t + j * 8, bd, bd_hi, idesc);
                 else tc_mma_ts2<true>(d_t, a_t + j * 8, bd, bd_hi, idesc);
               }
             }
@@ -351,8 +361,15 @@ razer_umma_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
       const float ts = a.extra_scale ? a.tensor_scale * *a.extra_scale : a.tensor_scale;
       const int done_tile = pending.tile;
       pending.tile = -1;
-      return segment_epilogue<NT, NACC, GROUPS>(
-          a, ctx, done_tile, pending.at_end, ts, seg++, epi_phase, abort_flag,
+      uint32_t live = 1u;                                  // sets of accumulators that an item of the segment went to
+      if (Cfg::SETS > 1) {
+        const int first = max(done_tile * spt - it_begin, 0), count = min((done_tile + 1) * spt, it_end) - it_begin - first;
+        live = 0;
+#pragma unroll
+        for (int q = 0; q < Cfg::SETS; ++q) live |= (uint32_t)((q + Cfg::SETS - first % Cfg::SETS) % Cfg::SETS < count) << q;
+      }
+      return segment_epilogue<NT, Cfg::PER_SET, Cfg::SETS, GROUPS>(
+          a, ctx, done_tile, pending.at_end, live, ts, seg++, epi_phase, abort_flag,
           [&](uint32_t bar, uint32_t parity, uint32_t which) { return wait_all(bar, parity, 7u + which); },
           [&](uint32_t which) { fail(7u + which); });
     };
@@ -588,7 +605,7 @@ int launch_gemm_umma(const razer_desc* d, const void* packed, const void* x, int
   a.total_items = p.total_items;
   a.x_map_3d = map_3d;
   switch (p.NT) {
-    case 16: return launch_cfg<16, 4, 4, 6, 4, 3, 12, 2>(tmap, tmap_w, a, p.grid, st);
+    case 16: return launch_cfg<16, 4, 4, 6, 4, 3, 12, 6>(tmap, tmap_w, a, p.grid, st);
     case 32: return launch_cfg<32, 4, 4, 6, 4, 3, 12, 2>(tmap, tmap_w, a, p.grid, st);
     case 64: return launch_cfg<64, 4, 4, 6, 3, 3, 12, 2>(tmap, tmap_w, a, p.grid, st);
     case 96: return launch_cfg<96, 4, 2, 6, 4, 3, 12, 1>(tmap, tmap_w, a, p.grid, st);

@@ -94,9 +94,11 @@ struct EpilogueCtx {
 // a: kernel arguments (y, slots, counters, g, M, token_tiles, steps_per_tile, total_items, split).  at_end: the segment reaches the
 // end of its tile.  GROUPS sets of four warps share the columns in units of 16.  wait(barrier, parity, which) is a bounded
 // wait of the whole warp, fail(which) records one that gave up: which = 0 accumulator, 1 rendezvous, 2 other CTAs.
-template <int NT, int NACC, int GROUPS, class KernelArgs, class Wait, class Fail>
-__device__ __forceinline__ bool segment_epilogue(const KernelArgs& a, const EpilogueCtx& x, int tile, bool at_end, float ts, uint32_t seg,
-                                                 uint32_t& epi_phase, volatile uint32_t* abort_flag, Wait wait, Fail fail) {
+// The tile's sum is spread over SETS sets of PER_SET accumulators, of which those in `live` hold something (set 0 does where SETS
+// is 1).
+template <int NT, int PER_SET, int SETS, int GROUPS, class KernelArgs, class Wait, class Fail>
+__device__ __forceinline__ bool segment_epilogue(const KernelArgs& a, const EpilogueCtx& x, int tile, bool at_end, uint32_t live, float ts,
+                                                 uint32_t seg, uint32_t& epi_phase, volatile uint32_t* abort_flag, Wait wait, Fail fail) {
   constexpr int UNITS = NT / 16, MAXC = 16 * ((UNITS + GROUPS - 1) / GROUPS);
   constexpr size_t SLOT = (size_t)NT * 128;                  // [NT / 4][128 rows][4] floats: a thread reads and writes 16 bytes at a time
   const int grid = gridDim.x, cta = blockIdx.x, spt = a.steps_per_tile;
@@ -107,15 +109,16 @@ __device__ __forceinline__ bool segment_epilogue(const KernelArgs& a, const Epil
   const int valid = min(n_cols, a.M - m0);                   // columns that are tokens
   const int n_out = rt * 128 + x.row;
   __nv_bfloat16* dst = a.y + (size_t)m0 * a.g.N + n_out;
-  // sixteen columns of the accumulator, summed over the NACC accumulators used in turn
+  // sixteen columns of the accumulator, summed over the accumulators used in turn
   auto load16 = [&](int c, float (&v)[16]) {
     uint32_t w[16];
     tc_ld16(x.tmem + col_lo + c, w);
     tc_wait_ld();
 #pragma unroll
-    for (int j = 0; j < 16; ++j) v[j] = __uint_as_float(w[j]);
+    for (int j = 0; j < 16; ++j) v[j] = SETS == 1 || (live & 1u) ? __uint_as_float(w[j]) : 0.0f;
 #pragma unroll
-    for (int q = 1; q < NACC; ++q) {
+    for (int q = 1; q < SETS * PER_SET; ++q) {
+      if (SETS > 1 && !((live >> (q / PER_SET)) & 1u)) continue;
       tc_ld16(x.tmem + q * NT + col_lo + c, w);
       tc_wait_ld();
 #pragma unroll

@@ -205,6 +205,28 @@ def test_gemm_token_tiles_and_partitions(b, M, N, K):
     _check_matmul(b, b.razer_gemm, desc, packed, codes, scales, 0.002, x, rows=rows_with_edge_tiles(N, 96, 76))
 
 
+def test_gemm_sixteen_tokens_keep_three_partial_sums_apart(b):
+    """Up to 16 tokens, three items of 256 columns in a row are summed apart and added up once per tile (a third of the
+    additions in a chain).  All weights are 1, and a tile's four items contribute 2^30, 1, 1 + m and -2^30: FP32 sums in one chain
+    lose the two in the middle (a unit of 2^30 in FP32 is 128), sums apart lose nothing, so y is exact.  148 row tiles of 1024
+    columns stay whole on a CTA each; the 16 rows beyond make a tile whose parts several CTAs hold, some without all three."""
+    M, K = 16, 1024
+    x = torch.zeros((M, K), dtype=torch.bfloat16)
+    x[:, 5], x[:, 256 + 5], x[:, 512 + 5], x[:, 768 + 5] = 2.0 ** 30, 1.0, 1.0 + torch.arange(M), -2.0 ** 30
+    want = (2.0 + torch.arange(M)).to(torch.bfloat16).cuda()[:, None]
+    for N in (148 * 128, 148 * 128 + 16):
+        codes = torch.full((N, K // 2), 0x22, dtype=torch.uint8)              # 1.0
+        scales = torch.full((N, K // 16), 0x38, dtype=torch.uint8)            # x 1.0
+        desc, packed = _pack(b, codes.numpy(), scales.numpy(), 1.0)
+        y = b.razer_gemm(desc, packed, x.cuda())
+        if N == 148 * 128:
+            assert torch.equal(y, want.expand(M, N))
+        x1 = inputs.activations(M, K, 77)
+        y1 = b.razer_gemm(desc, packed, x1.cuda())
+        ref = x1.double().sum(1)
+        assert torch.all((y1.cpu().double() - ref[:, None]).abs() <= 2.0 ** -8 * ref.abs()[:, None] + 2.0 ** -20 * x1.double().abs().sum(1)[:, None])
+
+
 # ------------------------------------------------------------------ activation quantization / W4A4
 
 @pytest.mark.parametrize("M,K,seed", [(256, 8192, 80), (7, 48, 81), (33, 1040, 82)])
