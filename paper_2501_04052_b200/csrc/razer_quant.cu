@@ -46,11 +46,12 @@ __device__ __forceinline__ uint32_t round_to_fp4_idx(float a) {
          (uint32_t)(a >= 1.75f) + (uint32_t)(a > 2.5f) + (uint32_t)(a >= 3.5f) + (uint32_t)(a > 5.0f);
 }
 
-// The short form of a block's arithmetic: valid for finite inputs below 2^100 and steps within 2^-60 .. 2^60.  (An element
+// The short form of a block's arithmetic: valid for finite inputs below 2^100, steps within 2^-60 .. 2^60 and quotients below 2^100
+// (a quotient that FP32 cannot hold would be infinite and its correction a NaN).  (An element
 // below 2^-100 may then miss its quotient's last bit, which is far below anything the error sums of a block whose
 // candidates differ can see: such an element's share is under 2^-80, a difference between candidates over 2^-40.)
 __device__ __forceinline__ bool short_form(float bmax, float denom) {
-  return bmax < 1.0e30f && denom > 8.6736174e-19f && denom < 1.1529215e18f;
+  return bmax < 1.0e30f && bmax < denom * 1.0e30f && denom > 8.6736174e-19f && denom < 1.1529215e18f;
 }
 // Two FP32 values in one 64-bit register: the packed instructions round each half like their scalar forms and take one issue
 // slot for both, which is what the quantizers are bound by.

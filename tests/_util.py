@@ -34,6 +34,39 @@ def rows_with_edge_tiles(N, n, seed, tile=128):
     return np.unique(np.concatenate([rng.integers(0, N, n), first, last]))
 
 
+def codes_of_scales(x, d32, scales, block, scale_fmt, sv_mag, remap_code=0x8):
+    """The element codes (packed, [R][C/2]) that the blocks' own scale bytes imply for x: with the scale and the special value that a
+    byte names, every element has one code (Eq. 3, 6, 7).  sv_mag = None: no special value."""
+    f32 = np.float32
+    R, C = x.shape
+    bits = 8 - ro.meta_bits(scale_fmt)
+    scode, meta = scales & ((1 << bits) - 1), scales >> bits
+    denom = (f32(d32) * ro.scale_grid(scale_fmt)[scode].astype(f32)).astype(f32)[:, :, None]
+    with np.errstate(all="ignore"):
+        xs = np.where(denom == 0, f32(0), x.reshape(R, C // block, block) / np.where(denom == 0, f32(1), denom)).astype(f32)
+        idx = ro.round_to_fp4(xs)
+        code = np.where(idx == 0, remap_code ^ 8, idx | (np.signbit(xs).astype(np.uint8) << 3)).astype(np.uint8)
+        if sv_mag is not None:
+            mags = np.array([0, .5, 1, 1.5, 2, 3, 4, 6], dtype=f32)[idx]
+            sv = np.array(ro.sv_candidates(sv_mag, scale_fmt), dtype=f32)[meta][:, :, None]
+            code = np.where(np.abs(xs - sv) < np.abs(xs - np.where(np.signbit(xs), -mags, mags)), remap_code, code).astype(np.uint8)
+    code = np.where(scode[:, :, None] == 0, remap_code ^ 8, code).reshape(R, C)
+    return (code[:, 0::2] | (code[:, 1::2] << 4)).astype(np.uint8)
+
+
+def blocks_agree(x, d32, got, want, near_tie, block, scale_fmt, sv_mag, remap_code=0x8, own_scales=False):
+    """Which blocks of a quantizer's result (codes, scale bytes) are right: those equal to the oracle's, and where the oracle's two best
+    candidates tie within rounding, those with another special value (own_scales: and its scale) whose codes are the ones that the
+    scale byte implies."""
+    (got_c, got_s), (want_c, want_s) = got, want
+    R, nb = got_s.shape
+    per_block = lambda eq: np.all(eq.reshape(R, nb, block // 2), axis=2)
+    same = (got_s == want_s) & per_block(got_c == want_c)
+    bits = 8 - ro.meta_bits(scale_fmt)
+    other = own_scales | ((got_s ^ want_s) & ((1 << bits) - 1) == 0)
+    return same, same | (near_tie & other & per_block(got_c == codes_of_scales(x, d32, got_s, block, scale_fmt, sv_mag, remap_code)))
+
+
 def oracle_reference(x_bits, codes, scales, tensor_scale, chunk_rows=2048, **kw):
     """Oracle outputs for all rows of (codes, scales), computed chunk by chunk over the weight rows to bound
     memory: (bf16 bits [M, n], unrounded FP64 result [M, n], tensor_scale * sum_k |x * D1| [M, n])."""

@@ -12,7 +12,7 @@ import torch
 from oracle import razer_oracle as ro
 from paper_2501_04052_b200 import inputs
 
-from _util import (elementwise_report, oracle_quantized_weights, oracle_reference, rel_fro_bits, rows_with_edge_tiles,
+from _util import (blocks_agree, elementwise_report, oracle_quantized_weights, oracle_reference, rel_fro_bits, rows_with_edge_tiles,
                    sample_rows, to_dev)
 
 pytestmark = pytest.mark.gpu
@@ -285,11 +285,12 @@ def test_quant_act_computed_scale_large(b, M, K):
             assert torch.isnan(b.razer_quant_act(x, scratch=scratch)[2]).all()
 
 
-@pytest.mark.parametrize("log2_scale", [None, -80, 0, 80])
+@pytest.mark.parametrize("log2_scale", [None, -80, -58, -50, -40, 0, 80])
 @pytest.mark.parametrize("sv_mag", [5.0, 8.0, None])
 def test_quant_act_extreme_magnitudes(b, log2_scale, sv_mag):
     """Rows from bf16 subnormals to 2^100, zero blocks among them, against the oracle: the blocks that the kernel's short form
-    cannot take go through the plain procedure, with the same decisions."""
+    cannot take go through the plain procedure, with the same decisions.  At the scales -58 to -40 the step alone and the
+    largest elements alone are within the short form's range, but the quotient is not (FP32 infinity)."""
     M, K = 60, 272
     x = inputs.activations(M, K, 84).float() * torch.pow(2.0, torch.linspace(-132, 100, M))[:, None]
     x[5, 32:64] = 0.0
@@ -300,8 +301,15 @@ def test_quant_act_extreme_magnitudes(b, log2_scale, sv_mag):
         want_c, want_s, want_d, dbg = ro.quantize_act(inputs.bf16_to_bits(x), sv_mag=sv_mag and (sv_mag,), return_debug=True,
                                                       tensor_scale=None if ts is None else np.float32(ts.item()))
     assert np.float32(out.item()) == want_d
-    blk_ok = (scales.cpu().numpy() == want_s) & np.all((codes.cpu().numpy() == want_c).reshape(M, K // 16, 8), axis=2)
-    assert np.all(blk_ok | dbg["near_tie"])
+    ok = blocks_agree(x.float().numpy(), want_d, (codes.cpu().numpy(), scales.cpu().numpy()), (want_c, want_s), dbg["near_tie"], 16,
+                      ro.SCALE_E4M3_META1, sv_mag and (sv_mag, sv_mag))[1]
+    assert np.all(ok), np.argwhere(~ok)[:5].tolist()
+    # prepared for the FP4 matmul: the same decisions, so a product with the same operand in the interchange format is the same
+    if sv_mag is None and ts is not None:
+        desc, packed = _pack(b, *(t.numpy() for t in inputs.random_codes(64, K, seed=7)), 0.01)
+        act, ats = b.razer_quant_act_fp4(x.cuda(), tensor_scale=ts.cuda())
+        assert torch.equal(b.razer_gemm_w4a4_fp4(desc, packed, act, ats, M).view(torch.int16),
+                           b.razer_gemm_w4a4(desc, packed, codes, scales, ats, use_native_fp4=True).view(torch.int16))
 
 
 @pytest.mark.parametrize("block,aware", [(16, False), (16, True), (32, False), (128, True)])
@@ -322,14 +330,15 @@ def test_quant_weight_extreme_magnitudes(b, block, aware):
     N, K = 70, 384
     w = inputs.student_t_weights(N, K, 8, outlier_frac=0.01) * torch.pow(2.0, torch.linspace(-140, 100, N))[:, None]
     w[3, 128:256] = 0.0
-    for log2_scale in (-70, -4, 70):
+    for log2_scale in (-70, -58, -50, -40, -4, 70):        # -58 to -40: only the quotient leaves the short form's range
         ts = torch.tensor([2.0 ** log2_scale])
         codes, scales, _ = b.razer_quant_weight(w.cuda(), tensor_scale=ts.cuda(), block=block, scale_aware=aware)
         with np.errstate(all="ignore"):
             quantize = ro.quantize_scale_aware if aware else ro.quantize_weight
             want_c, want_s, _, dbg = quantize(w.numpy(), tensor_scale=np.float32(ts.item()), block=block, return_debug=True)
-        blk_ok = (scales.cpu().numpy() == want_s) & np.all((codes.cpu().numpy() == want_c).reshape(N, K // block, block // 2), axis=2)
-        assert np.all(blk_ok | dbg["near_tie"])
+        ok = blocks_agree(w.numpy(), ts.item(), (codes.cpu().numpy(), scales.cpu().numpy()), (want_c, want_s), dbg["near_tie"], block,
+                          ro.SCALE_E3M3_META2, (5.0, 8.0), own_scales=aware)[1]
+        assert np.all(ok), (log2_scale, np.argwhere(~ok)[:5].tolist())
 
 
 @pytest.mark.parametrize("N,K", [(16, 1024), (17, 1040), (31, 2032), (1, 2064)])
