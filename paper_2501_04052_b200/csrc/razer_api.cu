@@ -112,6 +112,11 @@ static bool use_stream(const razer_desc* d, int M) {
 
 static size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
+// Workspace that one matmul against M tokens uses.
+static size_t matmul_call_bytes(const razer_desc* d, int M) {
+  return use_stream(d, M) ? gemv_stream_workspace_bytes(d, M) : umma_supported(d, M) ? umma_workspace_bytes(d, M) : simt_workspace_bytes(d, M);
+}
+
 // Workspace of a matmul against M tokens: enough for whichever kernel takes the shape.
 static size_t matmul_workspace_need(const razer_desc* d, int M) {
   size_t b = simt_workspace_bytes(d, M);
@@ -169,7 +174,7 @@ int razer_workspace_bytes(const razer_desc* d, int M, int op, size_t* bytes_out)
       break;
     case RAZER_OP_GEMM_W4A4: {
       const size_t g = matmul_workspace_need(d, M);
-      b = align_up((size_t)M * d->K * 2, 256) + g;                     // decoded activations + the bf16 matmul's own
+      b = align_up(g, 256) + align_up((size_t)M * d->K * 2, 256);      // the bf16 matmul's own + decoded activations
       const size_t f = gemm_fp4_workspace_bytes(d, M);                 // or the block-scaled FP4 path's
       b = b > f ? b : f;
       break;
@@ -408,12 +413,14 @@ int razer_gemm_w4a4(const razer_desc* d, const void* packed_w_dev, const uint8_t
     return launch_gemm_fp4(d, packed_w_dev, act_codes_dev, act_scales_dev, act_tensor_scale_dev, M, y_dev, workspace_dev,
                            workspace_bytes, (cudaStream_t)stream);
   }
-  const size_t act_bytes = align_up((size_t)M * d->K * 2, 256);
-  if (workspace_bytes < act_bytes) return set_error(RAZER_ERR_WORKSPACE, "workspace too small for the decoded activations");
-  cudaStream_t st = (cudaStream_t)stream;
-  RAZER_TRY(razer_decode_act(act_codes_dev, act_scales_dev, M, d->K, act_sv_mag, workspace_dev, stream));
-  return matmul_common(d, packed_w_dev, workspace_dev, M, y_dev, (char*)workspace_dev + act_bytes,
-                       workspace_bytes - act_bytes, 1.0f, act_tensor_scale_dev, st);
+  // The matmul's own part comes first: its status word and counters stay where they are whatever M and K.
+  const size_t own_bytes = align_up(matmul_call_bytes(d, M), 256), need = own_bytes + (size_t)M * d->K * 2;
+  if (workspace_bytes < need)
+    return set_error(RAZER_ERR_WORKSPACE, "workspace of %zu bytes needed, %zu given", need, workspace_bytes);
+  void* act = (char*)workspace_dev + own_bytes;
+  RAZER_TRY(razer_decode_act(act_codes_dev, act_scales_dev, M, d->K, act_sv_mag, act, stream));
+  return matmul_common(d, packed_w_dev, act, M, y_dev, workspace_dev, own_bytes, 1.0f, act_tensor_scale_dev,
+                       (cudaStream_t)stream);
 }
 
 }  // extern "C"

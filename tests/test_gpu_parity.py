@@ -754,6 +754,34 @@ def test_one_workspace_serves_all_shapes_and_token_counts_in_turn(b):
     b.razer_workspace_status(ws)
 
 
+def test_one_workspace_serves_both_w4a4_routes_in_turn(b):
+    """The same for the weight-activation matmul: exact route, FP4 route and prepared operand, with M and K falling and rising; what
+    one call keeps behind the status word and the counters (partial sums, decoded or re-laid-out activations) is nothing to the
+    next, and the status word is the kernels' own after every route."""
+    cases, sizes = [], []
+    for i, (M, N, K) in enumerate([(256, 8192, 2048), (128, 4096, 8192), (16, 1000, 1040), (300, 390, 2320), (4, 512, 4096), (65, 4096, 4096)]):
+        codes, scales = inputs.random_codes(N, K, seed=280 + i)
+        desc, packed = _pack(b, codes.numpy(), scales.numpy(), 0.002)
+        x = inputs.activations(M, K, 290 + i).cuda()
+        exact, plain = b.razer_quant_act(x), b.razer_quant_act(x, sv_mag=0.0)
+        act, ats = b.razer_quant_act_fp4(x)
+        for fn in (lambda ws, a=(desc, packed, *exact): b.razer_gemm_w4a4(*a, workspace=ws),
+                   lambda ws, a=(desc, packed, *plain): b.razer_gemm_w4a4(*a, workspace=ws, use_native_fp4=True),
+                   lambda ws, a=(desc, packed, act, ats, M): b.razer_gemm_w4a4_fp4(*a, workspace=ws)):
+            cases.append((fn, fn(None)))                                      # a workspace of its own
+        sizes.append(b.razer_workspace_bytes(desc, M, b.OP_GEMM_W4A4))
+    ws = torch.empty(max(sizes), dtype=torch.uint8, device="cuda")
+    b.razer_workspace_init(ws)
+    for step in (1, 5, 7, 11):                                                # four orders of the eighteen calls
+        for i in range(len(cases)):
+            fn, want = cases[(i * step) % len(cases)]
+            assert torch.equal(fn(ws), want), (step, i)
+            b.razer_workspace_status(ws)
+    ws.zero_()
+    cases[0][0](ws)                                                           # exact route, M = 256
+    assert not ws[:4].any()
+
+
 def test_weights_written_just_ahead_of_the_matmul_are_seen(b):
     """Stream-ordering contract of the header: the matmul kernels start reading the packed weights before the kernel
     directly ahead of them is known to have finished (programmatic dependent launch).  What is guaranteed: weights
