@@ -109,7 +109,7 @@ int razer_pack_layout(const razer_desc* d, const uint8_t* codes_dev, const uint8
 int razer_dequant(const razer_desc* d, const void* packed_dev, void* out_dev, int out_is_fp32,
                   void* stream);
 
-/* Scratch the matmul entry points need for `op` (RAZER_OP_*) with M activation rows.
+/* Scratch the matmul entry points need for `op` (RAZER_OP_*) with up to M activation rows.
  * The workspace must be 256-byte aligned and must have been prepared once with
  * razer_workspace_init; the matmul calls leave it prepared, so one workspace can serve any
  * number of calls, shapes included, one after another.  Calls that may overlap on the GPU

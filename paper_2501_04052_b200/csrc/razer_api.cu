@@ -1,4 +1,5 @@
 // extern "C" entry points of the RaZeR library: argument validation and dispatch only.
+#include <algorithm>
 #include <cstdarg>
 #include <cstdio>
 #include <cmath>
@@ -74,14 +75,16 @@ int launch_quant_act(const void*, int, int, float, const float*, uint32_t*, uint
 int launch_gemv_simt(const razer_desc*, const void*, const void*, int, const float*, void*, void*, size_t,
                      cudaStream_t);
 size_t simt_workspace_bytes(const razer_desc*, int M);
+size_t simt_workspace_bound(const razer_desc*, int M);
 int launch_gemm_fp4(const razer_desc*, const void*, const uint8_t*, const uint8_t*, const float*, int, void*, void*, size_t,
                     cudaStream_t);
-size_t gemm_fp4_workspace_bytes(const razer_desc*, int M);
+size_t gemm_fp4_workspace_bound(const razer_desc*, int M);
 int launch_gemm_fp4_prepared(const razer_desc*, const void*, const void*, const float*, int, void*, void*, size_t, cudaStream_t);
 int launch_quant_act_fp4(const void*, int, int, const float*, uint32_t*, void*, float*, cudaStream_t);
 int launch_gemm_umma(const razer_desc*, const void* packed, const void* x, int M, int ldx_K, float extra_scale,
                      const float* extra_scale_dev, void* y, void* ws, size_t ws_bytes, cudaStream_t, uint32_t* status_host);
 size_t umma_workspace_bytes(const razer_desc*, int M);
+size_t umma_workspace_bound(int M);
 bool umma_supported(const razer_desc*, int M);
 int launch_gemv_stream(const razer_desc*, const void* packed, const void* x, int M, float extra_scale,
                        const float* extra_scale_dev, void* y, void* ws, size_t ws_bytes, cudaStream_t, uint32_t* status_host);
@@ -117,12 +120,11 @@ static size_t matmul_call_bytes(const razer_desc* d, int M) {
   return use_stream(d, M) ? gemv_stream_workspace_bytes(d, M) : umma_supported(d, M) ? umma_workspace_bytes(d, M) : simt_workspace_bytes(d, M);
 }
 
-// Workspace of a matmul against M tokens: enough for whichever kernel takes the shape.
-static size_t matmul_workspace_need(const razer_desc* d, int M) {
-  size_t b = simt_workspace_bytes(d, M);
-  if (umma_supported(d, M)) b = b > umma_workspace_bytes(d, M) ? b : umma_workspace_bytes(d, M);
-  if (gemv_stream_supported(d, M)) b = b > gemv_stream_workspace_bytes(d, M) ? b : gemv_stream_workspace_bytes(d, M);
-  return b;
+// Workspace that is enough for any matmul against up to M tokens, whichever kernel takes it: a caller sizes it once for its largest
+// batch, and what a call uses does not grow with M alone (the token tile and the grid are chosen for each M).
+static size_t matmul_workspace_bound(const razer_desc* d, int M) {
+  const size_t parts[3] = {simt_workspace_bound(d, M), umma_supported(d, M) ? umma_workspace_bound(M) : 0, gemv_stream_workspace_bytes(d, 1)};
+  return std::max(parts[0], std::max(parts[1], parts[2]));
 }
 
 }  // namespace razer
@@ -170,12 +172,12 @@ int razer_workspace_bytes(const razer_desc* d, int M, int op, size_t* bytes_out)
       if (M > 64) return set_error(RAZER_ERR_INVALID_ARG, "razer_gemv takes 1 <= M <= 64 (got %d)", M);
       /* fall through */
     case RAZER_OP_GEMM:
-      b = matmul_workspace_need(d, M);
+      b = matmul_workspace_bound(d, M);
       break;
     case RAZER_OP_GEMM_W4A4: {
-      const size_t g = matmul_workspace_need(d, M);
+      const size_t g = matmul_workspace_bound(d, M);
       b = align_up(g, 256) + align_up((size_t)M * d->K * 2, 256);      // the bf16 matmul's own + decoded activations
-      const size_t f = gemm_fp4_workspace_bytes(d, M);                 // or the block-scaled FP4 path's
+      const size_t f = gemm_fp4_workspace_bound(d, M);                 // or the block-scaled FP4 path's
       b = b > f ? b : f;
       break;
     }

@@ -521,13 +521,17 @@ struct Plan {
 static const TileCost tile_costs[] = {{128, CH, CH, 0.139f, 0.08f, 0.6f, 2.9f, 0.30f, 4.6f, 0.50f},
                                       {256, CH, CH, 0.177f, 0.18f, 1.3f, 3.1f, 0.30f, 6.5f, 1.30f}};
 
+static bool admissible(const TileCost& t, const Fp4ActLayout& act) {
+  return act.force_nt ? t.NT == act.force_nt : t.NT <= act.tiles128 * 128;
+}
+
 static Plan make_plan(const razer_desc* d, int M) {
   Plan best;
   float best_cost = 0.0f;
   const Geometry g = make_geometry(d->N, d->K);
   const Fp4ActLayout act = make_fp4_act_layout(M, d->K);
   for (const TileCost& t : tile_costs) {
-    if (act.force_nt ? t.NT != act.force_nt : t.NT > act.tiles128 * 128) continue;
+    if (!admissible(t, act)) continue;
     Plan p;
     p.act = act;
     p.NT = t.NT;
@@ -596,16 +600,14 @@ Fp4ActLayout make_fp4_act_layout(int M, int K) {
   return L;
 }
 
-// workspace of the matmul proper: status word, tile counters, partial-tile slots
-size_t gemm_fp4_core_workspace_bytes(const razer_desc* d, int M) {
-  const fp4_path::Plan p = fp4_path::make_plan(d, M);
-  return WS_ZERO_BYTES + p.slots_bytes;
-}
-
-// ... plus the re-laid-out activation operand when the caller brings the interchange format
-size_t gemm_fp4_workspace_bytes(const razer_desc* d, int M) {
-  const fp4_path::Plan p = fp4_path::make_plan(d, M);
-  return WS_ZERO_BYTES + p.slots_bytes + p.act.codes_bytes + p.act.sfb_bytes;
+// No call against up to M tokens needs more: partial-tile slots, and the re-laid-out activation operand when the caller brings the
+// interchange format.
+size_t gemm_fp4_workspace_bound(const razer_desc* d, int M) {
+  const Fp4ActLayout act = make_fp4_act_layout(M, d->K);
+  int widest = 0;
+  for (const TileCost& t : fp4_path::tile_costs)
+    if (fp4_path::admissible(t, act) && t.NT > widest) widest = t.NT;
+  return WS_ZERO_BYTES + (size_t)sm_count() * widest * TILE_ROWS * sizeof(float) + act.codes_bytes + act.sfb_bytes;
 }
 
 // The matmul on a prepared activation operand (act_fp4: codes, then scale-factor tiles).

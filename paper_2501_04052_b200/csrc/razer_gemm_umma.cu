@@ -481,12 +481,14 @@ static const TileCost tile_costs[] = {
     {128, 4, 1, 0.228f, 0.15f, 0.7f, 2.9f, 0.75f, 6.0f, 0.45f}, {192, 2, 1, 0.268f, 0.20f, 1.2f, 3.7f, 0.60f, 6.3f, 0.67f},
     {256, 2, 1, 0.315f, 0.25f, 1.6f, 4.0f, 0.55f, 7.0f, 0.90f}};
 
+static bool admissible(const TileCost& t, int M) { return t.NT <= 16 || t.NT < 2 * M; }   // not half of the tile or more padding
+
 static UmmaPlan make_plan(const razer_desc* d, int M) {
   UmmaPlan best;
   float best_cost = 0.0f;
   const Geometry g = make_geometry(d->N, d->K);
   for (const TileCost& t : tile_costs) {
-    if (t.NT > 16 && t.NT >= 2 * M) continue;              // half of the tile or more would be padding
+    if (!admissible(t, M)) continue;
     UmmaPlan p;
     p.NT = t.NT;
     p.CH = t.CH;
@@ -511,6 +513,13 @@ bool umma_supported(const razer_desc* d, int M) {
 }
 
 size_t umma_workspace_bytes(const razer_desc* d, int M) { return WS_ZERO_BYTES + make_plan(d, M).slots_bytes; }
+// No call against up to M tokens needs more, whatever its shape.
+size_t umma_workspace_bound(int M) {
+  int widest = 0;
+  for (const TileCost& t : tile_costs)
+    if (admissible(t, M) && t.NT > widest) widest = t.NT;
+  return WS_ZERO_BYTES + (size_t)sm_count() * widest * TILE_ROWS * sizeof(float);
+}
 
 template <int NT, int CH, int CHX, int WST, int XST, int AST, int NDW, int NACC>
 static int launch_cfg(const CUtensorMap& tmap, const CUtensorMap& tmap_w, const UmmaArgs& args, int grid, cudaStream_t st) {

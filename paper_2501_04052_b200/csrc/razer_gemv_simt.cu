@@ -108,6 +108,15 @@ size_t simt_workspace_bytes(const razer_desc* d, int M) {
   return WS_ZERO_BYTES + (s > 1 ? (size_t)s * M * d->N * sizeof(float) : 0);
 }
 
+// No call against up to M tokens needs more.
+size_t simt_workspace_bound(const razer_desc* d, int M) {
+  const Geometry g = make_geometry(d->N, d->K);
+  size_t b = simt_workspace_bytes(d, M);
+  for (int m : {1, 3, 7}) b = m < M && simt_workspace_bytes(d, m) > b ? simt_workspace_bytes(d, m) : b;
+  for (int m = 8; m < M && simt_splits(g, m, 8) > 1; m += 8) b = simt_workspace_bytes(d, m) > b ? simt_workspace_bytes(d, m) : b;
+  return b;
+}
+
 int launch_gemv_simt(const razer_desc* d, const void* packed, const void* x, int M,
                      const float* extra_scale_dev, void* y, void* ws, size_t ws_bytes, cudaStream_t st) {
   const Geometry g = make_geometry(d->N, d->K);

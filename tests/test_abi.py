@@ -69,3 +69,26 @@ def test_host_side_validation(binding):
     assert b.lib().razer_quant_act(16, 4, 72, 5.0, None, None, None, None, None, None) == b.ERR_INVALID_ARG
     # the block-scaled FP4 path checks its workspace before it launches anything
     assert b.lib().razer_gemm_w4a4(ctypes.byref(good), 16, 16, 16, 16, 5.0, 4, 16, 256, 1 << 10, 1, None) == b.ERR_WORKSPACE
+
+
+@pytest.mark.parametrize("N,K", [(4096, 11008), (4096, 4096), (8192, 8192), (28672, 8192), (1024, 1024), (300, 2320), (16, 16)])
+def test_workspace_for_a_batch_serves_every_smaller_one(binding, N, K):
+    """razer_workspace_bytes(M) covers every call with up to M rows.  What a call needs is in the error that it gives when handed 256
+    bytes, before anything is launched."""
+    b = binding
+    desc = b.make_desc(N, K, 0.01)
+    ref, at = ctypes.byref(desc), 1 << 20                       # addresses are looked at for their alignment only
+    def need(call, *args):
+        assert call(*args) == b.ERR_WORKSPACE
+        return int(re.search(r"workspace of (\d+) bytes needed", b.last_error()).group(1))
+    lib = b.lib()
+    calls = {b.OP_GEMV: [lambda M: need(lib.razer_gemv, ref, at, at, M, at, at, 256, None)],
+             b.OP_GEMM: [lambda M: need(lib.razer_gemm, ref, at, at, M, at, at, 256, None)],
+             b.OP_GEMM_W4A4: [lambda M: need(lib.razer_gemm_w4a4, ref, at, at, at, at, 5.0, M, at, at, 256, 0, None),
+                              lambda M: need(lib.razer_gemm_w4a4, ref, at, at, at, at, 5.0, M, at, at, 256, 1, None),
+                              lambda M: need(lib.razer_gemm_w4a4_fp4, ref, at, at, at, M, at, at, 256, None)]}
+    for op, fns in calls.items():
+        most = 0
+        for M in range(1, 65 if op == b.OP_GEMV else 2100):
+            most = max(most, *(f(M) for f in fns))
+            assert b.razer_workspace_bytes(desc, M, op) >= most, (op, M)

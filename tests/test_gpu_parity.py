@@ -754,6 +754,19 @@ def test_one_workspace_serves_all_shapes_and_token_counts_in_turn(b):
     b.razer_workspace_status(ws)
 
 
+def test_workspace_sized_for_the_largest_batch(b):
+    """Sized once for 512 tokens, a workspace serves every kernel and token tile below, in any order, with unchanged results."""
+    N, K = 4096, 4096
+    codes, scales = inputs.random_codes(N, K, seed=270)
+    desc, packed = _pack(b, codes.numpy(), scales.numpy(), 0.002)
+    ws = torch.zeros(b.razer_workspace_bytes(desc, 512, b.OP_GEMM), dtype=torch.uint8, device="cuda")
+    xs = {M: inputs.activations(M, K, 271).cuda() for M in (512, 200, 1, 96, 16, 333, 128, 8, 33, 160, 64, 24, 256)}
+    want = {M: b.razer_gemm(desc, packed, x) for M, x in xs.items()}
+    for M in [*xs, *reversed(xs)]:
+        assert torch.equal(b.razer_gemm(desc, packed, xs[M], workspace=ws), want[M]), M
+    b.razer_workspace_status(ws)
+
+
 def test_one_workspace_serves_both_w4a4_routes_in_turn(b):
     """The same for the weight-activation matmul: exact route, FP4 route and prepared operand, with M and K falling and rising; what
     one call keeps behind the status word and the counters (partial sums, decoded or re-laid-out activations) is nothing to the
