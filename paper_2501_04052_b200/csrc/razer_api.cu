@@ -25,6 +25,7 @@ int set_error(int code, const char* fmt, ...) {
 
 int check_cuda(cudaError_t e, const char* what) {
   if (e == cudaSuccess) return RAZER_OK;
+  cudaGetLastError();                         // reported here: the next call's check of its own launch must not find it again
   return set_error(RAZER_ERR_CUDA, "%s: %s", what, cudaGetErrorString(e));
 }
 

@@ -720,6 +720,43 @@ def test_gemv_host_routes_of_x(b, M, N, K, offset):
     assert e.value.code == b.ERR_DEVICE_TIMEOUT and "7" in str(e.value)
 
 
+_FAILED_CALL_CHECK = r"""
+import sys, torch
+sys.path.insert(0, sys.argv[1])
+from paper_2501_04052_b200 import binding as b, inputs
+codes, scales = (t.cuda() for t in inputs.random_codes(256, 256, seed=1))
+desc = b.make_desc(256, 256, 0.01)
+ws = b.alloc_workspace(desc, 1, b.OP_GEMV, "cuda")
+torch.cuda.synchronize()
+g = torch.cuda.CUDAGraph()
+with torch.cuda.stream(torch.cuda.Stream()):
+    g.capture_begin()
+    try:
+        b.razer_workspace_status(ws)          # waits for the stream, which a stream that is being captured refuses
+        print("not refused")
+    except b.RazerError as e:
+        assert e.code == b.ERR_CUDA
+    try:
+        g.capture_end()
+    except Exception:
+        pass
+packed = b.razer_pack_layout(desc, codes, scales)
+d1 = b.razer_dequant(desc, packed, fp32=False)
+b.razer_workspace_status(ws)
+print("ok")
+"""
+
+
+def test_a_failed_call_is_reported_once():
+    """A CUDA error that one call has returned is not found again by the next call's check of its own launch."""
+    import os
+    import subprocess
+    import sys
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", _FAILED_CALL_CHECK, root], capture_output=True, text=True, timeout=600)
+    assert r.returncode == 0 and r.stdout.strip() == "ok", r.stdout + r.stderr
+
+
 def test_workspace_too_small_is_an_error(b):
     N, K = 512, 4096
     codes, scales = inputs.random_codes(N, K, seed=98)
