@@ -241,14 +241,17 @@ int razer_gemm(const razer_desc* d, const void* packed_dev, const void* x_dev, i
 }  // extern "C"
 
 namespace razer {
-// Device address of pinned host memory, or NULL.
-static void* device_view(const void* host) {
-  cudaPointerAttributes at;
-  if (cudaPointerGetAttributes(&at, host) != cudaSuccess) {
+// Device address of pinned host memory, or NULL where the `bytes` from `host` on are not all pinned (cudaHostRegister may have covered
+// only a part): a kernel that reads or writes beyond would fault, a copy reports it.
+static void* device_view(const void* host, size_t bytes) {
+  cudaPointerAttributes first, last;
+  if (cudaPointerGetAttributes(&first, host) != cudaSuccess || cudaPointerGetAttributes(&last, (const char*)host + bytes - 1) != cudaSuccess) {
     cudaGetLastError();                                      // not a CUDA-known pointer
     return nullptr;
   }
-  return at.type == cudaMemoryTypeHost ? at.devicePointer : nullptr;
+  const bool whole = first.type == cudaMemoryTypeHost && last.type == cudaMemoryTypeHost && first.devicePointer &&
+                     (char*)first.devicePointer + (bytes - 1) == (char*)last.devicePointer;
+  return whole ? first.devicePointer : nullptr;
 }
 
 // A pinned word of the calling thread in which a kernel shows that a wait gave up; given back when the thread ends.
@@ -295,10 +298,10 @@ int razer_gemv_host(const razer_desc* d, const void* packed_dev, const void* x_h
   cudaStream_t st = (cudaStream_t)stream;
   // Pinned host memory that the device can address takes the kernel's stores directly (no copy back), and gives x to a small
   // kernel that the matmul can follow as a dependent launch: a copy of a few KB by the copy engine costs about 6 us of this call.
-  void* y_mapped = device_view(y_host);
-  void* x_mapped = device_view(x_host);
+  const size_t x_bytes = (size_t)M * d->K * 2, y_bytes = (size_t)M * d->N * 2;
+  void* y_mapped = device_view(y_host, y_bytes);
+  void* x_mapped = device_view(x_host, x_bytes);
   void* y_target = y_mapped ? y_mapped : y_stage_dev;
-  const size_t x_bytes = (size_t)M * d->K * 2;
   if (x_mapped && reinterpret_cast<uintptr_t>(x_mapped) % 16 == 0 && x_bytes <= HOST_X_KERNEL_BYTES)
     RAZER_TRY(launch_copy_from_host(x_mapped, x_stage_dev, x_bytes, st));
   else
@@ -307,7 +310,7 @@ int razer_gemv_host(const razer_desc* d, const void* packed_dev, const void* x_h
   if (!workspace_dev || use_simt(d, M) || !status.ready()) {               // no status word, or no way to see it but a copy
     RAZER_TRY(matmul_common(d, packed_dev, x_stage_dev, M, y_target, workspace_dev, workspace_bytes, 1.0f, nullptr, st));
     if (!y_mapped)
-      RAZER_TRY(check_cuda(cudaMemcpyAsync(y_host, y_stage_dev, (size_t)M * d->N * 2, cudaMemcpyDeviceToHost, st), "copy of y to the host"));
+      RAZER_TRY(check_cuda(cudaMemcpyAsync(y_host, y_stage_dev, y_bytes, cudaMemcpyDeviceToHost, st), "copy of y to the host"));
     if (workspace_dev) return razer_workspace_status(workspace_dev, stream);   // synchronizes
     return check_cuda(cudaStreamSynchronize(st), "stream synchronize");
   }
@@ -315,7 +318,7 @@ int razer_gemv_host(const razer_desc* d, const void* packed_dev, const void* x_h
   *status.word = 0;
   RAZER_TRY(matmul_common(d, packed_dev, x_stage_dev, M, y_target, workspace_dev, workspace_bytes, 1.0f, nullptr, st, status.device_word));
   if (!y_mapped)
-    RAZER_TRY(check_cuda(cudaMemcpyAsync(y_host, y_stage_dev, (size_t)M * d->N * 2, cudaMemcpyDeviceToHost, st), "copy of y to the host"));
+    RAZER_TRY(check_cuda(cudaMemcpyAsync(y_host, y_stage_dev, y_bytes, cudaMemcpyDeviceToHost, st), "copy of y to the host"));
   RAZER_TRY(check_cuda(cudaStreamSynchronize(st), "stream synchronize"));
   const uint32_t code = *status.word;
   return code == 0 ? RAZER_OK : set_error(RAZER_ERR_DEVICE_TIMEOUT, "a device-side wait gave up (wait id %u)", code);

@@ -757,6 +757,36 @@ def test_a_failed_call_is_reported_once():
     assert r.returncode == 0 and r.stdout.strip() == "ok", r.stdout + r.stderr
 
 
+@pytest.mark.parametrize("which", ["x", "y"])
+def test_gemv_host_buffer_pinned_in_part(b, which):
+    """Only the first of a buffer's two pages is registered: no kernel may touch the other one.  The call copies instead, which
+    either works or is an error of the copy, and the next call is as good as ever."""
+    N = K = 4096                                                     # 8 KB of x and of y
+    codes, scales = inputs.random_codes(N, K, seed=101)
+    desc, packed = _pack(b, codes.numpy(), scales.numpy(), 0.01)
+    room = torch.empty(3 * 2048 * 2, dtype=torch.bfloat16)
+    page = room[(-room.data_ptr() % 4096) // 2:][:4096].view(1, 4096)
+    x, y = inputs.activations(1, K, 101).pin_memory(), torch.empty((1, N), dtype=torch.bfloat16).pin_memory()
+    xs, ys = torch.empty((1, K), dtype=torch.bfloat16, device="cuda"), torch.empty((1, N), dtype=torch.bfloat16, device="cuda")
+    ws = b.alloc_workspace(desc, 1, b.OP_GEMV, "cuda")
+    want = b.razer_gemv(desc, packed, x.cuda()).cpu()
+    page.copy_(x)
+    cudart = torch.cuda.cudart()
+    assert page.data_ptr() % 4096 == 0 and int(cudart.cudaHostRegister(page.data_ptr(), 4096, 0)) == 0
+    try:
+        try:
+            b.razer_gemv_host(desc, packed, page if which == "x" else x, page if which == "y" else y, xs, ys, ws)
+            assert torch.equal(page if which == "y" else y, want)
+        except b.RazerError as e:
+            assert e.code == b.ERR_CUDA and "copy" in str(e)
+        torch.cuda.synchronize()
+        b.razer_gemv_host(desc, packed, x, y, xs, ys, ws)
+        assert torch.equal(y, want)
+    finally:
+        torch.cuda.synchronize()
+        cudart.cudaHostUnregister(page.data_ptr())
+
+
 def test_workspace_too_small_is_an_error(b):
     N, K = 512, 4096
     codes, scales = inputs.random_codes(N, K, seed=98)
