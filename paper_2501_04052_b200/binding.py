@@ -170,8 +170,9 @@ def alloc_workspace(desc: RazerDesc, M: int, op: int, device) -> torch.Tensor:
 
 def _matmul(fn, desc, packed, x, y, workspace, op):
     # Every attribute read and call here is 50 to 150 ns of a call that takes 5 us in all: as few as there can be.
-    M, K = x.shape
-    assert x.is_cuda and x.dtype is torch.bfloat16 and x.is_contiguous() and K == desc.K
+    shape = x.shape
+    assert x.is_cuda and x.dtype is torch.bfloat16 and x.is_contiguous() and shape[1] == desc.K
+    M = shape[0]
     if y is None:
         y = torch.empty((M, desc.N), dtype=torch.bfloat16, device=x.device)
     if workspace is None:

@@ -71,6 +71,15 @@ def test_host_side_validation(binding):
     assert b.lib().razer_gemm_w4a4(ctypes.byref(good), 16, 16, 16, 16, 5.0, 4, 16, 256, 1 << 10, 1, None) == b.ERR_WORKSPACE
 
 
+def test_activations_on_the_host_are_refused_whatever_their_shape(binding):
+    import torch
+    desc = binding.make_desc(16, 32, 0.01)
+    for shape in ((32,), (2, 32), (2, 32, 1)):
+        for fn in (binding.razer_gemv, binding.razer_gemm):
+            with pytest.raises(AssertionError):
+                fn(desc, None, torch.zeros(shape, dtype=torch.bfloat16))
+
+
 @pytest.mark.parametrize("N,K", [(4096, 11008), (4096, 4096), (8192, 8192), (28672, 8192), (1024, 1024), (300, 2320), (16, 16)])
 def test_workspace_for_a_batch_serves_every_smaller_one(binding, N, K):
     """razer_workspace_bytes(M) covers every call with up to M rows.  What a call needs is in the error that it gives when handed 256

@@ -117,6 +117,16 @@ def test_gemv_ragged_shapes_random_codes(b, M):
     _check_matmul(b, b.razer_gemv, desc, packed, codes, scales, 0.004, x)
 
 
+def test_activations_with_trailing_axes_of_one(b):
+    """x's first two axes are its rows and columns; further ones of length one (a view of a caller's layout) change nothing."""
+    codes, scales = inputs.random_codes(300, 528, seed=33)
+    desc, packed = _pack(b, codes.numpy(), scales.numpy(), 0.01)
+    x = inputs.activations(3, 528, 33).cuda()
+    want = b.razer_gemv(desc, packed, x)
+    for view in ((3, 528, 1), (3, 528, 1, 1)):
+        assert torch.equal(b.razer_gemv(desc, packed, x.view(view)), want) and torch.equal(b.razer_gemm(desc, packed, x.view(view)), want)
+
+
 @pytest.mark.parametrize("sv_mag,remap_code", [((5.0, 7.0), 0x8), ((5.0, 9.0), 0x0), ((2.5, 12.0), 0x8)])
 def test_gemv_other_special_values(b, sv_mag, remap_code):
     N, K = 256, 1024
