@@ -248,7 +248,9 @@ __device__ __forceinline__ void epilogue_loop(const Args& a, const Work& work, i
     float acc[PER_LANE];
 #pragma unroll
     for (int j = 0; j < PER_LANE; ++j) acc[j] = 0.0f;
-    // CTA order (a fixed summation order); the loads of four CTAs' slots are in flight together
+    // CTA order (a fixed summation order); the loads of four CTAs' slots for two of the lane's outputs are in flight together.  (One
+    // output after another, a unit of 64 rows and 8 tokens took eight round trips to L2 for every four CTAs: 8 x 2500 x 6992 in such
+    // units 17.5 us, now 9.2; all eight outputs at once cost the decoding warps' code more than it gave, 1 x 28672 x 8192 29.6 -> 30.9.)
     for (int cb = c_first; cb <= c_last; cb += 4) {
       const float* src[4];
 #pragma unroll
@@ -258,14 +260,21 @@ __device__ __forceinline__ void epilogue_loop(const Args& a, const Work& work, i
         src[u] = a.slots + ((size_t)c * 2 + sl) * SLOT_FLOATS;
       }
 #pragma unroll
-      for (int j = 0; j < PER_LANE; ++j) {
+      for (int j = 0; j < PER_LANE; j += 2) {
         if (first + STEP * j < outputs) {
-          float part[4];
+          constexpr int LAST = PER_LANE - 1;
+          const int o[2] = {first + STEP * j, min(first + STEP * min(j + 1, LAST), outputs - 1)};   // where there is no second one: any other
+          float part[2][4];
 #pragma unroll
-          for (int u = 0; u < 4; ++u) part[u] = __ldcg(src[u] + first + STEP * j);
+          for (int i = 0; i < 2; ++i)
+#pragma unroll
+            for (int u = 0; u < 4; ++u) part[i][u] = __ldcg(src[u] + o[i]);
 #pragma unroll
           for (int u = 0; u < 4; ++u)
-            if (cb + u <= c_last) acc[j] += part[u];
+            if (cb + u <= c_last) {
+              acc[j] += part[0][u];
+              if (j < LAST) acc[j + 1] += part[1][u];
+            }
         }
       }
     }
@@ -307,11 +316,17 @@ struct StreamPlan {
 
 // One candidate: units of SW * TM strips; every CTA takes whole units only (split == false), or q whole units after a
 // piece of one of the remaining units, each of which is cut along K into equal pieces (processed first, combined
-// through the workspace).  The cost is the busiest CTA's time in SM cycles.  A round (each consumer warp takes TM strips of one
+// through the workspace).  The cost is about the busiest CTA's time in SM cycles.  A round (each consumer warp takes TM strips of one
 // chunk) costs the shared-memory wavefronts of its loads, 23 per strip and 8 per chunk and warp, which is what the decode is
-// bound by; a stage about 200 more, and 14 per token for the activations' copies; a segment 260 (partial sums); a split whose
-// combination nothing follows (q == 0) another 1700 at the end of the launch.  (Measured in place with the SM's clock: 870 to
-// 910 a round at TM = 2, 240 to 300 between the rounds of two stages.)
+// bound by; a stage 400 more, a segment 450; the launch 200 for every strip of its first stage and, at its end, 5 for every
+// partial sum that an epilogue lane adds.  Combining the parts of a unit costs the more the more outputs a lane has and the more CTAs
+// share it; where whole units follow, units are cut only if it is over before they are.  (Fitted to 336 sizes timed in every unit
+// shape, M 1 .. 8, N and K 256 .. 28672: the choice is within 1 % of the best of them in the mean, 11 % at worst.  Charged as 1700
+// whatever its size, the combination made it 4 % and 67 %, and slower than the kernel that decoded in registers (last figure):
+// 8 x 2500 x 6992 17.5 -> 7.1 us (11.7), 8 x 600 x 16000 11.0 -> 6.3 (8.1), 4 x 1024 x 11008 8.7 -> 6.1 (7.2), 8 x 1024 x 4096 7.5 -> 3.9 (6.7).)
+constexpr double STAGE_COST = 400, SEGMENT_COST = 450, STRIP_COST = 200, SUM_COST = 5;
+constexpr double SPLIT_COST = 100, COMBINE_COST = 1900, UNEVEN_COST = 300, TRIP_COST = 1400, OUTPUT_COST = 450;
+
 static inline StreamPlan stream_candidate(const razer_desc* d, int M, int G, int SW, int TM, bool split) {
   using namespace stream_path;
   StreamPlan p;
@@ -330,18 +345,27 @@ static inline StreamPlan stream_candidate(const razer_desc* d, int M, int G, int
   if (force_spw() == 1 || (force_spw() == 2 && TM <= 2 && 4 * stage1 <= ring)) p.SPW = force_spw();
   const int stages = ring / (p.SPW * stage1);
   p.red_bufs = (ring - red1) / (p.SPW * stage1) >= std::min(stages, 3) ? 2 : 1;
-  const double round = 16.0 * (23 * TM + 8) * (stages < 3 ? 1.12 : 1.0) + (200.0 + 14 * M) / p.SPW;
-  auto cycles = [&](int chunks) { return ((chunks + KW - 1) / KW) * round + 260; };
+  const int per_lane = (16 * SW * TM * M + 32 * EW - 1) / (32 * EW);   // outputs of an epilogue lane
+  const double round = 16.0 * (23 * TM + 8) * (stages < 3 ? 1.3 : 1.0) + STAGE_COST / p.SPW, sums = SUM_COST * KW * per_lane;
+  auto cycles = [&](int chunks) { return ((chunks + KW - 1) / KW) * round + SEGMENT_COST; };
+  p.cost = STRIP_COST * SW * TM + sums;
   const int q = p.units / G, rem = p.units - q * G;
   if (split && rem > 0) {
-    // pieces per unit: the count that leaves the busiest CTA the least to do
+    // pieces per unit: the count that costs the busiest CTA the least
     int best_p = 1;
     double best_cost = 0;
     const int max_p = std::max(1, std::min(8, p.kc / KW));              // a piece is at least one chunk per warp
     for (int pc = 1; pc <= max_p; ++pc) {
-      const int ctas = std::min(G, rem * pc);
-      const int most = (rem * pc + ctas - 1) / ctas;                    // pieces of the busiest CTA
-      const double c = cycles(most * ((p.kc + pc - 1) / pc)) + (most > 1 ? 260 : 0) + 50 * pc;
+      const int pieces = rem * pc, ctas = std::min(G, pieces);
+      const int most = (pieces + ctas - 1) / ctas;                      // pieces of the busiest CTA
+      double c = cycles(most * ((p.kc + pc - 1) / pc)) + (most > 1 ? SEGMENT_COST : 0);
+      if (pc > 1) {
+        const bool even = pieces == ctas;                               // a piece per CTA
+        const int parts = even ? pc : std::min(pc, (pc * ctas + pieces - 1) / pieces + 1);   // CTAs that share a unit
+        const double combine = COMBINE_COST + (even ? 0 : UNEVEN_COST) + TRIP_COST * ((parts + 3) / 4) + OUTPUT_COST * per_lane + sums;
+        if (q == 0) c += combine;
+        else if (combine > q * cycles(p.kc)) continue;
+      }
       if (pc == 1 || c < best_cost) { best_cost = c; best_p = pc; }
     }
     p.whole_base = rem;
@@ -349,7 +373,7 @@ static inline StreamPlan stream_candidate(const razer_desc* d, int M, int G, int
     p.pieces_per_unit = best_p;
     p.rem_ctas = std::min(G, rem * best_p);
     p.grid = q > 0 ? G : p.rem_ctas;
-    p.cost = q * cycles(p.kc) + best_cost + (q == 0 && best_p > 1 ? 1700 : 0);
+    p.cost += q * cycles(p.kc) + best_cost + SPLIT_COST;
   } else {
     const int qa = (p.units + G - 1) / G;
     p.whole_base = 0;
@@ -357,7 +381,7 @@ static inline StreamPlan stream_candidate(const razer_desc* d, int M, int G, int
     p.pieces_per_unit = 1;
     p.rem_ctas = 0;
     p.grid = (p.units + qa - 1) / qa;
-    p.cost = qa * cycles(p.kc);
+    p.cost += qa * cycles(p.kc);
   }
   p.slots_bytes = (size_t)G * 2 * SLOT_FLOATS * sizeof(float);
   return p;
