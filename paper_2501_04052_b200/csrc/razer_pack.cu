@@ -16,17 +16,21 @@ constexpr int SPAN_CHUNKS = 16;
 constexpr int SPAN_BLOCKS = SPAN_CHUNKS * CHUNK_BLOCKS;              // 16-element blocks of one row of a span
 constexpr int SPAN_BYTES = SPAN_CHUNKS * PIECE_BYTES;
 constexpr int SPAN_THREADS = 256;
+constexpr int FEW_CHUNKS = 4;
 
 // Reads the interchange-format blocks (8 code bytes + 1 scale byte), canonicalises them and writes them at their packed
 // positions.
 // `sub` = 16-element groups per scale block (block size / 16): the packed form always carries one scale byte per 16
 // elements, so a larger block's byte is repeated for each of its groups and the kernels need not know the block size.
+// CHUNKS per span: SPAN_CHUNKS, or few where the tensor makes few spans.
+template <int CHUNKS>
 __global__ void __launch_bounds__(SPAN_THREADS) pack_kernel(const uint8_t* __restrict__ codes, const uint8_t* __restrict__ scales,
                                                             uint8_t* __restrict__ packed, Geometry g, int remap_code, int sub) {
-  __shared__ __align__(16) uint8_t span[SPAN_BYTES];
-  const int spans = (g.k_chunks + SPAN_CHUNKS - 1) / SPAN_CHUNKS;
-  const int strip = (int)(blockIdx.x / (unsigned)spans), c0 = (int)(blockIdx.x % (unsigned)spans) * SPAN_CHUNKS;
-  const int n_chunks = min(SPAN_CHUNKS, g.k_chunks - c0);
+  constexpr int BLOCKS = CHUNKS * CHUNK_BLOCKS;         // 16-element blocks of one row of a span
+  __shared__ __align__(16) uint8_t span[CHUNKS * PIECE_BYTES];
+  const int spans = (g.k_chunks + CHUNKS - 1) / CHUNKS;
+  const int strip = (int)(blockIdx.x / (unsigned)spans), c0 = (int)(blockIdx.x % (unsigned)spans) * CHUNKS;
+  const int n_chunks = min(CHUNKS, g.k_chunks - c0);
   // bit 3 of each nibble of nz is set iff the nibble's magnitude (low three bits) is non-zero
   auto canon = [&](uint32_t w, bool negate) -> uint32_t {
     const uint32_t m = w & 0x77777777u;
@@ -44,8 +48,8 @@ __global__ void __launch_bounds__(SPAN_THREADS) pack_kernel(const uint8_t* __res
   };
   const int k16 = g.K / 16, ks = k16 / sub;
 #pragma unroll
-  for (int i = 0; i < STRIP_ROWS * SPAN_BLOCKS / SPAN_THREADS; ++i) {
-    const int b = (int)threadIdx.x + i * SPAN_THREADS, r = b / SPAN_BLOCKS, kb_in = b % SPAN_BLOCKS;
+  for (int i = 0; i < STRIP_ROWS * BLOCKS / SPAN_THREADS; ++i) {
+    const int b = (int)threadIdx.x + i * SPAN_THREADS, r = b / BLOCKS, kb_in = b % BLOCKS;
     const int n = strip * STRIP_ROWS + r, kb = c0 * CHUNK_BLOCKS + kb_in;
     uint32_t w0 = 0, w1 = 0, sb = 0;
     if (n < g.N && kb < k16) {
@@ -177,8 +181,8 @@ __global__ void __launch_bounds__(256) decode_act_kernel(const uint8_t* __restri
   }
 }
 
-static unsigned span_grid(const Geometry& g, int strips) {
-  return (unsigned)strips * (unsigned)((g.k_chunks + SPAN_CHUNKS - 1) / SPAN_CHUNKS);
+static unsigned span_grid(const Geometry& g, int strips, int chunks = SPAN_CHUNKS) {
+  return (unsigned)strips * (unsigned)((g.k_chunks + chunks - 1) / chunks);
 }
 
 static int grid_for(long long total, int threads) {
@@ -197,7 +201,12 @@ __global__ void pack_done_kernel() {}
 int launch_pack(const razer_desc* d, const uint8_t* codes, const uint8_t* scales, void* packed,
                 cudaStream_t st) {
   const Geometry g = make_geometry(d->N, d->K);
-  pack_kernel<<<span_grid(g, g.strips()), SPAN_THREADS, 0, st>>>(codes, scales, (uint8_t*)packed, g, d->remap_code, d->block / 16);
+  // Short spans where long ones would leave SMs idle or most of a span's width empty, us against long ones: 256 x 256 2.5, 3.3;
+  // 2048 x 1024 3.2, 3.6; 28672 x 256 5.3, 8.4.  Level at 2048 x 2048 (256 long spans) and 28672 x 512, long ones ahead at 1024 x 8192.
+  const bool few = span_grid(g, g.strips()) < 2 * 148 || g.k_chunks <= 8;
+  auto kern = few ? pack_kernel<FEW_CHUNKS> : pack_kernel<SPAN_CHUNKS>;
+  kern<<<span_grid(g, g.strips(), few ? FEW_CHUNKS : SPAN_CHUNKS), SPAN_THREADS, 0, st>>>(codes, scales, (uint8_t*)packed, g, d->remap_code,
+                                                                                      d->block / 16);
   count_launches(1);
   RAZER_TRY(check_cuda(cudaGetLastError(), "pack_kernel launch"));
   pack_done_kernel<<<1, 32, 0, st>>>();

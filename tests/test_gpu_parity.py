@@ -351,9 +351,10 @@ def test_quant_weight_extreme_magnitudes(b, block, aware):
         assert np.all(ok), (log2_scale, np.argwhere(~ok)[:5].tolist())
 
 
-@pytest.mark.parametrize("N,K", [(16, 1024), (17, 1040), (31, 2032), (1, 2064)])
+@pytest.mark.parametrize("N,K", [(16, 1024), (17, 1040), (31, 2032), (1, 2064), (4737, 512), (4737, 528), (4600, 528), (300, 8192)])
 def test_dequant_spans_and_unaligned_output(b, N, K):
-    """Widths at and around the sixteen chunks that a CTA lays out or decodes at a time, and outputs that are not 16-byte aligned."""
+    """Widths at and around the chunks that a CTA lays out (four or sixteen, by the tensor's size) or decodes (sixteen) at a time, and
+    outputs that are not 16-byte aligned."""
     codes, scales = inputs.random_codes(N, K, seed=12, scale_lo=0, scale_hi=64, zero_block_frac=0.05)
     desc, packed = _pack(b, codes.numpy(), scales.numpy(), 0.0123)
     want1 = ro.f64_to_bf16_bits(ro.dequant_d1(codes.numpy(), scales.numpy()).astype(np.float64))
