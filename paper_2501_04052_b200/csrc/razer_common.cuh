@@ -6,6 +6,8 @@
 #include <cuda_bf16.h>
 #include <stdint.h>
 #include <stddef.h>
+#include <cstdlib>
+#include <utility>
 
 #include "../../include/razer.h"
 
@@ -187,6 +189,27 @@ __device__ __forceinline__ uint4 lds128(uint32_t addr) {
 
 __device__ __forceinline__ float bf16_bits_to_float(uint32_t b) {
   return __uint_as_float(b << 16);
+}
+
+// A launch that may begin while the preceding kernel of the stream drains (programmatic dependent launch; RAZER_PDL=0 in the
+// environment, read once, turns it off): the kernel touches nothing that kernel may own before its grid_dep_wait().  `what` names it
+// in the error text.
+template <class... P, class... A>
+inline int launch_dependent(const char* what, void (*kern)(P...), long long grid, int threads, size_t smem, cudaStream_t st, A&&... args) {
+  static const bool pdl = [] { const char* e = getenv("RAZER_PDL"); return !(e && e[0] == '0'); }();
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = attr;
+  cfg.numAttrs = pdl ? 1 : 0;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, std::forward<A>(args)...);
+  count_launches(1);
+  return check_cuda(e, what);
 }
 
 }  // namespace razer

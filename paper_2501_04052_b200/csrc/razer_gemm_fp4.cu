@@ -37,6 +37,7 @@
 // Work partition, partial tiles and bounded waits are those of the bf16 tcgen05 kernel: a persistent grid,
 // contiguous stripes of (tile, stage) items, partial tiles through FP32 slots and a per-tile counter.
 #include <cuda.h>
+#include <algorithm>
 #include <cstdlib>
 
 #include "razer_common.cuh"
@@ -581,6 +582,17 @@ static bool split_special_values(const float sv[2], uint32_t base[2], uint32_t r
   return true;
 }
 
+template <int NT>
+static int launch_matmul(const CUtensorMap& tmap_x, const CUtensorMap& tmap_w, const Args& a, int grid, cudaStream_t st) {
+  static bool attr_set = false;
+  if (!attr_set) {
+    RAZER_TRY(check_cuda(cudaFuncSetAttribute(razer_fp4_kernel<NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg<NT>::SMEM_BYTES),
+                         "cudaFuncSetAttribute(max dynamic shared memory)"));
+    attr_set = true;
+  }
+  return launch_dependent("razer_fp4_kernel launch", razer_fp4_kernel<NT>, grid, THREADS, Cfg<NT>::SMEM_BYTES, st, tmap_x, tmap_w, a);
+}
+
 }  // namespace fp4_path
 
 Fp4ActLayout make_fp4_act_layout(int M, int K) {
@@ -669,38 +681,7 @@ int launch_gemm_fp4_prepared(const razer_desc* d, const void* packed, const void
                            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) return set_error(RAZER_ERR_CUDA, "cuTensorMapEncodeTiled (weights) failed with code %d", (int)r);
   }
-  static const bool pdl = [] { const char* e = getenv("RAZER_PDL"); return !(e && e[0] == '0'); }();
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)p.grid);
-  cfg.blockDim = dim3(THREADS);
-  cfg.stream = st;
-  cfg.attrs = attr;
-  cfg.numAttrs = pdl ? 1 : 0;
-  cudaError_t e;
-  if (p.NT == 128) {
-    static bool attr_set = false;
-    if (!attr_set) {
-      RAZER_TRY(check_cuda(cudaFuncSetAttribute(razer_fp4_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                (int)Cfg<128>::SMEM_BYTES), "cudaFuncSetAttribute(max dynamic shared memory)"));
-      attr_set = true;
-    }
-    cfg.dynamicSmemBytes = Cfg<128>::SMEM_BYTES;
-    e = cudaLaunchKernelEx(&cfg, razer_fp4_kernel<128>, tmap_x, tmap_w, a);
-  } else {
-    static bool attr_set = false;
-    if (!attr_set) {
-      RAZER_TRY(check_cuda(cudaFuncSetAttribute(razer_fp4_kernel<256>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                (int)Cfg<256>::SMEM_BYTES), "cudaFuncSetAttribute(max dynamic shared memory)"));
-      attr_set = true;
-    }
-    cfg.dynamicSmemBytes = Cfg<256>::SMEM_BYTES;
-    e = cudaLaunchKernelEx(&cfg, razer_fp4_kernel<256>, tmap_x, tmap_w, a);
-  }
-  count_launches(1);
-  return check_cuda(e, "razer_fp4_kernel launch");
+  return p.NT == 128 ? launch_matmul<128>(tmap_x, tmap_w, a, p.grid, st) : launch_matmul<256>(tmap_x, tmap_w, a, p.grid, st);
 }
 
 // Interchange-format activations: re-lay them out into the workspace (one small kernel), then the matmul.
@@ -714,25 +695,10 @@ int launch_gemm_fp4(const razer_desc* d, const void* packed, const uint8_t* act_
     return set_error(RAZER_ERR_WORKSPACE, "workspace of %zu bytes needed, %zu given", need, ws_bytes);
   uint8_t* codes_pad = (uint8_t*)ws + core;
   uint8_t* sfb = codes_pad + p.act.codes_bytes;
-  static const bool pdl = [] { const char* e = getenv("RAZER_PDL"); return !(e && e[0] == '0'); }();
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  {
-    const long long work = (long long)M * (p.act.KP / 32) + (long long)p.act.tiles128 * p.act.spt * CH * 128;
-    long long blocks = (work + 255) / 256;
-    if (blocks > 148 * 8) blocks = 148 * 8;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)blocks);
-    cfg.blockDim = dim3(256);
-    cfg.stream = st;
-    cfg.attrs = attr;
-    cfg.numAttrs = pdl ? 1 : 0;
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, fp4_act_prep_kernel, (const uint32_t*)act_codes, act_scales, M, d->K,
-                                             p.act.KP, p.act.tiles128, p.act.spt, (uint32_t*)codes_pad, (uint32_t*)sfb);
-    count_launches(1);
-    RAZER_TRY(check_cuda(e, "fp4_act_prep_kernel launch"));
-  }
+  const long long work = (long long)M * (p.act.KP / 32) + (long long)p.act.tiles128 * p.act.spt * CH * 128;
+  RAZER_TRY(launch_dependent("fp4_act_prep_kernel launch", fp4_act_prep_kernel, std::min((work + 255) / 256, 148LL * 8), 256, 0, st,
+                             (const uint32_t*)act_codes, act_scales, M, d->K, p.act.KP, p.act.tiles128, p.act.spt, (uint32_t*)codes_pad,
+                             (uint32_t*)sfb));
   return launch_gemm_fp4_prepared(d, packed, codes_pad, act_tensor_scale_dev, M, y, ws, core, st);
 }
 

@@ -531,22 +531,7 @@ static int launch_cfg(const CUtensorMap& tmap, const CUtensorMap& tmap_w, const 
                          "cudaFuncSetAttribute(max dynamic shared memory)"));
     attr_set = true;
   }
-  // Programmatic dependent launch (RAZER_PDL=0 turns it off): the kernel may begin while the preceding
-  // kernel of the stream drains; it touches nothing that kernel may own before its grid_dep_wait().
-  static const bool pdl = [] { const char* e = getenv("RAZER_PDL"); return !(e && e[0] == '0'); }();
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)grid);
-  cfg.blockDim = dim3(Cfg::THREADS);
-  cfg.dynamicSmemBytes = Cfg::SMEM_BYTES;
-  cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = pdl ? 1 : 0;
-  const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, tmap, tmap_w, args);
-  count_launches(1);
-  return check_cuda(e, "razer_umma_kernel launch");
+  return launch_dependent("razer_umma_kernel launch", kern, grid, Cfg::THREADS, Cfg::SMEM_BYTES, st, tmap, tmap_w, args);
 }
 
 int launch_gemm_umma(const razer_desc* d, const void* packed, const void* x, int M, int ldx_K, float extra_scale,

@@ -340,20 +340,7 @@ static int launch_stream_cfg(const stream_path::Args& a, int grid, cudaStream_t 
                          "cudaFuncSetAttribute(max dynamic shared memory)"));
     attr_set = true;
   }
-  static const bool pdl = [] { const char* e = getenv("RAZER_PDL"); return !(e && e[0] == '0'); }();
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)grid);
-  cfg.blockDim = dim3(stream_path::THREADS);
-  cfg.dynamicSmemBytes = stream_path::SMEM_BYTES;
-  cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = pdl ? 1 : 0;
-  const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, a);
-  count_launches(1);
-  return check_cuda(e, "razer_stream_kernel launch");
+  return launch_dependent("razer_stream_kernel launch", kern, grid, stream_path::THREADS, stream_path::SMEM_BYTES, st, a);
 }
 
 int launch_gemv_stream(const razer_desc* d, const void* packed, const void* x, int M, float extra_scale,

@@ -1,6 +1,4 @@
 // razer_pack_layout, razer_dequant, razer_decode_act: layout shuffle and exact decode kernels.
-#include <cstdlib>
-
 #include "razer_common.cuh"
 #include "razer_decode.cuh"
 #include "razer_ptx.cuh"
@@ -238,39 +236,16 @@ __global__ void __launch_bounds__(128) copy_from_host_kernel(const uint4* __rest
 }
 
 int launch_copy_from_host(const void* src, void* dst, size_t bytes, cudaStream_t st) {
-  static const bool pdl = [] { const char* e = getenv("RAZER_PDL"); return !(e && e[0] == '0'); }();
   const int n = (int)(bytes / 16);                                     // K is a multiple of 16 elements
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)((n + 127) / 128));
-  cfg.blockDim = dim3(128);
-  cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = pdl ? 1 : 0;
-  const cudaError_t e = cudaLaunchKernelEx(&cfg, copy_from_host_kernel, (const uint4*)src, (uint4*)dst, n);
-  count_launches(1);
-  return check_cuda(e, "copy_from_host_kernel launch");
+  return launch_dependent("copy_from_host_kernel launch", copy_from_host_kernel, (n + 127) / 128, 128, 0, st, (const uint4*)src, (uint4*)dst, n);
 }
 
 int launch_decode_act(const uint8_t* codes, const uint8_t* scales, int M, int K, float sv_mag,
                       void* out, cudaStream_t st) {
   const long long nb = (long long)M * (K / 16);
-  // dependent launch: it starts up while the kernel ahead (usually the quantizer that writes its input) drains
-  static const bool pdl = [] { const char* e = getenv("RAZER_PDL"); return !(e && e[0] == '0'); }();
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)grid_for(nb, 256));
-  cfg.blockDim = dim3(256);
-  cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = pdl ? 1 : 0;
-  const cudaError_t e = cudaLaunchKernelEx(&cfg, decode_act_kernel, codes, scales, (__nv_bfloat16*)out, nb, sv_mag);
-  count_launches(1);
-  return check_cuda(e, "decode_act_kernel launch");
+  // dependent: it starts up while the kernel ahead (usually the quantizer that writes its input) drains
+  return launch_dependent("decode_act_kernel launch", decode_act_kernel, grid_for(nb, 256), 256, 0, st, codes, scales, (__nv_bfloat16*)out,
+                          nb, sv_mag);
 }
 
 }  // namespace razer

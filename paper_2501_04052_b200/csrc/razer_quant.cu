@@ -18,6 +18,8 @@
 // A block that the short form cannot take (a NaN or an infinity, a step outside 2^-60 .. 2^60) goes through the plain
 // procedure.  Measured on B200: razer_quant_act of 2048 x 8192 53.5 -> 29.6 us, razer_quant_act_fp4 (no special value)
 // 57.5 -> 20.6 us; razer_quant_weight of 11008 x 4096 257.6 -> 96.6 us.
+#include <algorithm>
+
 #include "razer_common.cuh"
 #include "razer_ptx.cuh"
 
@@ -861,29 +863,23 @@ static int launch_quant_act_any(const void* x, int M, int K, float sv_mag, const
   const long long b = (n_work + threads - 1) / threads;
   const int grid = (int)(b < 1 ? 1 : (b > max_ctas ? max_ctas : b));
   const bool two = !scale_in && grid > 1 && n_blocks >= TWO_LAUNCH_BLOCKS;
+  if (two) {
+    const long long n_vec = 2 * n_blocks, amax_ctas = std::min((n_vec + 4 * threads - 1) / (4 * threads), 8 * 148LL);
+    RAZER_TRY(launch_dependent("act_amax_kernel launch", act_amax_kernel, amax_ctas, threads, 0, st, (const uint4*)x, n_vec, sync_scratch));
+    return launch_dependent("quant_act_fused_kernel launch", kern, grid, threads, 0, st, (const uint4*)x, n_blocks, sv_mag, scale_in,
+                            sync_scratch, (uint2*)codes, scales, scale_out, o, (uint32_t)amax_ctas);
+  }
   cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)grid);
   cfg.blockDim = dim3(threads);
   cfg.stream = st;
   cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeCooperative;
+  attr[0].val.cooperative = 1;
   cfg.attrs = attr;
-  uint32_t amax_ctas = 0;
-  if (two) {
-    const long long n_vec = 2 * n_blocks, a = (n_vec + 4 * threads - 1) / (4 * threads);
-    amax_ctas = (uint32_t)(a > 8 * 148 ? 8 * 148 : a);
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.gridDim = dim3(amax_ctas);
-    cfg.numAttrs = 1;
-    RAZER_TRY(check_cuda(cudaLaunchKernelEx(&cfg, act_amax_kernel, (const uint4*)x, n_vec, sync_scratch), "act_amax_kernel launch"));
-    count_launches(1);
-  } else {
-    attr[0].id = cudaLaunchAttributeCooperative;
-    attr[0].val.cooperative = 1;
-    cfg.numAttrs = scale_in || grid == 1 ? 0 : 1;                      // the grid only meets when it computes the scale
-  }
-  cfg.gridDim = dim3((unsigned)grid);
+  cfg.numAttrs = scale_in || grid == 1 ? 0 : 1;                        // the grid only meets when it computes the scale
   const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, (const uint4*)x, n_blocks, sv_mag, scale_in, sync_scratch, (uint2*)codes,
-                                           scales, scale_out, o, amax_ctas);
+                                           scales, scale_out, o, 0u);
   count_launches(1);
   return check_cuda(e, "quant_act_fused_kernel launch");
 }

@@ -966,6 +966,56 @@ def test_decode_kernel_unit_shapes(sw, tm, spw, split):
     assert r.returncode == 0 and "ok" in r.stdout, r.stdout + r.stderr
 
 
+_DEPENDENT_EDGES = r"""
+import ctypes, sys, torch
+sys.path.insert(0, sys.argv[1])
+from paper_2501_04052_b200 import binding as b, inputs
+N = K = 1024
+codes, scales = (t.cuda() for t in inputs.random_codes(N, K, seed=1))
+desc = b.make_desc(N, K, 0.01)
+packed = b.razer_pack_layout(desc, codes, scales)
+x = inputs.activations(1024, K, 2).cuda()                 # 2^20 elements: the quantizer takes two launches
+scratch = torch.zeros(2, dtype=torch.int32, device="cuda")
+ws = b.alloc_workspace(desc, 1024, b.OP_GEMM_W4A4, "cuda")
+def calls():
+    q = b.razer_quant_act(x, sv_mag=0.0, scratch=scratch)
+    y = [b.razer_gemm_w4a4(desc, packed, *q, workspace=ws, use_native_fp4=f) for f in (False, True)]
+    act, ts = b.razer_quant_act_fp4(x, scratch=scratch)
+    y.append(b.razer_gemm_w4a4_fp4(desc, packed, act, ts, 1024, workspace=ws))
+    y.append(b.razer_gemv(desc, packed, x[:4], workspace=ws))
+    return y
+want = calls()
+torch.cuda.synchronize()
+g = torch.cuda.CUDAGraph(keep_graph=True)
+with torch.cuda.graph(g):
+    got = calls()
+get_edges, graph, n = ctypes.CDLL("libcuda.so.1").cuGraphGetEdges_v2, ctypes.c_void_p(int(g.raw_cuda_graph())), ctypes.c_size_t(0)
+assert get_edges(graph, None, None, None, ctypes.byref(n)) == 0 and n.value >= 8
+ends, data = [(ctypes.c_void_p * n.value)() for _ in range(2)], (ctypes.c_ubyte * 8 * n.value)()   # data: from port, to port, type
+assert get_edges(graph, *ends, data, ctypes.byref(n)) == 0
+g.instantiate()
+g.replay()
+torch.cuda.synchronize()
+assert all(torch.equal(a, c) for a, c in zip(got, want))
+print(sum(e[2] != 0 for e in data), n.value)
+"""
+
+
+@pytest.mark.parametrize("pdl", ["0", "1"])
+def test_dependent_launch_switch(pdl):
+    """RAZER_PDL=0 turns programmatic dependent launch off in every kernel: a graph of the calls that use it has ordinary edges only.
+    Without it every launch of those calls follows the one ahead by a programmatic edge, and the results are the same."""
+    import os
+    import subprocess
+    import sys
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", _DEPENDENT_EDGES, root], env=dict(os.environ, RAZER_PDL=pdl), capture_output=True, text=True,
+                       timeout=600)
+    assert r.returncode == 0, r.stdout + r.stderr
+    programmatic, edges = map(int, r.stdout.split())
+    assert programmatic == (0 if pdl == "0" else edges), r.stdout
+
+
 def test_back_to_back_dependent_launches(b):
     """The matmul kernels start their weight stream while the preceding kernel of the stream still runs
     (programmatic dependent launch) and must read activations, workspace and outputs only after it has
