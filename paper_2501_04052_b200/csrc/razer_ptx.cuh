@@ -7,8 +7,8 @@
 
 namespace razer {
 
-constexpr uint32_t WAIT_LIMIT = 1u << 26;             // try_wait rounds before giving up, and
-constexpr uint64_t WAIT_LIMIT_NS = 2000000000ull;     // wall-clock bound of one wait (2 s)
+constexpr uint32_t WAIT_LIMIT = 1u << 26;             // try_wait rounds before a wait gives up, and
+constexpr uint64_t WAIT_LIMIT_NS = 2000000000ull;     // its wall-clock bound (2 s)
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
   return (uint32_t)__cvta_generic_to_shared(p);
@@ -43,17 +43,21 @@ __device__ __forceinline__ uint64_t global_ns() {
   return t;
 }
 // Bounded wait; false = gave up (or another thread already flagged a failure).  In line and without a call, so that the issuing
-// loops keep their uniform registers; the clock is read only once per 1024 polls (a poll waits up to its hint).
+// loops keep their uniform registers; the clock is read only once per WAIT_POLLS polls, of up to WAIT_SLICE_NS each: the first look
+// starts the count, and the wait gives up at the first one after the rest of WAIT_LIMIT_NS.
+constexpr uint32_t WAIT_POLLS = 256;
+constexpr uint64_t WAIT_REST_NS = WAIT_LIMIT_NS - 2ull * WAIT_POLLS * WAIT_SLICE_NS;
+static_assert(2ull * WAIT_POLLS * WAIT_SLICE_NS < WAIT_LIMIT_NS, "the looks before and after the count are part of the limit");
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile uint32_t* abort_flag) {
   if (mbar_try_wait(bar, parity)) return true;
   uint64_t t0 = 0;
   for (uint32_t i = 1;; ++i) {
     if (mbar_try_wait(bar, parity)) return true;
     if (*abort_flag) return false;
-    if ((i & 1023u) == 0) {
+    if (i % WAIT_POLLS == 0) {
       const uint64_t t = global_ns();
       if (t0 == 0) t0 = t;
-      else if (t - t0 > WAIT_LIMIT_NS) return false;
+      else if (t - t0 > WAIT_REST_NS || i >= WAIT_LIMIT) return false;
     }
   }
 }
