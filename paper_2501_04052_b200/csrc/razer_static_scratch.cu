@@ -14,7 +14,7 @@ namespace razer {
 
 int launch_gemm_umma(const razer_desc*, const void* packed, const void* x, int M, int ldx_K, float extra_scale,
                      const float* extra_scale_dev, void* y, void* ws, size_t ws_bytes, cudaStream_t, uint32_t* status_host);
-size_t umma_workspace_bytes(const razer_desc*, int M);
+size_t umma_workspace_bound(int M);
 
 // Every GPU that loads the library holds this array until the process exits.
 constexpr size_t STATIC_SCRATCH_BYTES = 4u << 20;
@@ -55,8 +55,10 @@ extern "C" int razer_gemv_static(const razer_desc* d, const void* packed_dev, co
   if (reinterpret_cast<uintptr_t>(packed_dev) % 16 || reinterpret_cast<uintptr_t>(x_dev) % 16 ||
       reinterpret_cast<uintptr_t>(y_dev) % 2)
     return set_error(RAZER_ERR_INVALID_ARG, "packed_dev and x_dev must be 16-byte aligned, y_dev 2-byte aligned");
-  // one word per 128-row tile is counted in: the documented limit on the number of rows
-  const size_t need = umma_workspace_bytes(d, M) + (size_t)make_geometry(d->N, d->K).row_tiles * sizeof(uint32_t);
+  // The limit on the rows is part of this entry point: a word for every 128-row tile and two slots of all SMs are counted, although
+  // the kernel now gets by with a counter and a slot per CTA.
+  const size_t need = WS_STATUS_BYTES + ((size_t)make_geometry(d->N, d->K).row_tiles * sizeof(uint32_t) + 255) / 256 * 256 +
+                      2 * (umma_workspace_bound(M) - WS_ZERO_BYTES);
   if (need > STATIC_SCRATCH_BYTES)
     return set_error(RAZER_ERR_UNSUPPORTED,
                      "this shape needs %zu bytes of scratch; the built-in array holds %zu (use razer_gemv with a "
