@@ -187,10 +187,6 @@ __device__ __forceinline__ uint4 lds128(uint32_t addr) {
   return v;
 }
 
-__device__ __forceinline__ float bf16_bits_to_float(uint32_t b) {
-  return __uint_as_float(b << 16);
-}
-
 // A launch that may begin while the preceding kernel of the stream drains (programmatic dependent launch; RAZER_PDL=0 in the
 // environment, read once, turns it off): the kernel touches nothing that kernel may own before its grid_dep_wait().  `what` names it
 // in the error text.

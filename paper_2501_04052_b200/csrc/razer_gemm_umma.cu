@@ -43,18 +43,6 @@
 
 namespace razer {
 
-// Shared-memory matrix descriptor of a K-major bf16 tile stored with the 128-byte swizzle:
-// rows are 128 bytes (64 elements), groups of 8 rows are 1024 bytes apart.
-__device__ __forceinline__ uint64_t make_b_desc(uint32_t saddr) {
-  uint64_t d = 0;
-  d |= (uint64_t)((saddr & 0x3FFFFu) >> 4);          // start address
-  d |= (uint64_t)1 << 16;                            // leading byte offset (unused for swizzled K-major)
-  d |= (uint64_t)(1024u >> 4) << 32;                 // stride byte offset: 8 rows x 128 B
-  d |= (uint64_t)1 << 46;                            // descriptor version of this architecture
-  d |= (uint64_t)2 << 61;                            // swizzle mode: 128 B
-  return d;
-}
-
 // Instruction descriptor: bf16 x bf16 -> f32, both operands K-major, M = 128, N = NT.
 __host__ __device__ constexpr uint32_t make_idesc(int nt) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(nt >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
@@ -62,7 +50,6 @@ __host__ __device__ constexpr uint32_t make_idesc(int nt) {
 
 // ------------------------------------------------------------------ kernel
 struct UmmaArgs {
-  const uint8_t* packed;
   __nv_bfloat16* y;
   float* slots;              // [grid] FP32 partial tiles of NT x 128
   uint32_t* counters;        // one per CTA: that of the partial tile it finishes; zero between calls
@@ -274,7 +261,8 @@ razer_umma_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
   } else if (warp == 1) {
     // ===================== MMA issuer =====================
     constexpr uint32_t idesc = make_idesc(NT);
-    // upper half of the shared-memory descriptor: 1024-byte group stride, descriptor version, 128-byte swizzle
+    // Shared-memory descriptor of a K-major bf16 tile in the 128-byte swizzle (rows of 128 bytes, 64 elements): upper half = 1024 bytes
+    // from one group of eight rows to the next, descriptor version, swizzle mode
     constexpr uint32_t bd_hi = (1024u >> 4) | (1u << 14) | (2u << 29);
     // One elected lane walks the items.  Electing once around the whole loop lets the compiler keep descriptors and
     // addresses in uniform registers; electing anew for every item cost about 37 cycles per tcgen05 instruction.
@@ -310,8 +298,8 @@ razer_umma_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
               if (j < nch * 4) {
                 const uint32_t bd = bd_lo + (uint32_t)(((k >> 2) * Cfg::X_BOX_BYTES + (k & 3) * 32) >> 4);
                 const uint32_t d_t = d_0 + (j % Cfg::PER_SET) * NT;
-                if (j < Cfg::PER_SET && fresh) tc_mma_ts2<false>(d_t, a_t + j * 8, bd, bd_hi, idesc);
-                else tc_mma_ts2<true>(d_t, a_t + j * 8, bd, bd_hi, idesc);
+                if (j < Cfg::PER_SET && fresh) tc_mma_ts<false>(d_t, a_t + j * 8, bd, bd_hi, idesc);
+                else tc_mma_ts<true>(d_t, a_t + j * 8, bd, bd_hi, idesc);
               }
             }
             tc_commit(bar_xempty + 8 * xr.slot);
@@ -579,7 +567,6 @@ int launch_gemm_umma(const razer_desc* d, const void* packed, const void* x, int
   }
 
   UmmaArgs a;
-  a.packed = (const uint8_t*)packed;
   a.y = (__nv_bfloat16*)y;
   a.status = (uint32_t*)ws;
   a.counters = (uint32_t*)((char*)ws + WS_STATUS_BYTES);

@@ -81,7 +81,7 @@ __device__ __forceinline__ void strip_step(float (&acc)[4], uint32_t piece, cons
   word_step(acc, c0.y, c1.y, r0, r1, s0, s1, xq[1]);
 }
 
-// The warp's slices J, J + 1, .. SPW - 1 of a stage (slice j is chunk c + j * CW): activation fragment, then decode
+// The warp's slices J, J + 1, .. SPW - 1 of a stage (slice j is chunk c + j * KW): activation fragment, then decode
 // + MMA for each of the unit's strips, fully unrolled with every shared-memory offset an immediate (a rolled
 // loop over the slices, with or without loading a slice ahead, measured 6 to 15 % slower).
 // CHECKED: the stage is the last of a segment and may hold fewer slices.
