@@ -139,11 +139,11 @@ int razer_gemm(const razer_desc* d, const void* packed_dev, const void* x_dev, i
 
 /* razer_gemv with HOST activations and HOST output: copies x (M*K bf16) into
  * x_stage_dev, runs razer_gemv, brings y (M*N bf16) back and synchronizes the stream.
- * x_host / y_host should be pinned for the copies to be asynchronous.  When y_host is
+ * x_host / y_host should be pinned for the copies to be asynchronous.  When all of y_host is
  * pinned memory that the device can address (what cudaHostAlloc / cudaHostRegister give
  * under unified addressing), the kernel stores y straight into it and y_stage_dev is not
- * touched; otherwise y goes through y_stage_dev and one more copy.  Pinned x_host of up to 256 KB on a
- * 16-byte boundary is fetched by a kernel instead of a copy.  Each calling thread keeps 64 bytes of pinned host memory
+ * touched; otherwise y goes through y_stage_dev and one more copy.  An x_host that is pinned as a whole, of up to 256 KB and
+ * on a 16-byte boundary, is fetched by a kernel instead of a copy.  Each calling thread keeps 64 bytes of pinned host memory
  * (the workspace's status is shown there) until it ends. */
 int razer_gemv_host(const razer_desc* d, const void* packed_dev, const void* x_host, int M,
                     void* y_host, void* x_stage_dev, void* y_stage_dev, void* workspace_dev,
@@ -202,8 +202,9 @@ int razer_quant_act(const void* x_dev, int M, int K, float sv_mag,
  * razer_quant_act; amax_scratch_dev: one device uint32 (needed when the scale is computed; the
  * call clears it itself).  Writes the interchange format that razer_pack_layout reads:
  * codes_dev [N][K/2], scales_dev [N][K/block] ([meta(2) | E3M3 code(6)]), special value =
- * remap_code (0x8 or 0x0), and the tensor scale to tensor_scale_out_dev.  Every FP32 step is a
- * single IEEE operation in a fixed order, so the result is reproducible bit for bit.
+ * remap_code (0x8 or 0x0), and the tensor scale to tensor_scale_out_dev.  Every decision
+ * is that of single IEEE FP32 operations in a fixed order, so the result is reproducible bit for
+ * bit.
  * Asynchronous on `stream`. */
 int razer_quant_weight(const float* w_dev, int N, int K, int block, int scale_aware,
                        const float sv_mag[2], int remap_code,

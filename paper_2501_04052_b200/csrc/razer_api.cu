@@ -280,7 +280,10 @@ struct HostStatus {
   }
 };
 
-// Up to here a kernel fetches x over the bus; beyond, the copy engine.
+// Up to here a kernel fetches x over the bus; beyond, the copy engine.  us a call, kernel / copy engine, on two machines: 2 KB 19.8 / 21.2
+// and 20.5 / 23.7, 22 KB 22.6 / 23.7 and 29.0 / 28.4, 64 KB 24.9 / 25.1 and 30.1 / 30.1, 256 KB 38.8 / 48.4 and 32.1 / 38.3, 1 MB 44.4 / 71.2
+// and 48.2 / 50.9, 3.5 MB 101 / 212 and 103 / 102.  So the two do not cross here: the kernel is level up to 64 KB and ahead beyond.  The line only
+// bounds how long it holds SMs for the bus.
 constexpr size_t HOST_X_KERNEL_BYTES = 256 * 1024;
 static bool use_simt(const razer_desc* d, int M) { return !use_stream(d, M) && !umma_supported(d, M); }
 }  // namespace razer

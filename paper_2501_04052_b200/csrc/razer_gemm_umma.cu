@@ -22,7 +22,8 @@
 // 64 x 8192 x 28672 50.1 -> 45.0, 16 x 8192 x 28672 45.7 -> 40.8.  At 16 tokens the decode takes 2500 cycles of the 4070 that a
 // group spends on an item; most of the rest it waits for its operand stage, 700 cycles from its last store to the MMAs'
 // completion.  Half-item operand stages, two to a group, came to 45.7 us (the MMA warp's waits double), all groups on one item with
-// two stages to 44.3, without the MMAs the launch takes 40.4.
+// two stages to 44.3, without the MMAs the launch takes 40.4.  (All with two accumulators; the six that the precision asks for take
+// 1 % longer.)  In a prefill the tensor pipe is active 81 % of a CTA's cycles; the shared-memory figure is counted from the layout.
 //
 // Work partition (Sec. 4.3 / App. E of the paper: stripes of about equal length that may span
 // several output tiles, partial results reduced through global memory): the grid is
@@ -460,8 +461,8 @@ struct UmmaPlan {
 };
 
 // Token tile and grid: the cheapest pair by the cost model (razer_tcgen05.cuh), fitted to a sweep of 18 shapes (M 16 .. 2048, K and N
-// 300 .. 28672, all widths, all grids).  On these the choice is within 11 % of the best of the sweep (16 x 28672 x 1024
-// aside), where the fixed rule before it (the narrowest tile that holds M, all SMs) was up to 4 times slower: 300 x 390 x 2320
+// 300 .. 28672, all widths, all grids).  On these the choice is within 11 % of the best of the sweep (further off at
+// 16 x 28672 x 1024, 14.3 -> 10.0 us), where the fixed rule before it (the narrowest tile that holds M, all SMs) was up to 4 times slower: 300 x 390 x 2320
 // 36.2 -> 8.1 us, 256 x 1024 x 1024 20.8 -> 4.8, 1000 x 300 x 8192 33.1 -> 14.5, 333 x 4096 x 11008 38.8 -> 32.4.
 static const TileCost tile_costs[] = {
     {16, 4, 4, 0.168f, 0.20f, 0.0f, 2.0f, 0.20f, 4.0f, 0.06f},  {32, 4, 4, 0.170f, 0.20f, 0.1f, 2.6f, 0.20f, 4.0f, 0.11f},
