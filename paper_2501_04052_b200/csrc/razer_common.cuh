@@ -187,6 +187,28 @@ __device__ __forceinline__ uint4 lds128(uint32_t addr) {
   return v;
 }
 
+// 32 bytes to or from global memory, in one access where the address allows it (`wide`, uniform): a thread with a 32-byte block of its
+// own makes every access of a warp touch 32 separate sectors, and halves issued apart cost twice the requests.
+__device__ __forceinline__ bool aligned32(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 31) == 0; }
+__device__ __forceinline__ void store32(void* p, const uint32_t (&v)[8], bool wide) {
+  if (wide) {
+    asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]),
+                 "r"(v[5]), "r"(v[6]), "r"(v[7])
+                 : "memory");
+  } else {
+    reinterpret_cast<uint4*>(p)[0] = make_uint4(v[0], v[1], v[2], v[3]);
+    reinterpret_cast<uint4*>(p)[1] = make_uint4(v[4], v[5], v[6], v[7]);
+  }
+}
+
+// Interchange order of a code word (element j in nibble j) to the packed order (nibbles p and p + 4 = elements 2p, 2p + 1).
+__device__ __forceinline__ uint32_t to_packed_order(uint32_t w) {
+  constexpr uint32_t LOW = 0x0F0F0F0Fu;
+  const uint32_t s4 = w >> 4, s8 = w >> 8;
+  // bytes 0 and 2 of the two words: elements 0, 2 and 4, 6; elements 1, 3 and 5, 7
+  return __byte_perm((w & LOW) | (s4 & ~LOW), (s4 & LOW) | (s8 & ~LOW), 0x6420);
+}
+
 // A launch that may begin while the preceding kernel of the stream drains (programmatic dependent launch; RAZER_PDL=0 in the
 // environment, read once, turns it off): the kernel touches nothing that kernel may own before its grid_dep_wait().  `what` names it
 // in the error text.

@@ -468,12 +468,6 @@ __global__ void fp4_act_prep_kernel(const uint32_t* __restrict__ codes, const ui
   const long long n_code = (long long)M * row_quads;
   const long long n_sf = (long long)tiles128 * spt * CH * 128;
   const bool vec = (K % 32) == 0 && (reinterpret_cast<uintptr_t>(codes) % 16) == 0;   // rows of the input start on 16 bytes
-  auto shuffle = [](uint32_t w) -> uint32_t {                          // element j of the word: nibble j -> nibble j / 2 + 4 (j % 2)
-    uint32_t o = 0;
-#pragma unroll
-    for (int j = 0; j < 8; ++j) o |= ((w >> (4 * j)) & 0xFu) << (4 * ((j >> 1) + 4 * (j & 1)));
-    return o;
-  };
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n_code + n_sf;
        i += (long long)gridDim.x * blockDim.x) {
     if (i < n_code) {
@@ -488,7 +482,7 @@ __global__ void fp4_act_prep_kernel(const uint32_t* __restrict__ codes, const ui
         if (4 * q + 2 < in_words) w.z = src[2];
         if (4 * q + 3 < in_words) w.w = src[3];
       }
-      reinterpret_cast<uint4*>(codes_out)[i] = make_uint4(shuffle(w.x), shuffle(w.y), shuffle(w.z), shuffle(w.w));
+      reinterpret_cast<uint4*>(codes_out)[i] = make_uint4(to_packed_order(w.x), to_packed_order(w.y), to_packed_order(w.z), to_packed_order(w.w));
     } else {
       const long long s = i - n_code;
       const int wi = (int)(s & 127);

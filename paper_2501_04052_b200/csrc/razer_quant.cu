@@ -670,7 +670,6 @@ __device__ __forceinline__ void load8(const float4* p, float* v, bool wide) {
     v[0] = a.x, v[1] = a.y, v[2] = a.z, v[3] = a.w, v[4] = b.x, v[5] = b.y, v[6] = b.z, v[7] = b.w;
   }
 }
-__device__ __forceinline__ bool aligned32(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 31) == 0; }
 
 // One thread per scale block of `sub` groups of 16 elements (ONE: sub == 1, the block stays in registers from its maximum
 // to its codes; larger blocks are walked three times).  A magnitude beyond 6 can win an element only where the block's
