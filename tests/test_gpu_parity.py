@@ -404,6 +404,27 @@ def test_quant_weight_bit_exact(b, N, K, seed, sv_mag, remap_code):
     assert np.linalg.norm(d2 - w.numpy()) / np.linalg.norm(w.numpy()) < 0.12
 
 
+@pytest.mark.parametrize("block", [16, 32, 64, 128])
+@pytest.mark.parametrize("sv_mag,remap_code", [((5.0, 8.0), 0x8), ((3.5, 6.5), 0x0), ((2.5, 12.0), 0x8)])
+def test_quant_weight_ties_between_candidates(b, block, sv_mag, remap_code):
+    """Scaled elements on a grid of eighths: every error is exact in FP32, candidates tie often, and elements sit exactly on the ends of the
+    intervals that a special value takes, so codes, signs and special values must be the first minimum's without exception.  Every other row
+    saturates its scale code, with elements up to 9.25 steps; a few blocks are zero."""
+    N, K = 96, 1152
+    gen = torch.Generator().manual_seed(block)
+    w = torch.randint(-40, 41, (N, K), generator=gen).float()
+    w = torch.where(torch.rand((N, K), generator=gen) < 0.6, torch.round(w / 4) * 4, w)
+    w.view(N, -1, block)[:, :, 3] = 48.0                       # block maximum: 6 steps
+    w.view(N, -1, block)[1::2, ::2, 5] = -74.0                 # or 9.25
+    w.view(N, -1, block)[::7, 1] = 0.0
+    w = w / 8
+    w[1::2] *= 1.875
+    given = torch.tensor([1.0])
+    codes, scales, _ = b.razer_quant_weight(w.cuda(), sv_mag=sv_mag, remap_code=remap_code, tensor_scale=given.cuda(), block=block)
+    want_c, want_s, _ = ro.quantize_weight(w.numpy(), sv_mag=sv_mag, remap_code=remap_code, tensor_scale=np.float32(1.0), block=block)
+    assert np.array_equal(scales.cpu().numpy(), want_s) and np.array_equal(codes.cpu().numpy(), want_c)
+
+
 @pytest.mark.parametrize("block", [32, 64, 128])
 def test_larger_blocks_quantize_pack_and_multiply(b, block):
     """Block sizes 32 / 64 / 128 (Sec. 5's block-size study, Sec. 4.3's deployment size): the GPU weight quantizer
