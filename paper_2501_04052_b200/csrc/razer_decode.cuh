@@ -79,4 +79,52 @@ __device__ __forceinline__ void decode_word(uint32_t w, uint32_t ss2, uint32_t s
   out[3] = mul_bf16x2(u3, ss2);
 }
 
+
+// The same pairs by table: [weight byte][special value][lane], two elements (value x 2^-126) to an entry, a copy per lane so that 32
+// random lookups never meet on a bank.  A pair costs a byte permute (which forms the address), a load and the multiply by the
+// scale; another permute each puts the pairs back in order, since a byte of a code word holds elements 0, 2 / 4, 6 / 1, 3 / 5, 7.
+// On B200 a packed bf16 operation takes two issue slots (one alternating with a logic operation measured 3.3 cycles for the pair),
+// so a word is 29 slots in registers and 20 this way.
+constexpr int PAIR_TABLE_BYTES = 65536;
+__device__ __forceinline__ void pair_table_fill(uint32_t base, int tid, int nthreads, uint32_t svp0, uint32_t svp1) {
+#pragma unroll 1
+  for (int e = tid; e < 512; e += nthreads) {
+    auto element = [&](uint32_t nib) { return nib ? ((nib & 7u) << 6) | ((nib & 8u) << 12) : ((e & 1) ? svp1 : svp0) & 0xFFFFu; };
+    const uint32_t v = element(((uint32_t)e >> 1) & 0xFu) | (element((uint32_t)e >> 5) << 16);
+#pragma unroll
+    for (int j = 0; j < 8; ++j)                             // each lane starts elsewhere in its row
+      asm volatile("st.shared.v4.u32 [%0], {%1, %1, %1, %1};" ::"r"(base + (uint32_t)e * 128 + (uint32_t)((j + tid) & 7) * 16), "r"(v) : "memory");
+  }
+}
+// Byte B of a code word; `row` = select bit (bit 7) | lane * 4.
+template <int B>
+__device__ __forceinline__ uint32_t pair_lookup(const uint8_t* table, uint32_t w, uint32_t row) {
+  return *reinterpret_cast<const uint32_t*>(table + __byte_perm(w, row, 0x7604 | (B << 4)));
+}
+// The pairs of two blocks, unscaled; `rows` = the chunk's select bits (bit 7 of each byte) | lane * 4 in every byte.
+__device__ __forceinline__ void lookup_blocks(const uint8_t* table, uint32_t rows, int blk, const uint2 (&cw)[CHUNK_BLOCKS], uint32_t (&pairs)[16]) {
+#pragma unroll
+  for (int b = 0; b < 2; ++b) {
+    const uint32_t row = __byte_perm(rows, 0, 0x4440 | (blk + b));
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const uint32_t w = h ? cw[blk + b].y : cw[blk + b].x;
+      uint32_t* p = pairs + 8 * b + 4 * h;
+      p[0] = pair_lookup<0>(table, w, row);                 // elements 0, 2
+      p[1] = pair_lookup<2>(table, w, row);                 // 1, 3
+      p[2] = pair_lookup<1>(table, w, row);                 // 4, 6
+      p[3] = pair_lookup<3>(table, w, row);                 // 5, 7
+    }
+  }
+}
+// ... scaled and put in order.
+__device__ __forceinline__ void finish_blocks(const uint32_t (&pairs)[16], uint32_t s0, uint32_t s1, uint32_t* out) {
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    const uint32_t s = q < 4 ? s0 : s1, x = mul_bf16x2(pairs[2 * q], s), y = mul_bf16x2(pairs[2 * q + 1], s);
+    out[2 * q] = __byte_perm(x, y, 0x5410);
+    out[2 * q + 1] = __byte_perm(x, y, 0x7632);
+  }
+}
+
 }  // namespace razer

@@ -13,17 +13,19 @@
 // and epilogue, the last = activation producer.  A warp reaches only the TMEM lanes 32 * (warp % 4) .. + 31; four warps form a
 // group that decodes an item, and the groups take the items in turn.
 //
-// The register-level decode is described in razer_decode.cuh.
+// Both decodes are described in razer_decode.cuh.  Up to 32 tokens by table: 16 x 8192 x 28672 41.3 (registers) -> 36.0 us, 16 x 4096 x 11008
+// 14.2 -> 13.1, 32 x 28672 x 8192 43.2 -> 38.7.  From 64 tokens on in registers: the table takes 64 KB from the rings, and its loads
+// meet the activations' in shared memory (64 x 8192 x 28672 45.3 us in registers, 49.7 by table, 48 half and half).
 //
-// What bounds it: the decode (about 3.4 instructions a weight) up to 128 tokens, from there on the MMAs (512 cycles per 128 x 256 x
-// 64) together with shared-memory bandwidth (571 cycles), and the combination of cut tiles.  Device times on B200, first for one
+// What bounds it: up to 32 tokens shared memory (270 wavefronts a chunk of about 305 cycles, copies and MMAs counted from the layout)
+// and issue (246 of 305 slots), then the decode (about 3.4 instructions a weight) up to 128 tokens, from there on the MMAs (512 cycles
+// per 128 x 256 x 64) together with shared-memory bandwidth (571 cycles), and the combination of cut tiles.  Device times on B200, first for one
 // ring of weights and activations and items of one chunk at 256 tokens, then for rings apart, two-chunk items and groups that
 // walk only their own items: 2048 x 14336 x 4096 204 -> 171 us (149 with the decode left out), 256 x 8192 x 8192 38.4 -> 32.7,
-// 64 x 8192 x 28672 50.1 -> 45.0, 16 x 8192 x 28672 45.7 -> 40.8.  At 16 tokens the decode takes 2500 cycles of the 4070 that a
-// group spends on an item; most of the rest it waits for its operand stage, 700 cycles from its last store to the MMAs'
-// completion.  Half-item operand stages, two to a group, came to 45.7 us (the MMA warp's waits double), all groups on one item with
-// two stages to 44.3, without the MMAs the launch takes 40.4.  (All with two accumulators; the six that the precision asks for take
-// 1 % longer.)  In a prefill the tensor pipe is active 81 % of a CTA's cycles; the shared-memory figure is counted from the layout.
+// 64 x 8192 x 28672 50.1 -> 45.0, 16 x 8192 x 28672 45.7 -> 40.8.  At 16 tokens, decoded in registers: half-item operand stages, two
+// to a group, 45.7 us (the MMA warp's waits double), all groups on one item with two stages 44.3, four groups with items of three
+// chunks 44.7 (by table 41.8), without the MMAs 40.4; the chunk loop rolled, by table, 44.5.  In a prefill the tensor pipe is active
+// 81 % of a CTA's cycles; the shared-memory figure is counted from the layout.
 //
 // Work partition (Sec. 4.3 / App. E of the paper: stripes of about equal length that may span
 // several output tiles, partial results reduced through global memory): the grid is
@@ -74,7 +76,7 @@ struct UmmaArgs {
 // a ring's length before had completed and both operands had been loaded again.  A work item is CH chunks, an activation
 // stage CHX of them: every item costs a group two barrier waits, a drained TMEM store and its bookkeeping, so items of one
 // chunk decode about a quarter slower than items of four, while activation boxes of 256 tokens fit only singly.
-template <int NT, int CH, int CHX, int WST, int XST, int AST, int NDW, int NACC>
+template <int NT, int CH, int CHX, int WST, int XST, int AST, int NDW, int NACC, bool TABLE>
 struct UmmaCfg {
   static constexpr int GROUPS = NDW / 4;                       // four warps (all TMEM lane quarters) decode one item together
   static constexpr int THREADS = 64 + 32 * NDW + 32;           // + W producer, MMA warp, X producer
@@ -92,9 +94,10 @@ struct UmmaCfg {
   static constexpr int TMEM_COLS = TMEM_COLS_NEEDED <= 64 ? 64 : TMEM_COLS_NEEDED <= 128 ? 128
                                    : TMEM_COLS_NEEDED <= 256 ? 256 : 512;
   static constexpr int NUM_BARS = 2 * (WST + XST + AST) + 4;
+  static constexpr int PAIR_BYTES = TABLE ? PAIR_TABLE_BYTES : 0;   // at the start of shared memory
   static constexpr int TABLE_BYTES = DECODE_TABLE_BYTES;        // scale table
   static constexpr size_t SMEM_BYTES =
-      1024 /*alignment slack*/ + (size_t)XST * X_BYTES + (size_t)WST * W_BYTES + NUM_BARS * 8 + 16 + 64 + TABLE_BYTES;
+      1024 /*alignment slack*/ + PAIR_BYTES + (size_t)XST * X_BYTES + (size_t)WST * W_BYTES + NUM_BARS * 8 + 16 + 64 + TABLE_BYTES;
   static_assert(TMEM_COLS_NEEDED <= 512, "TMEM budget exceeded");
   static_assert(SMEM_BYTES <= 232448, "shared memory budget exceeded");
   static_assert(CH % CHX == 0, "an item is whole activation stages");
@@ -114,17 +117,18 @@ struct Ring {
   }
 };
 
+extern __shared__ __align__(1024) uint8_t umma_smem[];      // a link-time address: the pair table is indexed from it without an addition
+
 // The MMA warp issues every item's MMAs.  (Letting the group that decoded an item issue it, once level at 16 tokens, lost
 // when the MMA warp came to elect its lane once: 8192 x 28672 at 16 tokens 49.3 against 45.9 us.)
-template <int NT, int CH, int CHX, int WST, int XST, int AST, int NDW, int NACC>
+template <int NT, int CH, int CHX, int WST, int XST, int AST, int NDW, int NACC, bool TABLE>
 __global__ void __launch_bounds__(96 + 32 * NDW, 1)
 razer_umma_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant__ CUtensorMap tmap_w,
                   const __grid_constant__ UmmaArgs a) {
-  using Cfg = UmmaCfg<NT, CH, CHX, WST, XST, AST, NDW, NACC>;
+  using Cfg = UmmaCfg<NT, CH, CHX, WST, XST, AST, NDW, NACC, TABLE>;
   constexpr int GROUPS = Cfg::GROUPS;
   constexpr int X_WARP = 2 + NDW;                       // the activation producer
-  extern __shared__ uint8_t smem_raw[];
-  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(umma_smem) + Cfg::PAIR_BYTES + 1023) & ~(uintptr_t)1023);
   const uint32_t smem_x = smem_u32(smem), smem_w = smem_x + XST * Cfg::X_BYTES;
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + (size_t)XST * Cfg::X_BYTES + (size_t)WST * Cfg::W_BYTES);
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(        // 16-byte aligned: the table behind it is written as uint4
@@ -196,7 +200,10 @@ razer_umma_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
     grid_dep_launch();                                    // the next kernel may start its own prologue
     for (; issued < n_items && issued < WST; ++issued) produce_w();
   }
-  if (warp >= 2) decode_tables_fill(tables, threadIdx.x - 64, Cfg::THREADS - 64);
+  if (warp >= 2) {
+    decode_tables_fill(tables, threadIdx.x - 64, Cfg::THREADS - 64);
+    if (TABLE) pair_table_fill(smem_addr(umma_smem), threadIdx.x - 64, Cfg::THREADS - 64, a.svp0, a.svp1);
+  }
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
                  "r"((uint32_t)Cfg::TMEM_COLS)
@@ -332,7 +339,7 @@ razer_umma_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
       return __all_sync(0xFFFFFFFFu, got);
     };
     const uint32_t ss_lane = smem_addr(tables) + lane * 4;
-    const uint32_t mul_lo = a.mul_lo, mul_hi = a.mul_hi;
+    const uint32_t mul_lo = a.mul_lo, mul_hi = a.mul_hi, lanes = (uint32_t)lane * 0x04040404u;
     // where this thread's weight row sits inside a stage ([strip 0..7][chunk 0..CH-1] pieces): strip row / 16, row r = row % 16 of it
     const int r16 = row % STRIP_ROWS;
     const uint32_t strip_at = smem_w + (uint32_t)(row / STRIP_ROWS) * (CH * PIECE_BYTES);
@@ -401,32 +408,51 @@ razer_umma_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
         uint32_t sw;
         uint2 cw[CHUNK_BLOCKS];
         load(0, sw, cw);
+        uint32_t pairs[2][16];
+        if (TABLE) lookup_blocks(umma_smem, (sw & 0x80808080u) | lanes, 0, cw, pairs[0]);
         if (!wait_all(bar_aempty + 8 * aslot, aphase ^ 1u, 6)) break;
         tc_fence_after();
+        if constexpr (TABLE) {
+          // half a chunk's lookups are on their way while the half before is scaled and put in order
 #pragma unroll
-        for (int c = 0; c < CH; ++c) {
-          if (c < nch) {
-            uint32_t ss2[CHUNK_BLOCKS];
+          for (int c = 0; c < CH; ++c) {
+            if (c < nch) {
+              uint32_t ss2[CHUNK_BLOCKS], v[8 * CHUNK_BLOCKS];
 #pragma unroll
-            for (int blk = 0; blk < CHUNK_BLOCKS; ++blk) ss2[blk] = decode_block_scale(ss_lane, sw, blk);
-            // the next chunk is fetched while this one is decoded (beyond the last one, or past the end of K: unused or zeros)
-            uint32_t sw_next = 0;
-            uint2 cw_next[CHUNK_BLOCKS];
-            if (c + 1 < CH) load(c + 1, sw_next, cw_next);
-            // (One store for the chunk lets the four blocks' decodes mix: 16 x 8192 x 28672 42.0 -> 40.9 us.  A lookup table instead,
-            // as in the decode kernel, came out level: its loads cost what its fewer instructions save.)
-            uint32_t v[8 * CHUNK_BLOCKS];
-#pragma unroll
-            for (int blk = 0; blk < CHUNK_BLOCKS; ++blk) {
-              const uint32_t svp = (sw & (PACKED_SELECT << (8 * blk))) ? a.svp1 : a.svp0;
-              decode_word(cw[blk].x, ss2[blk], svp, mul_lo, mul_hi, v + 8 * blk);
-              decode_word(cw[blk].y, ss2[blk], svp, mul_lo, mul_hi, v + 8 * blk + 4);
+              for (int blk = 0; blk < CHUNK_BLOCKS; ++blk) ss2[blk] = decode_block_scale(ss_lane, sw, blk);
+              lookup_blocks(umma_smem, (sw & 0x80808080u) | lanes, 2, cw, pairs[1]);
+              if (c + 1 < CH) load(c + 1, sw, cw);          // beyond the last chunk, or past the end of K: unused or zeros
+              finish_blocks(pairs[0], ss2[0], ss2[1], v);
+              if (c + 1 < CH) lookup_blocks(umma_smem, (sw & 0x80808080u) | lanes, 0, cw, pairs[0]);
+              finish_blocks(pairs[1], ss2[2], ss2[3], v + 16);
+              tc_st32(a_t + c * 32, v);
             }
-            tc_st32(a_t + c * 32, v);
-            if (c + 1 < CH) {
-              sw = sw_next;
+          }
+        } else {
 #pragma unroll
-              for (int blk = 0; blk < CHUNK_BLOCKS; ++blk) cw[blk] = cw_next[blk];
+          for (int c = 0; c < CH; ++c) {
+            if (c < nch) {
+              uint32_t ss2[CHUNK_BLOCKS];
+#pragma unroll
+              for (int blk = 0; blk < CHUNK_BLOCKS; ++blk) ss2[blk] = decode_block_scale(ss_lane, sw, blk);
+              // the next chunk is fetched while this one is decoded (beyond the last one, or past the end of K: unused or zeros)
+              uint32_t sw_next = 0;
+              uint2 cw_next[CHUNK_BLOCKS];
+              if (c + 1 < CH) load(c + 1, sw_next, cw_next);
+              // (One store for the chunk lets the four blocks' decodes mix.)
+              uint32_t v[8 * CHUNK_BLOCKS];
+#pragma unroll
+              for (int blk = 0; blk < CHUNK_BLOCKS; ++blk) {
+                const uint32_t svp = (sw & (PACKED_SELECT << (8 * blk))) ? a.svp1 : a.svp0;
+                decode_word(cw[blk].x, ss2[blk], svp, mul_lo, mul_hi, v + 8 * blk);
+                decode_word(cw[blk].y, ss2[blk], svp, mul_lo, mul_hi, v + 8 * blk + 4);
+              }
+              tc_st32(a_t + c * 32, v);
+              if (c + 1 < CH) {
+                sw = sw_next;
+#pragma unroll
+                for (int blk = 0; blk < CHUNK_BLOCKS; ++blk) cw[blk] = cw_next[blk];
+              }
             }
           }
         }
@@ -465,7 +491,7 @@ struct UmmaPlan {
 // 16 x 28672 x 1024, 14.3 -> 10.0 us), where the fixed rule before it (the narrowest tile that holds M, all SMs) was up to 4 times slower: 300 x 390 x 2320
 // 36.2 -> 8.1 us, 256 x 1024 x 1024 20.8 -> 4.8, 1000 x 300 x 8192 33.1 -> 14.5, 333 x 4096 x 11008 38.8 -> 32.4.
 static const TileCost tile_costs[] = {
-    {16, 4, 4, 0.168f, 0.20f, 0.0f, 2.0f, 0.20f, 4.0f, 0.06f},  {32, 4, 4, 0.170f, 0.20f, 0.1f, 2.6f, 0.20f, 4.0f, 0.11f},
+    {16, 4, 4, 0.140f, 0.20f, 0.0f, 2.0f, 0.20f, 4.0f, 0.06f},  {32, 4, 2, 0.152f, 0.20f, 0.1f, 2.6f, 0.20f, 4.0f, 0.11f},
     {64, 4, 4, 0.178f, 0.15f, 0.4f, 2.3f, 0.35f, 4.5f, 0.22f},  {96, 4, 2, 0.186f, 0.15f, 0.5f, 2.4f, 0.37f, 5.0f, 0.34f},
     {128, 4, 1, 0.228f, 0.15f, 0.7f, 2.9f, 0.75f, 6.0f, 0.45f}, {192, 2, 1, 0.268f, 0.20f, 1.2f, 3.7f, 0.60f, 6.3f, 0.67f},
     {256, 2, 1, 0.315f, 0.25f, 1.6f, 4.0f, 0.55f, 7.0f, 0.90f}};
@@ -510,10 +536,10 @@ size_t umma_workspace_bound(int M) {
   return WS_ZERO_BYTES + (size_t)sm_count() * widest * TILE_ROWS * sizeof(float);
 }
 
-template <int NT, int CH, int CHX, int WST, int XST, int AST, int NDW, int NACC>
+template <int NT, int CH, int CHX, int WST, int XST, int AST, int NDW, int NACC, bool TABLE>
 static int launch_cfg(const CUtensorMap& tmap, const CUtensorMap& tmap_w, const UmmaArgs& args, int grid, cudaStream_t st) {
-  using Cfg = UmmaCfg<NT, CH, CHX, WST, XST, AST, NDW, NACC>;
-  auto kern = razer_umma_kernel<NT, CH, CHX, WST, XST, AST, NDW, NACC>;
+  using Cfg = UmmaCfg<NT, CH, CHX, WST, XST, AST, NDW, NACC, TABLE>;
+  auto kern = razer_umma_kernel<NT, CH, CHX, WST, XST, AST, NDW, NACC, TABLE>;
   static bool attr_set = false;
   if (!attr_set) {
     RAZER_TRY(check_cuda(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::SMEM_BYTES),
@@ -587,13 +613,13 @@ int launch_gemm_umma(const razer_desc* d, const void* packed, const void* x, int
   a.total_items = p.total_items;
   a.x_map_3d = map_3d;
   switch (p.NT) {
-    case 16: return launch_cfg<16, 4, 4, 6, 4, 3, 12, 6>(tmap, tmap_w, a, p.grid, st);
-    case 32: return launch_cfg<32, 4, 4, 6, 4, 3, 12, 2>(tmap, tmap_w, a, p.grid, st);
-    case 64: return launch_cfg<64, 4, 4, 6, 3, 3, 12, 2>(tmap, tmap_w, a, p.grid, st);
-    case 96: return launch_cfg<96, 4, 2, 6, 4, 3, 12, 1>(tmap, tmap_w, a, p.grid, st);
-    case 128: return launch_cfg<128, 4, 1, 6, 6, 3, 12, 1>(tmap, tmap_w, a, p.grid, st);
-    case 192: return launch_cfg<192, 2, 1, 8, 5, 4, 16, 1>(tmap, tmap_w, a, p.grid, st);
-    default: return launch_cfg<256, 2, 1, 8, 4, 4, 16, 1>(tmap, tmap_w, a, p.grid, st);
+    case 16: return launch_cfg<16, 4, 4, 6, 4, 3, 12, 6, true>(tmap, tmap_w, a, p.grid, st);
+    case 32: return launch_cfg<32, 4, 2, 6, 4, 3, 12, 2, true>(tmap, tmap_w, a, p.grid, st);
+    case 64: return launch_cfg<64, 4, 4, 6, 3, 3, 12, 2, false>(tmap, tmap_w, a, p.grid, st);
+    case 96: return launch_cfg<96, 4, 2, 6, 4, 3, 12, 1, false>(tmap, tmap_w, a, p.grid, st);
+    case 128: return launch_cfg<128, 4, 1, 6, 6, 3, 12, 1, false>(tmap, tmap_w, a, p.grid, st);
+    case 192: return launch_cfg<192, 2, 1, 8, 5, 4, 16, 1, false>(tmap, tmap_w, a, p.grid, st);
+    default: return launch_cfg<256, 2, 1, 8, 4, 4, 16, 1, false>(tmap, tmap_w, a, p.grid, st);
   }
 }
 
