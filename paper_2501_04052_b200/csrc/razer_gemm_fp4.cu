@@ -289,9 +289,10 @@ razer_fp4_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_consta
         const bool seg_first = (i == 0) || cur.step == 0;
         const bool seg_last = (i + 1 == n_items) || cur.step == spt - 1;
         const int nch = min(CH, a.g.k_chunks - cur.step * CH);
-        if (!mbar_wait(bar_afull + 8 * cur.as, (uint32_t)cur.aph, abort_flag)) { fail(23); break; }
+        // the activations are there long before the weights are remapped: looked at first, so that it delays nothing
         if (!mbar_wait(bar_xfull + 8 * cur.xs, (uint32_t)cur.xph, abort_flag)) { fail(30); break; }
         if (seg_first && !mbar_wait(bar_accempty, (seg & 1u) ^ 1u, abort_flag)) { fail(24); break; }
+        if (!mbar_wait(bar_afull + 8 * cur.as, (uint32_t)cur.aph, abort_flag)) { fail(23); break; }
         tc_fence_after();
         const uint32_t xs = smem_u32(smem_x) + (uint32_t)cur.xs * C::X_BYTES;
         const uint32_t sfb_s = xs + C::X_CODE_BYTES;

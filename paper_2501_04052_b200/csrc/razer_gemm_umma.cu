@@ -284,8 +284,10 @@ razer_umma_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
         const bool seg_first = (i == 0) || step == 0;
         const bool seg_last = (i + 1 == n_items) || step == spt - 1;
         const int nch = min(CH, a.g.k_chunks - step * CH);
-        if (!mbar_wait(bar_afull + 8 * ar.slot, ar.phase, abort_flag)) { fail(3); break; }
+        // the activations are there long before the weights are decoded: looked at first, so that it delays nothing
+        if (!mbar_wait(bar_xfull + 8 * xr.slot, xr.phase, abort_flag)) { fail(10); break; }
         if (seg_first && !mbar_wait(bar_accempty, (seg & 1u) ^ 1u, abort_flag)) { fail(4); break; }
+        if (!mbar_wait(bar_afull + 8 * ar.slot, ar.phase, abort_flag)) { fail(3); break; }
         tc_fence_after();
         const uint32_t a_t = tmem_a0 + ar.slot * Cfg::A_STAGE_COLS;
         if (seg_first) seg_items = 0;
@@ -296,8 +298,10 @@ razer_umma_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
 #pragma unroll
         for (int h = 0; h < CH / CHX; ++h) {
           if (h * CHX < nch) {
-            if (!mbar_wait(bar_xfull + 8 * xr.slot, xr.phase, abort_flag)) { fail(10); alive = false; break; }
-            tc_fence_after();
+            if (h > 0) {
+              if (!mbar_wait(bar_xfull + 8 * xr.slot, xr.phase, abort_flag)) { fail(10); alive = false; break; }
+              tc_fence_after();
+            }
             const uint32_t bd_lo = ((smem_x + xr.slot * Cfg::X_BYTES) >> 4) | (1u << 16);   // start address and (unused) leading offset fields
 #pragma unroll
             for (int k = 0; k < CHX * 4; ++k) {
@@ -372,6 +376,8 @@ razer_umma_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
     // The group walks its own items only: bookkeeping for the others' cost as much as a third of a decode.
     bool all_closed = n_items == 0;
     step += group;
+    uint32_t turn = 0;                                   // the group's items so far
+    constexpr uint32_t WTURNS = WST / GROUPS, ATURNS = AST / GROUPS;   // stages and slots that serve a group
     for (int i = group;;) {
       const bool crossed = step >= spt && tile < last_tile;   // a segment ends before the group's next item
       if (pending.tile >= 0 && (crossed || i >= n_items || ahead == AST / GROUPS)) {   // (one call: it is large when inlined)
@@ -393,24 +399,23 @@ razer_umma_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
       }
       {
         const int nch = min(CH, a.g.k_chunks - step * CH);
-        const uint32_t wslot = (uint32_t)i % WST, wphase = ((uint32_t)i / WST) & 1u, aslot = (uint32_t)i % AST, aphase = ((uint32_t)i / AST) & 1u;
+        const uint32_t wslot = group + GROUPS * (turn % WTURNS), aslot = group + GROUPS * (turn % ATURNS);
         const uint32_t st = strip_at + wslot * Cfg::W_BYTES;
         const uint32_t a_t = tmem_a0 + aslot * Cfg::A_STAGE_COLS + lane_off;
-        if (!wait_all(bar_wfull + 8 * wslot, wphase, 5)) break;
         // a chunk's scale word and codes
-        auto load = [&](int c, uint32_t& sw, uint2 (&cw)[CHUNK_BLOCKS]) {
-          const uint32_t ck = st + c * PIECE_BYTES;
+        auto load = [&](uint32_t ck, uint32_t& sw, uint2 (&cw)[CHUNK_BLOCKS]) {
           const uint2 sq = lds64(ck + scale_off);           // the eight scale bytes of rows r % 8 and r % 8 + 8
 #pragma unroll
           for (int blk = 0; blk < CHUNK_BLOCKS; ++blk) cw[blk] = lds64(ck + blk * (STRIP_ROWS * 8) + (code_off ^ (32u * blk)));
           sw = __byte_perm(sq.x, sq.y, scale_sel);          // this row's four, in block order
         };
+        if (!wait_all(bar_wfull + 8 * wslot, (turn / WTURNS) & 1u, 5)) break;
         uint32_t sw;
         uint2 cw[CHUNK_BLOCKS];
-        load(0, sw, cw);
+        load(st, sw, cw);
         uint32_t pairs[2][16];
         if (TABLE) lookup_blocks(umma_smem, (sw & 0x80808080u) | lanes, 0, cw, pairs[0]);
-        if (!wait_all(bar_aempty + 8 * aslot, aphase ^ 1u, 6)) break;
+        if (!wait_all(bar_aempty + 8 * aslot, ((turn / ATURNS) & 1u) ^ 1u, 6)) break;
         tc_fence_after();
         if constexpr (TABLE) {
           // half a chunk's lookups are on their way while the half before is scaled and put in order
@@ -421,7 +426,7 @@ razer_umma_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
 #pragma unroll
               for (int blk = 0; blk < CHUNK_BLOCKS; ++blk) ss2[blk] = decode_block_scale(ss_lane, sw, blk);
               lookup_blocks(umma_smem, (sw & 0x80808080u) | lanes, 2, cw, pairs[1]);
-              if (c + 1 < CH) load(c + 1, sw, cw);          // beyond the last chunk, or past the end of K: unused or zeros
+              if (c + 1 < CH) load(st + (c + 1) * PIECE_BYTES, sw, cw);   // beyond the last chunk, or past the end of K: unused or zeros
               finish_blocks(pairs[0], ss2[0], ss2[1], v);
               if (c + 1 < CH) lookup_blocks(umma_smem, (sw & 0x80808080u) | lanes, 0, cw, pairs[0]);
               finish_blocks(pairs[1], ss2[2], ss2[3], v + 16);
@@ -438,7 +443,7 @@ razer_umma_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
               // the next chunk is fetched while this one is decoded (beyond the last one, or past the end of K: unused or zeros)
               uint32_t sw_next = 0;
               uint2 cw_next[CHUNK_BLOCKS];
-              if (c + 1 < CH) load(c + 1, sw_next, cw_next);
+              if (c + 1 < CH) load(st + (c + 1) * PIECE_BYTES, sw_next, cw_next);
               // (One store for the chunk lets the four blocks' decodes mix.)
               uint32_t v[8 * CHUNK_BLOCKS];
 #pragma unroll
@@ -458,12 +463,13 @@ razer_umma_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
         }
         __syncwarp();                                       // every lane has read the stage
         if (lane == 0) mbar_arrive(bar_wempty + 8 * wslot);
+        ++ahead;
+        ++turn;
+        i += GROUPS;
+        step += GROUPS;
         tc_wait_st();
         tc_fence_before();
         mbar_arrive(bar_afull + 8 * aslot);
-        ++ahead;
-        i += GROUPS;
-        step += GROUPS;
       }
     }
   }
