@@ -8,6 +8,7 @@ library and raises if it has not been built (python -m paper_2501_04052_b200.bui
 from __future__ import annotations
 
 import ctypes
+import importlib.util
 import os
 from ctypes import POINTER, c_char_p, c_float, c_int, c_int32, c_size_t, c_void_p
 
@@ -102,6 +103,22 @@ else:
         return torch.cuda.current_stream().cuda_stream
 
 
+# The compiled way of a plain matmul call (csrc/razer_call.cpp); without it everything goes through ctypes.
+def _load_call():
+    path = os.path.join(_HERE, "razer_call.so")
+    try:
+        spec = importlib.util.spec_from_file_location("razer_call", path)
+        module = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(module)
+        return module
+    except (ImportError, OSError):                       # not built, or for another torch or interpreter
+        return None
+
+
+_call = _load_call()
+_GEMV, _GEMM, _GEMV_HOST = (ctypes.cast(f, c_void_p).value for f in (_lib.razer_gemv, _lib.razer_gemm, _lib.razer_gemv_host))
+
+
 def _ptr(t) -> int:
     return 0 if t is None else t.data_ptr()
 
@@ -186,11 +203,23 @@ def _matmul(fn, desc, packed, x, y, workspace, op):
 
 def razer_gemv(desc, packed, x, y=None, workspace=None) -> torch.Tensor:
     """x bf16 [M, K] (M <= 64, device) -> y bf16 [M, N]."""
+    if _call is not None:
+        rc = _call.matmul(_GEMV, RazerDesc, desc, packed, x, y, workspace)
+        if rc == 0:
+            return y
+        if rc is not None:
+            _check(rc)
     return _matmul(_lib.razer_gemv, desc, packed, x, y, workspace, OP_GEMV)
 
 
 def razer_gemm(desc, packed, x, y=None, workspace=None) -> torch.Tensor:
     """x bf16 [M, K] (device) -> y bf16 [M, N]."""
+    if _call is not None:
+        rc = _call.matmul(_GEMM, RazerDesc, desc, packed, x, y, workspace)
+        if rc == 0:
+            return y
+        if rc is not None:
+            _check(rc)
     return _matmul(_lib.razer_gemm, desc, packed, x, y, workspace, OP_GEMM)
 
 
@@ -205,6 +234,10 @@ def razer_gemv_static(desc, packed, x, y) -> torch.Tensor:
 
 def razer_gemv_host(desc, packed, x_host, y_host, x_stage, y_stage, workspace) -> None:
     """x_host / y_host: pinned CPU bf16 tensors; x_stage / y_stage / workspace: device buffers."""
+    if _call is not None:
+        rc = _call.gemv_host(_GEMV_HOST, RazerDesc, desc, packed, x_host, y_host, x_stage, y_stage, workspace)
+        if rc is not None:
+            return _check(rc)
     assert not x_host.is_cuda and not y_host.is_cuda
     M = x_host.shape[0]
     _check(_lib.razer_gemv_host(ctypes.byref(desc), _ptr(packed), _ptr(x_host), M, _ptr(y_host), _ptr(x_stage),

@@ -521,11 +521,10 @@ static bool admissible(const TileCost& t, const Fp4ActLayout& act) {
   return act.force_nt ? t.NT == act.force_nt : t.NT <= act.tiles128 * 128;
 }
 
-static Plan make_plan(const razer_desc* d, int M) {
+static Plan work_out_plan(const razer_desc* d, int M, const Fp4ActLayout& act) {
   Plan best;
   float best_cost = 0.0f;
   const Geometry g = make_geometry(d->N, d->K);
-  const Fp4ActLayout act = make_fp4_act_layout(M, d->K);
   for (const TileCost& t : tile_costs) {
     if (!admissible(t, act)) continue;
     Plan p;
@@ -539,6 +538,11 @@ static Plan make_plan(const razer_desc* d, int M) {
   }
   best.slots_bytes = (size_t)best.grid * best.NT * TILE_ROWS * sizeof(float);
   return best;
+}
+
+static Plan make_plan(const razer_desc* d, int M) {
+  const Fp4ActLayout act = make_fp4_act_layout(M, d->K);
+  return remembered<Plan>(d->N, d->K, M, act.force_nt, [&] { return work_out_plan(d, M, act); });
 }
 
 // FP4 magnitude code (0 .5 1 1.5 2 3 4 6 -> 0..7) of v, or -1.

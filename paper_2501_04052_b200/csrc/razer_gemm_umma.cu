@@ -504,7 +504,7 @@ static const TileCost tile_costs[] = {
 
 static bool admissible(const TileCost& t, int M) { return t.NT <= 16 || t.NT < 2 * M; }   // not half of the tile or more padding
 
-static UmmaPlan make_plan(const razer_desc* d, int M) {
+static UmmaPlan work_out_plan(const razer_desc* d, int M) {
   UmmaPlan best;
   float best_cost = 0.0f;
   const Geometry g = make_geometry(d->N, d->K);
@@ -523,6 +523,10 @@ static UmmaPlan make_plan(const razer_desc* d, int M) {
   }
   best.slots_bytes = (size_t)best.grid * best.NT * TILE_ROWS * sizeof(float);
   return best;
+}
+
+static UmmaPlan make_plan(const razer_desc* d, int M) {
+  return remembered<UmmaPlan>(d->N, d->K, M, 0, [&] { return work_out_plan(d, M); });
 }
 
 bool umma_supported(const razer_desc* d, int M) {

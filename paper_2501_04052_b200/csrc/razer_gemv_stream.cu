@@ -321,13 +321,17 @@ __global__ void __launch_bounds__(THREADS, 1) razer_stream_kernel(const Args a) 
 
 }  // namespace stream_path
 
+static StreamPlan remembered_plan(const razer_desc* d, int M) {
+  return remembered<StreamPlan>(d->N, d->K, M, 0, [&] { return stream_plan(d, M); });
+}
+
 bool gemv_stream_supported(const razer_desc* d, int M) {
   (void)d;
   return M >= 1 && M <= stream_path::MAX_M;
 }
 
 size_t gemv_stream_workspace_bytes(const razer_desc* d, int M) {
-  const StreamPlan p = stream_plan(d, M);
+  const StreamPlan p = remembered_plan(d, M);
   return WS_ZERO_BYTES + p.slots_bytes;
 }
 
@@ -345,7 +349,7 @@ static int launch_stream_cfg(const stream_path::Args& a, int grid, cudaStream_t 
 
 int launch_gemv_stream(const razer_desc* d, const void* packed, const void* x, int M, float extra_scale,
                        const float* extra_scale_dev, void* y, void* ws, size_t ws_bytes, cudaStream_t st, uint32_t* status_host) {
-  const StreamPlan p = stream_plan(d, M);
+  const StreamPlan p = remembered_plan(d, M);
   const size_t need = WS_ZERO_BYTES + p.slots_bytes;
   if (!ws || ws_bytes < need)
     return set_error(RAZER_ERR_WORKSPACE, "workspace of %zu bytes needed, %zu given", need, ws_bytes);

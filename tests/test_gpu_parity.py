@@ -117,6 +117,44 @@ def test_gemv_ragged_shapes_random_codes(b, M):
     _check_matmul(b, b.razer_gemv, desc, packed, codes, scales, 0.004, x)
 
 
+@pytest.mark.parametrize("compiled", [True, False])
+def test_both_ways_into_the_library(b, monkeypatch, compiled):
+    """The compiled part of the binding and ctypes: the same results, and what one refuses the other refuses in the same way."""
+    if compiled:
+        assert b._call is not None
+    else:
+        monkeypatch.setattr(b, "_call", None)
+    N, K = 300, 528
+    codes, scales = inputs.random_codes(N, K, seed=5)
+    desc, packed = _pack(b, codes.numpy(), scales.numpy(), 0.01)
+    for M, fn, op in ((3, b.razer_gemv, b.OP_GEMV), (20, b.razer_gemv, b.OP_GEMV), (70, b.razer_gemm, b.OP_GEMM)):
+        x, ws = inputs.activations(M, K, M).cuda(), b.alloc_workspace(desc, M, op, "cuda")
+        y = torch.empty((M, N), dtype=torch.bfloat16, device="cuda")
+        assert fn(desc, packed, x, y, ws) is y
+        assert torch.equal(y, fn(desc, packed, x))                                        # buffers allocated by the binding
+        assert torch.equal(y, fn(desc, packed, torch.nn.Parameter(x, requires_grad=False), workspace=ws))
+        with torch.cuda.stream(torch.cuda.Stream()):
+            other = fn(desc, packed, x, torch.empty_like(y), ws)
+            torch.cuda.current_stream().synchronize()
+        assert torch.equal(y, other)
+        for bad in (x.float(), x[:, :-16], x.t().contiguous().t(), x.cpu()):
+            with pytest.raises(AssertionError):
+                fn(desc, packed, bad, y, ws)
+        with pytest.raises(IndexError):
+            fn(desc, packed, x.reshape(-1), y, ws)
+        for args, code in (((desc, packed, x, y, ws[:256]), b.ERR_WORKSPACE), ((desc, None, x, y, ws), b.ERR_INVALID_ARG),
+                           ((b.make_desc(N, K, -1.0), packed, x, y, ws), b.ERR_INVALID_ARG)):
+            with pytest.raises(b.RazerError) as e:
+                fn(*args)
+            assert e.value.code == code
+    xh, yh = inputs.activations(2, K, 9).pin_memory(), torch.empty((2, N), dtype=torch.bfloat16).pin_memory()
+    xd, yd, ws = torch.empty((2, K), dtype=torch.bfloat16, device="cuda"), torch.empty((2, N), dtype=torch.bfloat16, device="cuda"), b.alloc_workspace(desc, 2, b.OP_GEMV, "cuda")
+    b.razer_gemv_host(desc, packed, xh, yh, xd, yd, ws)
+    assert torch.equal(yh, b.razer_gemv(desc, packed, xh.cuda()).cpu())
+    with pytest.raises(AssertionError):
+        b.razer_gemv_host(desc, packed, xh.cuda(), yh, xd, yd, ws)
+
+
 def test_activations_with_trailing_axes_of_one(b):
     """x's first two axes are its rows and columns; further ones of length one (a view of a caller's layout) change nothing."""
     codes, scales = inputs.random_codes(300, 528, seed=33)
