@@ -83,8 +83,8 @@ __device__ __forceinline__ void decode_word(uint32_t w, uint32_t ss2, uint32_t s
 // The same pairs by table: [weight byte][special value][lane], two elements (value x 2^-126) to an entry, a copy per lane so that 32
 // random lookups never meet on a bank.  A pair costs a byte permute (which forms the address), a load and the multiply by the
 // scale; another permute each puts the pairs back in order, since a byte of a code word holds elements 0, 2 / 4, 6 / 1, 3 / 5, 7.
-// On B200 a packed bf16 operation takes two issue slots (one alternating with a logic operation measured 3.3 cycles for the pair),
-// so a word is 29 slots in registers and 20 this way.
+// Eight weights are 21 instructions in registers and 16 this way; in the tcgen05 kernel at 16 tokens 1032 warp instructions a chunk,
+// everything included, became 856.
 constexpr int PAIR_TABLE_BYTES = 65536;
 __device__ __forceinline__ void pair_table_fill(uint32_t base, int tid, int nthreads, uint32_t svp0, uint32_t svp1) {
 #pragma unroll 1

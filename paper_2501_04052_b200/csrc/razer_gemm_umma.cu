@@ -18,7 +18,7 @@
 // meet the activations' in shared memory (64 x 8192 x 28672 45.3 us in registers, 49.7 by table, 48 half and half).
 //
 // What bounds it: up to 32 tokens shared memory (270 wavefronts a chunk of about 305 cycles, copies and MMAs counted from the layout)
-// and issue (246 of 305 slots), then the decode (about 3.4 instructions a weight) up to 128 tokens, from there on the MMAs (512 cycles
+// and issue (214 of 305 slots), then the decode (about 3.4 instructions a weight) up to 128 tokens, from there on the MMAs (512 cycles
 // per 128 x 256 x 64) together with shared-memory bandwidth (571 cycles), and the combination of cut tiles.  Device times on B200, first for one
 // ring of weights and activations and items of one chunk at 256 tokens, then for rings apart, two-chunk items and groups that
 // walk only their own items: 2048 x 14336 x 4096 204 -> 171 us (149 with the decode left out), 256 x 8192 x 8192 38.4 -> 32.7,
