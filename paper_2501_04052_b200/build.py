@@ -24,42 +24,61 @@ NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", 
               "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr"]
 
 
-def _deps():
-    out = [os.path.join(CSRC, f) for f in os.listdir(CSRC)]
-    out.append(os.path.join(os.path.dirname(HERE), "include", "razer.h"))
-    return out
+HEADER = os.path.join(os.path.dirname(HERE), "include", "razer.h")
+CALL_SOURCE = os.path.join(CSRC, "razer_call.cpp")
+
+
+def _newer(target: str, deps) -> bool:
+    """`target` exists and none of `deps` is newer."""
+    return os.path.exists(target) and all(os.path.getmtime(p) <= os.path.getmtime(target) for p in deps)
 
 
 def needs_build() -> bool:
-    if not os.path.exists(LIB) or not os.path.exists(CALL):
-        return True
-    t = os.path.getmtime(LIB)
-    return any(os.path.getmtime(p) > t for p in _deps())
+    """The library: its own sources only, whatever became of the binding's compiled part."""
+    return not _newer(LIB, [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith((".cu", ".cuh"))] + [HEADER])
+
+
+def needs_call() -> bool:
+    """The compiled part: neither built nor, since its sources last changed, found impossible to build."""
+    return not any(_newer(p, [CALL_SOURCE, HEADER]) for p in (CALL, CALL + ".failed"))
+
+
+def _run(cmd) -> tuple[bool, str]:
+    try:
+        r = subprocess.run(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)
+        return r.returncode == 0, r.stdout
+    except OSError as e:
+        return False, str(e)
 
 
 def build_call(verbose: bool = False) -> None:
-    import torch
-    root = os.path.dirname(torch.__file__)
-    inc = [os.path.join(root, "include"), os.path.join(root, "include", "torch", "csrc", "api", "include"), sysconfig.get_paths()["include"],
-           os.path.join(os.path.dirname(os.path.dirname(os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc"))), "include")]
-    lib = os.path.join(root, "lib")
-    cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
-           *("-I" + d for d in inc), os.path.join(CSRC, "razer_call.cpp"), "-o", CALL, "-L" + lib, "-lc10", "-lc10_cuda", "-ltorch_cpu",
-           "-ltorch_python", "-Wl,-rpath," + lib]
+    """Never fails: without razer_call.so the binding goes through ctypes.  What an older build left is gone either way."""
+    for p in (CALL, CALL + ".failed"):
+        if os.path.exists(p):
+            os.remove(p)
     try:
-        r = subprocess.run(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)
-        failed, out = r.returncode != 0, r.stdout
-    except OSError as e:
-        failed, out = True, str(e)
-    if failed or verbose:
+        import torch
+        root = os.path.dirname(torch.__file__)
+        inc = [os.path.join(root, "include"), os.path.join(root, "include", "torch", "csrc", "api", "include"), sysconfig.get_paths()["include"],
+               os.path.join(os.path.dirname(os.path.dirname(os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc"))), "include")]
+        lib = os.path.join(root, "lib")
+        ok, out = _run([os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared",
+                        f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}", *("-I" + d for d in inc), CALL_SOURCE, "-o", CALL + ".tmp",
+                        "-L" + lib, "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python", "-Wl,-rpath," + lib])
+    except Exception as e:                               # no torch, or one that does not load
+        ok, out = False, repr(e)
+    if ok:
+        os.replace(CALL + ".tmp", CALL)
+    else:
+        with open(CALL + ".failed", "w") as f:
+            f.write(out)
+    if not ok or verbose:
         sys.stderr.write(f"--- razer_call.cpp\n{out}\n")
-    if failed:
-        sys.stderr.write("razer_call.so was not built: the binding will go through ctypes\n")
+    if not ok:
+        sys.stderr.write("razer_call.so was not built: the binding will go through ctypes (--force tries again)\n")
 
 
-def build(force: bool = False, verbose: bool = False) -> str:
-    if not force and not needs_build():
-        return LIB
+def build_lib(verbose: bool = False) -> None:
     nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
     objs = []
     procs = []
@@ -79,9 +98,16 @@ def build(force: bool = False, verbose: bool = False) -> str:
         failed |= p.returncode != 0
     if failed:
         raise RuntimeError("nvcc failed")
-    cmd = [nvcc, "-shared", "-o", LIB, *objs, "-gencode", "arch=compute_100a,code=sm_100a"]
-    build_call(verbose)
-    subprocess.run(cmd, check=True)
+    # beside it and then in its place: a process that has the library mapped keeps what it mapped
+    subprocess.run([nvcc, "-shared", "-o", LIB + ".tmp", *objs, "-gencode", "arch=compute_100a,code=sm_100a"], check=True)
+    os.replace(LIB + ".tmp", LIB)
+
+
+def build(force: bool = False, verbose: bool = False) -> str:
+    if force or needs_build():
+        build_lib(verbose)
+    if force or needs_call():
+        build_call(verbose)
     return LIB
 
 
