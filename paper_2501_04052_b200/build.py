@@ -35,7 +35,7 @@ def _newer(target: str, deps) -> bool:
 
 def needs_build() -> bool:
     """The library: its own sources only, whatever became of the binding's compiled part."""
-    return not _newer(LIB, [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith((".cu", ".cuh"))] + [HEADER])
+    return not _newer(LIB, [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith((".cu", ".cuh", ".h"))] + [HEADER])
 
 
 def needs_call() -> bool:

@@ -10,6 +10,7 @@
 #include <utility>
 
 #include "../../include/razer.h"
+#include "razer_plan_cache.h"
 
 namespace razer {
 
@@ -207,20 +208,6 @@ __device__ __forceinline__ uint32_t to_packed_order(uint32_t w) {
   const uint32_t s4 = w >> 4, s8 = w >> 8;
   // bytes 0 and 2 of the two words: elements 0, 2 and 4, 6; elements 1, 3 and 5, 7
   return __byte_perm((w & LOW) | (s4 & ~LOW), (s4 & LOW) | (s8 & ~LOW), 0x6420);
-}
-
-// The plan of a call, a pure function of its sizes (and of `variant`), remembered by the calling thread: working one out takes 0.5 to 1 us
-// of the host's time.  32 places, a size takes another's where they meet.
-template <class Plan, class Make>
-inline Plan remembered(int N, int K, int M, int variant, Make make) {
-  struct Entry { int N, K, M, variant; Plan plan; };
-  static thread_local Entry table[32];                    // N = 0: empty
-  Entry& e = table[((unsigned)N * 0x9E3779B1u ^ (unsigned)K * 0x85EBCA77u ^ (unsigned)M * 0xC2B2AE3Du) >> 27];
-  if (e.N != N || e.K != K || e.M != M || e.variant != variant) {
-    e.plan = make();
-    e.N = N, e.K = K, e.M = M, e.variant = variant;
-  }
-  return e.plan;
 }
 
 // A launch that may begin while the preceding kernel of the stream drains (programmatic dependent launch; RAZER_PDL=0 in the
