@@ -673,11 +673,131 @@ __device__ __forceinline__ void load8(const float4* p, float* v, bool wide) {
   }
 }
 
-// One thread per scale block of `sub` groups of 16 elements (ONE: sub == 1, the block stays in registers from its maximum
-// to its codes; larger blocks are walked three times).  A magnitude beyond 6 can win an element only where the block's
-// scaled maximum passes halfway between 6 and it, so a warp in which no block does skips its two candidates: their sums
-// would equal those without a special value.  The grid runs from the end of the tensor to its start, the reverse of the
-// maximum's order, so that the part of the input still in L2 is read first.
+// One thread's scale block of `sub` groups of 16 elements (ONE: sub == 1, the block stays in registers from its maximum
+// to its codes; larger blocks are walked three times); called by whole warps, `inside`: this thread has a block.  A magnitude beyond 6 can
+// win an element only where the block's scaled maximum passes halfway between 6 and it, so a warp in which no block does skips its two
+// candidates: their sums would equal those without a special value.
+template <bool AWARE, bool ONE>
+__device__ __forceinline__ void quant_weight_block(const float4* __restrict__ src, bool inside, int sub_arg, bool wide, float d32, float m0, float m1,
+                                                   uint32_t remap_code, uint2* __restrict__ codes, uint8_t* __restrict__ scale) {
+  const int sub = ONE ? 1 : sub_arg;
+  const uint32_t other_zero = remap_code ^ 8u;
+  const float d32x6 = __fmul_rn(d32, 6.0f);
+  float xv[16];
+  auto load = [&](int g) {
+#pragma unroll
+    for (int q = 0; q < 2; ++q) load8(src + 4 * g + 2 * q, xv + 8 * q, wide);
+  };
+  uint32_t mbits = 0;
+#pragma unroll 1
+  for (int g = 0; g < sub; ++g) {
+    load(g);
+#pragma unroll
+    for (int j = 0; j < 16; ++j) mbits = max(mbits, __float_as_uint(xv[j]) & 0x7FFFFFFFu);
+  }
+  const float bmax = __uint_as_float(mbits);
+  uint32_t scode = round_to_e4m3(__fdiv_rn(bmax, d32x6), 63u);       // Eq. 2
+  if (scode == 0) scode = 1;                                         // keep a non-empty block alive
+  float denom = __fmul_rn(d32, scale_value(scode));
+  bool fast = inside && mbits > 0 && mbits < 0x7F800000u && short_form(bmax, denom);
+  float own_denom[2] = {1.0f, 1.0f};
+  uint32_t own_scode[2] = {1u, 1u};
+  uint32_t top_neg = 0;
+  if (AWARE) {
+    bool found = false;                                              // sign of the first largest element
+#pragma unroll 1
+    for (int g = 0; g < sub; ++g) {
+      if (!ONE) load(g);
+#pragma unroll
+      for (int j = 0; j < 16; ++j) {
+        const bool is_top = !found && (__float_as_uint(xv[j]) & 0x7FFFFFFFu) == mbits;
+        if (is_top) { top_neg = __float_as_uint(xv[j]) >> 31; found = true; }
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      const float m = i ? m1 : m0;
+      uint32_t sc = round_to_e4m3(__fdiv_rn(bmax, __fmul_rn(d32, m)), 63u);
+      if (sc == 0) sc = 1;
+      own_scode[i] = sc;
+      own_denom[i] = __fmul_rn(d32, scale_value(sc));
+      fast = fast && short_form(bmax, own_denom[i]);
+    }
+  }
+  const float y = __frcp_rn(denom);
+  const float xmax = __fmul_rn(bmax, y) * 2.001f;
+  const bool on0 = __any_sync(0xFFFFFFFFu, fast && (m0 < 6.0f || xmax > 6.0f + m0));
+  const bool on1 = __any_sync(0xFFFFFFFFu, fast && (m1 < 6.0f || xmax > 6.0f + m1));
+  if (!inside) return;
+  if (!fast) {
+    if (mbits == 0) {
+      for (int g = 0; g < sub; ++g) codes[g] = make_uint2(other_zero * 0x11111111u, other_zero * 0x11111111u);
+      *scale = 0;
+    } else {
+      *scale = (uint8_t)quant_weight_block_plain<AWARE>(src, sub, d32, m0, m1, remap_code, codes);
+    }
+    return;
+  }
+  float e_base = 0.0f;
+  F2 e2[2] = {f2(0.0f, 0.0f), f2(0.0f, 0.0f)};
+  uint32_t take[2][2] = {{0, 0}, {0, 0}};
+  constexpr bool KEEP = ONE && !AWARE;
+#pragma unroll 1
+  for (int g = 0; g < sub; ++g) {
+    if (!ONE) load(g);
+    if (on0 && on1) weight_errors<true, true, KEEP>(xv, denom, y, m0, m1, e_base, e2, take);
+    else if (on0) weight_errors<true, false, KEEP>(xv, denom, y, m0, m1, e_base, e2, take);
+    else if (on1) weight_errors<false, true, KEEP>(xv, denom, y, m0, m1, e_base, e2, take);
+    else weight_errors<false, false, KEEP>(xv, denom, y, m0, m1, e_base, e2, take);
+  }
+  float e[4];                                                        // metadata order: +m0, +m1, -m0, -m1
+  split(e2[0], e[0], e[2]);
+  split(e2[1], e[1], e[3]);
+  if (!on0) e[0] = e[2] = e_base;
+  if (!on1) e[1] = e[3] = e_base;
+  if (AWARE) {
+#pragma unroll
+    for (int c = 0; c < 4; ++c) e[c] = __fmul_rn(__fmul_rn(denom, denom), e[c]);
+  }
+  uint32_t meta = 0;                                                 // first minimum: ties keep the earlier candidate
+  float best = e[0];
+#pragma unroll
+  for (int c = 1; c < 4; ++c)
+    if (e[c] < best) { best = e[c]; meta = c; }
+  float y_win = y;
+  if (AWARE) {
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      const float m = i ? m1 : m0;
+      if (m > 6.0f) {
+        const float d = own_denom[i], yo = __frcp_rn(d);
+        float eo = 0.0f;
+#pragma unroll 1
+        for (int g = 0; g < sub; ++g) {
+          if (!ONE) load(g);
+          eo = weight_error_one(xv, d, yo, m, top_neg, eo);
+        }
+        eo = __fmul_rn(__fmul_rn(d, d), eo);
+        if (eo < best) { best = eo; meta = top_neg * 2u + (uint32_t)i; scode = own_scode[i]; denom = d; y_win = yo; }
+      }
+    }
+  }
+  const float m_win = (meta & 1u) ? m1 : m0;
+#pragma unroll 1
+  for (int g = 0; g < sub; ++g) {
+    if (!ONE) load(g);
+    if (KEEP) {
+      const uint32_t won[2] = {(meta & 1u) ? take[1][0] : take[0][0], (meta & 1u) ? take[1][1] : take[0][1]};
+      *codes = codes_of_scaled(xv, won, meta >> 1, remap_code);
+    } else {
+      codes[g] = weight_codes(xv, denom, y_win, m_win, meta >> 1, remap_code);
+    }
+  }
+  *scale = (uint8_t)((meta << 6) | scode);
+}
+
+// The grid runs from the end of the tensor to its start, the reverse of the maximum's order, so that the part of the input still in L2 is
+// read first.
 template <bool AWARE, bool ONE>
 __global__ void __launch_bounds__(256, 4) quant_weight_kernel(const float4* __restrict__ w, long long n_blocks, int sub_arg, float m0, float m1,
                                                           uint32_t remap_code, const float* __restrict__ scale_in,
@@ -693,165 +813,18 @@ __global__ void __launch_bounds__(256, 4) quant_weight_kernel(const float4* __re
     d32 = (amax == 0.0f) ? 1.0f : __fdiv_rn(amax, __fmul_rn(1.875f, 6.0f));   // Eq. 1
   }
   if (blockIdx.x == 0 && threadIdx.x == 0) *scale_out = d32;
-  const uint32_t other_zero = remap_code ^ 8u;
-  const float d32x6 = __fmul_rn(d32, 6.0f);
   const long long stride = (long long)gridDim.x * blockDim.x;
   const long long turns = (n_blocks + stride - 1) / stride;
   for (long long turn = turns - 1; turn >= 0; --turn) {
     const long long t = turn * stride + (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const bool inside = t < n_blocks;
-    const float4* src = w + 4 * (inside ? t : 0) * sub;
-    float xv[16];
-    auto load = [&](int g) {
-#pragma unroll
-      for (int q = 0; q < 2; ++q) load8(src + 4 * g + 2 * q, xv + 8 * q, wide);
-    };
-    uint32_t mbits = 0;
-#pragma unroll 1
-    for (int g = 0; g < sub; ++g) {
-      load(g);
-#pragma unroll
-      for (int j = 0; j < 16; ++j) mbits = max(mbits, __float_as_uint(xv[j]) & 0x7FFFFFFFu);
-    }
-    const float bmax = __uint_as_float(mbits);
-    uint32_t scode = round_to_e4m3(__fdiv_rn(bmax, d32x6), 63u);       // Eq. 2
-    if (scode == 0) scode = 1;                                         // keep a non-empty block alive
-    float denom = __fmul_rn(d32, scale_value(scode));
-    bool fast = inside && mbits > 0 && mbits < 0x7F800000u && short_form(bmax, denom);
-    float own_denom[2] = {1.0f, 1.0f};
-    uint32_t own_scode[2] = {1u, 1u};
-    uint32_t top_neg = 0;
-    if (AWARE) {
-      bool found = false;                                              // sign of the first largest element
-#pragma unroll 1
-      for (int g = 0; g < sub; ++g) {
-        if (!ONE) load(g);
-#pragma unroll
-        for (int j = 0; j < 16; ++j) {
-          const bool is_top = !found && (__float_as_uint(xv[j]) & 0x7FFFFFFFu) == mbits;
-          if (is_top) { top_neg = __float_as_uint(xv[j]) >> 31; found = true; }
-        }
-      }
-#pragma unroll
-      for (int i = 0; i < 2; ++i) {
-        const float m = i ? m1 : m0;
-        uint32_t sc = round_to_e4m3(__fdiv_rn(bmax, __fmul_rn(d32, m)), 63u);
-        if (sc == 0) sc = 1;
-        own_scode[i] = sc;
-        own_denom[i] = __fmul_rn(d32, scale_value(sc));
-        fast = fast && short_form(bmax, own_denom[i]);
-      }
-    }
-    const float y = __frcp_rn(denom);
-    const float xmax = __fmul_rn(bmax, y) * 2.001f;
-    const bool on0 = __any_sync(0xFFFFFFFFu, fast && (m0 < 6.0f || xmax > 6.0f + m0));
-    const bool on1 = __any_sync(0xFFFFFFFFu, fast && (m1 < 6.0f || xmax > 6.0f + m1));
-    if (!inside) continue;
-    if (!fast) {
-      if (mbits == 0) {
-        for (int g = 0; g < sub; ++g) codes[t * sub + g] = make_uint2(other_zero * 0x11111111u, other_zero * 0x11111111u);
-        scales[t] = 0;
-      } else {
-        scales[t] = (uint8_t)quant_weight_block_plain<AWARE>(src, sub, d32, m0, m1, remap_code, codes + t * sub);
-      }
-      continue;
-    }
-    float e_base = 0.0f;
-    F2 e2[2] = {f2(0.0f, 0.0f), f2(0.0f, 0.0f)};
-    uint32_t take[2][2] = {{0, 0}, {0, 0}};
-    constexpr bool KEEP = ONE && !AWARE;
-#pragma unroll 1
-    for (int g = 0; g < sub; ++g) {
-      if (!ONE) load(g);
-      if (on0 && on1) weight_errors<true, true, KEEP>(xv, denom, y, m0, m1, e_base, e2, take);
-      else if (on0) weight_errors<true, false, KEEP>(xv, denom, y, m0, m1, e_base, e2, take);
-      else if (on1) weight_errors<false, true, KEEP>(xv, denom, y, m0, m1, e_base, e2, take);
-      else weight_errors<false, false, KEEP>(xv, denom, y, m0, m1, e_base, e2, take);
-    }
-    float e[4];                                                        // metadata order: +m0, +m1, -m0, -m1
-    split(e2[0], e[0], e[2]);
-    split(e2[1], e[1], e[3]);
-    if (!on0) e[0] = e[2] = e_base;
-    if (!on1) e[1] = e[3] = e_base;
-    if (AWARE) {
-#pragma unroll
-      for (int c = 0; c < 4; ++c) e[c] = __fmul_rn(__fmul_rn(denom, denom), e[c]);
-    }
-    uint32_t meta = 0;                                                 // first minimum: ties keep the earlier candidate
-    float best = e[0];
-#pragma unroll
-    for (int c = 1; c < 4; ++c)
-      if (e[c] < best) { best = e[c]; meta = c; }
-    float y_win = y;
-    if (AWARE) {
-#pragma unroll
-      for (int i = 0; i < 2; ++i) {
-        const float m = i ? m1 : m0;
-        if (m > 6.0f) {
-          const float d = own_denom[i], yo = __frcp_rn(d);
-          float eo = 0.0f;
-#pragma unroll 1
-          for (int g = 0; g < sub; ++g) {
-            if (!ONE) load(g);
-            eo = weight_error_one(xv, d, yo, m, top_neg, eo);
-          }
-          eo = __fmul_rn(__fmul_rn(d, d), eo);
-          if (eo < best) { best = eo; meta = top_neg * 2u + (uint32_t)i; scode = own_scode[i]; denom = d; y_win = yo; }
-        }
-      }
-    }
-    const float m_win = (meta & 1u) ? m1 : m0;
-#pragma unroll 1
-    for (int g = 0; g < sub; ++g) {
-      if (!ONE) load(g);
-      if (KEEP) {
-        const uint32_t won[2] = {(meta & 1u) ? take[1][0] : take[0][0], (meta & 1u) ? take[1][1] : take[0][1]};
-        codes[t] = codes_of_scaled(xv, won, meta >> 1, remap_code);
-      } else {
-        codes[t * sub + g] = weight_codes(xv, denom, y_win, m_win, meta >> 1, remap_code);
-      }
-    }
-    scales[t] = (uint8_t)((meta << 6) | scode);
+    const long long at = inside ? t : 0;
+    quant_weight_block<AWARE, ONE>(w + 4 * at * sub, inside, sub, wide, d32, m0, m1, remap_code, codes + at * sub, scales + at);
   }
 }
 
-// The same result for the usual magnitudes (m0 halfway between two FP4 values, m1 beyond 6) by gains instead of error sums: what a
-// special value m takes off a block's error is a sum over the elements that take it, and those lie in one interval, of
-// half-width WT around m0 or beyond LO1 = (6 + m1) / 2; an element at distance -t inside it gains K t.  That needs neither the rounded
-// value nor the squares, so a thread's 16 elements cost half the instructions.  The decision is that of the FP32 sums in
-// ascending order unless two candidates come within `delta`, more than all roundings of both ways together; then (one block in some
-// thousands) the sums are taken as they are defined.  t is exact wherever its sign matters (a within a factor of two of m0, v0, v1
-// or m1), so the elements that take the special value are the same ones.
-// SUB lanes share a block of 16 * SUB elements, so every block size reads its tensor once and alike.
-// Bound by instruction issue still (360 a thread and turn, 69 % of the slots; 180 MB in 45 us).  11008 x 4096 at a given scale, us with
-// the launch, quant_weight_kernel above / this: blocks of 16 67.6 / 49.2, 32 92.2 / 53.2, 64 98.3 / 57.3, 128 102.4 / 63.5.  80
-// registers and the next turn's loads ahead came out level, 48 registers likewise.
-// The winning candidate of one block by the sums themselves, one element at a time (few registers: it is needed once in thousands).
-__device__ __forceinline__ uint32_t choice_by_sums(const float* __restrict__ src, int n, float2 step, float m0, float m1) {
-  float e[4] = {0.0f, 0.0f, 0.0f, 0.0f};                               // metadata order: +m0, +m1, -m0, -m1
-#pragma unroll 1
-  for (int j = 0; j < n; ++j) {                                        // ascending element order, no fusion
-    const float x = src[j];
-    float q = __fmul_rn(x, step.y);
-    q = __fmaf_rn(__fmaf_rn(q, -step.x, x), step.y, q);
-    q = __fmaf_rn(__fmaf_rn(q, -step.x, x), step.y, q);                // the scaled element of Eq. 6, as div_f32 has it
-    const float a = fabsf(q), c = __uint_as_float((max(__float_as_uint(a), 0x3F800000u) & 0x7F800000u) + (22u << 23));
-    const float d_r = __fsub_rn(a, fminf(__fsub_rn(__fadd_rn(a, c), c), 6.0f)), s0 = __fsub_rn(a, m0), s1 = __fsub_rn(a, m1);
-    const float d0 = fabsf(s0) < fabsf(d_r) ? s0 : d_r, d1 = fabsf(s1) < fabsf(d_r) ? s1 : d_r;
-    const float q_r = __fmul_rn(d_r, d_r), q_0 = __fmul_rn(d0, d0), q_1 = __fmul_rn(d1, d1);
-    const bool neg = __float_as_uint(q) >> 31;
-    e[0] = __fadd_rn(e[0], neg ? q_r : q_0);
-    e[1] = __fadd_rn(e[1], neg ? q_r : q_1);
-    e[2] = __fadd_rn(e[2], neg ? q_0 : q_r);
-    e[3] = __fadd_rn(e[3], neg ? q_1 : q_r);
-  }
-  uint32_t first = 0;                                                  // first minimum: ties keep the earlier candidate
-  float best = e[0];
-#pragma unroll
-  for (int i = 1; i < 4; ++i)
-    if (e[i] < best) { best = e[i]; first = i; }
-  return first;
-}
+// What follows gives the same result for the usual magnitudes (m0 halfway between two FP4 values, m1 beyond 6) by gains instead of error
+// sums.
 __device__ __forceinline__ float max_nan(float a, float b) {          // a NaN stays one
   float r;
   asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
@@ -867,13 +840,35 @@ __device__ __forceinline__ uint32_t to_e4m3(float t) {                // nearest
   asm("cvt.rn.satfinite.e4m3x2.f32 %0, %1, %2;" : "=h"(v) : "f"(0.0f), "f"(t));
   return v & 0xFFu;
 }
-constexpr float QUICK_MAX = 9.4f;                                      // largest scaled element that the bounds below cover
+// What a special value m takes off a block's error is a sum over the elements that take it, and those lie in one interval, of half-width
+// `half_width` around m0 or beyond lo1 = (6 + m1) / 2; an element at distance -t inside it gains k t.  That needs neither the rounded
+// value nor the squares, so a thread's 16 elements cost half the instructions.  The decision is that of the FP32 sums in
+// ascending order unless two candidates come within `delta`, more than all roundings of both ways together.  t is exact wherever its
+// sign matters (a within a factor of two of m0, v0, v1 or m1), so the elements that take the special value are the same ones.
+// SUB lanes share a block of 16 * SUB elements, so every block size reads its tensor once and alike.
+//
+// Blocks left undecided (candidates too close, scaled elements beyond quick_max, values that the short form cannot take) are put down by
+// their warp and taken by quant_weight_block, a thread each, as soon as there are 32; a CTA's warps share out what is left at the end.
+// Few blocks of continuous weights are, many of weights that lie on a coarse grid (FP8, INT8, INT4 checkpoints) and nearly all at a
+// given scale a hundred times too small.
+//
+// Bound by instruction issue.  11008 x 4096 at a given scale, us in graph replays, quant_weight_kernel / this with undecided blocks walked
+// one element at a time by their whole warp and blocks beyond 9.4 steps by the plain procedure / this:
+//   blocks of 16: Student-t 61.3 / 43.6 / 42.8, rounded to bf16 61.4 / 54.4 / 44.6, FP8 grid 64.2 / 80.4 / 49.1, normal at 0.1 of its scale 94 / 255 / 64
+//   blocks of 128: 94.7 / 57.4 / 54.0, 94.6 / 73.7 / 55.9, 114.0 / 157.7 / 83.8, 107 / 1645 / 78
+// Blocks of 32 and more at 1e-3 of their scale and below (every code saturates) are slower by up to a third.  As many CTAs as are resident: the
+// undecided blocks fill warps better than with 16 to an SM (bf16, blocks of 128: 63.8).
 template <int SUB>
 __global__ void __launch_bounds__(256, 4) quant_weight_quick_kernel(const float4* __restrict__ w, long long n_groups, float m0, float m1,
                                                                     float half_width, uint32_t remap_code, const float* __restrict__ scale_in,
                                                                     const uint32_t* __restrict__ amax_bits, uint2* __restrict__ codes,
                                                                     uint8_t* __restrict__ scales, float* __restrict__ scale_out) {
+  constexpr int WARPS = 8;
+  constexpr float quick_max = 8192.0f / (SUB * SUB);                   // further out `delta` passes usual differences
   __shared__ float2 steps[64];                                         // scale code -> step, its correctly rounded reciprocal
+  __shared__ long long left[WARPS][64];                                // blocks left undecided, per warp
+  __shared__ int n_left[WARPS];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const bool wide = aligned32(w);
   const long long stride = (long long)gridDim.x * blockDim.x;
   const long long turns = (n_groups + stride - 1) / stride;
@@ -887,130 +882,156 @@ __global__ void __launch_bounds__(256, 4) quant_weight_quick_kernel(const float4
   }
   if (blockIdx.x == 0 && threadIdx.x == 0) *scale_out = d32;
   const float d32x6 = __fmul_rn(d32, 6.0f);
-  const bool usual = d32x6 > 1.0e-12f && d32x6 < 1.0e12f;              // every step and quotient well inside FP32
+  const bool usual = d32x6 > 1.0e-18f && d32x6 < 1.0e22f;              // some step is inside short_form's range
   const float inv6 = usual ? __frcp_rn(d32x6) : __uint_as_float(0x7FC00000u);
   if (threadIdx.x < 64) {
     const float d = __fmul_rn(d32, scale_value(threadIdx.x));
-    steps[threadIdx.x] = make_float2(d, usual && threadIdx.x > 0 ? __frcp_rn(d) : __uint_as_float(0x7FC00000u));   // NaN: not this way
+    steps[threadIdx.x] = make_float2(d, usual && short_form(0.0f, d) ? __frcp_rn(d) : __uint_as_float(0x7FC00000u));   // NaN: not this way
   }
   __syncthreads();
-  const uint32_t other_zero = remap_code ^ 8u;
   const float k0 = 4.0f * half_width, k1 = 2.0f * (m1 - 6.0f), lo1 = 0.5f * (m1 + 6.0f);
-  for (long long turn = turns - 1; turn >= 0; --turn) {
-    const long long t = turn * stride + (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const bool inside = t < n_groups;                                  // the same for all lanes of a block: n_groups and stride are multiples of SUB
-    float xs[16];
+  int count = 0;
+  for (long long turn = turns - 1; turn >= -1; --turn) {                // the last one: what is left
+    bool some = true;
+    long long block = 0;
+    if (turn >= 0) {
+      const long long t = turn * stride + (long long)blockIdx.x * blockDim.x + threadIdx.x;
+      const bool inside = t < n_groups;                                  // the same for all lanes of a block: n_groups and stride are multiples of SUB
+      float xs[16];
 #pragma unroll
-    for (int q = 0; q < 2; ++q) load8(w + 4 * (inside ? t : 0) + 2 * q, xs + 8 * q, wide);
-    float bmax = 0.0f;
+      for (int q = 0; q < 2; ++q) load8(w + 4 * (inside ? t : 0) + 2 * q, xs + 8 * q, wide);
+      float bmax = 0.0f;
 #pragma unroll
-    for (int j = 0; j < 16; j += 2) bmax = max3_nan(bmax, fabsf(xs[j]), fabsf(xs[j + 1]));
+      for (int j = 0; j < 16; j += 2) bmax = max3_nan(bmax, fabsf(xs[j]), fabsf(xs[j + 1]));
 #pragma unroll
-    for (int o = 1; o < SUB; o *= 2) bmax = max_nan(bmax, __shfl_xor_sync(0xFFFFFFFFu, bmax, o));
-    // Eq. 2: the quotient, correctly rounded where the code is not 0 or 1 anyway (the correction of div_f32)
-    float tq = bmax * inv6;
-    tq = __fmaf_rn(__fmaf_rn(tq, -d32x6, bmax), inv6, tq);
-    tq = __fmaf_rn(__fmaf_rn(tq, -d32x6, bmax), inv6, tq);
-    const uint32_t scode = max(min(to_e4m3(tq), 63u), 1u);             // never 0: keep a non-empty block alive
-    const float2 step = steps[scode];
-    const float xmax = bmax * step.y;
-    const bool quick = inside && bmax > 0.0f && bmax < 1.0e30f && xmax <= QUICK_MAX;   // false for a NaN anywhere
-    const bool on1 = __any_sync(0xFFFFFFFFu, quick && xmax > 0.999f * lo1);
-    const F2 nd2 = f2(-step.x, -step.x), y2 = f2(step.y, step.y);
-    F2 sum0 = f2(0.0f, 0.0f), dif0 = sum0, sum1 = sum0, dif1 = sum0;   // gains / -K of all elements; of the positive less the negative ones
-    uint32_t c[2], take0[2], take1[2] = {0, 0};
-    auto flip = [](float g, float x) { return __uint_as_float(__float_as_uint(g) ^ (__float_as_uint(x) & 0x80000000u)); };
+      for (int o = 1; o < SUB; o *= 2) bmax = max_nan(bmax, __shfl_xor_sync(0xFFFFFFFFu, bmax, o));
+      // Eq. 2: the quotient, correctly rounded where the code is not 0 or 1 anyway (the correction of div_f32)
+      float tq = bmax * inv6;
+      tq = __fmaf_rn(__fmaf_rn(tq, -d32x6, bmax), inv6, tq);
+      tq = __fmaf_rn(__fmaf_rn(tq, -d32x6, bmax), inv6, tq);
+      const uint32_t scode = max(min(to_e4m3(tq), 63u), 1u);             // never 0: keep a non-empty block alive
+      const float2 step = steps[scode];
+      const float xmax = bmax * step.y;
+      bool quick = inside && bmax < 1.0e30f && xmax <= quick_max;        // false for a NaN anywhere
+      if (__any_sync(0xFFFFFFFFu, quick)) {
+        const bool on1 = __any_sync(0xFFFFFFFFu, quick && xmax > 0.999f * lo1);
+        const F2 nd2 = f2(-step.x, -step.x), y2 = f2(step.y, step.y);
+        F2 sum0 = f2(0.0f, 0.0f), dif0 = sum0, sum1 = sum0, dif1 = sum0;   // gains / -K of all elements; of the positive less the negative ones
+        float far = 0.0f;                                                // the squared distances beyond 6
+        uint32_t c[2], take0[2], take1[2] = {0, 0};
+        auto flip = [](float g, float x) { return __uint_as_float(__float_as_uint(g) ^ (__float_as_uint(x) & 0x80000000u)); };
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      float* x = xs + 8 * h;
-      float t0[8];
+        for (int h = 0; h < 2; ++h) {
+          float* x = xs + 8 * h;
+          float t0[8];
 #pragma unroll
-      for (int j = 0; j < 8; j += 2) {
-        split(div_f32(f2(x[j], x[j + 1]), nd2, y2), x[j], x[j + 1]);   // the scaled block of Eq. 6
-        t0[j] = fabsf(fabsf(x[j]) - m0) - half_width;
-        t0[j + 1] = fabsf(fabsf(x[j + 1]) - m0) - half_width;
-        const float g0 = fminf(t0[j], 0.0f), g1 = fminf(t0[j + 1], 0.0f);
-        sum0 = add2(sum0, f2(g0, g1));
-        dif0 = add2(dif0, f2(flip(g0, x[j]), flip(g1, x[j + 1])));
-      }
-      c[h] = to_fp4x8(x[0], x[1], x[2], x[3], x[4], x[5], x[6], x[7]);
-      take0[h] = to_fp4x8(t0[0], t0[1], t0[2], t0[3], t0[4], t0[5], t0[6], t0[7]) & 0x88888888u;
-    }
-    if (on1) {
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const float* x = xs + 8 * h;
-        float t1[8];
-#pragma unroll
-        for (int j = 0; j < 8; j += 2) {
-          t1[j] = lo1 - fabsf(x[j]);
-          t1[j + 1] = lo1 - fabsf(x[j + 1]);
-          const float g0 = fminf(t1[j], 0.0f), g1 = fminf(t1[j + 1], 0.0f);
-          sum1 = add2(sum1, f2(g0, g1));
-          dif1 = add2(dif1, f2(flip(g0, x[j]), flip(g1, x[j + 1])));
+          for (int j = 0; j < 8; j += 2) {
+            split(div_f32(f2(x[j], x[j + 1]), nd2, y2), x[j], x[j + 1]);   // the scaled block of Eq. 6
+            t0[j] = fabsf(fabsf(x[j]) - m0) - half_width;
+            t0[j + 1] = fabsf(fabsf(x[j + 1]) - m0) - half_width;
+            const float g0 = fminf(t0[j], 0.0f), g1 = fminf(t0[j + 1], 0.0f);
+            sum0 = add2(sum0, f2(g0, g1));
+            dif0 = add2(dif0, f2(flip(g0, x[j]), flip(g1, x[j + 1])));
+          }
+          c[h] = to_fp4x8(x[0], x[1], x[2], x[3], x[4], x[5], x[6], x[7]);
+          take0[h] = to_fp4x8(t0[0], t0[1], t0[2], t0[3], t0[4], t0[5], t0[6], t0[7]) & 0x88888888u;
         }
-        take1[h] = to_fp4x8(t1[0], t1[1], t1[2], t1[3], t1[4], t1[5], t1[6], t1[7]) & 0x88888888u;
-      }
-    }
-    auto gains = [&](F2 sum, F2 dif, float k, float& pos, float& neg) {
-      float a, b, d, f;
-      split(sum, a, b);
-      split(dif, d, f);
-      a += b;
-      d += f;
+        if (on1) {
 #pragma unroll
-      for (int o = 1; o < SUB; o *= 2) {
-        a += __shfl_xor_sync(0xFFFFFFFFu, a, o);
-        d += __shfl_xor_sync(0xFFFFFFFFu, d, o);
-      }
-      pos = -0.5f * k * (a + d);
-      neg = -0.5f * k * (a - d);
-    };
-    float gain[4] = {0.0f, 0.0f, 0.0f, 0.0f};                          // metadata order: +m0, +m1, -m0, -m1
-    gains(sum0, dif0, k0, gain[0], gain[2]);
-    uint32_t meta = gain[2] > gain[0] ? 2u : 0u;
-    // How far roundings can bring two candidates together, n = 16 SUB elements.  No element up to 7 is further than 1 from FP4, none
-    // up to 3.5 than 1/2, none up to 1.75 than 1/4: that bounds every sum by E, two FP32 sums are off by less than 2 (n + 1) 2^-24 E,
-    // the gains by half as much.  Beyond 7, distances go up to 3.4 and gains to 40 an element.
-    const uint32_t from2 = (c[0] & 0x44444444u) | ((c[1] & 0x44444444u) >> 1), from4 = ((c[0] >> 1) & c[0] & 0x22222222u) | ((c[1] & (c[1] << 1) & 0x44444444u));
-    float bound = 1.0f + 0.25f * (float)__popc(from2) + 0.75f * (float)__popc(from4);
+          for (int h = 0; h < 2; ++h) {
+            const float* x = xs + 8 * h;
+            float t1[8];
 #pragma unroll
-    for (int o = 1; o < SUB; o *= 2) bound += __shfl_xor_sync(0xFFFFFFFFu, bound, o);
-    const float delta = xmax <= 7.0f ? bound * (SUB * 4.0e-6f) : SUB * SUB * 1.953125e-3f;
-    bool close = fabsf(gain[0] - gain[2]) <= delta && fmaxf(gain[0], gain[2]) > 0.0f;
-    if (on1) {
-      gains(sum1, dif1, k1, gain[1], gain[3]);
-      const float top0 = fmaxf(gain[0], gain[2]), low0 = fminf(gain[0], gain[2]);
-      const float top1 = fmaxf(gain[1], gain[3]), low1 = fminf(gain[1], gain[3]);
-      const float top = fmaxf(top0, top1), second = fmaxf(fminf(top0, top1), top0 > top1 ? low0 : low1);
-      close = top - second <= delta && top > 0.0f;
-      if (top1 > top0) meta = gain[3] > gain[1] ? 3u : 1u;
-    }
-    if (close && quick) meta = choice_by_sums(reinterpret_cast<const float*>(w + 4 * (t & ~(SUB - 1ll))), 16 * SUB, step, m0, m1);
-    if (!inside) continue;
-    if (!quick) {
-      if (bmax == 0.0f) {
-        codes[t] = make_uint2(other_zero * 0x11111111u, other_zero * 0x11111111u);
-        if (threadIdx.x % SUB == 0) scales[t / SUB] = 0;
-      } else if (threadIdx.x % SUB == 0) {
-        scales[t / SUB] = (uint8_t)quant_weight_block_plain<false>(w + 4 * t, SUB, d32, m0, m1, remap_code, codes + t);
-      }
-      continue;
-    }
-    uint32_t out[2];
+            for (int j = 0; j < 8; j += 2) {
+              t1[j] = lo1 - fabsf(x[j]);
+              t1[j + 1] = lo1 - fabsf(x[j + 1]);
+              const float g0 = fminf(t1[j], 0.0f), g1 = fminf(t1[j + 1], 0.0f);
+              sum1 = add2(sum1, f2(g0, g1));
+              dif1 = add2(dif1, f2(flip(g0, x[j]), flip(g1, x[j + 1])));
+            }
+            take1[h] = to_fp4x8(t1[0], t1[1], t1[2], t1[3], t1[4], t1[5], t1[6], t1[7]) & 0x88888888u;
+          }
+          if (__any_sync(0xFFFFFFFFu, quick && xmax > 7.0f)) {
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      uint32_t v = c[h];
-      const uint32_t taken = ((meta & 1u) ? take1[h] : take0[h]) & ((meta & 2u) ? v : ~v);   // elements of the special value's sign only
-      const uint32_t nz = nonzero_nibbles(v);
-      v &= nz | 0x77777777u;                                           // a true zero is always the other zero code
-      if (remap_code == 0u) v |= ~nz & 0x88888888u;
-      v &= ~((taken >> 3) * 15u);
-      if (remap_code != 0u) v |= taken;
-      out[h] = v;
+            for (int j = 0; j < 16; ++j) {
+              const float o = fmaxf(fabsf(xs[j]) - 6.0f, 0.0f);
+              far += o * o;
+            }
+          }
+        }
+        auto gains = [&](F2 sum, F2 dif, float k, float& pos, float& neg) {
+          float a, b, d, f;
+          split(sum, a, b);
+          split(dif, d, f);
+          a += b;
+          d += f;
+#pragma unroll
+          for (int o = 1; o < SUB; o *= 2) {
+            a += __shfl_xor_sync(0xFFFFFFFFu, a, o);
+            d += __shfl_xor_sync(0xFFFFFFFFu, d, o);
+          }
+          pos = -0.5f * k * (a + d);
+          neg = -0.5f * k * (a - d);
+        };
+        float gain[4] = {0.0f, 0.0f, 0.0f, 0.0f};                        // metadata order: +m0, +m1, -m0, -m1
+        gains(sum0, dif0, k0, gain[0], gain[2]);
+        uint32_t meta = gain[2] > gain[0] ? 2u : 0u;
+        // How far roundings can bring two candidates together, n = 16 SUB elements, u = 2^-24.  No element up to 7 is further than 1 from FP4,
+        // none up to 3.5 than 1/2, none up to 1.75 than 1/4: with the squares beyond 6 that bounds a block's error by E.  An FP32 sum of n
+        // squares is off by less than (n + 2) u E; a gain, which is part of the error, by less than 15 u E (8 packed additions, the two
+        // halves', three shuffles', the scale's, one of t itself).  Two of each: (2 n + 34) u E, at most 66 u E SUB = 3.94e-6 E SUB.
+        const uint32_t from2 = (c[0] & 0x44444444u) | ((c[1] & 0x44444444u) >> 1), from4 = ((c[0] >> 1) & c[0] & 0x22222222u) | ((c[1] & (c[1] << 1) & 0x44444444u));
+        float bound = 1.0f + 0.25f * (float)__popc(from2) + 0.75f * (float)__popc(from4) + far;
+#pragma unroll
+        for (int o = 1; o < SUB; o *= 2) bound += __shfl_xor_sync(0xFFFFFFFFu, bound, o);
+        const float delta = bound * (SUB * 4.0e-6f);
+        bool close = fabsf(gain[0] - gain[2]) <= delta && fmaxf(gain[0], gain[2]) > 0.0f;
+        if (on1) {
+          gains(sum1, dif1, k1, gain[1], gain[3]);
+          const float top0 = fmaxf(gain[0], gain[2]), low0 = fminf(gain[0], gain[2]);
+          const float top1 = fmaxf(gain[1], gain[3]), low1 = fminf(gain[1], gain[3]);
+          const float top = fmaxf(top0, top1), second = fmaxf(fminf(top0, top1), top0 > top1 ? low0 : low1);
+          close = top - second <= delta && top > 0.0f;
+          if (top1 > top0) meta = gain[3] > gain[1] ? 3u : 1u;
+        }
+        quick = quick && !close;
+        if (quick) {
+          uint32_t out[2];
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            uint32_t v = c[h];
+            const uint32_t taken = ((meta & 1u) ? take1[h] : take0[h]) & ((meta & 2u) ? v : ~v);   // elements of the special value's sign only
+            const uint32_t nz = nonzero_nibbles(v);
+            v &= nz | 0x77777777u;                                       // a true zero is always the other zero code
+            if (remap_code == 0u) v |= ~nz & 0x88888888u;
+            v &= ~((taken >> 3) * 15u);
+            if (remap_code != 0u) v |= taken;
+            out[h] = v;
+          }
+          codes[t] = make_uint2(out[0], out[1]);
+          if (threadIdx.x % SUB == 0) scales[t / SUB] = (uint8_t)(bmax > 0.0f ? (meta << 6) | scode : 0u);
+        }
+      }
+      const uint32_t undecided = __ballot_sync(0xFFFFFFFFu, inside && !quick && threadIdx.x % SUB == 0);
+      if (!undecided) continue;
+      if ((undecided >> lane) & 1u) left[warp][count + __popc(undecided & ((1u << lane) - 1u))] = t / SUB;
+      count += __popc(undecided);
+      __syncwarp();
+      if (count < 32) continue;
+      count -= 32;
+      block = left[warp][count + lane];
+    } else {
+      if (lane == 0) n_left[warp] = count;
+      if (!__syncthreads_or(count)) return;
+      int at = threadIdx.x, from = 0;
+      while (from < WARPS && at >= n_left[from]) at -= n_left[from++];
+      some = from < WARPS;
+      if (!__any_sync(0xFFFFFFFFu, some)) return;
+      if (some) block = left[from][at];
     }
-    codes[t] = make_uint2(out[0], out[1]);
-    if (threadIdx.x % SUB == 0) scales[t / SUB] = (uint8_t)((meta << 6) | scode);
+    // (the walking form for blocks of 16 too: the other one spills here)
+    quant_weight_block<false, false>(w + 4 * SUB * block, some, SUB, wide, d32, m0, m1, remap_code, codes + SUB * block, scales + block);
+    __syncwarp();
   }
 }
 
@@ -1032,7 +1053,7 @@ int launch_quant_weight(const float* w, int N, int K, int block, int scale_aware
   const bool halfway = m0 == 2.5f || m0 == 3.5f || m0 == 5.0f;         // between FP4 neighbours 2, 3 / 3, 4 / 4, 6
   if (!scale_aware && halfway && m1 > 6.0f) {
     const long long n_groups = n_blocks * sub, b = (n_groups + threads - 1) / threads;
-    const int g = (int)(b < 1 ? 1 : (b > 148LL * 16 ? 148LL * 16 : b));
+    const int g = (int)(b < 1 ? 1 : (b > 148LL * 4 ? 148LL * 4 : b));    // as many as are resident
     auto kern = sub == 1 ? quant_weight_quick_kernel<1> : sub == 2 ? quant_weight_quick_kernel<2> : sub == 4 ? quant_weight_quick_kernel<4>
                                                                                                    : quant_weight_quick_kernel<8>;
     // dependent: with a maximum ahead it starts up while that drains

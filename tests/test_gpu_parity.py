@@ -463,6 +463,63 @@ def test_quant_weight_ties_between_candidates(b, block, sv_mag, remap_code):
     assert np.array_equal(scales.cpu().numpy(), want_s) and np.array_equal(codes.cpu().numpy(), want_c)
 
 
+def _weights_like(b, got, w, d32, block, sv_mag=(5.0, 8.0), remap_code=0x8):
+    """Codes and scale bytes of the GPU against the oracle's at tensor scale d32, near-ties aside."""
+    want_c, want_s, _, dbg = ro.quantize_weight(w, sv_mag=sv_mag, remap_code=remap_code, tensor_scale=np.float32(d32), block=block, return_debug=True)
+    got_c, got_s = got[0].cpu().numpy(), got[1].cpu().numpy()
+    assert np.array_equal(got_s & 0x3F, want_s & 0x3F)
+    ok, right = blocks_agree(w, np.float32(d32), (got_c, got_s), (want_c, want_s), dbg["near_tie"], block, ro.SCALE_E3M3_META2, sv_mag, remap_code)
+    assert np.all(right), f"{int((~right).sum())} of {right.size} blocks"
+    return ok.mean()
+
+
+@pytest.mark.parametrize("block", [16, 32, 64, 128])
+@pytest.mark.parametrize("clip", [0.5, 0.1, 0.01, 1e-4])
+def test_quant_weight_given_scale_that_clips(b, block, clip):
+    """A tensor scale below the tensor's own: elements go beyond 6 steps, up to the point where every block saturates (0.01) and where the
+    short form's bound decides nothing any more (1e-4)."""
+    N, K = 130, 2048
+    w = inputs.student_t_weights(N, K, 31, outlier_frac=0.001)
+    d32 = np.float32(float(w.abs().max()) / 11.25 * clip)
+    got = b.razer_quant_weight(w.cuda(), tensor_scale=torch.tensor([float(d32)]).cuda(), block=block)
+    assert _weights_like(b, got, w.numpy(), d32, block) > 0.99
+
+
+@pytest.mark.parametrize("block", [16, 32, 64, 128])
+@pytest.mark.parametrize("scale", [2.0**-50, 2.0**45])
+def test_quant_weight_far_from_one(b, block, scale):
+    """Whole tensors near the ends of the range that the short form takes."""
+    w = inputs.student_t_weights(70, 1024, 32, outlier_frac=0.001) * scale
+    d32 = ro.quantize_weight(w.numpy(), block=block)[2]
+    assert _weights_like(b, b.razer_quant_weight(w.cuda(), block=block), w.numpy(), d32, block) > 0.999
+
+
+@pytest.mark.parametrize("block,N,K", [(16, 1, 16), (16, 3, 528), (16, 1300, 2048), (32, 1300, 2048), (64, 40, 1088), (128, 1300, 2048), (128, 7, 128)])
+@pytest.mark.parametrize("sv_mag,remap_code", [((5.0, 8.0), 0x8), ((2.5, 12.0), 0x0)])
+def test_quant_weight_undecided_blocks(b, block, N, K, sv_mag, remap_code):
+    """Weights on a coarse grid, where a good part of the blocks is left to the error sums: none, a few and more than a warp at a time, over one
+    and over several turns of the grid, some with a NaN or an infinity, some zero.  Steps are powers of two and errors exact, so the first
+    minimum is the answer without exception."""
+    gen = torch.Generator().manual_seed(N + block)
+    w = torch.randint(-12, 13, (N, K), generator=gen).float() / 2
+    w.view(N, -1, block)[:, :, 3] = 6.0                        # block maximum: 6 steps of one
+    blocks = w.view(-1, block)
+    if blocks.shape[0] > 64:
+        blocks[5::11] = 0.0
+    codes, scales, _ = b.razer_quant_weight(w.cuda(), sv_mag=sv_mag, remap_code=remap_code, tensor_scale=torch.ones(1, device="cuda"), block=block)
+    want_c, want_s, _ = ro.quantize_weight(w.numpy(), sv_mag=sv_mag, remap_code=remap_code, tensor_scale=np.float32(1.0), block=block)
+    assert np.array_equal(scales.cpu().numpy(), want_s) and np.array_equal(codes.cpu().numpy(), want_c)
+    # blocks with a NaN or an infinity leave the others as they are, whichever of a block's lanes holds it
+    odd = torch.randint(0, blocks.shape[0], (max(1, blocks.shape[0] // 9),), generator=gen)
+    at = torch.randint(0, block, odd.shape, generator=gen)
+    blocks[odd, at] = torch.where(torch.rand(odd.shape, generator=gen) < 0.5, float("nan"), float("inf"))
+    c2, s2, _ = b.razer_quant_weight(w.cuda(), sv_mag=sv_mag, remap_code=remap_code, tensor_scale=torch.ones(1, device="cuda"), block=block)
+    keep = np.ones(blocks.shape[0], bool)
+    keep[odd.numpy()] = False
+    assert np.array_equal(s2.cpu().numpy().reshape(-1)[keep], want_s.reshape(-1)[keep])
+    assert np.array_equal(c2.cpu().numpy().reshape(-1, block // 2)[keep], want_c.reshape(-1, block // 2)[keep])
+
+
 @pytest.mark.parametrize("block", [32, 64, 128])
 def test_larger_blocks_quantize_pack_and_multiply(b, block):
     """Block sizes 32 / 64 / 128 (Sec. 5's block-size study, Sec. 4.3's deployment size): the GPU weight quantizer
