@@ -285,14 +285,16 @@ razer_fp4_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_consta
     // elected once for the whole loop: descriptors and addresses stay in uniform registers
     if (elect_one()) {
       uint32_t seg = 0;
+      // what is there first is waited for first: the first item's weights, since its activations may belong to the preceding kernel, and
+      // from then on the activations
+      uint32_t bar0 = bar_afull, phase0 = 0, bar1 = bar_xfull, phase1 = 0;
       for (int i = 0; i < n_items; ++i) {
         const bool seg_first = (i == 0) || cur.step == 0;
         const bool seg_last = (i + 1 == n_items) || cur.step == spt - 1;
         const int nch = min(CH, a.g.k_chunks - cur.step * CH);
-        // the activations are there long before the weights are remapped: looked at first, so that it delays nothing
-        if (!mbar_wait(bar_xfull + 8 * cur.xs, (uint32_t)cur.xph, abort_flag)) { fail(30); break; }
+        if (!mbar_wait(bar0, phase0, abort_flag)) { fail(i > 0 ? 30 : 23); break; }
         if (seg_first && !mbar_wait(bar_accempty, (seg & 1u) ^ 1u, abort_flag)) { fail(24); break; }
-        if (!mbar_wait(bar_afull + 8 * cur.as, (uint32_t)cur.aph, abort_flag)) { fail(23); break; }
+        if (!mbar_wait(bar1, phase1, abort_flag)) { fail(i > 0 ? 23 : 30); break; }
         tc_fence_after();
         const uint32_t xs = smem_u32(smem_x) + (uint32_t)cur.xs * C::X_BYTES;
         const uint32_t sfb_s = xs + C::X_CODE_BYTES;
@@ -326,6 +328,8 @@ razer_fp4_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_consta
         tc_commit(bar_aempty + 8 * cur.as);
         if (seg_last) { tc_commit(bar_accfull); ++seg; }
         cur.next(spt);
+        bar0 = bar_xfull + 8 * cur.xs, phase0 = (uint32_t)cur.xph;
+        bar1 = bar_afull + 8 * cur.as, phase1 = (uint32_t)cur.aph;
       }
     }
     // the MMAs issued so far read shared memory and TMEM until they complete: wait for them (bounded, not

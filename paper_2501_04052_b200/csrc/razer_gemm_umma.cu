@@ -280,14 +280,17 @@ razer_umma_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
       bool alive = true;
       Ring<XST> xr;
       Ring<AST> ar;
+      // What is there first is waited for first (a wait that finds its stage full still takes 150 cycles): the first item's weights, since
+      // its activations may belong to the preceding kernel, and from then on the activations.  16 x 256 x 256 2.35 us with the activations
+      // first throughout, 2.14 this way; the two barriers are chosen an item ahead, since choosing them here cost 2 % at 192 tokens.
+      uint32_t bar0 = bar_afull, phase0 = 0, bar1 = bar_xfull, phase1 = 0;
       for (int i = 0; i < n_items; ++i) {
         const bool seg_first = (i == 0) || step == 0;
         const bool seg_last = (i + 1 == n_items) || step == spt - 1;
         const int nch = min(CH, a.g.k_chunks - step * CH);
-        // the activations are there long before the weights are decoded: looked at first, so that it delays nothing
-        if (!mbar_wait(bar_xfull + 8 * xr.slot, xr.phase, abort_flag)) { fail(10); break; }
+        if (!mbar_wait(bar0, phase0, abort_flag)) { fail(i > 0 ? 10 : 3); break; }
         if (seg_first && !mbar_wait(bar_accempty, (seg & 1u) ^ 1u, abort_flag)) { fail(4); break; }
-        if (!mbar_wait(bar_afull + 8 * ar.slot, ar.phase, abort_flag)) { fail(3); break; }
+        if (!mbar_wait(bar1, phase1, abort_flag)) { fail(i > 0 ? 3 : 10); break; }
         tc_fence_after();
         const uint32_t a_t = tmem_a0 + ar.slot * Cfg::A_STAGE_COLS;
         if (seg_first) seg_items = 0;
@@ -323,6 +326,8 @@ razer_umma_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
         if (seg_last) { tc_commit(bar_accfull); ++seg; }
         next_item();
         ar.next();
+        bar0 = bar_xfull + 8 * xr.slot, phase0 = xr.phase;
+        bar1 = bar_afull + 8 * ar.slot, phase1 = ar.phase;
       }
     }
     // The MMAs issued so far read shared memory and TMEM and write TMEM until they complete: commit them to a barrier
