@@ -518,8 +518,8 @@ struct Plan {
 // Fitted to a sweep of 16 shapes (M 16 .. 2048, K and N 300 .. 14336, both widths, all grids).  With 256 tokens wherever there are
 // more than 128, and stripes on all SMs, 512 x 4096 x 4096 took 18.0 us (14.0 by this choice), 300 x 390 x 2320 10.6 (7.9),
 // 2048 x 1024 x 1024 13.0 (6.4), 1000 x 300 x 8192 27.5 (12.2), 128 x 14336 x 4096 16.4 (13.8).
-static const TileCost tile_costs[] = {{128, CH, CH, 0.139f, 0.08f, 0.6f, 2.9f, 0.30f, 4.6f, 0.50f},
-                                      {256, CH, CH, 0.177f, 0.18f, 1.3f, 3.1f, 0.30f, 6.5f, 1.30f}};
+static const TileCost tile_costs[] = {{128, CH, CH, false, 1.6f, 1.8f, 0.139f, 0.08f, 0.6f, 2.9f, 0.30f, 4.6f, 0.50f, 0.0f, 0.0f},
+                                      {256, CH, CH, false, 1.6f, 1.8f, 0.177f, 0.18f, 1.3f, 3.1f, 0.30f, 6.5f, 1.30f, 0.0f, 0.0f}};
 
 static bool admissible(const TileCost& t, const Fp4ActLayout& act) {
   return act.force_nt ? t.NT == act.force_nt : t.NT <= act.tiles128 * 128;

@@ -492,20 +492,28 @@ razer_umma_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
 // ------------------------------------------------------------------ host side
 struct UmmaPlan {
   int NT, CH, CHX;             // token tile; chunks per item, per activation stage
+  bool table;                  // weights decoded by table
   int token_tiles, steps_per_tile, grid;
   long long tiles, total_items;
   size_t slots_bytes;
 };
 
-// Token tile and grid: the cheapest pair by the cost model (razer_tcgen05.cuh), fitted to a sweep of 18 shapes (M 16 .. 2048, K and N
-// 300 .. 28672, all widths, all grids).  On these the choice is within 11 % of the best of the sweep (further off at
-// 16 x 28672 x 1024, 14.3 -> 10.0 us), where the fixed rule before it (the narrowest tile that holds M, all SMs) was up to 4 times slower: 300 x 390 x 2320
-// 36.2 -> 8.1 us, 256 x 1024 x 1024 20.8 -> 4.8, 1000 x 300 x 8192 33.1 -> 14.5, 333 x 4096 x 11008 38.8 -> 32.4.
+// Token tile, decode and grid: the cheapest by the cost model (razer_tcgen05.cuh), fitted to 30,700 times of 1617 sizes (M 9 .. 2048, N and K
+// 256 .. 28672, all widths and grids, weights from HBM, launches back to back in a graph).  Of the best of a size's grids the choice is
+// 0.6 % off in the mean, 10 % at worst; by constants per width without `start`, `late` and `spread` it was 2.6 % off and up to 40 %
+// (157 x 3180 x 672 5.34 -> 4.29 us, 523 x 1024 x 1024 6.37 -> 4.88, 64 x 2341 x 816 3.88 -> 3.49).
+// Up to 32 tokens the table costs a start (it is filled by every CTA) and gains by the chunk: it is the faster one from 3 items of
+// four chunks a CTA on at 16 tokens (1 item +1.3 %, 2 and 3 level, 6 -4.5 %, 16 -11 %), from 6 on at 32 (1 to 5 +3 to +6 %, 8 -5 %, 16 -7 %).
 static const TileCost tile_costs[] = {
-    {16, 4, 4, 0.140f, 0.20f, 0.0f, 2.0f, 0.20f, 4.0f, 0.06f},  {32, 4, 2, 0.152f, 0.20f, 0.1f, 2.6f, 0.20f, 4.0f, 0.11f},
-    {64, 4, 4, 0.178f, 0.15f, 0.4f, 2.3f, 0.35f, 4.5f, 0.22f},  {96, 4, 2, 0.186f, 0.15f, 0.5f, 2.4f, 0.37f, 5.0f, 0.34f},
-    {128, 4, 1, 0.228f, 0.15f, 0.7f, 2.9f, 0.75f, 6.0f, 0.45f}, {192, 2, 1, 0.268f, 0.20f, 1.2f, 3.7f, 0.60f, 6.3f, 0.67f},
-    {256, 2, 1, 0.315f, 0.25f, 1.6f, 4.0f, 0.55f, 7.0f, 0.90f}};
+    {16, 4, 4, true, 0.879f, 0.095f, 0.113f, 0.611f, 0.83f, 2.868f, 0.201f, 3.914f, 0.189f, 0.036f, 4.337f},
+    {16, 4, 4, false, 0.933f, 0.006f, 0.121f, 0.847f, 0.633f, 2.706f, 0.191f, 4.336f, 0.159f, 0.116f, 4.053f},
+    {32, 4, 2, true, 1.316f, 0.2f, 0.13f, 0.52f, 0.384f, 2.288f, 0.185f, 3.497f, 0.202f, 0.221f, 3.806f},
+    {32, 4, 4, false, 1.016f, 0.0f, 0.127f, 0.743f, 0.622f, 2.533f, 0.173f, 3.826f, 0.191f, 0.161f, 4.159f},
+    {64, 4, 4, false, 0.753f, 0.703f, 0.141f, 0.666f, 0.862f, 2.94f, 0.22f, 4.07f, 0.31f, 0.702f, 1.154f},
+    {96, 4, 2, false, 0.565f, 1.498f, 0.156f, 0.485f, 1.257f, 3.283f, 0.211f, 4.532f, 0.457f, 0.525f, 0.607f},
+    {128, 4, 1, false, 0.299f, 1.573f, 0.192f, 0.337f, 1.68f, 3.805f, 0.293f, 5.405f, 0.749f, 0.587f, 0.504f},
+    {192, 2, 1, false, 0.0f, 2.182f, 0.233f, 0.31f, 2.861f, 5.058f, 0.276f, 6.369f, 1.003f, 0.349f, 0.0f},
+    {256, 2, 1, false, 0.0f, 1.57f, 0.267f, 0.375f, 3.371f, 6.306f, 0.25f, 7.699f, 1.495f, 0.56f, 0.0f}};
 
 static bool admissible(const TileCost& t, int M) { return t.NT <= 16 || t.NT < 2 * M; }   // not half of the tile or more padding
 
@@ -519,6 +527,7 @@ static UmmaPlan work_out_plan(const razer_desc* d, int M) {
     p.NT = t.NT;
     p.CH = t.CH;
     p.CHX = t.CHX;
+    p.table = t.table;
     p.token_tiles = (M + p.NT - 1) / p.NT;
     p.steps_per_tile = (g.k_chunks + p.CH - 1) / p.CH;
     p.tiles = (long long)g.row_tiles * p.token_tiles;
@@ -628,8 +637,8 @@ int launch_gemm_umma(const razer_desc* d, const void* packed, const void* x, int
   a.total_items = p.total_items;
   a.x_map_3d = map_3d;
   switch (p.NT) {
-    case 16: return launch_cfg<16, 4, 4, 6, 4, 3, 12, 6, true>(tmap, tmap_w, a, p.grid, st);
-    case 32: return launch_cfg<32, 4, 2, 6, 4, 3, 12, 2, true>(tmap, tmap_w, a, p.grid, st);
+    case 16: return p.table ? launch_cfg<16, 4, 4, 6, 4, 3, 12, 6, true>(tmap, tmap_w, a, p.grid, st) : launch_cfg<16, 4, 4, 6, 4, 3, 12, 6, false>(tmap, tmap_w, a, p.grid, st);
+    case 32: return p.table ? launch_cfg<32, 4, 2, 6, 4, 3, 12, 2, true>(tmap, tmap_w, a, p.grid, st) : launch_cfg<32, 4, 4, 6, 4, 3, 12, 2, false>(tmap, tmap_w, a, p.grid, st);
     case 64: return launch_cfg<64, 4, 4, 6, 3, 3, 12, 2, false>(tmap, tmap_w, a, p.grid, st);
     case 96: return launch_cfg<96, 4, 2, 6, 4, 3, 12, 1, false>(tmap, tmap_w, a, p.grid, st);
     case 128: return launch_cfg<128, 4, 1, 6, 6, 3, 12, 1, false>(tmap, tmap_w, a, p.grid, st);

@@ -155,6 +155,18 @@ def test_both_ways_into_the_library(b, monkeypatch, compiled):
         b.razer_gemv_host(desc, packed, xh.cuda(), yh, xd, yd, ws)
 
 
+@pytest.mark.parametrize("M", [9, 16, 17, 32, 33])
+@pytest.mark.parametrize("N,K", [(260, 208), (4200, 256), (1030, 1040), (130, 9232), (2300, 5008)])
+def test_gemv_both_decodes_up_to_32_tokens(b, M, N, K):
+    """Launches of one item a CTA to some twenty, on either side of where weights are decoded by table rather than in registers."""
+    codes, scales = inputs.random_codes(N, K, seed=M + K, scale_lo=0, scale_hi=64, zero_block_frac=0.02)
+    codes, scales = codes.numpy(), scales.numpy()
+    for sv_mag, remap_code in (((5.0, 8.0), 0x8), ((2.5, 12.0), 0x0)):
+        desc, packed = _pack(b, codes, scales, 0.004, sv_mag=sv_mag, remap_code=remap_code)
+        _check_matmul(b, b.razer_gemv, desc, packed, codes, scales, 0.004, inputs.activations(M, K, M), rows=sample_rows(N, 200, M), sv_mag=sv_mag,
+                      remap_code=remap_code)
+
+
 def test_activations_with_trailing_axes_of_one(b):
     """x's first two axes are its rows and columns; further ones of length one (a view of a caller's layout) change nothing."""
     codes, scales = inputs.random_codes(300, 528, seed=33)
