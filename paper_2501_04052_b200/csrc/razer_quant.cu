@@ -860,8 +860,8 @@ __device__ __forceinline__ uint32_t to_e4m3(float t) {                // nearest
 // undecided blocks fill warps better than with 16 to an SM (bf16, blocks of 128: 63.8).
 template <int SUB>
 __global__ void __launch_bounds__(256, 4) quant_weight_quick_kernel(const float4* __restrict__ w, long long n_groups, float m0, float m1,
-                                                                    float half_width, uint32_t remap_code, const float* __restrict__ scale_in,
-                                                                    const uint32_t* __restrict__ amax_bits, uint2* __restrict__ codes,
+                                                                    float half_width, uint32_t remap_code, const float* scale_in,
+                                                                    const uint32_t* amax_bits, uint2* __restrict__ codes,
                                                                     uint8_t* __restrict__ scales, float* __restrict__ scale_out) {
   constexpr int WARPS = 8;
   constexpr float quick_max = 8192.0f / (SUB * SUB);                   // further out `delta` passes usual differences
@@ -873,11 +873,12 @@ __global__ void __launch_bounds__(256, 4) quant_weight_quick_kernel(const float4
   const long long stride = (long long)gridDim.x * blockDim.x;
   const long long turns = (n_groups + stride - 1) / stride;
   grid_dep_wait();                                                     // for the maximum
+  // volatile: while this grid starts up the maximum is still being taken, so no load of it may move up or go by the constant cache
   float d32;
   if (scale_in) {
-    d32 = *scale_in;
+    d32 = *(volatile const float*)scale_in;
   } else {
-    const float amax = __uint_as_float(*amax_bits);
+    const float amax = __uint_as_float(*(volatile const uint32_t*)amax_bits);
     d32 = (amax == 0.0f) ? 1.0f : __fdiv_rn(amax, __fmul_rn(1.875f, 6.0f));   // Eq. 1
   }
   if (blockIdx.x == 0 && threadIdx.x == 0) *scale_out = d32;

@@ -532,6 +532,17 @@ def test_quant_weight_undecided_blocks(b, block, N, K, sv_mag, remap_code):
     assert np.array_equal(c2.cpu().numpy().reshape(-1, block // 2)[keep], want_c.reshape(-1, block // 2)[keep])
 
 
+def test_quant_weight_maxima_back_to_back(b):
+    """The quantizer starts up while the maximum ahead of it is still being taken: every call of a stream has its own tensor's scale."""
+    gen = torch.Generator().manual_seed(9)
+    ws = [torch.randn((n, 4096), generator=gen) * 4.0 ** i for i, n in enumerate((700, 3, 64, 2000))]
+    want = [np.float32(np.float32(w.abs().max()) / np.float32(11.25)) for w in ws]
+    dev = [w.cuda() for w in ws]
+    out = [b.razer_quant_weight(dev[i % 4])[2] for i in range(400)]
+    got = torch.cat(out).cpu().numpy()
+    assert np.array_equal(got, np.array([want[i % 4] for i in range(400)], dtype=np.float32))
+
+
 @pytest.mark.parametrize("block", [32, 64, 128])
 def test_larger_blocks_quantize_pack_and_multiply(b, block):
     """Block sizes 32 / 64 / 128 (Sec. 5's block-size study, Sec. 4.3's deployment size): the GPU weight quantizer
