@@ -167,6 +167,42 @@ def test_gemv_both_decodes_up_to_32_tokens(b, M, N, K):
                       remap_code=remap_code)
 
 
+def test_compiled_call_takes_plain_arguments_only(b):
+    """What the compiled part answers itself, and what it hands on (None)."""
+    N, K, M = 300, 528, 3
+    codes, scales = inputs.random_codes(N, K, seed=6)
+    desc, packed = _pack(b, codes.numpy(), scales.numpy(), 0.01)
+    x, y, ws = inputs.activations(M, K, 1).cuda(), torch.zeros((M, N), dtype=torch.bfloat16, device="cuda"), b.alloc_workspace(desc, M, b.OP_GEMV, "cuda")
+    want = b._matmul(b.lib().razer_gemv, desc, packed, x, None, None, b.OP_GEMV)
+    plain = (b._GEMV, b.RazerDesc, desc, packed, x, y, ws)
+    assert b._call.matmul(*plain) == 0 and torch.equal(y, want)
+    assert b._call.matmul(*plain[:6], ws[:256]) == b.ERR_WORKSPACE
+
+    class Sub(torch.Tensor):
+        pass
+
+    class Other(b.RazerDesc):
+        pass
+    for at, other in ((0, None), (2, None), (2, Other()), (3, None), (4, x.float()), (4, x.cpu()), (4, x.as_subclass(Sub)), (4, x[0]), (4, x[:, :-16]),
+                      (5, None), (5, y.as_subclass(Sub)), (5, y.to_sparse()), (6, None), (6, 7)):
+        args = list(plain)
+        args[at] = other
+        assert b._call.matmul(*args) is None, (at, other)
+    assert b._call.matmul(*plain[:6]) is None
+    # a subclass goes the other way, with the same result
+    assert torch.equal(b.razer_gemv(desc, packed, x.as_subclass(Sub), y, ws).as_subclass(torch.Tensor), want)
+    xh, yh = x.cpu().pin_memory(), torch.zeros((M, N), dtype=torch.bfloat16).pin_memory()
+    host = (b._GEMV_HOST, b.RazerDesc, desc, packed, xh, yh, x, y, ws)
+    assert b._call.gemv_host(*host) == 0 and torch.equal(yh, want.cpu())
+    for at, other in ((4, x), (5, y), (4, xh.as_subclass(Sub)), (4, torch.tensor(1.0)), (6, None), (8, None)):
+        args = list(host)
+        args[at] = other
+        assert b._call.gemv_host(*args) is None, (at, other)
+    for bad in ((x, yh), (xh, y)):
+        with pytest.raises(AssertionError):
+            b.razer_gemv_host(desc, packed, *bad, x, y, ws)
+
+
 def test_activations_with_trailing_axes_of_one(b):
     """x's first two axes are its rows and columns; further ones of length one (a view of a caller's layout) change nothing."""
     codes, scales = inputs.random_codes(300, 528, seed=33)
@@ -431,6 +467,30 @@ def test_dequant_spans_and_unaligned_output(b, N, K):
         assert np.array_equal(o2.cpu().numpy().view(np.uint32).reshape(N, K), want2.view(np.uint32))
 
 
+@pytest.mark.parametrize("offset_bytes", [16, 32, 48])
+def test_outputs_aligned_to_16_or_32_bytes(b, offset_bytes):
+    """Decoded weights and activations are stored 32 bytes at a time where the output is aligned to that, 16 where not."""
+    N, K = 37, 2064
+    codes, scales = inputs.random_codes(N, K, seed=13, scale_lo=0, scale_hi=64, zero_block_frac=0.05)
+    desc, packed = _pack(b, codes.numpy(), scales.numpy(), 0.0123)
+    want = {0: b.razer_dequant(desc, packed, fp32=False), 1: b.razer_dequant(desc, packed, fp32=True)}
+    for fp32, dtype in ((0, torch.bfloat16), (1, torch.float32)):
+        size = 4 if fp32 else 2
+        buf = torch.full((N * K + 64,), 7.0, dtype=dtype, device="cuda")
+        out = buf[offset_bytes // size:][:N * K]
+        b._check(b.lib().razer_dequant(desc, packed.data_ptr(), out.data_ptr(), fp32, None))
+        torch.cuda.synchronize()
+        assert torch.equal(out.view(N, K), want[fp32])
+        assert bool((buf[:offset_bytes // size] == 7).all()) and bool((buf[offset_bytes // size + N * K:] == 7).all())
+    ac, as_, _ = b.razer_quant_act(inputs.activations(19, K, 3).cuda())
+    ref = b.razer_decode_act(ac, as_)
+    buf = torch.full((19 * K + 64,), 7.0, dtype=torch.bfloat16, device="cuda")
+    out = buf[offset_bytes // 2:][:19 * K]
+    b._check(b.lib().razer_decode_act(ac.data_ptr(), as_.data_ptr(), 19, K, 5.0, out.data_ptr(), None))
+    torch.cuda.synchronize()
+    assert torch.equal(out.view(19, K), ref) and bool((buf[offset_bytes // 2 + 19 * K:] == 7).all()) and bool((buf[:offset_bytes // 2] == 7).all())
+
+
 @pytest.mark.parametrize("N,K,seed,sv_mag,remap_code", [(1024, 1024, 0, (5.0, 8.0), 0x8), (200, 80, 3, (5.0, 8.0), 0x8),
                                                          (129, 4160, 5, (5.0, 9.0), 0x0), (300, 528, 6, (2.5, 12.0), 0x8)])
 def test_quant_weight_bit_exact(b, N, K, seed, sv_mag, remap_code):
@@ -541,6 +601,25 @@ def test_quant_weight_maxima_back_to_back(b):
     out = [b.razer_quant_weight(dev[i % 4])[2] for i in range(400)]
     got = torch.cat(out).cpu().numpy()
     assert np.array_equal(got, np.array([want[i % 4] for i in range(400)], dtype=np.float32))
+
+
+@pytest.mark.parametrize("block", [16, 32, 64, 128])
+@pytest.mark.parametrize("sv_mag,remap_code", [((4.5, 8.0), 0x8), ((7.0, 10.0), 0x0), ((5.0, 2.5), 0x8), ((2.5, 5.0), 0x0)])
+def test_quant_weight_other_magnitudes_bit_exact(b, block, sv_mag, remap_code):
+    """Magnitudes outside the short cut of the usual ones (the first not halfway between FP4 values, or the second below 6): continuous weights,
+    near-ties aside, and weights on a grid of eighths at a scale of one, where every error is exact."""
+    w = inputs.student_t_weights(129, 1152, 40, outlier_frac=0.001)
+    got = b.razer_quant_weight(w.cuda(), sv_mag=sv_mag, remap_code=remap_code, block=block)
+    d32 = ro.quantize_weight(w.numpy(), sv_mag=sv_mag, remap_code=remap_code, block=block)[2]
+    assert np.float32(got[2].item()) == d32 and _weights_like(b, got, w.numpy(), d32, block, sv_mag, remap_code) > 0.999
+    gen = torch.Generator().manual_seed(block)
+    w = torch.randint(-40, 41, (96, 1152), generator=gen).float()
+    w.view(96, -1, block)[:, :, 3] = 48.0
+    w.view(96, -1, block)[::5, 1] = 0.0
+    w = w / 8
+    codes, scales, _ = b.razer_quant_weight(w.cuda(), sv_mag=sv_mag, remap_code=remap_code, tensor_scale=torch.ones(1, device="cuda"), block=block)
+    want_c, want_s, _ = ro.quantize_weight(w.numpy(), sv_mag=sv_mag, remap_code=remap_code, tensor_scale=np.float32(1.0), block=block)
+    assert np.array_equal(scales.cpu().numpy(), want_s) and np.array_equal(codes.cpu().numpy(), want_c)
 
 
 @pytest.mark.parametrize("block", [32, 64, 128])
