@@ -498,22 +498,23 @@ struct UmmaPlan {
   size_t slots_bytes;
 };
 
-// Token tile, decode and grid: the cheapest by the cost model (razer_tcgen05.cuh), fitted to 30,700 times of 1617 sizes (M 9 .. 2048, N and K
+// Token tile, decode and grid: the cheapest by the cost model (razer_tcgen05.cuh), fitted to 57,000 times of 2923 sizes (M 9 .. 2048, N and K
 // 256 .. 28672, all widths and grids, weights from HBM, launches back to back in a graph).  Of the best of a size's grids the choice is
-// 0.6 % off in the mean, 10 % at worst; by constants per width without `start`, `late` and `spread` it was 2.6 % off and up to 40 %
-// (157 x 3180 x 672 5.34 -> 4.29 us, 523 x 1024 x 1024 6.37 -> 4.88, 64 x 2341 x 816 3.88 -> 3.49).
-// Up to 32 tokens the table costs a start (it is filled by every CTA) and gains by the chunk: it is the faster one from 3 items of
-// four chunks a CTA on at 16 tokens (1 item +1.3 %, 2 and 3 level, 6 -4.5 %, 16 -11 %), from 6 on at 32 (1 to 5 +3 to +6 %, 8 -5 %, 16 -7 %).
+// 0.6 % off in the mean and 4 % or more at one size in 50; by fewer constants per width (one start for all, no `late`, no `spread`) it was 2.2 %
+// off: 53 x 512 x 4352 7.06 us instead of 6.37, 93 x 512 x 2816 6.88 (6.22), 239 x 1590 x 1648 7.69 (6.75), 64 x 2341 x 816 3.79 (3.46).
+// Up to 32 tokens the table costs a start (every CTA fills it) and gains by the chunk: at 16 tokens it is level with the registers at
+// 1 to 3 items of four chunks a CTA (1 item +1.3 %) and faster from there (6 -4.5 %, 16 -11 %), at 32 tokens from 6 on (1 to 5 +3 to +6 %, 8 -5 %,
+// 16 -7 %).
 static const TileCost tile_costs[] = {
-    {16, 4, 4, true, 0.879f, 0.095f, 0.113f, 0.611f, 0.83f, 2.868f, 0.201f, 3.914f, 0.189f, 0.036f, 4.337f},
-    {16, 4, 4, false, 0.933f, 0.006f, 0.121f, 0.847f, 0.633f, 2.706f, 0.191f, 4.336f, 0.159f, 0.116f, 4.053f},
-    {32, 4, 2, true, 1.316f, 0.2f, 0.13f, 0.52f, 0.384f, 2.288f, 0.185f, 3.497f, 0.202f, 0.221f, 3.806f},
-    {32, 4, 4, false, 1.016f, 0.0f, 0.127f, 0.743f, 0.622f, 2.533f, 0.173f, 3.826f, 0.191f, 0.161f, 4.159f},
-    {64, 4, 4, false, 0.753f, 0.703f, 0.141f, 0.666f, 0.862f, 2.94f, 0.22f, 4.07f, 0.31f, 0.702f, 1.154f},
-    {96, 4, 2, false, 0.565f, 1.498f, 0.156f, 0.485f, 1.257f, 3.283f, 0.211f, 4.532f, 0.457f, 0.525f, 0.607f},
-    {128, 4, 1, false, 0.299f, 1.573f, 0.192f, 0.337f, 1.68f, 3.805f, 0.293f, 5.405f, 0.749f, 0.587f, 0.504f},
-    {192, 2, 1, false, 0.0f, 2.182f, 0.233f, 0.31f, 2.861f, 5.058f, 0.276f, 6.369f, 1.003f, 0.349f, 0.0f},
-    {256, 2, 1, false, 0.0f, 1.57f, 0.267f, 0.375f, 3.371f, 6.306f, 0.25f, 7.699f, 1.495f, 0.56f, 0.0f}};
+    {16, 4, 4, true, 0.323f, 0.141f, 0.114f, 0.462f, 1.423f, 3.536f, 0.205f, 4.691f, 0.172f, 0.164f, 4.11f},
+    {16, 4, 4, false, 0.298f, 0.0f, 0.119f, 0.731f, 1.352f, 3.289f, 0.229f, 4.975f, 0.161f, 0.127f, 4.35f},
+    {32, 4, 2, true, 0.924f, 0.161f, 0.129f, 0.47f, 0.894f, 2.883f, 0.175f, 3.989f, 0.194f, 0.26f, 3.879f},
+    {32, 4, 4, false, 0.55f, 0.0f, 0.128f, 0.707f, 1.137f, 3.21f, 0.151f, 4.345f, 0.183f, 0.204f, 4.454f},
+    {64, 4, 4, false, 0.563f, 0.779f, 0.143f, 0.55f, 1.142f, 3.3f, 0.202f, 3.792f, 0.346f, 0.819f, 0.953f},
+    {96, 4, 2, false, 0.447f, 1.219f, 0.155f, 0.447f, 1.523f, 3.735f, 0.195f, 4.837f, 0.469f, 0.589f, 0.549f},
+    {128, 4, 1, false, 0.102f, 1.262f, 0.183f, 0.362f, 1.97f, 4.089f, 0.321f, 5.474f, 0.885f, 0.673f, 0.34f},
+    {192, 2, 1, false, 0.0f, 1.399f, 0.223f, 0.366f, 2.755f, 5.209f, 0.278f, 6.444f, 1.052f, 0.533f, 0.0f},
+    {256, 2, 1, false, 0.0f, 0.815f, 0.254f, 0.44f, 3.551f, 6.56f, 0.248f, 7.881f, 1.615f, 0.596f, 0.213f}};
 
 static bool admissible(const TileCost& t, int M) { return t.NT <= 16 || t.NT < 2 * M; }   // not half of the tile or more padding
 

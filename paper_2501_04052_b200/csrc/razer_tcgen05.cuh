@@ -314,7 +314,7 @@ static inline EncodeTiledFn encode_fn() {
 // razer_gemm_fp4.cu).  `start`: a launch, growing by `busy` with a CTA on every SM.  `chunk`: one 64-column chunk of a 128-row tile; it
 // grows by `load` likewise.  `whole`: storing a tile; `cut`, `part`: combining one cut evenly among several CTAs, and each CTA of it;
 // `stripe`: the two partial tiles of a stripe, `extra`: each CTA beyond three that shares one.  `late`: a grid of more than half of the
-// SMs, whose successor cannot start up beside it; `spread`: the same with a tile or more to every CTA, the more of them there are.
+// SMs, whose successor cannot start up beside it (with several tiles to a CTA that start-up is not what is waited for); `spread`: the same with a tile or more to every CTA, the more of them there are.
 struct TileCost { int NT, CH, CHX; bool table; float start, busy, chunk, load, whole, cut, part, stripe, extra, late, spread; };
 
 // The cheapest grid for `tiles` output tiles of `steps` items: every tile on one CTA, every tile cut evenly among 2 .. 16 CTAs, or
@@ -325,7 +325,7 @@ static inline float best_grid(const TileCost& t, long long tiles, int steps, int
   auto consider = [&](long long g, int tiles_per_cta, int cut) {            // whole tiles per CTA, or CTAs per tile, or stripes (0, 0)
     const float busy = (float)g / sms;
     float c = t.start + t.busy * busy + (float)((total + g - 1) / g * t.CH) * t.chunk * (1.0f + t.load * busy);
-    if (2 * g > sms) c += t.late;
+    if (2 * g > sms || tiles_per_cta > 1) c += t.late;
     if (tiles_per_cta > 0) {
       c += t.whole * (0.6f + 0.4f * tiles_per_cta) + (2 * g > sms ? t.spread * (busy - 0.5f) : 0.0f);
     } else if (cut > 0) {
