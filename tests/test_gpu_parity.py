@@ -314,6 +314,19 @@ def test_gemm_stripes_and_several_whole_tiles(b, M, N, K):
     _check_matmul(b, b.razer_gemm, desc, packed, codes, scales, 0.002, x, rows=rows_with_edge_tiles(N, 128, 80))
 
 
+@pytest.mark.parametrize("M,N,K", [(10, 68, 2272), (10, 20463, 80), (27, 17668, 64), (30, 3999, 10992), (498, 132, 3200), (19, 19597, 80),
+                                   (58, 6003, 1008), (37, 21233, 64), (50, 3999, 8208), (80, 5003, 1008), (454, 157, 3184), (124, 9731, 4112),
+                                   (255, 21336, 64), (197, 5385, 64), (194, 3379, 3168)])
+def test_gemm_more_token_tiles_and_partitions(b, M, N, K):
+    """Tiles and partitions that the sizes above leave out: 16 and 32 tokens decoded in registers with cut tiles and with several tiles to a CTA, by
+    table likewise, 64 to 256 tokens with whole, cut and several tiles, 128 in stripes."""
+    codes, scales = inputs.random_codes(N, K, seed=M, zero_block_frac=0.02)
+    codes, scales = codes.numpy(), scales.numpy()
+    desc, packed = _pack(b, codes, scales, 0.002)
+    x = inputs.activations(M, K, 77, outlier_channel_frac=0.01)
+    _check_matmul(b, b.razer_gemm, desc, packed, codes, scales, 0.002, x, rows=rows_with_edge_tiles(N, 96, 76))
+
+
 def test_gemm_sixteen_tokens_keep_three_partial_sums_apart(b):
     """Up to 16 tokens, three items of 256 columns in a row are summed apart and added up once per tile (a third of the
     additions in a chain).  All weights are 1, and a tile's four items contribute 2^30, 1, 1 + m and -2^30: FP32 sums in one chain
