@@ -14,6 +14,8 @@ from ctypes import POINTER, c_char_p, c_float, c_int, c_int32, c_size_t, c_void_
 
 import torch
 
+from .build import call_path
+
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.environ.get("RAZER_LIB") or os.path.join(_HERE, "librazer.so")   # RAZER_LIB: load another build of the library
 
@@ -103,19 +105,27 @@ else:
         return torch.cuda.current_stream().cuda_stream
 
 
-# The compiled way of a plain matmul call (csrc/razer_call.cpp); without it everything goes through ctypes.
+# The compiled way of a plain matmul call (csrc/razer_call.cpp); without it everything goes through ctypes.  It has torch's and the
+# interpreter's layouts built in: only the file built for these two is loaded (build.call_path).  call_route() says which way calls go and why.
 def _load_call():
-    path = os.path.join(_HERE, "razer_call.so")
+    path = call_path(torch.__version__)
     try:
         spec = importlib.util.spec_from_file_location("razer_call", path)
         module = importlib.util.module_from_spec(spec)
         spec.loader.exec_module(module)
-        return module
-    except (ImportError, OSError):                       # not built, or for another torch or interpreter
-        return None
+        return module, f"compiled ({path})"
+    except (ImportError, OSError) as e:                  # not built
+        return None, f"ctypes ({e})"
 
 
-_call = _load_call()
+_call, _route = _load_call()
+
+
+def call_route() -> str:
+    """How razer_gemv, razer_gemm and razer_gemv_host reach the library for plain arguments."""
+    return _route
+
+
 _GEMV, _GEMM, _GEMV_HOST = (ctypes.cast(f, c_void_p).value for f in (_lib.razer_gemv, _lib.razer_gemm, _lib.razer_gemv_host))
 
 

@@ -86,3 +86,25 @@ def test_a_compiled_part_that_no_longer_builds_is_not_left_behind(tree):
     os.utime(tree.path("csrc", "razer_call.cpp"), (later, later))
     assert tree.build().returncode == 0
     assert tree.calls() == ["CXX"] and tree.files(".so") == ["librazer.so"]
+
+
+def test_compiled_part_is_for_one_torch_and_one_interpreter(tree, monkeypatch):
+    """Its file says what it was built for; where that is not what is installed it is not loaded, and build() makes another one."""
+    import sysconfig
+
+    import torch
+    from paper_2501_04052_b200 import binding as b
+    assert sysconfig.get_config_var("SOABI") in build.call_path() and build.call_path(torch.__version__) == build.call_path()
+    assert len({build.call_path(v) for v in ("2.11.0+cu128", "2.11.0+cpu", "2.12.0+cu128", "none")}) == 4
+    assert b._load_call()[0] is not None and b.call_route().startswith("compiled")
+    monkeypatch.setattr(torch, "__version__", "0.0.1")
+    module, route = b._load_call()
+    assert module is None and route.startswith("ctypes") and "torch-0_0_1" in route
+    # a file for another torch: built anew, the other one gone
+    assert tree.build().returncode == 0
+    mine, = (f for f in tree.files(".so") if f.startswith("razer_call."))
+    other = tree.path("razer_call.cpython-399-x86_64-linux-gnu.torch-9_9_9.so")
+    os.rename(tree.path(mine), other)
+    tree.calls()
+    assert tree.build().returncode == 0 and tree.calls() == ["CXX"]
+    assert os.path.exists(tree.path(mine)) and not os.path.exists(other)
