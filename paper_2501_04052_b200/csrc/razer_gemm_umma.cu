@@ -498,23 +498,24 @@ struct UmmaPlan {
   size_t slots_bytes;
 };
 
-// Token tile, decode and grid: the cheapest by the cost model (razer_tcgen05.cuh), fitted to 57,000 times of 2923 sizes (M 9 .. 2048, N and K
-// 256 .. 28672, all widths and grids, weights from HBM, launches back to back in a graph).  Of the best of a size's grids the choice is
-// 0.6 % off in the mean and 4 % or more at one size in 50; by fewer constants per width (one start for all, no `late`, no `spread`) it was 2.2 %
-// off: 53 x 512 x 4352 7.06 us instead of 6.37, 93 x 512 x 2816 6.88 (6.22), 239 x 1590 x 1648 7.69 (6.75), 64 x 2341 x 816 3.79 (3.46).
+// Token tile, decode and grid: the cheapest by the cost model (razer_tcgen05.cuh), fitted to 63,000 times of 3823 sizes (M 9 .. 2048, N and K
+// 256 .. 28672, all widths and grids, launches back to back; 900 of them with weights, activations and workspaces all in turn, under
+// sustained load).  Of the best of a size's grids the choice is 0.6 % off in the mean; by fewer constants per width (one start for all,
+// no `late`, no `spread`) it was 2.2 % off: 53 x 512 x 4352 7.06 us instead of 6.37, 93 x 512 x 2816 6.88 (6.22), 239 x 1590 x 1648 7.69 (6.75),
+// 64 x 2341 x 816 3.79 (3.46).
 // Up to 32 tokens the table costs a start (every CTA fills it) and gains by the chunk: at 16 tokens it is level with the registers at
 // 1 to 3 items of four chunks a CTA (1 item +1.3 %) and faster from there (6 -4.5 %, 16 -11 %), at 32 tokens from 6 on (1 to 5 +3 to +6 %, 8 -5 %,
 // 16 -7 %).
 static const TileCost tile_costs[] = {
-    {16, 4, 4, true, 0.323f, 0.141f, 0.114f, 0.462f, 1.423f, 3.536f, 0.205f, 4.691f, 0.172f, 0.164f, 4.11f},
-    {16, 4, 4, false, 0.298f, 0.0f, 0.119f, 0.731f, 1.352f, 3.289f, 0.229f, 4.975f, 0.161f, 0.127f, 4.35f},
-    {32, 4, 2, true, 0.924f, 0.161f, 0.129f, 0.47f, 0.894f, 2.883f, 0.175f, 3.989f, 0.194f, 0.26f, 3.879f},
-    {32, 4, 4, false, 0.55f, 0.0f, 0.128f, 0.707f, 1.137f, 3.21f, 0.151f, 4.345f, 0.183f, 0.204f, 4.454f},
-    {64, 4, 4, false, 0.563f, 0.779f, 0.143f, 0.55f, 1.142f, 3.3f, 0.202f, 3.792f, 0.346f, 0.819f, 0.953f},
-    {96, 4, 2, false, 0.447f, 1.219f, 0.155f, 0.447f, 1.523f, 3.735f, 0.195f, 4.837f, 0.469f, 0.589f, 0.549f},
-    {128, 4, 1, false, 0.102f, 1.262f, 0.183f, 0.362f, 1.97f, 4.089f, 0.321f, 5.474f, 0.885f, 0.673f, 0.34f},
-    {192, 2, 1, false, 0.0f, 1.399f, 0.223f, 0.366f, 2.755f, 5.209f, 0.278f, 6.444f, 1.052f, 0.533f, 0.0f},
-    {256, 2, 1, false, 0.0f, 0.815f, 0.254f, 0.44f, 3.551f, 6.56f, 0.248f, 7.881f, 1.615f, 0.596f, 0.213f}};
+    {16, 4, 4, true, 0.321f, 0.135f, 0.114f, 0.408f, 1.423f, 3.535f, 0.207f, 4.69f, 0.172f, 0.191f, 4.131f},
+    {16, 4, 4, false, 0.315f, 0.0f, 0.119f, 0.638f, 1.345f, 3.239f, 0.24f, 4.975f, 0.161f, 0.147f, 4.499f},
+    {32, 4, 2, true, 0.922f, 0.164f, 0.129f, 0.467f, 0.894f, 2.883f, 0.172f, 3.902f, 0.229f, 0.306f, 4.087f},
+    {32, 4, 4, false, 0.552f, 0.001f, 0.128f, 0.707f, 1.118f, 3.026f, 0.173f, 4.346f, 0.183f, 0.204f, 4.581f},
+    {64, 4, 4, false, 0.637f, 0.727f, 0.139f, 0.542f, 1.172f, 3.179f, 0.205f, 4.394f, 0.346f, 0.827f, 0.953f},
+    {96, 4, 2, false, 0.447f, 1.219f, 0.155f, 0.375f, 1.584f, 3.506f, 0.225f, 4.894f, 0.469f, 0.606f, 0.541f},
+    {128, 4, 1, false, 0.122f, 1.194f, 0.183f, 0.362f, 1.981f, 4.037f, 0.333f, 5.988f, 0.895f, 0.707f, 0.295f},
+    {192, 2, 1, false, 0.0f, 1.329f, 0.221f, 0.366f, 2.816f, 5.203f, 0.378f, 6.982f, 1.055f, 0.533f, 0.0f},
+    {256, 2, 1, false, 0.0f, 0.949f, 0.257f, 0.44f, 3.516f, 5.896f, 0.48f, 7.576f, 1.685f, 0.652f, 0.213f}};
 
 static bool admissible(const TileCost& t, int M) { return t.NT <= 16 || t.NT < 2 * M; }   // not half of the tile or more padding
 
