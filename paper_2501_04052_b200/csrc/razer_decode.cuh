@@ -1,6 +1,7 @@
-// Register-level decode of packed RaZeR blocks to bf16 pairs: the tcgen05 matmul kernel, and what the others share of it.
+// Decode of packed RaZeR blocks to bf16 pairs for the tcgen05 matmul kernel, in registers and by table, and what the other kernels share
+// of it.
 //
-// Per pair of elements, with no comparison and no conversion instruction: the stored nibble
+// In registers, per pair of elements, with no comparison and no conversion instruction: the stored nibble
 // is isolated in both 16-bit halves of the word, one integer multiply-add drops two shifted
 // copies of it, one logic op keeps sign -> bit 15 and E1 E0 M -> bits 8:6 (a bf16 pattern worth
 // value x 2^-126, subnormal for 0.5) and ORs in the special value, which one fused

@@ -6,14 +6,14 @@
 // (128 weight rows = 128 TMEM lanes), the activation tile is the B operand (NT tokens,
 // K-major in shared memory, 128-byte swizzle, written by TMA), the accumulator D[128 x NT]
 // lives in TMEM.  Weights never exist as bf16 in shared or global memory: TMA boxes bring the packed 4.5-bit chunks into
-// shared memory, the "dequant" warps (thread = weight row) decode one 16-element block at a time in registers and write the
-// bf16 pairs straight into TMEM with tcgen05.st, and the MMA reads A from TMEM.
+// shared memory, the "dequant" warps (thread = weight row) decode a chunk of 64 columns at a time, in registers or by table, and write
+// the bf16 pairs straight into TMEM with tcgen05.st, and the MMA reads A from TMEM.
 //
 // Warp roles (96 + 32 * NDW threads): warp 0 = weight producer, warp 1 = TMEM owner + MMA issuer, warps 2 .. 1 + NDW = dequant
 // and epilogue, the last = activation producer.  A warp reaches only the TMEM lanes 32 * (warp % 4) .. + 31; four warps form a
 // group that decodes an item, and the groups take the items in turn.
 //
-// Both decodes are described in razer_decode.cuh.  Up to 32 tokens by table: 16 x 8192 x 28672 41.3 (registers) -> 36.0 us, 16 x 4096 x 11008
+// Both decodes are described in razer_decode.cuh.  Up to 32 tokens by table where a launch is long enough (make_plan): 16 x 8192 x 28672 41.3 (registers) -> 36.0 us, 16 x 4096 x 11008
 // 14.2 -> 13.1, 32 x 28672 x 8192 43.2 -> 38.7.  From 64 tokens on in registers: the table takes 64 KB from the rings, and its loads
 // meet the activations' in shared memory (64 x 8192 x 28672 45.3 us in registers, 49.7 by table, 48 half and half).
 //

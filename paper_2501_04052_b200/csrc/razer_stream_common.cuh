@@ -20,7 +20,7 @@ constexpr int EW = 2;                               // epilogue warps, each with
 constexpr int THREADS = 32 * (CW + EW + 2);         // + a producer warp each for weights and activations
 constexpr int MAX_STAGES = 8;
 constexpr int MAX_M = 8;
-constexpr int LUT_BYTES = 65536;                    // [weight byte][special value][lane]: two elements as bf16x2
+constexpr int LUT_BYTES = PAIR_TABLE_BYTES;         // [weight byte][special value][lane]: two elements as bf16x2 (here not times 2^-126)
 constexpr int SCALES_BYTES = 128 * 32 * 4;                  // [scale byte without the select bit][lane]: +-scale as bf16x2
 constexpr int MAX_ROWS = 64;
 constexpr int SLOT_FLOATS = MAX_ROWS * MAX_M;       // one CTA's partial result of a unit
