@@ -316,10 +316,10 @@ def test_gemm_stripes_and_several_whole_tiles(b, M, N, K):
 
 @pytest.mark.parametrize("M,N,K", [(10, 68, 2272), (10, 20463, 80), (27, 17668, 64), (30, 3999, 10992), (498, 132, 3200), (19, 19597, 80),
                                    (58, 6003, 1008), (37, 21233, 64), (50, 3999, 8208), (80, 5003, 1008), (454, 157, 3184), (124, 9731, 4112),
-                                   (255, 21336, 64), (197, 5385, 64), (194, 3379, 3168)])
+                                   (255, 21336, 64), (197, 5385, 64), (194, 3379, 3168), (20, 11003, 1040), (129, 19010, 528), (250, 4071, 8208)])
 def test_gemm_more_token_tiles_and_partitions(b, M, N, K):
     """Tiles and partitions that the sizes above leave out: 16 and 32 tokens decoded in registers with cut tiles and with several tiles to a CTA, by
-    table likewise, 64 to 256 tokens with whole, cut and several tiles, 128 in stripes."""
+    table likewise, 64 to 256 tokens with whole, cut and several tiles, 128 and 192 in stripes."""
     codes, scales = inputs.random_codes(N, K, seed=M, zero_block_frac=0.02)
     codes, scales = codes.numpy(), scales.numpy()
     desc, packed = _pack(b, codes, scales, 0.002)
