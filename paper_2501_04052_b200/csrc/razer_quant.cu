@@ -19,7 +19,7 @@
 // A block that the short form cannot take (a NaN or an infinity, a step outside 2^-60 .. 2^60, a quotient beyond 2^100) goes
 // through the plain procedure.  Measured on B200, everything in this file included: razer_quant_act of 2048 x 8192 54.2 -> 27.2 us,
 // razer_quant_act_fp4 (no special value) 58.1 -> 19.6; razer_quant_weight of 11008 x 4096 256.6 -> 94.6, of which the maximum 32, and
-// by gains instead of error sums (quant_weight_quick_kernel) 76.4.
+// by gains instead of error sums (quant_weight_quick_kernel) 71.3.
 #include <algorithm>
 
 #include "razer_common.cuh"
@@ -849,8 +849,8 @@ __device__ __forceinline__ uint32_t to_e4m3(float t) {                // nearest
 //
 // Blocks left undecided (candidates too close, scaled elements beyond quick_max, values that the short form cannot take) are put down by
 // their warp and taken by quant_weight_block, a thread each, as soon as there are 32; a CTA's warps share out what is left at the end.
-// Few blocks of continuous weights are, many of weights that lie on a coarse grid (FP8, INT8, INT4 checkpoints) and nearly all at a
-// given scale a hundred times too small.
+// Few blocks of continuous weights are, many of weights that lie on a coarse grid (FP8, INT8, INT4 checkpoints), and nearly all large blocks at
+// a given scale a hundred times too small.
 //
 // Bound by instruction issue.  11008 x 4096 at a given scale, us in graph replays, quant_weight_kernel / this with undecided blocks walked
 // one element at a time by their whole warp and blocks beyond 9.4 steps by the plain procedure / this:
